@@ -473,6 +473,8 @@ attn_redo_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant_
                  const AttnParams p, const int* __restrict__ redo_list) {
   using L = AttnSmem<BLK, D>;
   extern __shared__ __align__(1024) uint8_t smem[];
+  pdl_wait();
+  pdl_launch();
   const int n_redo = p.status->redo_count;
   const int warp = threadIdx.x >> 5;
   for (int k = blockIdx.x; k < n_redo; k += gridDim.x) {
@@ -551,6 +553,8 @@ __global__ void __launch_bounds__(128) merge_splits_kernel(const float* __restri
                                                            int64_t o_sb, int64_t o_sh, int64_t o_sn,
                                                            float* __restrict__ lse, const int32_t* __restrict__ row_map,
                                                            int row_map_stride, int n_out) {
+  pdl_wait();
+  pdl_launch();
   merge_splits_rows<BLK, D>(blockIdx.x, threadIdx.x, part_o, part_lse2, n_split, NQT, Nq, H, total_rows, o, o_sb, o_sh,
                             o_sn, lse, row_map, row_map_stride, n_out);
 }

@@ -185,6 +185,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
+  pdl_wait();
+  pdl_launch();
 
   // A wait that gives up when the CTA has been stopped (a time limit was reached somewhere).
   auto wait_or_stop = [&](int bar, uint32_t parity, int where, int tag) -> bool {
@@ -278,14 +280,20 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     // items ahead of the one whose V tiles it is loading.
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     int pub_item = -1, pub_cnt = 0;
+    bool first = true;
     // takes the next valid work item off the global queue and publishes it as item m of this CTA
     auto publish = [&](int m) -> bool {
       const int slot = m % kPRing;
       if (m >= kPRing && !wait_all(ITEM_EMPTY + slot, ((m / kPRing) - 1) & 1, kPersistItemEmpty, m)) return false;
       while (true) {
-        int id = 0;
-        if (lane == 0) id = atomicAdd(&p.status->next_item, 1);
-        id = __shfl_sync(FULLM, id, 0);
+        // The CTA's first item is its own index, the others come off the queue behind those of the whole grid: with
+        // one item or less per CTA, a CTA that is a little early must not take a second one from a late CTA.
+        int id = blockIdx.x;
+        if (!first) {
+          if (lane == 0) id = gridDim.x + atomicAdd(&p.status->next_item, 1);
+          id = __shfl_sync(FULLM, id, 0);
+        }
+        first = false;
         if (id >= n_items) {
           pub_item = -1;
           pub_cnt = 0;

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/avsa.h"
 
 namespace avsa {
@@ -29,8 +31,34 @@ __device__ __forceinline__ void report_status(StatusRecord* st, int code, int wh
   }
 }
 
+// ------------------------------------------------------------------------------------ programmatic dependent launch
+// Every kernel of the library's calls is launched as a programmatic dependent of the kernel before it on the stream:
+// it is set up while that one drains, waits (pdl_wait) before it touches memory that an earlier kernel may read or
+// write, and then lets its own successor be set up (pdl_launch).  A grid retires only after its own wait, so whatever
+// is ordered behind it is ordered behind everything before it as well.  Between ordinary launches the GPU idles
+// 1.5-4 us each; the smallest layer-step (eleven launches) took 33 us with them.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Resets the status record at the start of every call (first node of the call's launch sequence).
 static __global__ void clear_status_kernel(StatusRecord* st) {
+  pdl_wait();
+  pdl_launch();
   st->code = 0;
   st->where = 0;
   st->item = 0;

@@ -85,6 +85,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
     prefetch_tmap(&tmq);
     prefetch_tmap(&tmk);
   }
+  pdl_wait();
   // negated log2-domain LSEs (one packed FMA then gives s*c - lse2); queries beyond Nq get -inf: exp2 = 0
   // (straight from the splits' partial LSEs when pass 1 left its merge for later: the same maximum-and-sum as the
   // merge kernel, in the log2 domain)
@@ -242,6 +243,9 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   }
   tc_fence_before();
   __syncthreads();
+  // only now: staged earlier, the small CTAs of the next grid crowd onto the SMs that this grid leaves idle
+  // (128 of 148 used, ltx shape: the head sum behind it took 43 us instead of 17)
+  pdl_launch();
   if (warp == 2) tmem_dealloc(tmem, 512);
 }
 
@@ -328,6 +332,7 @@ colsum_rev_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
+  pdl_wait();
 
   auto wait_or_abort = [&](int bar, uint32_t parity, int where, int aux) -> bool {
     if (mbar_try_wait(BAR(bar), parity)) return true;
@@ -442,6 +447,7 @@ colsum_rev_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
+  pdl_launch();      // not earlier, as in colsum_kernel
   if (warp == 2) tmem_dealloc(tmem, 256);
 }
 
@@ -449,6 +455,8 @@ colsum_rev_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant
 __global__ void __launch_bounds__(256) lse_to_log2_kernel(const float* __restrict__ lse, int Nq, int Nq_pad, int BH,
                                                           float* __restrict__ lse2) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+  pdl_wait();
+  pdl_launch();
   if (idx >= static_cast<int64_t>(BH) * Nq_pad) return;
   const int bh = static_cast<int>(idx / Nq_pad), i = static_cast<int>(idx % Nq_pad);
   lse2[idx] = i < Nq ? -lse[static_cast<int64_t>(bh) * Nq + i] * 1.4426950408889634f : -INFINITY;
@@ -481,6 +489,8 @@ __device__ __forceinline__ void head_sum_keys(int block, int tid, const float* _
 }
 __global__ void __launch_bounds__(256) head_sum_kernel(const float* __restrict__ partial, int NCH, int B, int H,
                                                        int Nk, float beta, float gamma, float* __restrict__ scores) {
+  pdl_wait();
+  pdl_launch();
   head_sum_keys(blockIdx.x, threadIdx.x, partial, NCH, B, H, Nk, beta, gamma, scores);
 }
 
@@ -495,6 +505,8 @@ __global__ void __launch_bounds__(256) cross_finalize_kernel(int hs_blocks, cons
                                                              int Nq, int total_rows, __nv_bfloat16* __restrict__ o,
                                                              int64_t o_sb, int64_t o_sh, int64_t o_sn,
                                                              float* __restrict__ lse) {
+  pdl_wait();
+  pdl_launch();
   if (static_cast<int>(blockIdx.x) < hs_blocks) {
     head_sum_keys(blockIdx.x, threadIdx.x, partial, NCH, B, H, Nk, beta, gamma, scores);
   } else {
@@ -512,6 +524,8 @@ __global__ void __launch_bounds__(256) head_sum_wide_kernel(const float* __restr
                                                             int Nk, float beta, float gamma, float* __restrict__ scores) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_launch();
   if (idx >= static_cast<int64_t>(B) * Nk) return;
   const int b = static_cast<int>(idx / Nk), i = static_cast<int>(idx % Nk);
   const int J = H * NCH;
@@ -595,15 +609,15 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
   float* part_lse = reinterpret_cast<float*>(ws + c.off_part_lse);
   float* lse = lse_out != nullptr ? lse_out : reinterpret_cast<float*>(ws + c.off_lse);
   float* partial = reinterpret_cast<float*>(ws + c.off_partial);
-  clear_status_kernel<<<1, 1, 0, st>>>(status);
+  if (launch_pdl(clear_status_kernel, 1, 1, 0, st, status) != cudaSuccess) return AVSA_ERR_CUDA;
   bool merge_late = false;
   // ---- pass 1
   {
-    using L = AttnSmem<BLK, D>;
     CUtensorMap tq, tk, tv;
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tv, v.ptr, B, H, Nk, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
+    using L = AttnSmem<BLK, D>;
     using LP = PersistSmem<BLK, D>;
     AttnParams prm = {};
     prm.part_o = part_o;
@@ -633,9 +647,12 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
       if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE_DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                L::kTotal) != cudaSuccess)
         return AVSA_ERR_CUDA;
-      attn_persist_kernel<BLK, D, MODE_RANGE_DIRECT><<<pgrid, kAttnThreads, LP::kTotal, st>>>(
-          tq, tk, tv, to, prm, redo, nullptr, static_cast<int>(items));
-      attn_redo_kernel<BLK, D, MODE_RANGE_DIRECT><<<pgrid, kAttnThreads, L::kTotal, st>>>(tq, tk, tv, to, prm, redo);
+      if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE_DIRECT>, pgrid, kAttnThreads, LP::kTotal, st, tq, tk, tv, to, prm,
+                     redo, nullptr, static_cast<int>(items)) != cudaSuccess)
+        return AVSA_ERR_CUDA;
+      if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE_DIRECT>, pgrid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo) !=
+          cudaSuccess)
+        return AVSA_ERR_CUDA;
     } else {
       if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                LP::kTotal) != cudaSuccess)
@@ -643,16 +660,20 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
       if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                L::kTotal) != cudaSuccess)
         return AVSA_ERR_CUDA;
-      attn_persist_kernel<BLK, D, MODE_RANGE><<<pgrid, kAttnThreads, LP::kTotal, st>>>(tq, tk, tv, tq, prm, redo, nullptr,
-                                                                                       static_cast<int>(items));
-      attn_redo_kernel<BLK, D, MODE_RANGE><<<pgrid, kAttnThreads, L::kTotal, st>>>(tq, tk, tv, tq, prm, redo);
+      if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, pgrid, kAttnThreads, LP::kTotal, st, tq, tk, tv, tq, prm, redo,
+                     nullptr, static_cast<int>(items)) != cudaSuccess)
+        return AVSA_ERR_CUDA;
+      if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, pgrid, kAttnThreads, L::kTotal, st, tq, tk, tv, tq, prm, redo) !=
+          cudaSuccess)
+        return AVSA_ERR_CUDA;
       merge_late = scores != nullptr && !c.reverse;      // then the merge rides in the call's last grid
       if (!merge_late) {
         const int total_rows = B * H * Nq;
         constexpr int RPB = 128 / (D / 4);
-        merge_splits_kernel<BLK, D><<<(total_rows + RPB - 1) / RPB, 128, 0, st>>>(
-            part_o, part_lse, c.n_split, c.NQT, Nq, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h,
-            q.stride_n, lse, nullptr, 0, Nq);
+        if (launch_pdl(merge_splits_kernel<BLK, D>, (total_rows + RPB - 1) / RPB, 128, 0, st, part_o, part_lse, c.n_split,
+                       c.NQT, Nq, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h, q.stride_n, lse,
+                       nullptr, 0, Nq) != cudaSuccess)
+          return AVSA_ERR_CUDA;
       }
     }
   }
@@ -661,7 +682,9 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     using L = ColsumRevSmem<D>;
     float* lse2 = reinterpret_cast<float*>(ws + c.off_lse2);
     const int64_t n2 = static_cast<int64_t>(B) * H * c.NQC * 128;
-    lse_to_log2_kernel<<<static_cast<unsigned>((n2 + 255) / 256), 256, 0, st>>>(lse, Nq, c.NQC * 128, B * H, lse2);
+    if (launch_pdl(lse_to_log2_kernel, static_cast<unsigned>((n2 + 255) / 256), 256, 0, st, lse, Nq, c.NQC * 128, B * H,
+                   lse2) != cudaSuccess)
+      return AVSA_ERR_CUDA;
     CUtensorMap tq, tk;
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
@@ -679,10 +702,12 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     rp.n_range = c.rev_ranges;
     rp.chunks_per_range = c.rev_cpr;
     rp.scale_log2 = scale * 1.4426950408889634f;
-    colsum_rev_kernel<D><<<dim3(c.rev_ranges, H, B), kColThreads, smem, st>>>(tq, tk, rp);
+    if (launch_pdl(colsum_rev_kernel<D>, dim3(c.rev_ranges, H, B), kColThreads, smem, st, tq, tk, rp) != cudaSuccess)
+      return AVSA_ERR_CUDA;
     const int64_t n = static_cast<int64_t>(B) * Nk;
-    head_sum_wide_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, st>>>(partial, c.rev_slots, B, H, Nk, beta, gamma,
-                                                                            scores);
+    if (launch_pdl(head_sum_wide_kernel, static_cast<unsigned>((n + 7) / 8), 256, 0, st, partial, c.rev_slots, B, H, Nk, beta,
+                   gamma, scores) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   }
   // ---- pass 2, queries resident (at most 512 queries)
   if (scores != nullptr && !c.reverse) {
@@ -711,18 +736,20 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     cp.tiles_per_range = c.tpr;
     cp.scale_log2 = scale * 1.4426950408889634f;
     dim3 grid(c.n_range, H, B);
-    colsum_kernel<D><<<grid, kColThreads, smem, st>>>(tq, tk, cp);
+    if (launch_pdl(colsum_kernel<D>, grid, kColThreads, smem, st, tq, tk, cp) != cudaSuccess) return AVSA_ERR_CUDA;
     const int64_t n = static_cast<int64_t>(B) * Nk;
     const int hs_blocks = static_cast<int>((n + 255) / 256);
     if (merge_late) {
       const int total_rows = B * H * Nq;
       constexpr int RPB = 128 / (D / 4);
       const int merge_blocks = ((total_rows + RPB - 1) / RPB + 1) / 2;
-      cross_finalize_kernel<BLK, D><<<hs_blocks + merge_blocks, 256, 0, st>>>(
-          hs_blocks, partial, c.NCH, B, H, Nk, beta, gamma, scores, part_o, part_lse, c.n_split, c.NQT, Nq, total_rows,
-          static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h, q.stride_n, lse);
+      if (launch_pdl(cross_finalize_kernel<BLK, D>, hs_blocks + merge_blocks, 256, 0, st, hs_blocks, partial, c.NCH, B, H, Nk,
+                     beta, gamma, scores, part_o, part_lse, c.n_split, c.NQT, Nq, total_rows, static_cast<__nv_bfloat16*>(o),
+                     q.stride_b, q.stride_h, q.stride_n, lse) != cudaSuccess)
+        return AVSA_ERR_CUDA;
     } else {
-      head_sum_kernel<<<hs_blocks, 256, 0, st>>>(partial, c.NCH, B, H, Nk, beta, gamma, scores);
+      if (launch_pdl(head_sum_kernel, hs_blocks, 256, 0, st, partial, c.NCH, B, H, Nk, beta, gamma, scores) != cudaSuccess)
+        return AVSA_ERR_CUDA;
     }
   }
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restri
   constexpr int RPP = 256 / TPR;      // rows per pass
   __shared__ float part[RPP][D + 4];
   // lets the block-score grid be staged while this one drains (it waits for this grid before it reads)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_launch();
 
   const int nb = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
   const int b = bh / H, h = bh % H;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restri
   // kernels behind (which wait for their predecessor only); by then the select is long done, and no
   // earlier CTA ever holds an SM slot waiting.
   const unsigned lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  if (lin + kPoolTailCtas >= gridDim.x * gridDim.y * gridDim.z) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (lin + kPoolTailCtas >= gridDim.x * gridDim.y * gridDim.z) pdl_wait();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -184,8 +184,9 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
   uint8_t* ptok = prot_tok + static_cast<int64_t>(b) * N;
   uint8_t* pblk = prot_blk + static_cast<int64_t>(b) * NB;
   // nothing launched next on the stream depends on this kernel until the list emission, so let the
-  // pooling kernel start right away (programmatic dependent launch)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // pooling kernel start right away (but not before this grid's own predecessors are done: pooling does not wait)
+  pdl_wait();
+  pdl_launch();
   if (b == 0 && tid == 0) {
     status->code = 0;
     status->where = 0;
@@ -364,7 +365,8 @@ __global__ void __launch_bounds__(128) row_select_kernel(const float* __restrict
                                                          int protect_cols, int total_rows, int32_t* __restrict__ col_idx,
                                                          int32_t* __restrict__ col_cnt) {
   __shared__ int all_bins[4][256];
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the block flags come from the kernel before
+  pdl_wait();   // the block flags come from the kernel before
+  pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 4 + warp;      // row = (b*H + h)*NB + qb
   if (row >= total_rows) return;
@@ -411,8 +413,8 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   static_assert(NT == 4, "the key ring holds two tile pairs per 16-channel group");
   // Staged behind the pooling grid (programmatic dependent launch) and waits for it here; the pooling grid in
   // turn retires only after the token select, so the block flags are final too.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch();
+  pdl_wait();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t = lane & 3;
   const int bh = blockIdx.y, i0 = blockIdx.x * kStripRows;
@@ -540,6 +542,8 @@ __global__ void __launch_bounds__(256) block_sum_kernel(const float* __restrict_
                                                         float* __restrict__ bsum) {
   const int b = blockIdx.y, lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  pdl_wait();
+  pdl_launch();
   if (j >= NB) return;
   const float* s = scores + static_cast<int64_t>(b) * N;
   const int lo = j * blk, hi = min(N, lo + blk);
@@ -554,6 +558,8 @@ __global__ void __launch_bounds__(256) block_sum_kernel(const float* __restrict_
 __global__ void __launch_bounds__(256) expand_blocks_kernel(const uint8_t* __restrict__ prot_blk, int N, int blk, int NB,
                                                             int64_t total, uint8_t* __restrict__ prot_tok) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+  pdl_wait();
+  pdl_launch();
   if (idx >= total) return;
   const int64_t b = idx / N;
   const int i = static_cast<int>(idx % N);
@@ -565,29 +571,28 @@ __global__ void __launch_bounds__(256) expand_blocks_kernel(const uint8_t* __res
 // while the pooling grid drains, took thread slots from its last CTAs and the call came out slower (0.118 against
 // 0.103 ms on the Ovi-class shape).
 template <int D, int KPL, int WARPS>
-static cudaError_t launch_score_select_as(cudaLaunchConfig_t& cfg, int NB, const float* qbar, const float* kbar,
+static cudaError_t launch_score_select_as(cudaStream_t st, int B, int NB, const float* qbar, const float* kbar,
                                           float* bs, const uint8_t* pblk, int H, float scale, int k_keep, int pr, int pc,
                                           int32_t* col_idx, int32_t* col_cnt) {
-  cfg.blockDim = dim3(WARPS * 32, 1, 1);
-  cfg.dynamicSmemBytes = (static_cast<size_t>(2 * kStripRows) * (D + 4) + static_cast<size_t>(kStripRows) * strip_pitch<D>(NB)) *
+  const size_t smem = (static_cast<size_t>(2 * kStripRows) * (D + 4) + static_cast<size_t>(kStripRows) * strip_pitch<D>(NB)) *
                              sizeof(float) + WARPS * 256 * sizeof(int) + WARPS * 4 * 2 * 32 * 16;
   // always the same limit (the largest NB the call accepts), so concurrent callers never race on its value
   constexpr int kMaxSmem = (2 * kStripRows * (D + 4) + kStripRows * strip_pitch<D>(kMaxBlocksPerRow)) * 4 + WARPS * 256 * 4 + WARPS * 4 * 2 * 32 * 16;
   cudaError_t e = cudaFuncSetAttribute(score_select_kernel<D, KPL, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMaxSmem);
   if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, score_select_kernel<D, KPL, WARPS>, qbar, kbar, bs, pblk, H, NB, scale, k_keep, pr, pc,
-                            col_idx, col_cnt);
+  return launch_pdl(score_select_kernel<D, KPL, WARPS>, dim3((NB + kStripRows - 1) / kStripRows, B * H, 1), WARPS * 32, smem, st,
+                    qbar, kbar, bs, pblk, H, NB, scale, k_keep, pr, pc, col_idx, col_cnt);
 }
 template <int D>
-static cudaError_t launch_score_select(cudaLaunchConfig_t& cfg, int NB, const float* qbar, const float* kbar, float* bs,
+static cudaError_t launch_score_select(cudaStream_t st, int B, int NB, const float* qbar, const float* kbar, float* bs,
                                        const uint8_t* pblk, int H, float scale, int k_keep, int pr, int pc,
                                        int32_t* col_idx, int32_t* col_cnt) {
   if (NB <= 256)
-    return launch_score_select_as<D, 8, 8>(cfg, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+    return launch_score_select_as<D, 8, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   if (NB <= 512)
-    return launch_score_select_as<D, 16, 8>(cfg, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
-  return launch_score_select_as<D, 64, 8>(cfg, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+    return launch_score_select_as<D, 16, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+  return launch_score_select_as<D, 64, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
 }
 
 // The staged token select may use up to kSelectSmemKeys keys of dynamic shared memory.  The limit is always set
@@ -655,19 +660,24 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
     // block sums, then the token select run over the NB sums: its "token" flags are the block flags (its own
     // block lift goes to a scratch array); the token flags are filled in at the end of the call
     float* bsum = reinterpret_cast<float*>(base + w.bsum);
-    if (n_protect > 0) block_sum_kernel<<<dim3((NB + 7) / 8, B), 256, 0, st>>>(scores, N, blk, NB, bsum);
+    if (n_protect > 0 &&
+        launch_pdl(block_sum_kernel, dim3((NB + 7) / 8, B), 256, 0, st, scores, N, blk, NB, bsum) != cudaSuccess)
+      return AVSA_ERR_CUDA;
     const size_t key_bytes = static_cast<size_t>(NB) * sizeof(uint32_t);
     if (!allow_select_smem()) return AVSA_ERR_CUDA;
-    token_select_kernel<true><<<B, 1024, key_bytes, st>>>(bsum, NB, n_protect, 32, (NB + 31) / 32, 1, pblk,
-                                                         base + w.junk, static_cast<StatusRecord*>(ws));
+    if (launch_pdl(token_select_kernel<true>, B, 1024, key_bytes, st, bsum, NB, n_protect, 32, (NB + 31) / 32, 1, pblk,
+                   base + w.junk, static_cast<StatusRecord*>(ws)) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   } else if (N <= kSelectSmemKeys) {
     const size_t key_bytes = static_cast<size_t>(N) * sizeof(uint32_t);
     if (!allow_select_smem()) return AVSA_ERR_CUDA;
-    token_select_kernel<true><<<B, 1024, key_bytes, st>>>(scores, N, n_protect, blk, NB, min_tokens, ptok, pblk,
-                                                         static_cast<StatusRecord*>(ws));
+    if (launch_pdl(token_select_kernel<true>, B, 1024, key_bytes, st, scores, N, n_protect, blk, NB, min_tokens, ptok, pblk,
+                   static_cast<StatusRecord*>(ws)) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   } else {
-    token_select_kernel<false><<<B, 1024, 0, st>>>(scores, N, n_protect, blk, NB, min_tokens, ptok, pblk,
-                                                   static_cast<StatusRecord*>(ws));
+    if (launch_pdl(token_select_kernel<false>, B, 1024, 0, st, scores, N, n_protect, blk, NB, min_tokens, ptok, pblk,
+                   static_cast<StatusRecord*>(ws)) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   }
   const int total_rows = B * H * NB;
   const int pr = (flags & AVSA_PROTECT_ROWS) ? 1 : 0, pc = (flags & AVSA_PROTECT_COLS) ? 1 : 0;
@@ -676,49 +686,37 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
     const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(q.ptr);
     const __nv_bfloat16* kp = static_cast<const __nv_bfloat16*>(k.ptr);
     // the pooling kernel does not read anything the token select writes: allow it to start early
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(NB, B * H, 2);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const int64_t qsb = q.stride_b, qsh = q.stride_h, qsn = q.stride_n, ksb = k.stride_b, ksh = k.stride_h,
-                  ksn = k.stride_n;
+    const dim3 pool_grid(NB, B * H, 2);
     cudaError_t e;
     if (d == 128)
-      e = cudaLaunchKernelEx(&cfg, pool_kernel<128>, qp, qsb, qsh, qsn, kp, ksb, ksh, ksn, qbar, kbar, H, N, blk);
+      e = launch_pdl(pool_kernel<128>, pool_grid, 256, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b,
+                     k.stride_h, k.stride_n, qbar, kbar, H, N, blk);
     else
-      e = cudaLaunchKernelEx(&cfg, pool_kernel<64>, qp, qsb, qsh, qsn, kp, ksb, ksh, ksn, qbar, kbar, H, N, blk);
+      e = launch_pdl(pool_kernel<64>, pool_grid, 256, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b,
+                     k.stride_h, k.stride_n, qbar, kbar, H, N, blk);
     if (e != cudaSuccess) return AVSA_ERR_CUDA;
     // block scores and lists of 16 query blocks per CTA, staged behind the pooling grid
-    cfg.gridDim = dim3((NB + kStripRows - 1) / kStripRows, B * H, 1);
-    const float* qbc = qbar;
-    const float* kbc = kbar;
     if (d == 128)
-      e = launch_score_select<128>(cfg, NB, qbc, kbc, block_scores, pbc, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+      e = launch_score_select<128>(st, B, NB, qbar, kbar, block_scores, pbc, H, scale, k_keep, pr, pc, col_idx, col_cnt);
     else
-      e = launch_score_select<64>(cfg, NB, qbc, kbc, block_scores, pbc, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+      e = launch_score_select<64>(st, B, NB, qbar, kbar, block_scores, pbc, H, scale, k_keep, pr, pc, col_idx, col_cnt);
     if (e != cudaSuccess) return AVSA_ERR_CUDA;
   } else {
     const unsigned rgrid = static_cast<unsigned>((total_rows + 3) / 4);
-    const float* bsc = block_scores;
     cudaError_t e = cudaSuccess;
     if (NB <= 256)
-      row_select_kernel<8><<<rgrid, 128, 0, st>>>(bsc, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
+      e = launch_pdl(row_select_kernel<8>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     else if (NB <= 512)
-      row_select_kernel<16><<<rgrid, 128, 0, st>>>(bsc, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
+      e = launch_pdl(row_select_kernel<16>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     else
-      row_select_kernel<64><<<rgrid, 128, 0, st>>>(bsc, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
-    e = cudaGetLastError();
+      e = launch_pdl(row_select_kernel<64>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     if (e != cudaSuccess) return AVSA_ERR_CUDA;
   }
   if (by_block_sum) {
     const int64_t total = static_cast<int64_t>(B) * N;
-    expand_blocks_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(pblk, N, blk, NB, total, ptok);
+    if (launch_pdl(expand_blocks_kernel, static_cast<unsigned>((total + 255) / 256), 256, 0, st, pblk, N, blk, NB, total,
+                   ptok) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }

@@ -18,6 +18,8 @@ __global__ void __launch_bounds__(1024) compact_rows_kernel(const uint8_t* __res
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint8_t* f = prot_tok + static_cast<int64_t>(b) * N;
   int32_t* out = rows + static_cast<int64_t>(b) * n_pad;
+  pdl_wait();
+  pdl_launch();
   if (b == 0 && tid == 0) {
     status->code = 0;
     status->where = 0;
@@ -63,6 +65,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* _
   const int r = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
   const int c = threadIdx.x % TPR;
   const int h = blockIdx.y, b = blockIdx.z, H = gridDim.y;
+  pdl_wait();
+  pdl_launch();
   if (r >= n_pad) return;
   const int src = rows[static_cast<int64_t>(b) * n_pad + r];
   uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -102,28 +106,31 @@ template <int BLK, int D>
 static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d& q, const avsa_bf16_4d& k,
                          const avsa_bf16_4d& v, const uint8_t* prot_tok, void* o, float* lse, float scale, uint8_t* ws,
                          const ProtPlan& c, cudaStream_t st) {
-  using L = AttnSmem<BLK, D>;
   StatusRecord* status = reinterpret_cast<StatusRecord*>(ws);
   int32_t* rows = reinterpret_cast<int32_t*>(ws + c.off_rows);
   __nv_bfloat16* qp = reinterpret_cast<__nv_bfloat16*>(ws + c.off_qp);
   float* part_o = reinterpret_cast<float*>(ws + c.off_part_o);
   float* part_lse = reinterpret_cast<float*>(ws + c.off_part_lse);
-  compact_rows_kernel<<<B, 1024, 0, st>>>(prot_tok, N, n_protect, c.n_pad, rows, status);
+  if (launch_pdl(compact_rows_kernel, B, 1024, 0, st, prot_tok, N, n_protect, c.n_pad, rows, status) != cudaSuccess)
+    return AVSA_ERR_CUDA;
   constexpr int RPB = 256 / (D / 8);
-  gather_rows_kernel<D><<<dim3((c.n_pad + RPB - 1) / RPB, H, B), 256, 0, st>>>(
-      static_cast<const __nv_bfloat16*>(q.ptr), q.stride_b, q.stride_h, q.stride_n, rows, c.n_pad, qp);
+  if (launch_pdl(gather_rows_kernel<D>, dim3((c.n_pad + RPB - 1) / RPB, H, B), 256, 0, st,
+                 static_cast<const __nv_bfloat16*>(q.ptr), q.stride_b, q.stride_h, q.stride_n, rows, c.n_pad, qp) !=
+      cudaSuccess)
+    return AVSA_ERR_CUDA;
   CUtensorMap tq, tk, tv;
   if (!encode_bf16_tile_map(&tq, qp, B, H, c.n_pad, D, static_cast<int64_t>(H) * c.n_pad * D,
                             static_cast<int64_t>(c.n_pad) * D, D, BLK))
     return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tk, k.ptr, B, H, N, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tv, v.ptr, B, H, N, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
+  using L = AttnSmem<BLK, D>;
   using LP = PersistSmem<BLK, D>;
-  if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           LP::kTotal) != cudaSuccess)
-    return AVSA_ERR_CUDA;
   if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            L::kTotal) != cudaSuccess)
+    return AVSA_ERR_CUDA;
+  if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           LP::kTotal) != cudaSuccess)
     return AVSA_ERR_CUDA;
   AttnParams prm = {};
   prm.part_o = part_o;
@@ -141,14 +148,18 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   int* redo = reinterpret_cast<int*>(ws + c.off_redo);
   const long long items = static_cast<long long>(B) * H * c.NQT * c.n_split;
   const int grid = persistent_grid(items);
-  attn_persist_kernel<BLK, D, MODE_RANGE><<<grid, kAttnThreads, LP::kTotal, st>>>(tq, tk, tv, tq, prm, redo, nullptr,
-                                                                                  static_cast<int>(items));
-  attn_redo_kernel<BLK, D, MODE_RANGE><<<grid, kAttnThreads, L::kTotal, st>>>(tq, tk, tv, tq, prm, redo);
+  if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, LP::kTotal, st, tq, tk, tv, tq, prm, redo,
+                 nullptr, static_cast<int>(items)) != cudaSuccess)
+    return AVSA_ERR_CUDA;
+  if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, tq, prm, redo) !=
+      cudaSuccess)
+    return AVSA_ERR_CUDA;
   const int total_rows = B * H * c.n_pad;
   constexpr int MRPB = 128 / (D / 4);
-  merge_splits_kernel<BLK, D><<<(total_rows + MRPB - 1) / MRPB, 128, 0, st>>>(
-      part_o, part_lse, c.n_split, c.NQT, c.n_pad, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b,
-      q.stride_h, q.stride_n, lse, rows, c.n_pad, N);
+  if (launch_pdl(merge_splits_kernel<BLK, D>, (total_rows + MRPB - 1) / MRPB, 128, 0, st, part_o, part_lse, c.n_split, c.NQT,
+                 c.n_pad, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h, q.stride_n, lse, rows,
+                 c.n_pad, N) != cudaSuccess)
+    return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -176,7 +187,8 @@ extern "C" int avsa_protected_rows_attn(int B, int H, int N, int d, int blk, avs
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
   if (n_protect == 0) {
-    clear_status_kernel<<<1, 1, 0, as_stream(stream)>>>(static_cast<StatusRecord*>(ws));
+    if (launch_pdl(clear_status_kernel, 1, 1, 0, as_stream(stream), static_cast<StatusRecord*>(ws)) != cudaSuccess)
+      return AVSA_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
   }
   uint8_t* base = static_cast<uint8_t*>(ws);

@@ -17,6 +17,8 @@ __global__ void __launch_bounds__(1024) prep_sparse_kernel(StatusRecord* st, con
   __shared__ int warp_tot[32];
   __shared__ int total_heavy;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  pdl_launch();
   if (tid == 0) {
     st->code = 0;
     st->where = 0;
@@ -93,26 +95,28 @@ __global__ void __launch_bounds__(32) bounded_wait_selftest_kernel(StatusRecord*
 template <int BLK, int D>
 static int launch_sparse_attn(int B, int H, int N, const avsa_bf16_4d& q, const avsa_bf16_4d& k,
                               const avsa_bf16_4d& v, void* o, const AttnParams& prm, int* redo, cudaStream_t st) {
-  using L = AttnSmem<BLK, D>;
   CUtensorMap tq, tk, tv, to;
   if (!encode_bf16_tile_map(&tq, q.ptr, B, H, N, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tk, k.ptr, B, H, N, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tv, v.ptr, B, H, N, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&to, o, B, H, N, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
-  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) !=
-      cudaSuccess)
-    return AVSA_ERR_CUDA;
   // The persistent fast kernel first; it lists the (rare) work items whose rows outgrow its fixed reference
   // maxima, and the exact-rescaling kernel behind it recomputes exactly those.
   const long long items = static_cast<long long>(prm.NQT) * H * B;
+  using L = AttnSmem<BLK, D>;
   using LP = PersistSmem<BLK, D>;
+  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) !=
+      cudaSuccess)
+    return AVSA_ERR_CUDA;
   if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            LP::kTotal) != cudaSuccess)
     return AVSA_ERR_CUDA;
-  attn_persist_kernel<BLK, D, MODE_LIST><<<persistent_grid(items), kAttnThreads, LP::kTotal, st>>>(
-      tq, tk, tv, to, prm, redo, redo + items, static_cast<int>(items));
-  const int redo_grid = persistent_grid(items);
-  attn_redo_kernel<BLK, D><<<redo_grid, kAttnThreads, L::kTotal, st>>>(tq, tk, tv, to, prm, redo);
+  if (launch_pdl(attn_persist_kernel<BLK, D, MODE_LIST>, persistent_grid(items), kAttnThreads, LP::kTotal, st, tq, tk, tv,
+                 to, prm, redo, redo + items, static_cast<int>(items)) != cudaSuccess)
+    return AVSA_ERR_CUDA;
+  if (launch_pdl(attn_redo_kernel<BLK, D, MODE_LIST>, persistent_grid(items), kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm,
+                 redo) != cudaSuccess)
+    return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -167,8 +171,9 @@ extern "C" int avsa_sparse_self_attn(int B, int H, int N, int d, int blk, avsa_b
   if (tail_heads < 1) tail_heads = 1;
   if (tail_heads > static_cast<long long>(B) * H) tail_heads = static_cast<long long>(B) * H;
   const int tail_start = static_cast<int>((static_cast<long long>(B) * H - tail_heads) * prm.NQT);
-  prep_sparse_kernel<<<1, 1024, 0, st>>>(prm.status, col_cnt, static_cast<int>(n_items), tail_start, prm.NKB,
-                                         redo + n_items);
+  if (launch_pdl(prep_sparse_kernel, 1, 1024, 0, st, prm.status, col_cnt, static_cast<int>(n_items), tail_start, prm.NKB,
+                 redo + n_items) != cudaSuccess)
+    return AVSA_ERR_CUDA;
   if (d == 128) return launch_sparse_attn<128, 128>(B, H, N, q, k, v, o_bf16, prm, redo, st);
   return launch_sparse_attn<64, 64>(B, H, N, q, k, v, o_bf16, prm, redo, st);
 }
