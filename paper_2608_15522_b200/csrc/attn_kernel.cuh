@@ -14,9 +14,9 @@
 //
 // MODE_LIST   key tiles come from an explicit ascending list; the output tile is converted to bf16
 //             and TMA-stored; optional natural-log LSE.
-// MODE_RANGE  key tiles are a contiguous range (one split of the key axis); the output is a partial
-//             result (fp32 rows normalised by their own sum, plus the log2-domain LSE of the split).
-// MODE_RANGE_DIRECT  the whole key axis as one range (few keys): output written like MODE_LIST.
+// MODE_RANGE  key tiles are a contiguous range.  Part of the key axis: the output is a partial result (fp32 rows
+//             normalised by their own sum) for merge_splits_rows.  The whole key axis: output written like MODE_LIST
+//             (unless the caller wants partials throughout).  The log2-domain LSE of the range is written either way.
 #pragma once
 #include "avsa_common.cuh"
 #include "sm100_ptx.cuh"
@@ -33,7 +33,7 @@ static_assert(4 * 32 * kServiceRegs + 8 * 32 * kSoftmaxRegs <= kAttnThreads * kL
 constexpr int kStages = 3;
 constexpr float kRescaleThreshold = 8.0f;   // log2 units: O is rescaled only when a row max grew by more
 
-enum { MODE_LIST = 0, MODE_RANGE = 1, MODE_RANGE_DIRECT = 2 };
+enum { MODE_LIST = 0, MODE_RANGE = 1 };
 
 enum AttnWhere {
   kWhereQFull = 1, kWhereKEmpty, kWhereVEmpty, kWhereKFull, kWhereVFull, kWherePFull, kWhereSFull, kWhereFinal,
@@ -54,15 +54,88 @@ struct AttnSmem {
   static constexpr int kTotal = kMisc + 16;
 };
 
+// How MODE_RANGE cuts its work.  The query tiles of a head are taken `chunk` at a time; a unit is such a chunk against
+// the whole key axis.  CTAs that work on the same part of a unit's key axis do so side by side, one query tile each, so
+// the tiles come from DRAM once per chunk.
+//   Stream (L > 0): the units' key tiles, one unit after the other, form one stream; the grid is `groups` groups of
+// `chunk` CTAs, and group g takes tiles [g L, (g+1) L).  Every CTA gets the same number of tiles up to one, in at most
+// L/NKB + 2 contiguous segments.  For calls of few tiles per CTA, where equal pieces do not divide over the CTAs (128
+// query tiles on 148 SMs: 20 idle; 340 us as one item each, 323 as a stream).
+//   Queue (L == 0): the first unitsA units are cut into nA pieces of tpsA tiles, the rest into smaller ones (nB, tpsB),
+// and the CTAs take them off a queue.  The SMs are not equally fast (a GPC's SMs share their way to L2; equal shares end
+// up to 10 % apart), so for long calls the queue with small pieces at its end is the better balance: 1782 us as a stream,
+// 1646 us as a queue for the dense rows of the long sequence.
+// A query tile whose keys fall into several parts is merged from them.
+struct RangeSplit {
+  int chunk, cpb;           // query tiles per chunk, chunks per head
+  int units;                // B*H*cpb
+  int NQT, NKB;
+  int ctas;                 // grid size
+  int groups, L;            // stream
+  int unitsA, nA, tpsA, nB, tpsB;   // queue
+  // Partial results are numbered part * chunk + query tile of the chunk.  Stream: the part of group g and unit u is
+  // g + u (both grow along the stream, so the sum is unique).  Queue: the parts are the pieces in queue order.
+  __host__ __device__ int parts() const { return L > 0 ? groups + units : unitsA * nA + (units - unitsA) * nB; }
+  __host__ __device__ int slots() const { return parts() * chunk; }
+  // parts [first, first + n) hold the keys of unit u
+  __host__ __device__ int unit_parts(int u, int& first) const {
+    if (L > 0) {
+      const int g = u * NKB / L;
+      first = g + u;
+      return (u * NKB + NKB - 1) / L - g + 1;
+    }
+    first = u < unitsA ? u * nA : unitsA * nA + (u - unitsA) * nB;
+    return u < unitsA ? nA : nB;
+  }
+  __host__ __device__ bool whole_rows() const {      // no query tile is split
+    return L > 0 ? L % NKB == 0 : (nA == 1 || unitsA == 0) && (nB == 1 || unitsA == units);
+  }
+  // Item: stream: unit * ctas + CTA (below 2^31: one query tile of 128 rows is 16 KB at least, so 2^31 / 148 of them do
+  // not fit the card); queue: the slot.
+  struct Item {
+    int u, j, kb0, cnt, slot;      // cnt <= 0: nothing there
+  };
+  __host__ __device__ Item item(int id) const {
+    Item it;
+    it.j = id % chunk;
+    if (L > 0) {
+      it.u = id / ctas;
+      const int g = (id % ctas) / chunk;
+      const int lo = g * L > it.u * NKB ? g * L : it.u * NKB;
+      const int hi = (g + 1) * L < (it.u + 1) * NKB ? (g + 1) * L : (it.u + 1) * NKB;
+      it.kb0 = lo - it.u * NKB;
+      it.cnt = hi - lo;
+      it.slot = (g + it.u) * chunk + it.j;
+    } else {
+      const int q = id / chunk, qb = q - unitsA * nA;
+      const int tps = qb < 0 ? tpsA : tpsB;
+      it.u = qb < 0 ? q / nA : unitsA + qb / nB;
+      it.kb0 = (qb < 0 ? q % nA : qb % nB) * tps;
+      it.cnt = (NKB - it.kb0 < tps ? NKB - it.kb0 : tps);
+      it.slot = id;
+    }
+    if ((it.u % cpb) * chunk + it.j >= NQT) it.cnt = 0;
+    return it;
+  }
+};
+
+// kStoreNone: no bf16 output asked for; kStoreTile: whole tiles by TMA; kStoreRows: row by row through a row map
+enum { kStoreNone = 0, kStoreTile, kStoreRows };
+
 struct AttnParams {
   // MODE_LIST
   const int32_t* col_idx;   // [B,H,NB,NB]
   const int32_t* col_cnt;   // [B,H,NB]
-  float* lse;               // [B,H,Nq] natural log, optional
+  float* lse;               // [B,H,Nq] natural log, optional (MODE_RANGE: of the rows written directly)
   // MODE_RANGE
-  float* part_o;            // [items][BLK][D] fp32
-  float* part_lse2;         // [items][BLK]
-  int n_split, tiles_per_split;
+  RangeSplit rs;
+  float* part_o;            // [slots][BLK][D] fp32
+  float* part_lse2;         // [slots][BLK]
+  int store;                // kStoreNone / kStoreTile / kStoreRows: how query tiles that are not split go out
+  __nv_bfloat16* o;         // kStoreRows: row r of batch item b goes to row row_map[b*Nq + r] (left out if negative)
+  int64_t o_sb, o_sh, o_sn;
+  const int32_t* row_map;
+  int n_out;                // rows of `o` and of `lse`
   // both
   StatusRecord* status;
   int H;
@@ -71,36 +144,74 @@ struct AttnParams {
   float scale_log2;         // softmax_scale * log2(e)
 };
 
-// One work item of the tile kernel: query tile `bx` (MODE_LIST) or query tile / key split `bx`
-// (range modes) of head `by`, batch item `bz`.  Called once per flagged work item by attn_redo_kernel;
+// One work item: query tile, key tiles (`cnt` of them; MODE_RANGE: from kb0 on), valid keys of the last one, and
+// (MODE_RANGE) where its partial result goes.
+struct AttnItem {
+  int item, cnt, qt, h, b, kb0, slot, valid;
+};
+// MODE_LIST: item = (b*H + h)*NQT + qt; MODE_RANGE: see RangeSplit::item.
+template <int BLK, int MODE>
+__device__ __forceinline__ AttnItem decode_item(const AttnParams& p, int item) {
+  AttnItem it;
+  it.item = item;
+  int bh, last;
+  if (MODE == MODE_LIST) {
+    it.kb0 = 0;
+    it.slot = 0;
+    it.cnt = p.col_cnt[item];
+    it.qt = item % p.NQT;
+    bh = item / p.NQT;
+    last = it.cnt >= 1 && it.cnt <= p.NKB ? p.col_idx[static_cast<int64_t>(item) * p.NKB + it.cnt - 1] : 0;
+  } else {
+    const RangeSplit::Item r = p.rs.item(item);
+    it.kb0 = r.kb0;
+    it.slot = r.slot;
+    it.cnt = r.cnt;
+    it.qt = (r.u % p.rs.cpb) * p.rs.chunk + r.j;
+    bh = r.u / p.rs.cpb;
+    last = r.kb0 + r.cnt - 1;
+  }
+  it.h = bh % p.H;
+  it.b = bh / p.H;
+  it.valid = last == p.NKB - 1 ? p.Nk - last * BLK : BLK;
+  return it;
+}
+
+// kStoreRows: `HALF` accumulator columns of one row, scaled, from column col0 on
+template <int HALF>
+__device__ __forceinline__ void store_mapped_row(const AttnParams& p, int b, int h, int out_row, int col0, const uint32_t* o,
+                                                 float inv) {
+  if (out_row < 0 || out_row >= p.n_out) return;
+  uint4* dst = reinterpret_cast<uint4*>(p.o + b * p.o_sb + h * p.o_sh + out_row * p.o_sn + col0);
+#pragma unroll
+  for (int g = 0; g < HALF / 8; g++) {
+    uint4 val;
+    val.x = pack_bf16x2(__uint_as_float(o[g * 8 + 0]) * inv, __uint_as_float(o[g * 8 + 1]) * inv);
+    val.y = pack_bf16x2(__uint_as_float(o[g * 8 + 2]) * inv, __uint_as_float(o[g * 8 + 3]) * inv);
+    val.z = pack_bf16x2(__uint_as_float(o[g * 8 + 4]) * inv, __uint_as_float(o[g * 8 + 5]) * inv);
+    val.w = pack_bf16x2(__uint_as_float(o[g * 8 + 6]) * inv, __uint_as_float(o[g * 8 + 7]) * inv);
+    dst[g] = val;
+  }
+}
+
+// One work item of the tile kernel with exact rescaling.  Called once per flagged work item by attn_redo_kernel;
 // every thread of the CTA must call it.
 template <int BLK, int D, int MODE>
 __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUtensorMap* tmk, const CUtensorMap* tmv,
-                                              const CUtensorMap* tmo, const AttnParams& p, int bx, int by, int bz) {
+                                              const CUtensorMap* tmo, const AttnParams& p, int item) {
   using L = AttnSmem<BLK, D>;
   constexpr bool kListIn = (MODE == MODE_LIST);          // explicit list of key tiles (else a contiguous range)
-  constexpr bool kDirectOut = (MODE != MODE_RANGE);      // final bf16 tile + LSE (else a partial result)
   constexpr int NPANEL = D / 64;
   constexpr int PANEL_BYTES = BLK * 128;        // one 64-channel panel of a K/V tile
   constexpr int QPANEL_BYTES = 128 * 128;
   extern __shared__ __align__(1024) uint8_t smem[];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int h = by, b = bz;
-  int qt, split = 0, kb0 = 0, cnt;
-  const int32_t* list = nullptr;
-  if (kListIn) {
-    qt = bx;
-    const int row_id = (b * p.H + h) * p.NQT + qt;
-    list = p.col_idx + static_cast<int64_t>(row_id) * p.NKB;
-    cnt = p.col_cnt[row_id];
-  } else {
-    qt = bx / p.n_split;
-    split = bx % p.n_split;
-    kb0 = split * p.tiles_per_split;
-    cnt = min(p.NKB, kb0 + p.tiles_per_split) - kb0;
-  }
-  const int item = ((b * p.H + h) * p.NQT + qt) * (kListIn ? 1 : p.n_split) + split;
+  const AttnItem it = decode_item<BLK, MODE>(p, item);
+  const int qt = it.qt, h = it.h, b = it.b, kb0 = it.kb0, cnt = it.cnt;
+  const int32_t* list = kListIn ? p.col_idx + static_cast<int64_t>(item) * p.NKB : nullptr;
+  const bool whole = kListIn || cnt == p.NKB;            // final rows (else a partial result)
+  const bool tile_out = kListIn || p.store == kStoreTile;
   // ---- validation: nothing is loaded through a bad list entry
   {
     int bad = (cnt < 1 || cnt > p.NKB) ? 1 : 0;
@@ -150,7 +261,7 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
     prefetch_tmap(tmq);
     prefetch_tmap(tmk);
     prefetch_tmap(tmv);
-    if (kDirectOut) prefetch_tmap(tmo);
+    if (tile_out) prefetch_tmap(tmo);
   }
   if (warp == 2) {
     // (the allocation permit is kept: attn_redo_kernel runs this body several times in one CTA, and with one
@@ -308,8 +419,7 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
     const int row = ((warp & 3) << 5) + lane;    // row of the tile == TMEM lane
     const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const int nw = n_tiles[w];
-    const int last_kb = (kListIn) ? list[cnt - 1] : kb0 + cnt - 1;
-    const int ragged_valid = (last_kb == p.NKB - 1) ? (p.Nk - last_kb * BLK) : BLK;   // valid keys of the last tile
+    const int ragged_valid = it.valid;      // valid keys of the last tile
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
     for (int i = 0; i < nw && ok; i++) {
@@ -405,6 +515,9 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
       const float f0 = a0 / Lsum, f1 = a1 / Lsum;
       // group w handles channels [w*D/2, (w+1)*D/2) of every row
       constexpr int HALF = D / 2;
+      const int64_t grow = static_cast<int64_t>(qt) * BLK + row;
+      int out_row = static_cast<int>(grow);
+      if (whole && !kListIn && p.store == kStoreRows) out_row = row < BLK ? p.row_map[static_cast<int64_t>(b) * p.Nq + grow] : -1;
       uint8_t* stage = smem + L::kQ;     // the Q tile is dead once every MMA has finished
 #pragma unroll
       for (int c = 0; c < HALF / 32; c++) {
@@ -420,7 +533,10 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
           if (have1) v[j] = fmaf(__uint_as_float(o1[j]), f1, v[j]);
         }
         if (row < BLK) {
-          if (kDirectOut) {
+          if (whole && !tile_out) {
+            if (p.store == kStoreRows)
+              store_mapped_row<32>(p, b, h, out_row, col0, reinterpret_cast<const uint32_t*>(v), 1.0f);
+          } else if (whole) {
 #pragma unroll
             for (int g = 0; g < 4; g++) {
               const int col = col0 + g * 8;
@@ -433,7 +549,7 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
               *reinterpret_cast<uint4*>(stage + panel * QPANEL_BYTES + row * 128 + ((chunk ^ (row & 7)) << 4)) = val;
             }
           } else {
-            float4* dst = reinterpret_cast<float4*>(p.part_o + (static_cast<int64_t>(item) * BLK + row) * D + col0);
+            float4* dst = reinterpret_cast<float4*>(p.part_o + (static_cast<int64_t>(it.slot) * BLK + row) * D + col0);
 #pragma unroll
             for (int g = 0; g < 8; g++) dst[g] = make_float4(v[g * 4], v[g * 4 + 1], v[g * 4 + 2], v[g * 4 + 3]);
           }
@@ -441,18 +557,15 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
       }
       if (w == 0 && row < BLK) {
         const float lse2 = m + log2f(Lsum);
-        if (kDirectOut) {
-          if (p.lse != nullptr && qt * BLK + row < p.Nq)
-            p.lse[(static_cast<int64_t>(b) * p.H + h) * p.Nq + qt * BLK + row] = lse2 * 0.6931471805599453f;
-        } else {
-          p.part_lse2[static_cast<int64_t>(item) * BLK + row] = lse2;
-        }
+        if (whole && p.lse != nullptr && grow < p.Nq && out_row >= 0 && out_row < p.n_out)
+          p.lse[(static_cast<int64_t>(b) * p.H + h) * p.n_out + out_row] = lse2 * 0.6931471805599453f;
+        if (!kListIn) p.part_lse2[static_cast<int64_t>(it.slot) * BLK + row] = lse2;
       }
-      if (kDirectOut) fence_proxy_async();
+      if (whole && tile_out) fence_proxy_async();
     }
     tc_fence_before();
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (kDirectOut && ok && warp == 4 && lane == 0) {
+    if (whole && tile_out && ok && warp == 4 && lane == 0) {
       for (int pn = 0; pn < NPANEL; pn++)
         tma_store_4d(tmo, smem_u32(smem + L::kQ) + pn * QPANEL_BYTES, pn * 64, qt * BLK, h, b);
       tma_store_commit();
@@ -462,6 +575,76 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
   tc_fence_before();
   __syncthreads();
   if (warp == 2) tmem_dealloc(tmem, 512);
+}
+
+// The cut of B*H heads x NQT query tiles x NKB key tiles (see RangeSplit).  `out_of_l2`: the keys and values of all
+// heads together do not stay in L2, so every unit streams its tiles from DRAM.  Costs in units of one key tile
+// (128 keys against 128 queries, 0.7 us): an item's own start and end take about four (measured on one-tile items), a
+// merge grid about four; the slowest SM needs 8 % more for an equal share; and beyond ~70 tile streams side by side the
+// DRAM (6.5 TB/s against 64 KB per tile and stream) sets the pace instead of the tensor pipe.
+inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_of_l2) {
+  RangeSplit best = {};
+  double best_cost = 0.0;
+  // (more than 32 query tiles side by side share no more, and small chunks divide the CTAs better)
+  const int cmax = NQT < 32 ? NQT : 32;
+  for (int chunk = cmax < ctas ? cmax : ctas; chunk >= 1; chunk--) {
+    RangeSplit r = {};
+    r.chunk = chunk;
+    r.cpb = (NQT + chunk - 1) / chunk;
+    r.units = BH * r.cpb;
+    r.NQT = NQT;
+    r.NKB = NKB;
+    const long long tiles = static_cast<long long>(r.units) * NKB;
+    if (tiles >= (1ll << 31) - ctas && best.L != 0) break;      // stream positions are ints; larger chunks make fewer
+    long long groups = ctas / chunk;
+    if (groups > tiles) groups = tiles;
+    const long long even = (tiles + groups - 1) / groups;
+    const long long rows = (even + NKB - 1) / NKB * NKB;         // the same, no query tile split
+    for (int v = 0; v < (rows != even ? 2 : 1); v++) {
+      const long long L = v == 0 ? rows : even;
+      r.L = static_cast<int>(L);
+      r.groups = static_cast<int>((tiles + L - 1) / L);
+      r.ctas = r.groups * chunk;
+      const double pace = out_of_l2 && r.groups > 70 ? r.groups / 70.0 : 1.0;
+      const double segs = v == 0 ? static_cast<double>(L / NKB) : static_cast<double>(L) / NKB + 1.0;
+      const double cost = 1.08 * L * pace + 4.0 * segs + (v == 0 ? 0.0 : 4.0 + 0.1 * NKB / L);
+      if (best.L == 0 || cost < best_cost * 0.999) {
+        best = r;
+        best_cost = cost;
+      }
+    }
+  }
+  // the queue: pieces of 48 tiles or more (a part of a row costs three tiles more than a whole one: its fp32 rows are
+  // written and read again), the last round of them cut into smaller ones
+  const int cpb = (NQT + 31) / 32;
+  const double share = static_cast<double>(BH) * NQT * NKB / ctas;       // tiles per CTA
+  for (int n = 1; n == 1 || NKB / n >= 48; n++) {
+    RangeSplit r = {};
+    r.chunk = (NQT + cpb - 1) / cpb;
+    r.cpb = cpb;
+    r.units = BH * cpb;
+    r.NQT = NQT;
+    r.NKB = NKB;
+    r.ctas = ctas;
+    r.tpsA = (NKB + n - 1) / n;
+    r.nA = (NKB + r.tpsA - 1) / r.tpsA;
+    // the end: 7 tpsA / tpsB for the parts' own costs, 0.7 tpsB of uneven finish; least near sqrt(10 tpsA)
+    r.tpsB = r.tpsA;
+    while (r.tpsB > 16 && r.tpsB * r.tpsB > 20 * r.tpsA) r.tpsB = (r.tpsB + 1) / 2;
+    r.nB = (NKB + r.tpsB - 1) / r.tpsB;
+    const bool cut_tail = r.tpsB < r.tpsA;
+    const double tail = cut_tail ? static_cast<double>(r.tpsA) * ctas * cpb / (static_cast<double>(NQT) * NKB) : 0.0;
+    if (share < 3.0 * r.tpsA || tail + 1.0 > r.units) continue;
+    r.unitsA = cut_tail ? r.units - static_cast<int>(tail + 1.0) : r.units;
+    const double main_share = cut_tail ? share - r.tpsA : share;
+    const double cost = share + (r.nA > 1 ? 7.0 : 4.0) * main_share / r.tpsA + (cut_tail ? 7.0 * r.tpsA / r.tpsB : 0.0) +
+                        0.7 * r.tpsB + (r.whole_rows() ? 0.0 : 4.0);
+    if (cost < best_cost) {
+      best = r;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 // Exact-rescaling pass behind the fast kernels: recomputes the work items they listed (normally none: then
@@ -478,10 +661,7 @@ attn_redo_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant_
   const int n_redo = p.status->redo_count;
   const int warp = threadIdx.x >> 5;
   for (int k = blockIdx.x; k < n_redo; k += gridDim.x) {
-    const int item = redo_list[k];                     // list mode: (b*H + h)*NQT + qt; range modes: that * n_split + split
-    const int per_bh = p.NQT * (MODE == MODE_LIST ? 1 : p.n_split);
-    const int bx = item % per_bh, bh = item / per_bh;
-    attn_fwd_body<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p, bx, bh % p.H, bh / p.H);
+    attn_fwd_body<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p, redo_list[k]);
     // back to the launch state for the next item: every warp at the launch register count, barriers invalidated
     if (warp < 4) {
       asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
@@ -497,39 +677,56 @@ attn_redo_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------------
-// Merge of the key-axis splits written by MODE_RANGE: for every query row, combine the normalised
-// partial outputs with weights exp2(lse2_split - max) and write bf16 rows and the natural-log LSE.
+// Merge of the partial results written by MODE_RANGE: for every query row, combine the normalised
+// partial outputs with weights exp2(lse2_part - max) and write bf16 rows and the natural-log LSE.
+// Rows whose key axis was not split are left alone: the tile kernel wrote them itself.
 // With a row map the result of compact row r goes to row row_map[b][r] of the output (rows mapped to
 // a negative index are skipped): that is how recomputed protected rows are scattered back.
 // ------------------------------------------------------------------------------------------------
+struct MergeParams {
+  RangeSplit rs;
+  const float* part_o;
+  const float* part_lse2;
+  int Nq, H;
+  int row0, total_rows;      // rows [row0, row0 + total_rows) of all B*H*Nq: no row before them is split
+  __nv_bfloat16* o;
+  int64_t o_sb, o_sh, o_sn;
+  float* lse;
+  const int32_t* row_map;
+  int row_map_stride, n_out;
+};
+
 // (`block`, `tid`: index of a group of 128 threads and the thread's place in it, so that another kernel can run
 // this work in part of its grid)
 template <int BLK, int D>
-__device__ __forceinline__ void merge_splits_rows(int block, int tid, const float* __restrict__ part_o,
-                                                  const float* __restrict__ part_lse2, int n_split, int NQT, int Nq,
-                                                  int H, int total_rows, __nv_bfloat16* __restrict__ o, int64_t o_sb,
-                                                  int64_t o_sh, int64_t o_sn, float* __restrict__ lse,
-                                                  const int32_t* __restrict__ row_map, int row_map_stride, int n_out) {
+__device__ __forceinline__ void merge_splits_rows(int block, int tid, const MergeParams& m) {
   constexpr int TPR = D / 4;
-  const int rg = block * (128 / TPR) + tid / TPR;
+  const int rl = block * (128 / TPR) + tid / TPR;
   const int c4 = tid % TPR;
-  if (rg >= total_rows) return;
-  const int bh = rg / Nq, qrow = rg % Nq;
-  const int b = bh / H, h = bh % H;
-  int out_row = qrow;
-  if (row_map != nullptr) {
-    out_row = row_map[static_cast<int64_t>(b) * row_map_stride + qrow];
-    if (out_row < 0 || out_row >= n_out) return;
-  }
+  if (rl >= m.total_rows) return;
+  const int rg = m.row0 + rl;
+  const int bh = rg / m.Nq, qrow = rg % m.Nq;
+  const int b = bh / m.H, h = bh % m.H;
   const int qt = qrow / BLK, r = qrow % BLK;
-  const int64_t item0 = (static_cast<int64_t>(bh) * NQT + qt) * n_split;
+  const int u = bh * m.rs.cpb + qt / m.rs.chunk;
+  int first;
+  const int n = m.rs.unit_parts(u, first);
+  if (n == 1) return;
+  int out_row = qrow;
+  if (m.row_map != nullptr) {
+    out_row = m.row_map[static_cast<int64_t>(b) * m.row_map_stride + qrow];
+    if (out_row < 0 || out_row >= m.n_out) return;
+  }
+  const int64_t row0 = (static_cast<int64_t>(first) * m.rs.chunk + qt % m.rs.chunk) * BLK + r, step = static_cast<int64_t>(m.rs.chunk) * BLK;
   float M = -INFINITY;
-  for (int s = 0; s < n_split; s++) M = fmaxf(M, part_lse2[(item0 + s) * BLK + r]);
+#pragma unroll 4
+  for (int s = 0; s < n; s++) M = fmaxf(M, __ldg(m.part_lse2 + row0 + s * step));
   float W = 0.f;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s = 0; s < n_split; s++) {
-    const float w = exp2f(part_lse2[(item0 + s) * BLK + r] - M);
-    const float4 v = *reinterpret_cast<const float4*>(part_o + ((item0 + s) * BLK + r) * D + c4 * 4);
+#pragma unroll 4
+  for (int s = 0; s < n; s++) {
+    const float w = exp2f(__ldg(m.part_lse2 + row0 + s * step) - M);
+    const float4 v = __ldg(reinterpret_cast<const float4*>(m.part_o + (row0 + s * step) * D + c4 * 4));
     W += w;
     acc.x = fmaf(w, v.x, acc.x);
     acc.y = fmaf(w, v.y, acc.y);
@@ -537,26 +734,26 @@ __device__ __forceinline__ void merge_splits_rows(int block, int tid, const floa
     acc.w = fmaf(w, v.w, acc.w);
   }
   const float inv = 1.0f / W;
-  if (o != nullptr) {
+  if (m.o != nullptr) {
     uint2 pk;
     pk.x = pack_bf16x2(acc.x * inv, acc.y * inv);
     pk.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2*>(o + b * o_sb + h * o_sh + out_row * o_sn + c4 * 4) = pk;
+    *reinterpret_cast<uint2*>(m.o + b * m.o_sb + h * m.o_sh + out_row * m.o_sn + c4 * 4) = pk;
   }
-  if (c4 == 0 && lse != nullptr) lse[static_cast<int64_t>(bh) * n_out + out_row] = (M + log2f(W)) * 0.6931471805599453f;
+  if (c4 == 0 && m.lse != nullptr) m.lse[static_cast<int64_t>(bh) * m.n_out + out_row] = (M + log2f(W)) * 0.6931471805599453f;
+}
+
+inline void set_merge_rows(MergeParams& m, int BH) {
+  const int bh0 = m.rs.L == 0 && m.rs.nA == 1 ? m.rs.unitsA / m.rs.cpb : 0;
+  m.row0 = bh0 * m.Nq;
+  m.total_rows = (BH - bh0) * m.Nq;
 }
 
 template <int BLK, int D>
-__global__ void __launch_bounds__(128) merge_splits_kernel(const float* __restrict__ part_o,
-                                                           const float* __restrict__ part_lse2, int n_split, int NQT,
-                                                           int Nq, int H, int total_rows, __nv_bfloat16* __restrict__ o,
-                                                           int64_t o_sb, int64_t o_sh, int64_t o_sn,
-                                                           float* __restrict__ lse, const int32_t* __restrict__ row_map,
-                                                           int row_map_stride, int n_out) {
+__global__ void __launch_bounds__(128) merge_splits_kernel(const __grid_constant__ MergeParams m) {
   pdl_wait();
   pdl_launch();
-  merge_splits_rows<BLK, D>(blockIdx.x, threadIdx.x, part_o, part_lse2, n_split, NQT, Nq, H, total_rows, o, o_sb, o_sh,
-                            o_sn, lse, row_map, row_map_stride, n_out);
+  merge_splits_rows<BLK, D>(blockIdx.x, threadIdx.x, m);
 }
 
 }  // namespace avsa

@@ -55,8 +55,8 @@ struct PersistSmem {
   static constexpr int kBars = kStage + kQBytes;
   static constexpr int kNumBars = 2 * kPQB + 2 * kPKS + 2 * kPVS + 18 + 2 * kPRing;
   static constexpr int kStats = kBars + kNumBars * 8;          // float mref[128], lsum[2][128]
-  static constexpr int kItems = kStats + 3 * 128 * 4;          // int {item, cnt}[kPRing], two redo flags
-  static constexpr int kMisc = kItems + 8 * kPRing + 16;       // tmem base, stop flag
+  static constexpr int kItems = kStats + 3 * 128 * 4;          // AttnItem[kPRing], two redo flags
+  static constexpr int kMisc = kItems + 32 * kPRing + 16;      // tmem base, stop flag
   static constexpr int kTotal = kMisc + 16;
 };
 
@@ -68,34 +68,10 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&r)[8]) 
                : "memory");
 }
 
-// One work item: which query tile, which key tiles.
-struct PersistItem {
-  int qt, h, b, kb0;
-  const int32_t* list;
-};
-template <int MODE>
-__device__ __forceinline__ PersistItem decode_item(const AttnParams& p, int item) {
-  PersistItem it;
-  int rest = item;
-  it.kb0 = 0;
-  it.list = nullptr;
-  if (MODE == MODE_LIST) {
-    it.list = p.col_idx + static_cast<int64_t>(item) * p.NKB;
-  } else {
-    it.kb0 = (item % p.n_split) * p.tiles_per_split;
-    rest = item / p.n_split;
-  }
-  it.qt = rest % p.NQT;
-  const int bh = rest / p.NQT;
-  it.h = bh % p.H;
-  it.b = bh / p.H;
-  return it;
-}
-
 // MODE_LIST: work item = query tile with an explicit list of key tiles, output bf16 rows + optional LSE
-// (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE / MODE_RANGE_DIRECT: work
-// item = (query tile, split of the key axis), key tiles kb0 .. kb0+cnt-1; output normalised fp32 partials +
-// log2 LSE per split (merge_splits_kernel combines them), or bf16 rows directly when there is one split.
+// (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE: the CTA's items are its segments of
+// the stream described at RangeSplit, fixed by its index; output bf16 rows where the key axis is not split, else
+// normalised fp32 partials for merge_splits_rows, and the log2 LSE of the range.
 template <int BLK, int D, int MODE>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
@@ -103,7 +79,6 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
                     const AttnParams p, int* __restrict__ redo_list, const int* __restrict__ order, int n_items) {
   using L = PersistSmem<BLK, D>;
   constexpr bool kListIn = (MODE == MODE_LIST);
-  constexpr bool kDirectOut = (MODE != MODE_RANGE);
   constexpr int NPANEL = D / 64;
   constexpr int PANEL_BYTES = BLK * 128;
   constexpr int QPANEL_BYTES = 128 * 128;
@@ -129,11 +104,13 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   constexpr int NCH = BLK / 32;
   float* mref_s = reinterpret_cast<float*>(smem + L::kStats);
   float* lsum_s = mref_s + 128;                                              // [2][128]
-  volatile int* items = reinterpret_cast<volatile int*>(smem + L::kItems);   // {item, cnt} x kPRing, then two redo flags
+  AttnItem* ring = reinterpret_cast<AttnItem*>(smem + L::kItems);
+  volatile int* items = reinterpret_cast<volatile int*>(smem + L::kItems);   // the same memory: the redo flags follow the ring
+  static_assert(sizeof(AttnItem) == 32, "ring entries of 32 bytes");
   // One redo flag per item parity: the flag of item n is cleared after item n's second row-sum barrier, and the
   // first thread that can set the flag of item n + 2 has passed that barrier itself, so a set never meets a
   // pending clear (with a single flag, a fast warp of the other group could set it for item n + 1 first).
-  constexpr int REDO = 2 * kPRing;
+  constexpr int REDO = 8 * kPRing;
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + L::kMisc);   // [0] tmem base, [1] stop
 
   if (tid == 0) {
@@ -175,7 +152,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     prefetch_tmap(&tmq);
     prefetch_tmap(&tmk);
     prefetch_tmap(&tmv);
-    if (kDirectOut) prefetch_tmap(&tmo);
+    if (kListIn || p.store == kStoreTile) prefetch_tmap(&tmo);
   }
   if (warp == 2) {
     tmem_alloc(smem_u32(smem + L::kMisc), 512);
@@ -205,13 +182,13 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   auto wait_all = [&](int bar, uint32_t parity, int where, int tag) -> bool {
     return __all_sync(FULLM, wait_or_stop(bar, parity, where, tag));
   };
-  // consumer side of the item ring: item n sits in slot n mod kPRing
-  auto get_item = [&](int n, int& item, int& cnt) -> bool {     // false: stopped, or the queue is empty
+  // consumer side of the item ring: item n sits in slot n mod kPRing, decoded (its divisions, a dozen of them in range
+  // mode, stood at the head of every role's item: 30 us of the reverse direction's 42 two-tile items)
+  auto get_item = [&](int n, AttnItem& it) -> bool {     // false: stopped, or the queue is empty
     const int slot = n % kPRing;
     if (!wait_all(ITEM_FULL + slot, (n / kPRing) & 1, kPersistItem, n)) return false;
-    item = items[2 * slot];
-    cnt = items[2 * slot + 1];
-    return item >= 0;
+    it = ring[slot];
+    return it.item >= 0;
   };
   auto item_done = [&](int n) {
     __syncwarp();
@@ -225,10 +202,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     int q_loads = 0;
     bool ok = true;
     for (int n = 0; ok; n++) {
-      int item, cnt;
-      if (!get_item(n, item, cnt)) break;
-      const PersistItem it = decode_item<MODE>(p, item);
-      const int qt = it.qt, h = it.h, b = it.b;
+      AttnItem it;
+      if (!get_item(n, it)) break;
+      const int qt = it.qt, h = it.h, b = it.b, cnt = it.cnt;
+      const int32_t* list = kListIn ? p.col_idx + static_cast<int64_t>(it.item) * p.NKB : nullptr;
       const int qb = n % kPQB;
       if (n >= kPQB) {
         // the last Q K^T of the item that used this Q buffer has run
@@ -244,7 +221,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       }
       for (int t0 = 0; t0 < cnt && ok; t0 += 32) {
         int mine = it.kb0 + t0 + lane;
-        if (kListIn) mine = (t0 + lane < cnt) ? it.list[t0 + lane] : 0;
+        if (kListIn) mine = (t0 + lane < cnt) ? list[t0 + lane] : 0;
         const int nn = min(32, cnt - t0);
         for (int j = 0; j < nn; j++) {
           const int kb = __shfl_sync(FULLM, mine, j);
@@ -279,34 +256,40 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     // V is needed last in a tile's life, so this warp has the slack to fetch work: it keeps the item ring two
     // items ahead of the one whose V tiles it is loading.
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-    int pub_item = -1, pub_cnt = 0;
-    bool first = true;
+    AttnItem pub;            // the last item published; pub.item < 0: the queue is empty
+    bool first = true;       // queue
+    int seg = 0;             // stream
     // takes the next valid work item off the global queue and publishes it as item m of this CTA
     auto publish = [&](int m) -> bool {
       const int slot = m % kPRing;
       if (m >= kPRing && !wait_all(ITEM_EMPTY + slot, ((m / kPRing) - 1) & 1, kPersistItemEmpty, m)) return false;
       while (true) {
+        int id = blockIdx.x;
+        pub.item = -1;
+        if (!kListIn && p.rs.L > 0) {
+          // stream: the CTA's segments in order, those without a query tile left out
+          const int u = (blockIdx.x / p.rs.chunk) * p.rs.L / p.rs.NKB + seg++;
+          if (u >= p.rs.units) break;
+          pub = decode_item<BLK, MODE>(p, u * p.rs.ctas + id);
+          if (pub.cnt == 0) continue;
+          if (pub.cnt < 0) pub.item = -1;
+          break;
+        }
         // The CTA's first item is its own index, the others come off the queue behind those of the whole grid: with
         // one item or less per CTA, a CTA that is a little early must not take a second one from a late CTA.
-        int id = blockIdx.x;
         if (!first) {
           if (lane == 0) id = gridDim.x + atomicAdd(&p.status->next_item, 1);
           id = __shfl_sync(FULLM, id, 0);
         }
         first = false;
-        if (id >= n_items) {
-          pub_item = -1;
-          pub_cnt = 0;
-          break;
-        }
+        if (id >= n_items) break;
+        if (kListIn) id = order[id];                  // queue position -> query tile (long lists first)
+        pub = decode_item<BLK, MODE>(p, id);
         if (!kListIn) {
-          const int kb0 = (id % p.n_split) * p.tiles_per_split;
-          pub_item = id;
-          pub_cnt = min(p.NKB, kb0 + p.tiles_per_split) - kb0;
+          if (pub.cnt <= 0) continue;
           break;
         }
-        id = order[id];                  // queue position -> query tile (long lists first)
-        const int c = p.col_cnt[id];
+        const int c = pub.cnt;
         bool bad = (c < 1 || c > p.NKB);
         if (!bad) {
           // nothing is loaded through a bad list: entries in range and strictly ascending
@@ -322,16 +305,11 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
           }
           bad = __any_sync(FULLM, bad);
         }
-        if (!bad) {
-          pub_item = id;
-          pub_cnt = c;
-          break;
-        }
+        if (!bad) break;
         if (lane == 0) report_status(p.status, AVSA_ERR_BAD_MASK, kWhereList, id, c);   // refused, not deferred
       }
       if (lane == 0) {
-        items[2 * slot] = pub_item;
-        items[2 * slot + 1] = pub_cnt;
+        ring[slot] = pub;
         mbar_arrive(BAR(ITEM_FULL + slot));     // release: the slot is written before the phase completes
       }
       __syncwarp();
@@ -339,19 +317,18 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     };
     int vc = 0;              // V tiles loaded so far, over all items
     bool ok = publish(0);
-    int a_item = pub_item, a_cnt = pub_cnt;       // item n, whose V tiles are loaded next
-    int b_item = -1, b_cnt = 0;                   // item n + 1
-    if (ok && a_item >= 0) {
+    AttnItem cur = pub, next;                     // item n, whose V tiles are loaded next, and item n + 1
+    next.item = -1;
+    if (ok && cur.item >= 0) {
       ok = publish(1);
-      b_item = pub_item;
-      b_cnt = pub_cnt;
+      next = pub;
     }
-    for (int n = 0; ok && a_item >= 0; n++) {
-      const PersistItem it = decode_item<MODE>(p, a_item);
-      const int h = it.h, b = it.b;
+    for (int n = 0; ok && cur.item >= 0; n++) {
+      const int h = cur.h, b = cur.b, a_cnt = cur.cnt;
+      const int32_t* list = kListIn ? p.col_idx + static_cast<int64_t>(cur.item) * p.NKB : nullptr;
       for (int t0 = 0; t0 < a_cnt && ok; t0 += 32) {
-        int mine = it.kb0 + t0 + lane;
-        if (kListIn) mine = (t0 + lane < a_cnt) ? it.list[t0 + lane] : 0;
+        int mine = cur.kb0 + t0 + lane;
+        if (kListIn) mine = (t0 + lane < a_cnt) ? list[t0 + lane] : 0;
         const int nn = min(32, a_cnt - t0);
         for (int j = 0; j < nn; j++) {
           const int kb = __shfl_sync(FULLM, mine, j);
@@ -376,16 +353,11 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       }
       if (!ok) break;
       // keep the ring two items ahead (nothing more once the end of the queue has been published)
-      int c_item = -1, c_cnt = 0;
-      if (b_item >= 0) {
+      cur = next;
+      if (next.item >= 0) {
         ok = publish(n + 2);
-        c_item = pub_item;
-        c_cnt = pub_cnt;
+        next = pub;
       }
-      a_item = b_item;
-      a_cnt = b_cnt;
-      b_item = c_item;
-      b_cnt = c_cnt;
     }
     if (lane == 0 && misc[1] != 0u)
       for (int c = max(0, vc - kPVS); c < vc; c++) mbar_wait(BAR(V_FULL + c % kPVS), (c / kPVS) & 1);
@@ -403,8 +375,9 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     int used[2] = {0, 0};       // S tiles written so far into each group's buffer
     bool ok = true;
     for (int n = 0; ok; n++) {
-      int item, cnt;
-      if (!get_item(n, item, cnt)) break;
+      AttnItem it;
+      if (!get_item(n, it)) break;
+      const int cnt = it.cnt;
       const int qb = n % kPQB;
       const uint32_t q_lo = q_lo0 + qb * (L::kQBytes >> 4);
       ok = wait_all(Q_FULL + qb, (n / kPQB) & 1, kWhereQFull, n);
@@ -461,8 +434,9 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     int used[2] = {0, 0};       // P tiles read so far from each group's buffer
     bool ok = true;
     for (int n = 0; ok; n++) {
-      int item, cnt;
-      if (!get_item(n, item, cnt)) break;
+      AttnItem it;
+      if (!get_item(n, it)) break;
+      const int cnt = it.cnt;
       for (int t = 0; t < cnt && ok; t++) {
         const int j = t & 1, sv = vc % kPVS;
         ok = wait_all(V_FULL + sv, (vc / kPVS) & 1, kWhereVFull, t);
@@ -505,14 +479,12 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     const uint32_t tm_s = tmem + w * BLK + lane_off;                    // this group's S buffer
     const uint32_t tm_p = tmem + TM_P + w * (BLK / 2) + lane_off;       // and its P buffer
     int used = 0;               // tiles this group has taken so far, over all items
+    int n_staged = 0;           // items whose rows went through the staging buffer
     bool ok = true;
     for (int n = 0; ok; n++) {
-      int item, cnt;
-      if (!get_item(n, item, cnt)) break;
-      const PersistItem it = decode_item<MODE>(p, item);
-      const int qt = it.qt, h = it.h, b = it.b;
-      const int last_kb = kListIn ? it.list[cnt - 1] : it.kb0 + cnt - 1;
-      const int ragged_valid = (last_kb == p.NKB - 1) ? (p.Nk - last_kb * BLK) : BLK;
+      AttnItem it;
+      if (!get_item(n, it)) break;
+      const int cnt = it.cnt, ragged_valid = it.valid;
       float m_ref = 0.f;
       uint64_t sum2[4] = {0ull, 0ull, 0ull, 0ull};
       for (int t = w; t < cnt && ok; t += 2) {       // the groups take alternate key tiles
@@ -595,7 +567,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       lsum_s[w * 128 + row] = l_run;
       // the staged output tile of the item before must have been read by its TMA store before anybody writes the
       // staging buffer again; the thread that issued the store makes sure of it before it joins the barrier below
-      if (kDirectOut && tid == 128) tma_store_wait_read();
+      if (tid == 128) tma_store_wait_read();
       // (time-limited barriers, not bar.sync: a group that gave up must not leave the other one waiting for ever)
       mbar_arrive(BAR(LSUM_A));
       ok = __all_sync(FULLM, wait_or_stop(LSUM_A, n & 1, kPersistLsum, n));
@@ -607,7 +579,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       if (!ok) break;
       if (tid == 128) {
         items[REDO + (n & 1)] = 0;
-        if (redo) redo_list[atomicAdd(&p.status->redo_count, 1)] = item;
+        if (redo) redo_list[atomicAdd(&p.status->redo_count, 1)] = it.item;
       }
       ok = __all_sync(FULLM, wait_or_stop(O_FULL, n & 1, kPersistOFull, n));
       if (!ok) break;
@@ -620,9 +592,23 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       tmem_wait_ld();
       tc_fence_before();
       mbar_arrive(BAR(O_FREE));           // the accumulator is in registers: the next item's P V may start
-      const int64_t grow = static_cast<int64_t>(qt) * BLK + row;
+      const int64_t grow = static_cast<int64_t>(it.qt) * BLK + row;
       const float inv = 1.0f / Lsum;
-      if (kDirectOut) {
+      const bool whole = kListIn || cnt == p.NKB;
+      const bool tile_out = kListIn || p.store == kStoreTile;
+      if (!kListIn && !redo && w == 0 && row < BLK)
+        p.part_lse2[static_cast<int64_t>(it.slot) * BLK + row] = m_ref + log2f(Lsum);
+      if (whole && !tile_out) {
+        if (!redo && row < BLK) {
+          int out_row = static_cast<int>(grow);
+          if (p.store == kStoreRows) {
+            out_row = p.row_map[static_cast<int64_t>(it.b) * p.Nq + grow];
+            store_mapped_row<HALF>(p, it.b, it.h, out_row, w * HALF, o0, inv);
+          }
+          if (w == 0 && p.lse != nullptr && grow < p.Nq && out_row >= 0 && out_row < p.n_out)
+            p.lse[(static_cast<int64_t>(it.b) * p.H + it.h) * p.n_out + out_row] = (m_ref + log2f(Lsum)) * 0.6931471805599453f;
+        }
+      } else if (whole) {
         // The tile goes out through shared memory (128-byte swizzled) and one TMA store.  Rows written straight
         // from registers, even as whole 32-byte sectors, kept these warps busy for about 2000 cycles per item
         // (1024 sector requests at 256-byte stride); the store's read of the staging buffer is only waited for
@@ -641,20 +627,21 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
             *reinterpret_cast<uint4*>(stage + panel * QPANEL_BYTES + row * 128 + ((chunk ^ (row & 7)) << 4)) = val;
           }
           if (!redo && w == 0 && p.lse != nullptr && grow < p.Nq)
-            p.lse[(static_cast<int64_t>(b) * p.H + h) * p.Nq + grow] = (m_ref + log2f(Lsum)) * 0.6931471805599453f;
+            p.lse[(static_cast<int64_t>(it.b) * p.H + it.h) * p.Nq + grow] = (m_ref + log2f(Lsum)) * 0.6931471805599453f;
         }
         fence_proxy_async();
         mbar_arrive(BAR(STAGE_FULL));
         if (tid == 128) {
-          if (wait_or_stop(STAGE_FULL, n & 1, kPersistStage, n) && !redo) {
+          if (wait_or_stop(STAGE_FULL, n_staged & 1, kPersistStage, n) && !redo) {
             for (int pn = 0; pn < NPANEL; pn++)
-              tma_store_4d(&tmo, smem_u32(smem + L::kStage) + pn * QPANEL_BYTES, pn * 64, qt * BLK, h, b);
+              tma_store_4d(&tmo, smem_u32(smem + L::kStage) + pn * QPANEL_BYTES, pn * 64, it.qt * BLK, it.h, it.b);
             tma_store_commit();
           }
         }
+        n_staged++;
       } else if (!redo && row < BLK) {
-        // normalised fp32 partial of this split + its log2 LSE, for merge_splits_kernel
-        float* prow = p.part_o + (static_cast<int64_t>(item) * BLK + row) * D + w * HALF;
+        // normalised fp32 partial of this range, for merge_splits_rows
+        float* prow = p.part_o + (static_cast<int64_t>(it.slot) * BLK + row) * D + w * HALF;
 #pragma unroll
         for (int g = 0; g < HALF / 8; g++) {
           uint32_t r[8];
@@ -662,11 +649,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
           for (int i = 0; i < 8; i++) r[i] = __float_as_uint(__uint_as_float(o0[g * 8 + i]) * inv);
           st_global_v8(prow + g * 8, r);
         }
-        if (w == 0) p.part_lse2[static_cast<int64_t>(item) * BLK + row] = m_ref + log2f(Lsum);
       }
       item_done(n);
     }
-    if (kDirectOut && tid == 128) tma_store_wait_read();     // the last store has read the staging buffer
+    if (tid == 128) tma_store_wait_read();     // the last store has read the staging buffer
   }
   tc_fence_before();
   __syncthreads();

@@ -67,6 +67,9 @@ static __global__ void clear_status_kernel(StatusRecord* st) {
   st->next_item = 0;
 }
 
+// Keys and values of at most this many bytes are taken to stay in L2 (126 MB) between their readers.
+constexpr long long kL2KeepBytes = 64ll << 20;
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

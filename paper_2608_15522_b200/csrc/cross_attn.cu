@@ -19,9 +19,9 @@ constexpr int kColThreads = 384;
 constexpr int kColStages = 3;
 
 struct ColsumParams {
-  const float* lse;        // [B,H,Nq] natural log; used when part_lse2 is null
-  const float* part_lse2;  // or the log2-domain LSEs of pass 1's key splits, [B,H,NQT,n_split,blk], merged here
-  int n_split, NQT, blk;
+  const float* part_lse2;  // log2-domain LSEs of pass 1's key ranges, [slots][blk], merged here
+  RangeSplit rs;           // how pass 1 was cut
+  int blk;
   float* partial;          // [NCH][B,H,Nk]
   StatusRecord* status;
   int H, Nq, Nk, NKT;      // NKT = key tiles of 128
@@ -87,22 +87,21 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   }
   pdl_wait();
   // negated log2-domain LSEs (one packed FMA then gives s*c - lse2); queries beyond Nq get -inf: exp2 = 0
-  // (straight from the splits' partial LSEs when pass 1 left its merge for later: the same maximum-and-sum as the
-  // merge kernel, in the log2 domain)
+  // (straight from the partial LSEs of pass 1's key ranges: the same maximum-and-sum as in merge_splits_rows, so that
+  // nothing has to be merged between the passes)
   for (int j = tid; j < NCH * W; j += kColThreads) {
     float v = -INFINITY;
     if (j < p.Nq) {
-      if (p.part_lse2 != nullptr) {
-        const int64_t item0 = ((static_cast<int64_t>(b) * p.H + h) * p.NQT + j / p.blk) * p.n_split;
-        const float* pl = p.part_lse2 + item0 * p.blk + j % p.blk;
-        float M = -INFINITY;
-        for (int s = 0; s < p.n_split; s++) M = fmaxf(M, pl[s * p.blk]);
-        float Wsum = 0.f;
-        for (int s = 0; s < p.n_split; s++) Wsum += exp2f(pl[s * p.blk] - M);
-        v = -(M + log2f(Wsum));
-      } else {
-        v = -p.lse[(static_cast<int64_t>(b) * p.H + h) * p.Nq + j] * 1.4426950408889634f;
-      }
+      const int qt = j / p.blk, u = (b * p.H + h) * p.rs.cpb + qt / p.rs.chunk;
+      int first;
+      const int n = p.rs.unit_parts(u, first);
+      const float* pl = p.part_lse2 + (static_cast<int64_t>(first) * p.rs.chunk + qt % p.rs.chunk) * p.blk + j % p.blk;
+      const int step = p.rs.chunk * p.blk;
+      float M = -INFINITY;
+      for (int s = 0; s < n; s++) M = fmaxf(M, pl[s * step]);
+      float Wsum = 0.f;
+      for (int s = 0; s < n; s++) Wsum += exp2f(pl[s * step] - M);
+      v = -(M + log2f(Wsum));
     }
     lse2[j] = v;
   }
@@ -500,19 +499,15 @@ __global__ void __launch_bounds__(256) head_sum_kernel(const float* __restrict__
 template <int BLK, int D>
 __global__ void __launch_bounds__(256) cross_finalize_kernel(int hs_blocks, const float* __restrict__ partial, int NCH, int B,
                                                              int H, int Nk, float beta, float gamma,
-                                                             float* __restrict__ scores, const float* __restrict__ part_o,
-                                                             const float* __restrict__ part_lse2, int n_split, int NQT,
-                                                             int Nq, int total_rows, __nv_bfloat16* __restrict__ o,
-                                                             int64_t o_sb, int64_t o_sh, int64_t o_sn,
-                                                             float* __restrict__ lse) {
+                                                             float* __restrict__ scores,
+                                                             const __grid_constant__ MergeParams m) {
   pdl_wait();
   pdl_launch();
   if (static_cast<int>(blockIdx.x) < hs_blocks) {
     head_sum_keys(blockIdx.x, threadIdx.x, partial, NCH, B, H, Nk, beta, gamma, scores);
   } else {
     const int block = (static_cast<int>(blockIdx.x) - hs_blocks) * 2 + (threadIdx.x >> 7);
-    merge_splits_rows<BLK, D>(block, threadIdx.x & 127, part_o, part_lse2, n_split, NQT, Nq, H, total_rows, o, o_sb, o_sh,
-                              o_sn, lse, nullptr, 0, Nq);
+    merge_splits_rows<BLK, D>(block, threadIdx.x & 127, m);
   }
 }
 
@@ -550,7 +545,8 @@ __global__ void __launch_bounds__(256) head_sum_wide_kernel(const float* __restr
 }
 
 struct CrossPlan {
-  int blk, NQT, NKB, n_split, tps;           // pass 1 (key tiles of blk)
+  int blk, NQT, NKB;                         // pass 1 (key tiles of blk)
+  RangeSplit rs;
   int NKT, NCH, W, n_range, tpr;             // pass 2 (key tiles of 128)
   bool reverse;                              // pass 2 with the keys resident (Nq > 512, Nk <= 512)
   int NQC, rev_ranges, rev_cpr, rev_slots;   // query chunks of 128, CTAs per (b,h), chunks per CTA, partial slots
@@ -562,15 +558,9 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   c.blk = d;   // (blk, d) = (128,128) or (64,64)
   c.NQT = (Nq + c.blk - 1) / c.blk;
   c.NKB = (Nk + c.blk - 1) / c.blk;
-  // One work item per SM (one CTA each): a single wave.  Two items per SM were measured slower on the
-  // Ovi-class shape (210 vs 196 us for the call): every item pays its own pipeline fill, partial-result
-  // write-out and merge work.
   const int target = persistent_grid(1 << 30);
-  int want_split = target / (B * H * c.NQT);
-  if (want_split < 1) want_split = 1;
-  if (want_split > c.NKB) want_split = c.NKB;
-  c.tps = (c.NKB + want_split - 1) / want_split;
-  c.n_split = (c.NKB + c.tps - 1) / c.tps;
+  const long long kv_bytes = 4ll * B * H * Nk * d;
+  c.rs = make_range_split(B * H, c.NQT, c.NKB, target, kv_bytes > kL2KeepBytes);
   c.NKT = (Nk + 127) / 128;
   c.NCH = Nq > 256 ? 2 : 1;
   c.W = (((Nq + c.NCH - 1) / c.NCH) + 15) / 16 * 16;
@@ -588,14 +578,14 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   c.rev_ranges = (c.NQC + c.rev_cpr - 1) / c.rev_cpr;
   c.rev_slots = c.rev_ranges * 2;
   size_t off = kStatusBytes;
-  const size_t items = static_cast<size_t>(B) * H * c.NQT * c.n_split;
-  c.off_part_o = off; off += align_up(items * c.blk * d * sizeof(float), 256);
-  c.off_part_lse = off; off += align_up(items * c.blk * sizeof(float), 256);
+  const size_t slots1 = static_cast<size_t>(c.rs.slots());
+  c.off_part_o = off; off += c.rs.whole_rows() ? 0 : align_up(slots1 * c.blk * d * sizeof(float), 256);
+  c.off_part_lse = off; off += align_up(slots1 * c.blk * sizeof(float), 256);
   c.off_lse = off; off += align_up(static_cast<size_t>(B) * H * Nq * sizeof(float), 256);
   c.off_lse2 = off; off += c.reverse ? align_up(static_cast<size_t>(B) * H * c.NQC * 128 * sizeof(float), 256) : 0;
   const size_t slots = c.reverse ? static_cast<size_t>(c.rev_slots) : static_cast<size_t>(c.NCH);
   c.off_partial = off; off += align_up(slots * B * H * Nk * sizeof(float), 256);
-  c.off_redo = off; off += align_up(items * sizeof(int), 256);
+  c.off_redo = off; off += align_up(slots1 * sizeof(int), 256);
   c.total = off;
   return c;
 }
@@ -610,20 +600,41 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
   float* lse = lse_out != nullptr ? lse_out : reinterpret_cast<float*>(ws + c.off_lse);
   float* partial = reinterpret_cast<float*>(ws + c.off_partial);
   if (launch_pdl(clear_status_kernel, 1, 1, 0, st, status) != cudaSuccess) return AVSA_ERR_CUDA;
-  bool merge_late = false;
-  // ---- pass 1
+  const bool merge = !c.rs.whole_rows();      // some query tiles come in parts
+  const bool merge_late = merge && scores != nullptr && !c.reverse;      // then the merge rides in the call's last grid
+  MergeParams m = {};
+  m.rs = c.rs;
+  m.part_o = part_o;
+  m.part_lse2 = part_lse;
+  m.Nq = Nq;
+  m.H = H;
+  set_merge_rows(m, B * H);
+  m.o = static_cast<__nv_bfloat16*>(o);
+  m.o_sb = q.stride_b;
+  m.o_sh = q.stride_h;
+  m.o_sn = q.stride_n;
+  m.lse = lse;
+  m.n_out = Nq;
+  constexpr int RPB = 128 / (D / 4);
+  const int merge_blocks = (m.total_rows + RPB - 1) / RPB;
+  // ---- pass 1: the persistent fast kernel (one CTA per SM), with the exact-rescaling kernel behind it for the items
+  // whose rows outgrow their first-tile reference
   {
-    CUtensorMap tq, tk, tv;
+    using L = AttnSmem<BLK, D>;
+    using LP = PersistSmem<BLK, D>;
+    CUtensorMap tq, tk, tv, to;
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tv, v.ptr, B, H, Nk, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
-    using L = AttnSmem<BLK, D>;
-    using LP = PersistSmem<BLK, D>;
+    to = tq;      // not used without an output
+    if (o != nullptr && !encode_bf16_tile_map(&to, o, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
     AttnParams prm = {};
     prm.part_o = part_o;
     prm.part_lse2 = part_lse;
-    prm.n_split = c.n_split;
-    prm.tiles_per_split = c.tps;
+    prm.rs = c.rs;
+    prm.store = o != nullptr ? kStoreTile : kStoreNone;
+    prm.n_out = Nq;
+    prm.lse = lse;
     prm.status = status;
     prm.H = H;
     prm.Nq = Nq;
@@ -631,51 +642,22 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     prm.Nk = Nk;
     prm.NKB = c.NKB;
     prm.scale_log2 = scale * 1.4426950408889634f;
-    // Pass 1 runs on the persistent fast kernel (one CTA per SM over the (query tile, key split) items), with the
-    // exact-rescaling kernel behind it for the items whose rows outgrow their first-tile reference.
     int* redo = reinterpret_cast<int*>(ws + c.off_redo);
-    const long long items = static_cast<long long>(B) * H * c.NQT * c.n_split;
-    const int pgrid = persistent_grid(items);
-    if (c.n_split == 1 && o != nullptr) {
-      // the whole key axis fits one work item (few keys): write O and the LSE directly, no partials to merge
-      CUtensorMap to;
-      if (!encode_bf16_tile_map(&to, o, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
-      prm.lse = lse;
-      if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE_DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               LP::kTotal) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE_DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               L::kTotal) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE_DIRECT>, pgrid, kAttnThreads, LP::kTotal, st, tq, tk, tv, to, prm,
-                     redo, nullptr, static_cast<int>(items)) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE_DIRECT>, pgrid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo) !=
-          cudaSuccess)
-        return AVSA_ERR_CUDA;
-    } else {
-      if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               LP::kTotal) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               L::kTotal) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, pgrid, kAttnThreads, LP::kTotal, st, tq, tk, tv, tq, prm, redo,
-                     nullptr, static_cast<int>(items)) != cudaSuccess)
-        return AVSA_ERR_CUDA;
-      if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, pgrid, kAttnThreads, L::kTotal, st, tq, tk, tv, tq, prm, redo) !=
-          cudaSuccess)
-        return AVSA_ERR_CUDA;
-      merge_late = scores != nullptr && !c.reverse;      // then the merge rides in the call's last grid
-      if (!merge_late) {
-        const int total_rows = B * H * Nq;
-        constexpr int RPB = 128 / (D / 4);
-        if (launch_pdl(merge_splits_kernel<BLK, D>, (total_rows + RPB - 1) / RPB, 128, 0, st, part_o, part_lse, c.n_split,
-                       c.NQT, Nq, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h, q.stride_n, lse,
-                       nullptr, 0, Nq) != cudaSuccess)
-          return AVSA_ERR_CUDA;
-      }
-    }
+    const int grid = c.rs.ctas;
+    if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             LP::kTotal) != cudaSuccess)
+      return AVSA_ERR_CUDA;
+    if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) !=
+        cudaSuccess)
+      return AVSA_ERR_CUDA;
+    if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, LP::kTotal, st, tq, tk, tv, to, prm, redo,
+                   nullptr, c.rs.slots()) != cudaSuccess)
+      return AVSA_ERR_CUDA;
+    if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo) !=
+        cudaSuccess)
+      return AVSA_ERR_CUDA;
+    if (merge && !merge_late && launch_pdl(merge_splits_kernel<BLK, D>, merge_blocks, 128, 0, st, m) != cudaSuccess)
+      return AVSA_ERR_CUDA;
   }
   // ---- pass 2, keys resident (many queries, at most 512 keys)
   if (scores != nullptr && c.reverse) {
@@ -719,10 +701,8 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     if (cudaFuncSetAttribute(colsum_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
       return AVSA_ERR_CUDA;
     ColsumParams cp;
-    cp.lse = lse;
-    cp.part_lse2 = merge_late ? part_lse : nullptr;
-    cp.n_split = c.n_split;
-    cp.NQT = c.NQT;
+    cp.part_lse2 = part_lse;
+    cp.rs = c.rs;
     cp.blk = c.blk;
     cp.partial = partial;
     cp.status = status;
@@ -740,12 +720,8 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     const int64_t n = static_cast<int64_t>(B) * Nk;
     const int hs_blocks = static_cast<int>((n + 255) / 256);
     if (merge_late) {
-      const int total_rows = B * H * Nq;
-      constexpr int RPB = 128 / (D / 4);
-      const int merge_blocks = ((total_rows + RPB - 1) / RPB + 1) / 2;
-      if (launch_pdl(cross_finalize_kernel<BLK, D>, hs_blocks + merge_blocks, 256, 0, st, hs_blocks, partial, c.NCH, B, H, Nk,
-                     beta, gamma, scores, part_o, part_lse, c.n_split, c.NQT, Nq, total_rows, static_cast<__nv_bfloat16*>(o),
-                     q.stride_b, q.stride_h, q.stride_n, lse) != cudaSuccess)
+      if (launch_pdl(cross_finalize_kernel<BLK, D>, hs_blocks + (merge_blocks + 1) / 2, 256, 0, st, hs_blocks, partial, c.NCH, B,
+                     H, Nk, beta, gamma, scores, m) != cudaSuccess)
         return AVSA_ERR_CUDA;
     } else {
       if (launch_pdl(head_sum_kernel, hs_blocks, 256, 0, st, partial, c.NCH, B, H, Nk, beta, gamma, scores) != cudaSuccess)

@@ -75,7 +75,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* _
 }
 
 struct ProtPlan {
-  int n_pad, NQT, NKB, n_split, tps;
+  int n_pad, NQT, NKB;
+  RangeSplit rs;
   size_t off_rows, off_qp, off_part_o, off_part_lse, off_redo, total;
 };
 
@@ -85,19 +86,15 @@ static ProtPlan make_prot_plan(int B, int H, int N, int d, int blk, int n_protec
   if (c.NQT < 1) c.NQT = 1;
   c.n_pad = c.NQT * blk;
   c.NKB = (N + blk - 1) / blk;
-  // key-axis splits: work items of about 64 tiles, and at least two waves of 148 items when possible
-  int want = (c.NKB + 63) / 64;
-  const int items1 = B * H * c.NQT;
-  while (items1 * want < 296 && want < c.NKB) want++;
-  c.tps = (c.NKB + want - 1) / want;
-  c.n_split = (c.NKB + c.tps - 1) / c.tps;
+  const long long kv_bytes = 4ll * B * H * N * d;
+  c.rs = make_range_split(B * H, c.NQT, c.NKB, persistent_grid(1 << 30), kv_bytes > kL2KeepBytes);
   size_t off = kStatusBytes;
-  const size_t items = static_cast<size_t>(items1) * c.n_split;
+  const size_t slots = static_cast<size_t>(c.rs.slots());
   c.off_rows = off; off += align_up(static_cast<size_t>(B) * c.n_pad * sizeof(int32_t), 256);
   c.off_qp = off; off += align_up(static_cast<size_t>(B) * H * c.n_pad * d * 2, 256);
-  c.off_part_o = off; off += align_up(items * blk * d * sizeof(float), 256);
-  c.off_part_lse = off; off += align_up(items * blk * sizeof(float), 256);
-  c.off_redo = off; off += align_up(items * sizeof(int), 256);
+  c.off_part_o = off; off += c.rs.whole_rows() ? 0 : align_up(slots * blk * d * sizeof(float), 256);
+  c.off_part_lse = off; off += align_up(slots * blk * sizeof(float), 256);
+  c.off_redo = off; off += align_up(slots * sizeof(int), 256);
   c.total = off;
   return c;
 }
@@ -135,8 +132,15 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   AttnParams prm = {};
   prm.part_o = part_o;
   prm.part_lse2 = part_lse;
-  prm.n_split = c.n_split;
-  prm.tiles_per_split = c.tps;
+  prm.rs = c.rs;
+  prm.store = kStoreRows;
+  prm.o = static_cast<__nv_bfloat16*>(o);
+  prm.o_sb = q.stride_b;
+  prm.o_sh = q.stride_h;
+  prm.o_sn = q.stride_n;
+  prm.row_map = rows;
+  prm.n_out = N;
+  prm.lse = lse;
   prm.status = status;
   prm.H = H;
   prm.Nq = c.n_pad;
@@ -144,21 +148,33 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   prm.Nk = N;
   prm.NKB = c.NKB;
   prm.scale_log2 = scale * 1.4426950408889634f;
-  // persistent fast kernel over the (row tile, key split) items, then the exact kernel for what it handed over
+  // persistent fast kernel over the row tiles and all keys, then the exact kernel for what it handed over
   int* redo = reinterpret_cast<int*>(ws + c.off_redo);
-  const long long items = static_cast<long long>(B) * H * c.NQT * c.n_split;
-  const int grid = persistent_grid(items);
+  const int grid = c.rs.ctas;
   if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, LP::kTotal, st, tq, tk, tv, tq, prm, redo,
-                 nullptr, static_cast<int>(items)) != cudaSuccess)
+                 nullptr, c.rs.slots()) != cudaSuccess)
     return AVSA_ERR_CUDA;
   if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, tq, prm, redo) !=
       cudaSuccess)
     return AVSA_ERR_CUDA;
-  const int total_rows = B * H * c.n_pad;
+  MergeParams m = {};
+  m.rs = c.rs;
+  m.part_o = part_o;
+  m.part_lse2 = part_lse;
+  m.Nq = c.n_pad;
+  m.H = H;
+  set_merge_rows(m, B * H);
+  m.o = static_cast<__nv_bfloat16*>(o);
+  m.o_sb = q.stride_b;
+  m.o_sh = q.stride_h;
+  m.o_sn = q.stride_n;
+  m.lse = lse;
+  m.row_map = rows;
+  m.row_map_stride = c.n_pad;
+  m.n_out = N;
   constexpr int MRPB = 128 / (D / 4);
-  if (launch_pdl(merge_splits_kernel<BLK, D>, (total_rows + MRPB - 1) / MRPB, 128, 0, st, part_o, part_lse, c.n_split, c.NQT,
-                 c.n_pad, H, total_rows, static_cast<__nv_bfloat16*>(o), q.stride_b, q.stride_h, q.stride_n, lse, rows,
-                 c.n_pad, N) != cudaSuccess)
+  if (!c.rs.whole_rows() &&
+      launch_pdl(merge_splits_kernel<BLK, D>, (m.total_rows + MRPB - 1) / MRPB, 128, 0, st, m) != cudaSuccess)
     return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }

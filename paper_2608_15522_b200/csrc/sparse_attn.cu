@@ -159,6 +159,7 @@ extern "C" int avsa_sparse_self_attn(int B, int H, int N, int d, int blk, avsa_b
   prm.H = H;
   prm.Nq = N;
   prm.Nk = N;
+  prm.n_out = N;
   prm.NQT = prm.NKB = (N + blk - 1) / blk;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
   prm.scale_log2 = scale * 1.4426950408889634f;

@@ -509,6 +509,31 @@ def test_cross_attention_long_query_axis_two_chunks():
     _close_scores(_np64(s), want_s, "scores, two query chunks")
 
 
+@pytest.mark.parametrize("B,H,Nq,Nk,d,scores", [
+    (1, 1, 1, 1, 128, True),           # one query, one key
+    (1, 1, 600, 3000, 128, False),     # 5 query tiles in chunks of 4, 24 key tiles cut into twelve ranges
+    (1, 2, 300, 2900, 128, True),      # 3 query tiles, split rows, the LSEs of the score pass from the parts
+    (2, 3, 140, 333, 64, True),        # few tiles: whole rows, written by the tile kernel itself
+    (1, 22, 2427, 200, 128, True),     # reverse: 19 query tiles in chunks of 4, whole rows, score pass over the keys
+    (1, 2, 130, 6400, 64, True),
+])
+def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
+    """Every way the (query tile, key tile) work is cut over the CTAs: whole rows, split rows, chunks that do not divide
+    the query tiles; with O, and with only the LSE asked for (same LSEs)."""
+    g = torch.Generator().manual_seed(Nq * 7 + Nk)
+    q, k, v = (torch.randn((B, H, n, d), generator=g).to(torch.bfloat16) for n in (Nq, Nk, Nk))
+    want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+    o, lse, s, ws = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), want_scores=scores, score_gamma=1.0 / (H * Nq))
+    _status_ok(ws)
+    _close(_np64(o), want_o, "split O")
+    _close_lse(_np64(lse), want_lse, "split lse")
+    if scores:
+        _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "split scores")
+    _, lse2, _, ws2 = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), want_scores=False, want_o=False)
+    _status_ok(ws2)
+    assert torch.equal(lse, lse2)
+
+
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_reverse_direction(name):
     """Video queries attending to audio keys (the other half of the bidirectional pair): outputs, LSE, and the
