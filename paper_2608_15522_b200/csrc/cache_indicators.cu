@@ -41,7 +41,8 @@ __global__ void __launch_bounds__(kIndThreads) l1_partials_kernel(const __nv_bfl
   const __nv_bfloat16* cb = (video ? yhat_v : yhat_a) + b * batch_stride;
   const uint8_t* pb = (video && prot != nullptr) ? prot + static_cast<int64_t>(b) * N : nullptr;
   float* partial = video ? part_v : part_a;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();
+  pdl_launch();
   const int chunks = C / 8;
   float d_all = 0.f, m_all = 0.f, d_p = 0.f, m_p = 0.f;
   for (int row = cta * kIndWarps + warp; row < N; row += ncta * kIndWarps) {
@@ -94,27 +95,12 @@ __global__ void __launch_bounds__(kFinThreads) indicators_finalize_kernel(const 
                                                                   const float* __restrict__ s_anchor, int N,
                                                                   float lambda_p, float lambda_s, float tau, float eps,
                                                                   float* __restrict__ out, StatusRecord* status) {
-  __shared__ float red[kFinThreads][9];
+  __shared__ float red[kFinThreads / 32][9];
   const int b = blockIdx.x, tid = threadIdx.x;
-  asm volatile("griddepcontrol.wait;" ::: "memory");      // the partial sums come from the kernel before
-  if (b == 0 && tid == 0) {
-    status->code = 0;
-    status->where = 0;
-    status->item = 0;
-    status->aux = 0;
-  }
   // nine sums at once, each in a fixed order: thread t takes entries t, t+1024, ...; then a fixed tree
   float acc[9];
 #pragma unroll
   for (int i = 0; i < 9; i++) acc[i] = 0.f;
-  for (int g = tid; g < gv; g += kFinThreads) {
-    const float4 v = *reinterpret_cast<const float4*>(part_v + (static_cast<int64_t>(b) * gv + g) * 4);
-    acc[0] += v.x; acc[1] += v.y; acc[2] += v.z; acc[3] += v.w;
-  }
-  for (int g = tid; g < ga; g += kFinThreads) {
-    const float4 v = *reinterpret_cast<const float4*>(part_a + (static_cast<int64_t>(b) * ga + g) * 4);
-    acc[4] += v.x; acc[5] += v.y;
-  }
   if (s_cur != nullptr && s_anchor != nullptr) {
     const float* sc = s_cur + static_cast<int64_t>(b) * N;
     const float* sa = s_anchor + static_cast<int64_t>(b) * N;
@@ -134,16 +120,42 @@ __global__ void __launch_bounds__(kFinThreads) indicators_finalize_kernel(const 
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < 9; i++) red[tid][i] = acc[i];
-  __syncthreads();
-  for (int off = kFinThreads / 2; off > 0; off >>= 1) {
-    if (tid < off)
-#pragma unroll
-      for (int i = 0; i < 9; i++) red[tid][i] += red[tid + off][i];
-    __syncthreads();
+  // The saliency products above need nothing from the partial-sum grid, which in turn lets this grid start only after
+  // everything before it on the stream is done: they run under its last CTAs (5 of the 11 us this kernel took).
+  pdl_wait();
+  pdl_launch();
+  if (b == 0 && tid == 0) {
+    status->code = 0;
+    status->where = 0;
+    status->item = 0;
+    status->aux = 0;
   }
-  const float* sums = red[0];
+  for (int g = tid; g < gv; g += kFinThreads) {
+    const float4 v = *reinterpret_cast<const float4*>(part_v + (static_cast<int64_t>(b) * gv + g) * 4);
+    acc[0] += v.x; acc[1] += v.y; acc[2] += v.z; acc[3] += v.w;
+  }
+  for (int g = tid; g < ga; g += kFinThreads) {
+    const float4 v = *reinterpret_cast<const float4*>(part_a + (static_cast<int64_t>(b) * ga + g) * 4);
+    acc[4] += v.x; acc[5] += v.y;
+  }
+  // the 1024 threads' sums in a fixed tree: within the warps, then over the 32 warps
+#pragma unroll
+  for (int i = 0; i < 9; i++)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+  if ((tid & 31) == 0)
+#pragma unroll
+    for (int i = 0; i < 9; i++) red[tid >> 5][i] = acc[i];
+  __syncthreads();
+  if (tid < 32) {
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+      acc[i] = red[tid][i];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+    }
+  }
+  const float* sums = acc;
   if (tid == 0) {
     const float dv = sums[0] / (sums[1] + eps);
     const float dp = sums[2] / (sums[3] + eps);
@@ -197,24 +209,12 @@ extern "C" int avsa_cache_indicators(int B, int Nv, int Na, int C, const void* y
   uint8_t* base = static_cast<uint8_t*>(ws);
   float* pv = reinterpret_cast<float*>(base + p.off_v);
   float* pa = reinterpret_cast<float*>(base + p.off_a);
-  l1_partials_kernel<<<dim3(p.gv + p.ga, B), kIndThreads, 0, st>>>(
-      static_cast<const __nv_bfloat16*>(y_v), static_cast<const __nv_bfloat16*>(yhat_v), Nv,
-      static_cast<const __nv_bfloat16*>(y_a), static_cast<const __nv_bfloat16*>(yhat_a), Na, C, prot_tok, p.gv, p.ga, pv,
-      pa);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(B, 1, 1);
-  cfg.blockDim = dim3(kFinThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const float* pvc = pv;
-  const float* pac = pa;
-  if (cudaLaunchKernelEx(&cfg, indicators_finalize_kernel, pvc, p.gv, pac, p.ga, s_cur, s_anchor, Nv, lambda_p,
-                         lambda_s, tau, eps, out, static_cast<StatusRecord*>(ws)) != cudaSuccess)
+  if (launch_pdl(l1_partials_kernel, dim3(p.gv + p.ga, B), kIndThreads, 0, st, static_cast<const __nv_bfloat16*>(y_v),
+                 static_cast<const __nv_bfloat16*>(yhat_v), Nv, static_cast<const __nv_bfloat16*>(y_a),
+                 static_cast<const __nv_bfloat16*>(yhat_a), Na, C, prot_tok, p.gv, p.ga, pv, pa) != cudaSuccess)
+    return AVSA_ERR_CUDA;
+  if (launch_pdl(indicators_finalize_kernel, B, kFinThreads, 0, st, pv, p.gv, pa, p.ga, s_cur, s_anchor, Nv, lambda_p, lambda_s,
+                 tau, eps, out, static_cast<StatusRecord*>(ws)) != cudaSuccess)
     return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
