@@ -1,4 +1,7 @@
-"""ctypes binding of libavsa.so: same names as the C ABI, argument marshalling only.
+"""Binding of libavsa.so: same names as the C ABI, argument marshalling only.
+
+The calls that run on the GPU go through the extension module ``_avsa_host`` (csrc/host_call.cc), which reads the
+tensors' pointers and strides and calls the library; everything else goes through ctypes.
 
 PyTorch appears here for device memory and the current stream; every step of the path runs in the
 library's CUDA kernels.  There is no CPU fallback: without the built library, or on a machine
@@ -7,6 +10,8 @@ without a CUDA device, the calls raise.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -57,6 +62,28 @@ class _Bf16Tensor4(ctypes.Structure):
 
 
 _lib = None
+_host_module = None
+
+
+def _host():
+    """The extension module that marshals the GPU calls, bound to the loaded library."""
+    global _host_module
+    if _host_module is None:
+        lib = load_library()
+        path = next((p for p in (os.path.join(_HERE, "_avsa_host" + e) for e in importlib.machinery.EXTENSION_SUFFIXES)
+                     if os.path.exists(p)), None)
+        if path is None:
+            raise RuntimeError(f"_avsa_host is missing in {_HERE}: run `python -m paper_2608_15522_b200.build` "
+                               "(there is no fallback path)")
+        spec = importlib.util.spec_from_file_location("_avsa_host", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+        module.bind(address(lib.avsa_cross_attn_scores), address(lib.avsa_build_block_mask),
+                    address(lib.avsa_sparse_self_attn), address(lib.avsa_protected_rows_attn),
+                    address(lib.avsa_cache_indicators), torch.bfloat16, torch._C._cuda_getCurrentRawStream)
+        _host_module = module
+    return _host_module
 
 
 def load_library() -> ctypes.CDLL:
@@ -129,10 +156,6 @@ def _t4(x: torch.Tensor) -> _Bf16Tensor4:
     return _Bf16Tensor4(x.data_ptr(), x.stride(0), x.stride(1), x.stride(2))
 
 
-def _null_t4() -> _Bf16Tensor4:
-    return _Bf16Tensor4(None, 0, 0, 0)
-
-
 def _ptr(x: Optional[torch.Tensor]):
     return None if x is None else ctypes.c_void_p(x.data_ptr())
 
@@ -141,9 +164,7 @@ def _stream(device) -> ctypes.c_void_p:
     return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
 
 
-def _workspace(nbytes: int, device, ws: Optional[torch.Tensor]) -> torch.Tensor:
-    if ws is not None:
-        return ws          # the library checks its size
+def _workspace(nbytes: int, device) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
@@ -178,22 +199,20 @@ def avsa_cross_attn_scores_workspace_bytes(B, H, Nq, Nk, d) -> int:
 def avsa_cross_attn_scores(q, k, v, scores=None, score_beta=0.0, score_gamma=1.0, softmax_scale=0.0,
                            want_o=True, want_scores=True, o=None, lse=None, ws=None):
     """Eq. 1-2.  q [B,H,Nq,d], k/v [B,H,Nk,d] bf16 CUDA.  Returns (o, lse, scores, ws)."""
-    lib = load_library()
-    B, H, Nq, d = q.shape
-    Nk = k.shape[2]
-    dev = q.device
     if want_o and o is None:
-        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=dev)
+        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
     if lse is None:
-        lse = torch.empty((B, H, Nq), dtype=torch.float32, device=dev)
+        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
     if want_scores and scores is None:
-        scores = torch.empty((B, Nk), dtype=torch.float32, device=dev)
+        scores = torch.empty((q.shape[0], k.shape[2]), dtype=torch.float32, device=q.device)
         score_beta = 0.0
-    ws = _workspace(avsa_cross_attn_scores_workspace_bytes(B, H, Nq, Nk, d), dev, ws)
-    st = lib.avsa_cross_attn_scores(B, H, Nq, Nk, d, _t4(q), _t4(k), _t4(v), _ptr(o if want_o else None), _ptr(lse),
-                                    _ptr(scores if want_scores else None), float(score_beta), float(score_gamma),
-                                    float(softmax_scale), _ptr(ws), ws.numel(), _stream(dev))
-    _check(st, "avsa_cross_attn_scores")
+    if ws is None:
+        B, H, Nq, d = q.shape
+        ws = _workspace(avsa_cross_attn_scores_workspace_bytes(B, H, Nq, k.shape[2], d), q.device)
+    st = (_host_module or _host()).cross(q, k, v, o if want_o else None, lse, scores if want_scores else None, score_beta,
+                                         score_gamma, softmax_scale, ws)
+    if st != AVSA_OK:
+        raise AvsaError(st, "avsa_cross_attn_scores")
     return o, lse, scores, ws
 
 
@@ -208,37 +227,36 @@ def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTE
     With AVSA_USE_GIVEN_BLOCK_SCORES pass ``block_scores`` [B,H,NB,NB] fp32 and ``shape`` = (B,H,N,d);
     q and k may then be None.
     """
-    lib = load_library()
     if q is not None:
-        B, H, N, d = q.shape
+        B, H, N, d = shape = q.shape
         dev = q.device
     else:
         B, H, N, d = shape
         dev = block_scores.device
-    NB = (N + blk - 1) // blk
     out = out or {}
     if block_scores is None:
         block_scores = out.get("block_scores")
+    col_idx = out.get("col_idx")
+    col_cnt = out.get("col_cnt")
+    prot_tok = out.get("prot_tok")
+    prot_blk = out.get("prot_blk")
+    NB = (N + blk - 1) // blk
     if block_scores is None:
         block_scores = torch.empty((B, H, NB, NB), dtype=torch.float32, device=dev)
-    col_idx = out.get("col_idx")
     if col_idx is None:
         col_idx = torch.empty((B, H, NB, NB), dtype=torch.int32, device=dev)
-    col_cnt = out.get("col_cnt")
     if col_cnt is None:
         col_cnt = torch.empty((B, H, NB), dtype=torch.int32, device=dev)
-    prot_tok = out.get("prot_tok")
     if prot_tok is None:
         prot_tok = torch.empty((B, N), dtype=torch.uint8, device=dev)
-    prot_blk = out.get("prot_blk")
     if prot_blk is None:
         prot_blk = torch.empty((B, NB), dtype=torch.uint8, device=dev)
-    ws = _workspace(avsa_build_block_mask_workspace_bytes(B, H, N, d, blk), dev, ws)
-    st = lib.avsa_build_block_mask(B, H, N, d, blk, _t4(q) if q is not None else _null_t4(),
-                                   _t4(k) if k is not None else _null_t4(), _ptr(scores), int(n_protect), int(k_keep),
-                                   int(flags), float(softmax_scale), _ptr(block_scores), _ptr(col_idx), _ptr(col_cnt),
-                                   _ptr(prot_tok), _ptr(prot_blk), _ptr(ws), ws.numel(), _stream(dev))
-    _check(st, "avsa_build_block_mask")
+    if ws is None:
+        ws = _workspace(avsa_build_block_mask_workspace_bytes(B, H, N, d, blk), dev)
+    st = (_host_module or _host()).mask(tuple(shape), blk, q, k, scores, n_protect, k_keep, flags, softmax_scale, block_scores,
+                                        col_idx, col_cnt, prot_tok, prot_blk, ws)
+    if st != AVSA_OK:
+        raise AvsaError(st, "avsa_build_block_mask")
     return dict(block_scores=block_scores, col_idx=col_idx, col_cnt=col_cnt, prot_tok=prot_tok, prot_blk=prot_blk, ws=ws)
 
 
@@ -270,17 +288,16 @@ def avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk) -> int:
 
 def avsa_sparse_self_attn(q, k, v, col_idx, col_cnt, blk, softmax_scale=0.0, want_lse=False, o=None, lse=None, ws=None):
     """Eq. 10.  Returns (o, lse or None, ws)."""
-    lib = load_library()
-    B, H, N, d = q.shape
-    dev = q.device
     if o is None:
-        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=dev)
+        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
     if want_lse and lse is None:
-        lse = torch.empty((B, H, N), dtype=torch.float32, device=dev)
-    ws = _workspace(avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk), dev, ws)
-    st = lib.avsa_sparse_self_attn(B, H, N, d, blk, _t4(q), _t4(k), _t4(v), _ptr(col_idx), _ptr(col_cnt), _ptr(o),
-                                   _ptr(lse), float(softmax_scale), _ptr(ws), ws.numel(), _stream(dev))
-    _check(st, "avsa_sparse_self_attn")
+        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
+    if ws is None:
+        B, H, N, d = q.shape
+        ws = _workspace(avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk), q.device)
+    st = (_host_module or _host()).sparse(q, k, v, col_idx, col_cnt, blk, o, lse, softmax_scale, ws)
+    if st != AVSA_OK:
+        raise AvsaError(st, "avsa_sparse_self_attn")
     return o, lse, ws
 
 
@@ -307,13 +324,12 @@ def avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, n_protect) -> int:
 def avsa_protected_rows_attn(q, k, v, prot_tok, n_protect, blk, o, lse=None, softmax_scale=0.0, ws=None):
     """Eq. 9 / Eq. 11 on tokens: overwrites the rows of the protected tokens in ``o`` (and ``lse``) with dense
     attention rows.  Returns ws."""
-    lib = load_library()
-    B, H, N, d = q.shape
-    dev = q.device
-    ws = _workspace(avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, int(n_protect)), dev, ws)
-    st = lib.avsa_protected_rows_attn(B, H, N, d, blk, _t4(q), _t4(k), _t4(v), _ptr(prot_tok), int(n_protect), _ptr(o),
-                                      _ptr(lse), float(softmax_scale), _ptr(ws), ws.numel(), _stream(dev))
-    _check(st, "avsa_protected_rows_attn")
+    if ws is None:
+        B, H, N, d = q.shape
+        ws = _workspace(avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, int(n_protect)), q.device)
+    st = (_host_module or _host()).protected_rows(q, k, v, prot_tok, n_protect, blk, o, lse, softmax_scale, ws)
+    if st != AVSA_OK:
+        raise AvsaError(st, "avsa_protected_rows_attn")
     return ws
 
 
@@ -325,18 +341,13 @@ def avsa_cache_indicators(y_v, yhat_v, y_a, yhat_a, prot_tok=None, s_cur=None, s
                           lambda_s=0.1, tau=0.2, eps=1e-6, out=None, ws=None):
     """Eq. 12-15.  y_v/yhat_v bf16 [B,Nv,C], y_a/yhat_a bf16 [B,Na,C] (contiguous).  Returns (out [B,8], ws) with
     out[:, :6] = dv, da, dp, ds, dsync, reuse."""
-    lib = load_library()
-    B, Nv, C = y_v.shape
-    Na = y_a.shape[1]
-    dev = y_v.device
-    for t in (y_v, yhat_v, y_a, yhat_a):
-        if t.dtype != torch.bfloat16 or not t.is_contiguous() or not t.is_cuda:
-            raise ValueError("expected contiguous CUDA bf16 tensors")
     if out is None:
-        out = torch.empty((B, 8), dtype=torch.float32, device=dev)
-    ws = _workspace(avsa_cache_indicators_workspace_bytes(B, Nv, Na, C), dev, ws)
-    st = lib.avsa_cache_indicators(B, Nv, Na, C, _ptr(y_v), _ptr(yhat_v), _ptr(y_a), _ptr(yhat_a), _ptr(prot_tok),
-                                   _ptr(s_cur), _ptr(s_anchor), float(lambda_p), float(lambda_s), float(tau),
-                                   float(eps), _ptr(out), _ptr(ws), ws.numel(), _stream(dev))
-    _check(st, "avsa_cache_indicators")
+        out = torch.empty((y_v.shape[0], 8), dtype=torch.float32, device=y_v.device)
+    if ws is None:
+        B, Nv, C = y_v.shape
+        ws = _workspace(avsa_cache_indicators_workspace_bytes(B, Nv, y_a.shape[1], C), y_v.device)
+    st = (_host_module or _host()).indicators(y_v, yhat_v, y_a, yhat_a, prot_tok, s_cur, s_anchor, lambda_p, lambda_s, tau, eps,
+                                              out, ws)
+    if st != AVSA_OK:
+        raise AvsaError(st, "avsa_cache_indicators")
     return out, ws

@@ -1,14 +1,16 @@
-"""Builds libavsa.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libavsa.so and the host extension that calls it in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libavsa.so")
+HOST = os.path.join(HERE, "_avsa_host" + sysconfig.get_config_var("EXT_SUFFIX"))      # marshalling for this interpreter
 SOURCES = ["api.cu", "mask.cu", "sparse_attn.cu", "cross_attn.cu", "protected_rows.cu", "cache_indicators.cu"]
 HEADERS = sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")) + [os.path.join("..", "..", "include", "avsa.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -23,15 +25,24 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST))
+    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["host_call.cc"]]
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def _build_host() -> None:
+    src = os.path.join(CSRC, "host_call.cc")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wall", "-Wno-cast-function-type",
+           "-I" + sysconfig.get_paths()["include"], src, "-o", HOST]
+    r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on host_call.cc:\n{r.stdout}")
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compiles every .cu of the library and links libavsa.so; returns its path."""
+    """Compiles every .cu of the library, links libavsa.so and builds the host extension; returns the library's path."""
     if not force and not _stale():
         return LIB
     nvcc = _nvcc()
@@ -54,6 +65,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}")
+    _build_host()
     return LIB
 
 
