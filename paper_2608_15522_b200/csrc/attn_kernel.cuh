@@ -587,6 +587,7 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
   double best_cost = 0.0;
   // (more than 32 query tiles side by side share no more, and small chunks divide the CTAs better)
   const int cmax = NQT < 32 ? NQT : 32;
+  const double streams = ctas > 70 * cmax ? static_cast<double>(ctas) / cmax : 70.0;      // (one per CTA cannot be helped)
   for (int chunk = cmax < ctas ? cmax : ctas; chunk >= 1; chunk--) {
     RangeSplit r = {};
     r.chunk = chunk;
@@ -605,7 +606,7 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
       r.L = static_cast<int>(L);
       r.groups = static_cast<int>((tiles + L - 1) / L);
       r.ctas = r.groups * chunk;
-      const double pace = out_of_l2 && r.groups > 70 ? r.groups / 70.0 : 1.0;
+      const double pace = out_of_l2 && r.groups > streams ? r.groups / streams : 1.0;
       const double segs = v == 0 ? static_cast<double>(L / NKB) : static_cast<double>(L) / NKB + 1.0;
       const double cost = 1.08 * L * pace + 4.0 * segs + (v == 0 ? 0.0 : 4.0 + 0.1 * NKB / L);
       if (best.L == 0 || cost < best_cost * 0.999) {

@@ -925,3 +925,24 @@ def test_a_wait_that_nothing_ends_times_out_and_leaves_the_context_usable():
     NB = w.n_blocks
     idx = np.broadcast_to(np.arange(NB, dtype=np.int32), (w.B, w.H, NB, NB)).copy()
     _run_sparse_case(w, 1, idx, np.full((w.B, w.H, NB), NB, np.int32))
+
+
+@pytest.mark.parametrize("B,H,N,d,n_protect", [(2, 1, 1007, 64, 37), (2, 2, 513, 128, 1), (1, 3, 2600, 64, 700), (3, 1, 130, 128, 130)])
+def test_protected_rows_odd_lengths(B, H, N, d, n_protect):
+    """Flags at any alignment (odd N, several batch items), one to all rows: the flagged rows are dense rows, the others
+    stay as they were, with and without an LSE."""
+    g = torch.Generator().manual_seed(N + n_protect)
+    q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    flags = torch.zeros((B, N), dtype=torch.uint8)
+    for b in range(B):
+        flags[b, torch.randperm(N, generator=g)[:n_protect]] = 1
+    o = torch.full((B, H, N, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((B, H, N), 7.0, dtype=torch.float32, device="cuda")
+    ws = av.avsa_protected_rows_attn(q.cuda(), k.cuda(), v.cuda(), flags.cuda(), n_protect, d, o, lse=lse)
+    _status_ok(ws)
+    want_o, want_l = orc.dense_attention(_np64(q), _np64(k), _np64(v))
+    on = flags.bool().numpy()[:, None, :].repeat(H, axis=1)
+    got_o, got_l = _np64(o), _np64(lse)
+    _close(got_o[on], want_o[on], "protected rows O")
+    _close_lse(got_l[on], want_l[on], "protected rows lse")
+    assert (got_o[~on] == 7.0).all() and (got_l[~on] == 7.0).all()
