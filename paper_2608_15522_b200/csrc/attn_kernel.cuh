@@ -648,32 +648,43 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
   return best;
 }
 
+// The roles of the tile kernels redistribute the registers that the CTA was launched with; this puts them back.
+__device__ __forceinline__ void attn_launch_regs() {
+  if (threadIdx.x < 128) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 168;");
+  }
+  __syncthreads();
+}
+
+// attn_fwd_body in a CTA at its launch register shares, with idle shared memory and no tensor memory, as often as needed
+// (lists that reach it have been checked before: it does not refuse them)
+template <int BLK, int D, int MODE>
+__device__ __forceinline__ void attn_exact_item(const CUtensorMap* tmq, const CUtensorMap* tmk, const CUtensorMap* tmv,
+                                                const CUtensorMap* tmo, const AttnParams& p, int item) {
+  using L = AttnSmem<BLK, D>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  attn_fwd_body<BLK, D, MODE>(tmq, tmk, tmv, tmo, p, item);
+  attn_launch_regs();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < L::kNumBars; i++) mbar_inval(smem_u32(smem + L::kBars) + i * 8);
+  }
+  __syncthreads();
+}
+
 // Exact-rescaling pass behind the fast kernels: recomputes the work items they listed (normally none: then
 // every CTA of this small grid returns at once).  CTA c takes entries c, c + gridDim.x, ...
-template <int BLK, int D, int MODE = MODE_LIST>
+template <int BLK, int D, int MODE>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_redo_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                  const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmo,
                  const AttnParams p, const int* __restrict__ redo_list) {
-  using L = AttnSmem<BLK, D>;
-  extern __shared__ __align__(1024) uint8_t smem[];
   pdl_wait();
   pdl_launch();
   const int n_redo = p.status->redo_count;
-  const int warp = threadIdx.x >> 5;
   for (int k = blockIdx.x; k < n_redo; k += gridDim.x) {
-    attn_fwd_body<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p, redo_list[k]);
-    // back to the launch state for the next item: every warp at the launch register count, barriers invalidated
-    if (warp < 4) {
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
-    } else {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 168;");
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int i = 0; i < L::kNumBars; i++) mbar_inval(smem_u32(smem + L::kBars) + i * 8);
-    }
-    __syncthreads();
+    attn_exact_item<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p, redo_list[k]);
   }
 }
 

@@ -30,6 +30,10 @@
 // A row whose sum, relative to m_ref, ends above 2^64 (or not finite) outgrew its reference: its work item is
 // appended to `redo_list` (count in the status record) and attn_redo_kernel, a small grid launched behind this
 // kernel, recomputes the listed items with exact rescaling.  List validation and bounded waits as in attn_fwd_body.
+//
+// FOLD: for short calls the CTA recomputes its own items itself once the queue is empty, and the redo grid is not
+// launched at all (2.5 us of host time and 1.7 us on the device, where the smallest layer-step takes 30).  Only for short
+// calls, because the exact body inside the kernel costs the fast roles 3 % of their pace, even as a function of its own.
 #pragma once
 #include "attn_kernel.cuh"
 
@@ -57,8 +61,27 @@ struct PersistSmem {
   static constexpr int kStats = kBars + kNumBars * 8;          // float mref[128], lsum[2][128]
   static constexpr int kItems = kStats + 3 * 128 * 4;          // AttnItem[kPRing], two redo flags
   static constexpr int kMisc = kItems + 32 * kPRing + 16;      // tmem base, stop flag
-  static constexpr int kTotal = kMisc + 16;
+  // FOLD: count, then the items to recompute, above the memory that attn_fwd_body works in
+  static constexpr int kRedo = kMisc + 16 > AttnSmem<BLK, D>::kTotal ? kMisc + 16 : AttnSmem<BLK, D>::kTotal;
+  static constexpr int kRedoCap = 192;
+  static constexpr int kTotal = kRedo + 16 + kRedoCap * 4;
+  static_assert(kRedo % 16 == 0 && kTotal <= 232448, "shared memory of a CTA exceeded");
 };
+
+// Calls of at most this many (query tile, key tile) pairs per CTA run with FOLD (with lists, of which a third or so is
+// kept; without, half as many: 45 tiles a CTA were 72.5 us with FOLD and 71.0 without).  Their few items fit the lists of
+// the CTAs: 148 x 64 items at most, against 148 x 188 places (a CTA whose list is full takes no more items).
+constexpr int kFoldTiles = 64;
+inline bool fold_redo(long long tile_pairs) { return tile_pairs <= static_cast<long long>(kFoldTiles) * persistent_grid(1 << 30); }
+
+template <int BLK, int D, int MODE>
+__device__ __noinline__ void persist_exact_phase(const CUtensorMap* tmq, const CUtensorMap* tmk, const CUtensorMap* tmv,
+                                                 const CUtensorMap* tmo, const AttnParams& p) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const volatile int* mine = reinterpret_cast<const volatile int*>(smem + PersistSmem<BLK, D>::kRedo);
+  const int n = mine[0];
+  for (int i = 0; i < n; i++) attn_exact_item<BLK, D, MODE>(tmq, tmk, tmv, tmo, p, mine[4 + i]);
+}
 
 enum PersistWhere { kPersistItem = 71, kPersistItemEmpty, kPersistQEmpty, kPersistOFull, kPersistOFree, kPersistLsum, kPersistStage };
 
@@ -72,7 +95,7 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&r)[8]) 
 // (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE: the CTA's items are its segments of
 // the stream described at RangeSplit, fixed by its index; output bf16 rows where the key axis is not split, else
 // normalised fp32 partials for merge_splits_rows, and the log2 LSE of the range.
-template <int BLK, int D, int MODE>
+template <int BLK, int D, int MODE, bool FOLD>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmo,
@@ -113,7 +136,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   constexpr int REDO = 8 * kPRing;
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + L::kMisc);   // [0] tmem base, [1] stop
 
+  volatile int* mine = reinterpret_cast<volatile int*>(smem + L::kRedo);
+
   if (tid == 0) {
+    if (FOLD) mine[0] = 0;
     for (int s = 0; s < kPQB; s++) {
       mbar_init(BAR(Q_FULL + s), 1);
       mbar_init(BAR(Q_EMPTY + s), 1);
@@ -156,7 +182,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   }
   if (warp == 2) {
     tmem_alloc(smem_u32(smem + L::kMisc), 512);
-    tmem_relinquish();
+    if (!FOLD) tmem_relinquish();      // (attn_fwd_body allocates again)
   }
   tc_fence_before();
   __syncthreads();
@@ -277,6 +303,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         }
         // The CTA's first item is its own index, the others come off the queue behind those of the whole grid: with
         // one item or less per CTA, a CTA that is a little early must not take a second one from a late CTA.
+        if (FOLD && __any_sync(FULLM, mine[0] >= L::kRedoCap - kPRing)) break;
         if (!first) {
           if (lane == 0) id = gridDim.x + atomicAdd(&p.status->next_item, 1);
           id = __shfl_sync(FULLM, id, 0);
@@ -579,7 +606,13 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       if (!ok) break;
       if (tid == 128) {
         items[REDO + (n & 1)] = 0;
-        if (redo) redo_list[atomicAdd(&p.status->redo_count, 1)] = it.item;
+        if (redo) {
+          redo_list[atomicAdd(&p.status->redo_count, 1)] = it.item;
+          if (FOLD) {
+            mine[4 + mine[0]] = it.item;
+            mine[0] = mine[0] + 1;
+          }
+        }
       }
       ok = __all_sync(FULLM, wait_or_stop(O_FULL, n & 1, kPersistOFull, n));
       if (!ok) break;
@@ -657,6 +690,29 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   tc_fence_before();
   __syncthreads();
   if (warp == 2) tmem_dealloc(tmem, 512);
+  if (FOLD && mine[0] > 0 && misc[1] == 0u) {          // uniform over the CTA; hardly ever taken
+    if (tid == 0) {
+      for (int i = 0; i < L::kNumBars; i++) mbar_inval(bar0 + i * 8);
+    }
+    attn_launch_regs();
+    persist_exact_phase<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p);
+  }
+}
+
+// The persistent kernel and, unless it recomputes its items itself, the redo grid behind it.
+template <int BLK, int D, int MODE>
+inline bool launch_attention(int grid, bool fold, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
+                             const CUtensorMap& tv, const CUtensorMap& to, const AttnParams& prm, int* redo, const int* order,
+                             int n_items) {
+  using L = PersistSmem<BLK, D>;
+  auto kernel = fold ? attn_persist_kernel<BLK, D, MODE, true> : attn_persist_kernel<BLK, D, MODE, false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) != cudaSuccess) return false;
+  if (launch_pdl(kernel, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo, order, n_items) != cudaSuccess) return false;
+  if (fold) return true;
+  constexpr int kExactSmem = AttnSmem<BLK, D>::kTotal;
+  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kExactSmem) != cudaSuccess)
+    return false;
+  return launch_pdl(attn_redo_kernel<BLK, D, MODE>, grid, kAttnThreads, kExactSmem, st, tq, tk, tv, to, prm, redo) == cudaSuccess;
 }
 
 }  // namespace avsa

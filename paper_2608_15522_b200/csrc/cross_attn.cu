@@ -620,11 +620,9 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
   m.n_out = Nq;
   constexpr int RPB = 128 / (D / 4);
   const int merge_blocks = (m.total_rows + RPB - 1) / RPB;
-  // ---- pass 1: the persistent fast kernel (one CTA per SM), with the exact-rescaling kernel behind it for the items
-  // whose rows outgrow their first-tile reference
+  // ---- pass 1: the persistent fast kernel (one CTA per SM); items whose rows outgrow their first-tile reference are
+  // recomputed with exact rescaling
   {
-    using L = AttnSmem<BLK, D>;
-    using LP = PersistSmem<BLK, D>;
     CUtensorMap tq, tk, tv, to;
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
@@ -646,18 +644,8 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     prm.NKB = c.NKB;
     prm.scale_log2 = scale * 1.4426950408889634f;
     int* redo = reinterpret_cast<int*>(ws + c.off_redo);
-    const int grid = c.rs.ctas;
-    if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             LP::kTotal) != cudaSuccess)
-      return AVSA_ERR_CUDA;
-    if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) !=
-        cudaSuccess)
-      return AVSA_ERR_CUDA;
-    if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, LP::kTotal, st, tq, tk, tv, to, prm, redo,
-                   nullptr, c.rs.slots()) != cudaSuccess)
-      return AVSA_ERR_CUDA;
-    if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo) !=
-        cudaSuccess)
+    if (!launch_attention<BLK, D, MODE_RANGE>(c.rs.ctas, fold_redo(2ll * B * H * c.NQT * c.NKB), st, tq, tk, tv, to,
+                                              prm, redo, nullptr, c.rs.slots()))
       return AVSA_ERR_CUDA;
     if (merge && !merge_late && launch_pdl(merge_splits_kernel<BLK, D>, merge_blocks, 128, 0, st, m) != cudaSuccess)
       return AVSA_ERR_CUDA;

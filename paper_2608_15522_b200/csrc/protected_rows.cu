@@ -145,14 +145,6 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
     return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tk, k.ptr, B, H, N, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tv, v.ptr, B, H, N, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
-  using L = AttnSmem<BLK, D>;
-  using LP = PersistSmem<BLK, D>;
-  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           L::kTotal) != cudaSuccess)
-    return AVSA_ERR_CUDA;
-  if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           LP::kTotal) != cudaSuccess)
-    return AVSA_ERR_CUDA;
   AttnParams prm = {};
   prm.part_o = part_o;
   prm.part_lse2 = part_lse;
@@ -172,14 +164,9 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   prm.Nk = N;
   prm.NKB = c.NKB;
   prm.scale_log2 = scale * 1.4426950408889634f;
-  // persistent fast kernel over the row tiles and all keys, then the exact kernel for what it handed over
   int* redo = reinterpret_cast<int*>(ws + c.off_redo);
-  const int grid = c.rs.ctas;
-  if (launch_pdl(attn_persist_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, LP::kTotal, st, tq, tk, tv, tq, prm, redo,
-                 nullptr, c.rs.slots()) != cudaSuccess)
-    return AVSA_ERR_CUDA;
-  if (launch_pdl(attn_redo_kernel<BLK, D, MODE_RANGE>, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, tq, prm, redo) !=
-      cudaSuccess)
+  if (!launch_attention<BLK, D, MODE_RANGE>(c.rs.ctas, fold_redo(2ll * B * H * c.NQT * c.NKB), st, tq, tk, tv, tq,
+                                            prm, redo, nullptr, c.rs.slots()))
     return AVSA_ERR_CUDA;
   MergeParams m = {};
   m.rs = c.rs;

@@ -100,22 +100,11 @@ static int launch_sparse_attn(int B, int H, int N, const avsa_bf16_4d& q, const 
   if (!encode_bf16_tile_map(&tk, k.ptr, B, H, N, D, k.stride_b, k.stride_h, k.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tv, v.ptr, B, H, N, D, v.stride_b, v.stride_h, v.stride_n, BLK)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&to, o, B, H, N, D, q.stride_b, q.stride_h, q.stride_n, BLK)) return AVSA_ERR_CUDA;
-  // The persistent fast kernel first; it lists the (rare) work items whose rows outgrow its fixed reference
-  // maxima, and the exact-rescaling kernel behind it recomputes exactly those.
+  // The persistent fast kernel lists the (rare) work items whose rows outgrow its fixed reference maxima; exactly those
+  // are recomputed with exact rescaling.
   const long long items = static_cast<long long>(prm.NQT) * H * B;
-  using L = AttnSmem<BLK, D>;
-  using LP = PersistSmem<BLK, D>;
-  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) !=
-      cudaSuccess)
-    return AVSA_ERR_CUDA;
-  if (cudaFuncSetAttribute(attn_persist_kernel<BLK, D, MODE_LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           LP::kTotal) != cudaSuccess)
-    return AVSA_ERR_CUDA;
-  if (launch_pdl(attn_persist_kernel<BLK, D, MODE_LIST>, persistent_grid(items), kAttnThreads, LP::kTotal, st, tq, tk, tv,
-                 to, prm, redo, redo + items, static_cast<int>(items)) != cudaSuccess)
-    return AVSA_ERR_CUDA;
-  if (launch_pdl(attn_redo_kernel<BLK, D, MODE_LIST>, persistent_grid(items), kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm,
-                 redo) != cudaSuccess)
+  if (!launch_attention<BLK, D, MODE_LIST>(persistent_grid(items), fold_redo(items * prm.NKB), st, tq, tk, tv, to, prm, redo,
+                                           redo + items, static_cast<int>(items)))
     return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }

@@ -946,3 +946,38 @@ def test_protected_rows_odd_lengths(B, H, N, d, n_protect):
     _close(got_o[on], want_o[on], "protected rows O")
     _close_lse(got_l[on], want_l[on], "protected rows lse")
     assert (got_o[~on] == 7.0).all() and (got_l[~on] == 7.0).all()
+
+
+@pytest.mark.parametrize("heads", [20, 40])
+def test_rows_that_outgrow_their_reference_in_short_and_long_calls(heads):
+    """Steeply growing logits: a short call recomputes such items inside the tile kernel, a long one in a grid of its
+    own (more than 64 tile pairs per SM, 32 without lists); list and range modes."""
+    d, n, na = 128, 2070, 300
+    g = torch.Generator().manual_seed(heads)
+    q, k, v = (torch.randn((1, heads, n, d), generator=g) for _ in range(3))
+    u = 1.0 / np.sqrt(d)
+    q = (q + 8.0 * u).to(torch.bfloat16)
+    ramp = torch.arange(n, dtype=torch.float32).div(d, rounding_mode="floor") * 16.0
+    k = (k + (ramp * u).view(1, 1, -1, 1)).to(torch.bfloat16)
+    v = v.to(torch.bfloat16)
+    NB = (n + d - 1) // d
+    idx = np.broadcast_to(np.arange(NB, dtype=np.int32), (1, heads, NB, NB)).copy()
+    cnt = np.full((1, heads, NB), NB, np.int32)
+    cnt[:, :, ::2] = 3
+    o, lse, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(),
+                                          torch.from_numpy(cnt).cuda(), d, want_lse=True)
+    _status_ok(ws)
+    n_redo, items = av.avsa_sparse_self_attn_redo_items(ws)
+    assert n_redo >= heads * (NB // 2) and len(set(items.tolist())) == n_redo
+    hs = [0, heads - 1]
+    want_o, want_l = orc.masked_attention(_np64(q)[:, hs], _np64(k)[:, hs], _np64(v)[:, hs], idx[:, hs], cnt[:, hs], d)
+    _close(_np64(o)[:, hs], want_o, "outgrown O")
+    _close_lse(_np64(lse)[:, hs], want_l, "outgrown lse")
+    qa = q[:, :, :na].contiguous()
+    kc, vc = (torch.cat([t] * 5, dim=2) if heads > 20 else t for t in (k, v))
+    oc, lc, _, wc = av.avsa_cross_attn_scores(qa.cuda(), kc.cuda(), vc.cuda(), want_scores=False)
+    _status_ok(wc)
+    assert av.avsa_redo_count(wc) > 0
+    want_o, want_l, _ = orc.cross_attention(_np64(qa)[:, hs], _np64(kc)[:, hs], _np64(vc)[:, hs])
+    _close(_np64(oc)[:, hs], want_o, "outgrown cross O")
+    _close_lse(_np64(lc)[:, hs], want_l, "outgrown cross lse")
