@@ -270,67 +270,53 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
 // ------------------------------------------------------------------------------------------------
 // (iv) per-(head, query block) top-k_keep of a block-score row, protection OR (Eq. 9), ascending
 // list emission.  One warp per row; the row's keys live in registers (KPL per lane, element j*32+lane
-// in slot j).  The radix select stops as soon as the bin that holds the k-th key is taken whole.
-// `src` is the row of block scores (global or shared memory), `bins` 256 ints of shared memory owned
-// by this warp.
+// in slot j).  The k-th largest key is found bit by bit from the highest bit in which the row's keys differ, counting the
+// keys at or above a candidate over the warp, and the search stops at the first candidate with exactly k above it: a
+// dozen rounds of about 16 instructions for a row of 256 distinct scores.  (A radix select with shared-memory histograms
+// took some 2000 instructions a row; on the Ovi-class shape, 6144 rows, the SMs issued 11 us of them.)
+// `src` is the row of block scores (global or shared memory).
 // ------------------------------------------------------------------------------------------------
 template <int KPL>
 __device__ __forceinline__ void select_row(const float* src, const uint8_t* __restrict__ pb, bool row_prot, int NB,
-                                           int k_keep, int protect_cols, int* bins, int lane,
-                                           int32_t* __restrict__ out, int32_t* __restrict__ cnt_out) {
+                                           int k_keep, int protect_cols, int lane, int32_t* __restrict__ out,
+                                           int32_t* __restrict__ cnt_out) {
   const unsigned lt = (1u << lane) - 1u;
   const bool keep_all = row_prot || k_keep >= NB;
   uint32_t keys[KPL];
   uint32_t T = 0;
-  int want = 0;
+  int want = 0;      // keys equal to T that are taken, lowest index first
   if (!keep_all) {
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
 #pragma unroll
     for (int j = 0; j < KPL; j++) {
       const int i = j * 32 + lane;
-      keys[j] = (i < NB) ? rank_key(src[i]) : 0u;
+      keys[j] = (i < NB) ? rank_key(src[i]) : 0u;      // 0 is below every key
+      kmax = max(kmax, keys[j]);
+      if (i < NB) kmin = min(kmin, keys[j]);
     }
-    uint32_t prefix = 0, mask = 0;
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    T = kmax;
     want = k_keep;
-    for (int pass = 0; pass < 4; pass++) {
-      const int shift = 24 - 8 * pass;
-      // digit range of the keys: when they all share the leading byte (sign and high exponent bits: the usual
-      // case) the first pass needs no histogram at all; later bytes hardly ever agree, so only it is checked
-      if (pass == 0) {
-        uint32_t dmin = 255u, dmax = 0u;
+    if (kmin != kmax) {
+      int bit = 31 - __clz(kmin ^ kmax);
+      T = kmax & ~((2u << bit) - 1u);      // what all keys share above that bit
+      int above = 0;                       // keys above every value that T can still take
+      for (; bit >= 0; bit--) {
+        const uint32_t cand = T | (1u << bit);
+        int c = 0;
 #pragma unroll
-        for (int j = 0; j < KPL; j++) {
-          const uint32_t dg = keys[j] >> 24;
-          if (j * 32 + lane < NB) {
-            dmin = min(dmin, dg);
-            dmax = max(dmax, dg);
-          }
-        }
-        dmin = __reduce_min_sync(0xffffffffu, dmin);
-        dmax = __reduce_max_sync(0xffffffffu, dmax);
-        if (dmin == dmax) {
-          prefix = dmin << 24;
-          mask = 255u << 24;
-          continue;
+        for (int j = 0; j < KPL; j++) c += keys[j] >= cand ? 1 : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c >= k_keep) {
+          T = cand;
+          if (c == k_keep) break;          // exactly the keys at or above T
+        } else {
+          above = c;
         }
       }
-#pragma unroll
-      for (int i = 0; i < 8; i++) bins[i * 32 + lane] = 0;
-      __syncwarp();
-#pragma unroll
-      for (int j = 0; j < KPL; j++) {
-        const bool in = (j * 32 + lane < NB) && ((keys[j] & mask) == prefix);
-        if (in) atomicAdd(&bins[(keys[j] >> shift) & 255u], 1);
-      }
-      __syncwarp();
-      int dg, ab, ib;
-      warp_pick_digit(bins, want, lane, dg, ab, ib);
-      want -= ab;
-      prefix |= static_cast<uint32_t>(dg) << shift;
-      mask |= 255u << shift;
-      __syncwarp();
-      if (ib == want) break;     // the whole bin is taken
+      want = bit >= 0 ? NB : k_keep - above;
     }
-    T = prefix;
   }
   int pos = 0, eq_seen = 0;
 #pragma unroll
@@ -364,7 +350,6 @@ __global__ void __launch_bounds__(128) row_select_kernel(const float* __restrict
                                                          int H, int NB, int k_keep, int protect_rows,
                                                          int protect_cols, int total_rows, int32_t* __restrict__ col_idx,
                                                          int32_t* __restrict__ col_cnt) {
-  __shared__ int all_bins[4][256];
   pdl_wait();   // the block flags come from the kernel before
   pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -374,7 +359,7 @@ __global__ void __launch_bounds__(128) row_select_kernel(const float* __restrict
   const int b = row / (NB * H);
   const uint8_t* pb = prot_blk + static_cast<int64_t>(b) * NB;
   select_row<KPL>(bs + static_cast<int64_t>(row) * NB, pb, protect_rows && pb[qb] != 0, NB, k_keep, protect_cols,
-                  all_bins[warp], lane, col_idx + static_cast<int64_t>(row) * NB, col_cnt + row);
+                  lane, col_idx + static_cast<int64_t>(row) * NB, col_cnt + row);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -408,8 +393,7 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   uint32_t* sq_lo = sq_hi + kStripRows * PITCH;                          // split into their two tf32 halves once
   const int SP = strip_pitch<D>(NB);
   float* strip = strip_smem + 2 * kStripRows * PITCH;       // [16][SP] block scores of the strip
-  int* all_bins = reinterpret_cast<int*>(strip + kStripRows * SP);      // [WARPS][256]
-  float4* ring = reinterpret_cast<float4*>(all_bins + WARPS * 256);     // [WARPS][4 slots][2 tiles][32 lanes]
+  float4* ring = reinterpret_cast<float4*>(strip + kStripRows * SP);    // [WARPS][4 slots][2 tiles][32 lanes]
   static_assert(NT == 4, "the key ring holds two tile pairs per 16-channel group");
   // Staged behind the pooling grid (programmatic dependent launch) and waits for it here; the pooling grid in
   // turn retires only after the token select, so the block flags are final too.
@@ -527,7 +511,7 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
     const float* src = strip + r * SP;
     float* dst = bs + row * NB;
     for (int i = lane; i < NB; i += 32) dst[i] = src[i];
-    select_row<KPL>(src, pb, protect_rows && pb[qi] != 0, NB, k_keep, protect_cols, all_bins + warp * 256, lane,
+    select_row<KPL>(src, pb, protect_rows && pb[qi] != 0, NB, k_keep, protect_cols, lane,
                     col_idx + row * NB, col_cnt + row);
   }
 }
@@ -575,9 +559,9 @@ static cudaError_t launch_score_select_as(cudaStream_t st, int B, int NB, const 
                                           float* bs, const uint8_t* pblk, int H, float scale, int k_keep, int pr, int pc,
                                           int32_t* col_idx, int32_t* col_cnt) {
   const size_t smem = (static_cast<size_t>(2 * kStripRows) * (D + 4) + static_cast<size_t>(kStripRows) * strip_pitch<D>(NB)) *
-                             sizeof(float) + WARPS * 256 * sizeof(int) + WARPS * 4 * 2 * 32 * 16;
+                             sizeof(float) + WARPS * 4 * 2 * 32 * 16;
   // always the same limit (the largest NB the call accepts), so concurrent callers never race on its value
-  constexpr int kMaxSmem = (2 * kStripRows * (D + 4) + kStripRows * strip_pitch<D>(kMaxBlocksPerRow)) * 4 + WARPS * 256 * 4 + WARPS * 4 * 2 * 32 * 16;
+  constexpr int kMaxSmem = (2 * kStripRows * (D + 4) + kStripRows * strip_pitch<D>(kMaxBlocksPerRow)) * 4 + WARPS * 4 * 2 * 32 * 16;
   cudaError_t e = cudaFuncSetAttribute(score_select_kernel<D, KPL, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMaxSmem);
   if (e != cudaSuccess) return e;
@@ -592,6 +576,8 @@ static cudaError_t launch_score_select(cudaStream_t st, int B, int NB, const flo
     return launch_score_select_as<D, 8, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   if (NB <= 512)
     return launch_score_select_as<D, 16, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+  if (NB <= 1024)      // (64 keys a lane are 230 registers, one CTA per SM)
+    return launch_score_select_as<D, 32, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   return launch_score_select_as<D, 64, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
 }
 
@@ -708,6 +694,8 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
       e = launch_pdl(row_select_kernel<8>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     else if (NB <= 512)
       e = launch_pdl(row_select_kernel<16>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
+    else if (NB <= 1024)
+      e = launch_pdl(row_select_kernel<32>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     else
       e = launch_pdl(row_select_kernel<64>, rgrid, 128, 0, st, block_scores, pbc, H, NB, k_keep, pr, pc, total_rows, col_idx, col_cnt);
     if (e != cudaSuccess) return AVSA_ERR_CUDA;

@@ -981,3 +981,36 @@ def test_rows_that_outgrow_their_reference_in_short_and_long_calls(heads):
     want_o, want_l, _ = orc.cross_attention(_np64(qa)[:, hs], _np64(kc)[:, hs], _np64(vc)[:, hs])
     _close(_np64(oc)[:, hs], want_o, "outgrown cross O")
     _close_lse(_np64(lc)[:, hs], want_l, "outgrown cross lse")
+
+
+@pytest.mark.parametrize("NB", [1, 32, 33, 256, 257, 512, 513, 1024, 1025])
+def test_mask_select_over_row_lengths(NB):
+    """The select's key slots per lane at their limits: distinct scores, heavy ties, one bit of difference, a sign change,
+    infinities and NaN, all with few and many kept."""
+    blk = 64
+    N = NB * blk - 3
+    rng = np.random.default_rng(NB)
+    bs = rng.standard_normal((1, 1, NB, NB)).astype(np.float32)
+    for r, row in enumerate(bs[0, 0]):
+        if r % 6 == 1:
+            row[:] = rng.integers(0, 3, NB)
+        elif r % 6 == 2:
+            row[:] = 1.5
+            row[rng.integers(NB)] = np.nextafter(np.float32(1.5), np.float32(2.0))
+        elif r % 6 == 3:
+            row[:] *= np.float32(1e-42)
+        elif r % 6 == 4:
+            row[rng.integers(NB)] = np.inf
+            row[rng.integers(NB)] = -np.inf
+            row[rng.integers(NB)] = np.nan
+        elif r % 6 == 5:
+            row[:] = -np.inf
+    s = rng.random((1, N)).astype(np.float32)
+    for k_keep in sorted({1, max(1, NB // 7), max(1, NB - 1), NB}):
+        idx, cnt, _, _ = orc.build_block_mask(bs, s, 3, k_keep, blk, N)
+        out = av.avsa_build_block_mask(None, None, torch.from_numpy(s).cuda(), 3, k_keep, blk,
+                                       flags=av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES,
+                                       block_scores=torch.from_numpy(bs).cuda(), shape=(1, 1, N, 64))
+        _status_ok(out["ws"])
+        assert np.array_equal(out["col_cnt"].cpu().numpy(), cnt)
+        assert np.array_equal(out["col_idx"].cpu().numpy(), idx)
