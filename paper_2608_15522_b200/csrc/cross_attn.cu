@@ -8,8 +8,10 @@
 namespace avsa {
 
 // ------------------------------------------------------------------------------------------------
-// pass 2: column sums of the attention map.  One CTA keeps the queries of one (batch, head) in
-// shared memory and walks a range of 128-key tiles.  S^T[key, query] accumulates in tensor memory
+// pass 2: column sums of the attention map.  A CTA keeps the queries of one (batch, head) pair in shared memory and walks
+// a range of its 128-key tiles: either one of n_range equal cuts of a pair, or (n_range == 0) one of even cuts of all
+// pairs' tiles in a row, which may lead from one pair into the next: the CTA then loads queries and LSEs again with
+// its pipeline empty (about three tiles).  S^T[key, query] accumulates in tensor memory
 // (two buffers of up to 256 columns); two groups of 128 threads (one thread per key row) turn
 // alternate buffers into row sums of exp2(S^T c - lse2[query]).
 //   warp 0 TMA producer, warp 1 MMA issuer, warp 2 tensor-memory allocation,
@@ -26,7 +28,7 @@ struct ColsumParams {
   StatusRecord* status;
   int H, Nq, Nk, NKT;      // NKT = key tiles of 128
   int NCH, W;              // query chunks and their width (multiple of 16, <= 256)
-  int n_range, tiles_per_range;
+  int BH, n_range, tiles_per_cta;
   float scale_log2;
 };
 
@@ -52,13 +54,9 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   constexpr int KPANEL_BYTES = 128 * 128;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int range = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int kt0 = range * p.tiles_per_range;
-  const int ntile = min(p.NKT, kt0 + p.tiles_per_range) - kt0;
-  const int item = (b * p.H + h) * p.n_range + range;
+  const int item = blockIdx.x;
   const int W = p.W, NCH = p.NCH;
   const int q_chunk_bytes = W * D * 2, q_panel_bytes = W * 128;
-  if (ntile <= 0) return;
   if ((smem_u32(smem) & 1023u) != 0u) {
     if (tid == 0) report_status(p.status, AVSA_ERR_CUDA, kWhereSmemAlign, item, 0);
     return;
@@ -85,26 +83,6 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
     prefetch_tmap(&tmq);
     prefetch_tmap(&tmk);
   }
-  pdl_wait();
-  // negated log2-domain LSEs (one packed FMA then gives s*c - lse2); queries beyond Nq get -inf: exp2 = 0
-  // (straight from the partial LSEs of pass 1's key ranges: the same maximum-and-sum as in merge_splits_rows, so that
-  // nothing has to be merged between the passes)
-  for (int j = tid; j < NCH * W; j += kColThreads) {
-    float v = -INFINITY;
-    if (j < p.Nq) {
-      const int qt = j / p.blk, u = (b * p.H + h) * p.rs.cpb + qt / p.rs.chunk;
-      int first;
-      const int n = p.rs.unit_parts(u, first);
-      const float* pl = p.part_lse2 + (static_cast<int64_t>(first) * p.rs.chunk + qt % p.rs.chunk) * p.blk + j % p.blk;
-      const int step = p.rs.chunk * p.blk;
-      float M = -INFINITY;
-      for (int s = 0; s < n; s++) M = fmaxf(M, pl[s * step]);
-      float Wsum = 0.f;
-      for (int s = 0; s < n; s++) Wsum += exp2f(pl[s * step] - M);
-      v = -(M + log2f(Wsum));
-    }
-    lse2[j] = v;
-  }
   if (warp == 2) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(misc)), 512);
     tmem_relinquish();
@@ -113,6 +91,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
+  pdl_wait();
 
   auto wait_or_abort = [&](int bar, uint32_t parity, int where, int aux) -> bool {
     if (misc[1] != 0u) return false;
@@ -122,122 +101,163 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
     return false;
   };
 
-  const int n_units = ntile * NCH;
-  if (warp == 0) {
-    if (lane == 0) {
-      mbar_expect_tx(BAR(Q_FULL), NCH * q_chunk_bytes);
-      for (int ch = 0; ch < NCH; ch++)
-        for (int pn = 0; pn < NPANEL; pn++)
-          tma_load_4d(smem_u32(smem + L::kQ) + ch * q_chunk_bytes + pn * q_panel_bytes, &tmq, BAR(Q_FULL), pn * 64,
-                      ch * W, h, b);
-      bool ok = true;
-      for (int t = 0; t < ntile && ok; t++) {
-        const int s = t % kColStages, f = t / kColStages;
-        if (f > 0) ok = wait_or_abort(K_EMPTY + s, (f - 1) & 1, kColKEmpty, t);
-        if (!ok) break;
-        mbar_expect_tx(BAR(K_FULL + s), L::kKTile);
-        for (int pn = 0; pn < NPANEL; pn++)
-          tma_load_4d(smem_u32(smem + L::kK) + s * L::kKTile + pn * KPANEL_BYTES, &tmk, BAR(K_FULL + s), pn * 64,
-                      (kt0 + t) * 128, h, b);
+  int pos = blockIdx.x * p.tiles_per_cta, pos_end = p.BH * p.NKT;
+  if (p.n_range > 0) {
+    const int pair = blockIdx.x / p.n_range;
+    pos = pair * p.NKT + (blockIdx.x % p.n_range) * p.tiles_per_cta;
+    pos_end = (pair + 1) * p.NKT;
+  }
+  pos_end = min(pos_end, pos + p.tiles_per_cta);
+  int kc = 0;                               // key tiles of the segments before
+  for (int seg = 0; pos < pos_end; seg++) {
+    const int bh = pos / p.NKT, kt0 = pos % p.NKT, h = bh % p.H, b = bh / p.H;
+    const int ntile = min(p.NKT - kt0, pos_end - pos);
+    // negated log2-domain LSEs (one packed FMA then gives s*c - lse2); queries beyond Nq get -inf: exp2 = 0
+    // (straight from the partial LSEs of pass 1's key ranges: the same maximum-and-sum as in merge_splits_rows, so that
+    // nothing has to be merged between the passes)
+    // (warp 0 has no part in this: the first tiles and the queries are on their way meanwhile)
+    for (int j = tid - 32; j < NCH * W; j += kColThreads - 32) {
+      if (warp == 0) break;
+      float v = -INFINITY;
+      if (j < p.Nq) {
+        const int qt = j / p.blk, u = bh * p.rs.cpb + qt / p.rs.chunk;
+        int first;
+        const int n = p.rs.unit_parts(u, first);
+        const float* pl = p.part_lse2 + (static_cast<int64_t>(first) * p.rs.chunk + qt % p.rs.chunk) * p.blk + j % p.blk;
+        const int step = p.rs.chunk * p.blk;
+        float M = -INFINITY;
+        for (int s = 0; s < n; s++) M = fmaxf(M, pl[s * step]);
+        float Wsum = 0.f;
+        for (int s = 0; s < n; s++) Wsum += exp2f(pl[s * step] - M);
+        v = -(M + log2f(Wsum));
       }
+      lse2[j] = v;
     }
-  } else if (warp == 1) {
-    // The whole warp runs the loop (uniform control flow), one elected lane issues; descriptor words are
-    // prepared ahead so that the issuing lane does little besides issuing.
-    const bool leader = elect_one_sync();
-    const uint32_t idesc = make_idesc_bf16(128, W, 0, 0);
-    constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-    auto desc64 = [](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
-    const uint32_t k_lo0 = ((smem_u32(smem + L::kK) & 0x3FFFFu) >> 4) | (1u << 16);
-    const uint32_t q_lo0 = ((smem_u32(smem + L::kQ) & 0x3FFFFu) >> 4) | (1u << 16);
-    auto wait_all = [&](int bar, uint32_t parity, int where, int aux) -> bool {
-      return __all_sync(0xffffffffu, wait_or_abort(bar, parity, where, aux));
-    };
-    bool ok = wait_all(Q_FULL, 0, kColQFull, 0);
-    for (int t = 0; t < ntile && ok; t++) {
-      const int s = t % kColStages, f = t / kColStages;
-      ok = wait_all(K_FULL + s, f & 1, kColKFull, t);
-      if (!ok) break;
-      const uint32_t k_lo = k_lo0 + s * (L::kKTile >> 4);
-      for (int ch = 0; ch < NCH && ok; ch++) {
-        const int u = t * NCH + ch, g = u & 1, i = u >> 1;
-        if (i > 0) ok = wait_all(S_EMPTY + g, (i - 1) & 1, kColSEmpty, u);
+    if (warp != 0) asm volatile("bar.sync 1, 352;" ::: "memory");      // the table is there (kColThreads - 32 threads)
+    const int n_units = ntile * NCH;
+    if (warp == 0) {
+      if (lane == 0) {
+        mbar_expect_tx(BAR(Q_FULL), NCH * q_chunk_bytes);
+        for (int ch = 0; ch < NCH; ch++)
+          for (int pn = 0; pn < NPANEL; pn++)
+            tma_load_4d(smem_u32(smem + L::kQ) + ch * q_chunk_bytes + pn * q_panel_bytes, &tmq, BAR(Q_FULL), pn * 64,
+                        ch * W, h, b);
+        bool ok = true;
+        for (int t = 0; t < ntile && ok; t++) {
+          const int s = (kc + t) % kColStages, f = (kc + t) / kColStages;
+          if (f > 0) ok = wait_or_abort(K_EMPTY + s, (f - 1) & 1, kColKEmpty, t);
+          if (!ok) break;
+          mbar_expect_tx(BAR(K_FULL + s), L::kKTile);
+          for (int pn = 0; pn < NPANEL; pn++)
+            tma_load_4d(smem_u32(smem + L::kK) + s * L::kKTile + pn * KPANEL_BYTES, &tmk, BAR(K_FULL + s), pn * 64,
+                        (kt0 + t) * 128, h, b);
+        }
+      }
+    } else if (warp == 1) {
+      // The whole warp runs the loop (uniform control flow), one elected lane issues; descriptor words are
+      // prepared ahead so that the issuing lane does little besides issuing.
+      const bool leader = elect_one_sync();
+      const uint32_t idesc = make_idesc_bf16(128, W, 0, 0);
+      constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+      auto desc64 = [](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
+      const uint32_t k_lo0 = ((smem_u32(smem + L::kK) & 0x3FFFFu) >> 4) | (1u << 16);
+      const uint32_t q_lo0 = ((smem_u32(smem + L::kQ) & 0x3FFFFu) >> 4) | (1u << 16);
+      auto wait_all = [&](int bar, uint32_t parity, int where, int aux) -> bool {
+        return __all_sync(0xffffffffu, wait_or_abort(bar, parity, where, aux));
+      };
+      bool ok = wait_all(Q_FULL, seg & 1, kColQFull, 0);
+      for (int t = 0; t < ntile && ok; t++) {
+        const int s = (kc + t) % kColStages, f = (kc + t) / kColStages;
+        ok = wait_all(K_FULL + s, f & 1, kColKFull, t);
+        if (!ok) break;
+        const uint32_t k_lo = k_lo0 + s * (L::kKTile >> 4);
+        for (int ch = 0; ch < NCH && ok; ch++) {
+          const int u = (kc + t) * NCH + ch, g = u & 1, i = u >> 1;
+          if (i > 0) ok = wait_all(S_EMPTY + g, (i - 1) & 1, kColSEmpty, u);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t q_lo = q_lo0 + ch * (q_chunk_bytes >> 4);
+          if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ks++) {
+              const uint32_t koff = ((ks >> 2) * KPANEL_BYTES + (ks & 3) * 32) >> 4;
+              const uint32_t qoff = ((ks >> 2) * q_panel_bytes + (ks & 3) * 32) >> 4;
+              umma_ss(tmem + g * 256, desc64(k_lo + koff), desc64(q_lo + qoff), idesc, ks > 0 ? 1u : 0u);
+            }
+            umma_commit(BAR(S_FULL + g));
+            if (ch == NCH - 1) umma_commit(BAR(K_EMPTY + s));
+          }
+          __syncwarp();
+        }
+      }
+    } else if (warp >= 4) {
+      const int g = (warp - 4) >> 2;
+      const int row = ((warp & 3) << 5) + lane;
+      const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
+      bool ok = true;
+      const int u0 = kc * NCH;      // units of the segments before: unit u goes to buffer and group u mod 2
+      for (int u = u0 + ((g ^ u0) & 1); u < u0 + n_units && ok; u += 2) {
+        const int i = u >> 1, t = u / NCH - kc, ch = u % NCH;
+        ok = wait_or_abort(S_FULL + g, i & 1, kColSFull, u);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t q_lo = q_lo0 + ch * (q_chunk_bytes >> 4);
-        if (leader) {
+        const float* l2 = lse2 + ch * W;
+        const uint32_t base = tmem + g * 256 + lane_off;
+        const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
+        uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+        // sum over 32 (or 16) queries of exp2(s*c - lse2), two values per packed FMA / add
+        auto reduce32 = [&](const uint32_t (&sv)[32], const float* nl) {
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ks++) {
-            const uint32_t koff = ((ks >> 2) * KPANEL_BYTES + (ks & 3) * 32) >> 4;
-            const uint32_t qoff = ((ks >> 2) * q_panel_bytes + (ks & 3) * 32) >> 4;
-            umma_ss(tmem + g * 256, desc64(k_lo + koff), desc64(q_lo + qoff), idesc, ks > 0 ? 1u : 0u);
+          for (int j = 0; j < 32; j += 4) {
+            const ulonglong2 nv = *reinterpret_cast<const ulonglong2*>(nl + j);      // four negated LSEs
+            float x0, x1, x2, x3;
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nv.x), x0, x1);
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3])), c2, nv.y), x2, x3);
+            acc[(j >> 2) & 3] = add_f32x2(acc[(j >> 2) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+            acc[((j >> 2) + 2) & 3] = add_f32x2(acc[((j >> 2) + 2) & 3], pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
           }
-          umma_commit(BAR(S_FULL + g));
-          if (ch == NCH - 1) umma_commit(BAR(K_EMPTY + s));
+        };
+        const int n32 = W / 32;           // whole 32-column pieces; W is a multiple of 16, so 16 columns may remain
+        uint32_t sa[32], sb[32];
+        if (n32 > 0) tmem_ld32(base, sa);
+        for (int c = 0; c < n32; c += 2) {
+          tmem_wait_ld();
+          if (c + 1 < n32) tmem_ld32(base + (c + 1) * 32, sb);      // in flight under the exponentials of piece c
+          reduce32(sa, l2 + c * 32);
+          if (c + 1 < n32) {
+            tmem_wait_ld();
+            if (c + 2 < n32) tmem_ld32(base + (c + 2) * 32, sa);
+            reduce32(sb, l2 + (c + 1) * 32);
+          }
         }
-        __syncwarp();
+        if (n32 * 32 < W) {
+          uint32_t st[16];
+          tmem_ld16(base + n32 * 32, st);
+          tmem_wait_ld();
+          const float* nl = l2 + n32 * 32;
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            float x0, x1;
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(st[j]), __uint_as_float(st[j + 1])), c2,
+                                   *reinterpret_cast<const uint64_t*>(nl + j)), x0, x1);
+            acc[(j >> 1) & 3] = add_f32x2(acc[(j >> 1) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+          }
+        }
+        float sum0, sum1;
+        unpack_f32x2(add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3])), sum0, sum1);
+        tc_fence_before();
+        mbar_arrive(BAR(S_EMPTY + g));
+        const int key = (kt0 + t) * 128 + row;
+        if (key < p.Nk)
+          p.partial[(static_cast<int64_t>(ch) * p.BH + bh) * p.Nk + key] = sum0 + sum1;
       }
     }
-  } else if (warp >= 4) {
-    const int g = (warp - 4) >> 2;
-    const int row = ((warp & 3) << 5) + lane;
-    const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    bool ok = true;
-    for (int u = g; u < n_units && ok; u += 2) {
-      const int i = u >> 1, t = u / NCH, ch = u % NCH;
-      ok = wait_or_abort(S_FULL + g, i & 1, kColSFull, u);
-      if (!ok) break;
-      tc_fence_after();
-      const float* l2 = lse2 + ch * W;
-      const uint32_t base = tmem + g * 256 + lane_off;
-      const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
-      uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-      // sum over 32 (or 16) queries of exp2(s*c - lse2), two values per packed FMA / add
-      auto reduce32 = [&](const uint32_t (&sv)[32], const float* nl) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          const ulonglong2 nv = *reinterpret_cast<const ulonglong2*>(nl + j);      // four negated LSEs
-          float x0, x1, x2, x3;
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nv.x), x0, x1);
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3])), c2, nv.y), x2, x3);
-          acc[(j >> 2) & 3] = add_f32x2(acc[(j >> 2) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-          acc[((j >> 2) + 2) & 3] = add_f32x2(acc[((j >> 2) + 2) & 3], pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
-        }
-      };
-      const int n32 = W / 32;           // whole 32-column pieces; W is a multiple of 16, so 16 columns may remain
-      uint32_t sa[32], sb[32];
-      if (n32 > 0) tmem_ld32(base, sa);
-      for (int c = 0; c < n32; c += 2) {
-        tmem_wait_ld();
-        if (c + 1 < n32) tmem_ld32(base + (c + 1) * 32, sb);      // in flight under the exponentials of piece c
-        reduce32(sa, l2 + c * 32);
-        if (c + 1 < n32) {
-          tmem_wait_ld();
-          if (c + 2 < n32) tmem_ld32(base + (c + 2) * 32, sa);
-          reduce32(sb, l2 + (c + 1) * 32);
-        }
-      }
-      if (n32 * 32 < W) {
-        uint32_t st[16];
-        tmem_ld16(base + n32 * 32, st);
-        tmem_wait_ld();
-        const float* nl = l2 + n32 * 32;
-#pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-          float x0, x1;
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(st[j]), __uint_as_float(st[j + 1])), c2,
-                                 *reinterpret_cast<const uint64_t*>(nl + j)), x0, x1);
-          acc[(j >> 1) & 3] = add_f32x2(acc[(j >> 1) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-        }
-      }
-      float sum0, sum1;
-      unpack_f32x2(add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3])), sum0, sum1);
-      tc_fence_before();
-      mbar_arrive(BAR(S_EMPTY + g));
-      const int key = (kt0 + t) * 128 + row;
-      if (key < p.Nk)
-        p.partial[(static_cast<int64_t>(ch) * gridDim.z * p.H + static_cast<int64_t>(b) * p.H + h) * p.Nk + key] =
-            sum0 + sum1;
+    pos += ntile;
+    kc += ntile;
+    if (pos < pos_end) {
+      // nobody reads the queries and LSEs any more (roles that gave up come here too: the waits of the others end then)
+      __syncthreads();
+      if (misc[1] != 0u) break;
     }
   }
   tc_fence_before();
@@ -547,7 +567,7 @@ __global__ void __launch_bounds__(256) head_sum_wide_kernel(const float* __restr
 struct CrossPlan {
   int blk, NQT, NKB;                         // pass 1 (key tiles of blk)
   RangeSplit rs;
-  int NKT, NCH, W, n_range, tpr;             // pass 2 (key tiles of 128)
+  int NKT, NCH, W, n_range, tpc, ctas2;      // pass 2 (key tiles of 128), cuts per pair, tiles per CTA, CTAs
   bool reverse;                              // pass 2 with the keys resident (Nq > 512, Nk <= 512)
   int NQC, rev_ranges, rev_cpr, rev_slots;   // query chunks of 128, CTAs per (b,h), chunks per CTA, partial slots
   size_t off_part_o, off_part_lse, off_lse, off_lse2, off_partial, off_redo, total;
@@ -567,11 +587,24 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   c.NKT = (Nk + 127) / 128;
   c.NCH = Nq > 256 ? 2 : 1;
   c.W = (((Nq + c.NCH - 1) / c.NCH) + 15) / 16 * 16;
-  int want_range = target / (B * H);
+  // equal cuts of every pair, or even cuts through all of them where that is shorter by more than the reload it costs
+  // (32 heads x 384 tiles, 512 queries on 148 SMs: 96 tiles on 128 of them 645 us for the call, 84 on all 612; 32 x 157 with
+  // 100 queries: 110 us as 40 tiles on 128, 112 as 34 on all)
+  const int BH = B * H;
+  int want_range = target / BH;
   if (want_range < 1) want_range = 1;
   if (want_range > c.NKT) want_range = c.NKT;
-  c.tpr = (c.NKT + want_range - 1) / want_range;
-  c.n_range = (c.NKT + c.tpr - 1) / c.tpr;
+  c.tpc = (c.NKT + want_range - 1) / want_range;
+  c.n_range = (c.NKT + c.tpc - 1) / c.tpc;
+  const long long tiles2 = static_cast<long long>(BH) * c.NKT;
+  const long long waves = (static_cast<long long>(BH) * c.n_range + target - 1) / target;
+  const int even = static_cast<int>((tiles2 + target - 1) / target);
+  const int reload = 3 * 512 / (c.NCH * c.W);       // three tiles of 512 queries, more of them with fewer
+  if (even + reload * ((even + c.NKT - 1) / c.NKT) < waves * c.tpc) {
+    c.n_range = 0;
+    c.tpc = even;
+  }
+  c.ctas2 = static_cast<int>(c.n_range > 0 ? static_cast<long long>(BH) * c.n_range : (tiles2 + c.tpc - 1) / c.tpc);
   c.reverse = Nq > 512;
   c.NQC = (Nq + 127) / 128;
   int want_rev = target / (B * H);
@@ -703,11 +736,11 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     cp.NKT = c.NKT;
     cp.NCH = c.NCH;
     cp.W = c.W;
+    cp.BH = B * H;
     cp.n_range = c.n_range;
-    cp.tiles_per_range = c.tpr;
+    cp.tiles_per_cta = c.tpc;
     cp.scale_log2 = scale * 1.4426950408889634f;
-    dim3 grid(c.n_range, H, B);
-    if (launch_pdl(colsum_kernel<D>, grid, kColThreads, smem, st, tq, tk, cp) != cudaSuccess) return AVSA_ERR_CUDA;
+    if (launch_pdl(colsum_kernel<D>, c.ctas2, kColThreads, smem, st, tq, tk, cp) != cudaSuccess) return AVSA_ERR_CUDA;
     const int64_t n = static_cast<int64_t>(B) * Nk;
     const int hs_blocks = static_cast<int>((n + 255) / 256);
     if (merge_late) {

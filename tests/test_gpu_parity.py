@@ -516,6 +516,8 @@ def test_cross_attention_long_query_axis_two_chunks():
     (2, 3, 140, 333, 64, True),        # few tiles: whole rows, written by the tile kernel itself
     (1, 22, 2427, 200, 128, True),     # reverse: 19 query tiles in chunks of 4, whole rows, score pass over the keys
     (1, 2, 130, 6400, 64, True),
+    (1, 100, 40, 1000, 64, True),      # score pass: 800 key tiles cut evenly through the heads
+    (1, 96, 300, 520, 128, True),      # the same with the queries in two chunks
 ])
 def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
     """Every way the (query tile, key tile) work is cut over the CTAs: whole rows, split rows, chunks that do not divide
