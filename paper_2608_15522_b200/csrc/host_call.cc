@@ -97,10 +97,17 @@ bool read_optional_view(PyObject* t, avsa_bf16_4d* out) {      // None is the nu
   *out = avsa_bf16_4d{nullptr, 0, 0, 0};
   return t == Py_None || read_view(t, out);
 }
-// current stream of the tensor's device
+// current stream of the tensor's device (a tensor in host memory has none: its index is -1, which the reader of the
+// stream would take for the current device)
 bool read_stream(PyObject* t, void** out) {
   PyObject* dev = PyObject_CallMethodNoArgs(t, s_get_device);
   if (dev == nullptr) return false;
+  const long index = PyLong_AsLong(dev);
+  if (index < 0) {
+    Py_DECREF(dev);
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "expected a tensor on a CUDA device");
+    return false;
+  }
   PyObject* r = PyObject_CallOneArg(o_raw_stream, dev);
   Py_DECREF(dev);
   if (r == nullptr) return false;

@@ -1,4 +1,6 @@
 """The marshalling extension refuses what the library could not describe (no GPU needed: nothing is launched)."""
+import ctypes
+
 import pytest
 import torch
 
@@ -33,3 +35,43 @@ def test_missing_tensors_raise_instead_of_reaching_the_library():
                  lambda: av.avsa_sparse_self_attn(None, t, t, t, t, 64, o=t, ws=t)):
         with pytest.raises((AttributeError, ValueError)):
             call()
+
+
+# ------------------------------------------------------------------------- the library's entry points replaced by recorders
+_i, _f, _p, _sz, _u, _T = ctypes.c_int, ctypes.c_float, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_uint, av._Bf16Tensor4
+_SIGNATURES = {
+    "cross": [_i] * 5 + [_T] * 3 + [_p] * 3 + [_f] * 3 + [_p, _sz, _p],
+    "mask": [_i] * 5 + [_T] * 2 + [_p, _i, _i, _u, _f] + [_p] * 6 + [_sz, _p],
+    "sparse": [_i] * 5 + [_T] * 3 + [_p] * 4 + [_f, _p, _sz, _p],
+    "protected": [_i] * 5 + [_T] * 3 + [_p, _i, _p, _p, _f, _p, _sz, _p],
+    "indicators": [_i] * 4 + [_p] * 7 + [_f] * 4 + [_p, _p, _sz, _p],
+}
+
+
+@pytest.fixture
+def recorded():
+    """The extension bound to recorders instead of the library: calls[...] is what would have been called, with what."""
+    calls, keep = [], []
+
+    def recorder(name, types):
+        def entry(*args):
+            calls.append((name, [(a.ptr, a.stride_b, a.stride_h, a.stride_n) if isinstance(a, _T) else a for a in args]))
+            return 0
+        keep.append(ctypes.CFUNCTYPE(_i, *types)(entry))
+        return ctypes.cast(keep[-1], _p).value
+
+    host = av._host()
+    host.bind(*(recorder(n, t) for n, t in _SIGNATURES.items()), torch.bfloat16, lambda device: 4096 + device)
+    yield calls
+    av._host_module = None      # bound to the library again
+    av._host()
+
+
+def test_given_block_scores_in_host_memory_are_refused(recorded):
+    """Without q and k the block scores say which device the call runs on; in host memory there is none, and the kernels
+    would be handed host pointers."""
+    bs = torch.zeros((1, 2, 4, 4))
+    with pytest.raises(ValueError, match="CUDA device"):
+        av.avsa_build_block_mask(None, None, None, 0, 1, 64, flags=av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES,
+                                 block_scores=bs, shape=(1, 2, 256, 64))
+    assert recorded == []
