@@ -37,6 +37,12 @@ bool read_int(PyObject* v, int* out) {
   Py_DECREF(n);
   return !PyErr_Occurred();
 }
+// an argument that binding.py does not convert: only an int, as a C prototype would have it (block size 64.9 is not 64)
+bool read_strict_int(PyObject* v, int* out) {
+  if (PyLong_Check(v)) return read_int(v, out);
+  PyErr_Format(PyExc_TypeError, "expected an int, got %s", Py_TYPE(v)->tp_name);
+  return false;
+}
 bool read_float(PyObject* v, float* out) {
   PyObject* f = PyNumber_Float(v);
   if (f == nullptr) return false;
@@ -174,7 +180,7 @@ PyObject* py_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int blk, n_protect, k_keep, flags;
   float scale;
   size_t ws_bytes;
-  if (!read_tuple(Py_NewRef(a[0]), sh, 4) || !read_int(a[1], &blk) || !read_optional_view(a[2], &q) ||
+  if (!read_tuple(Py_NewRef(a[0]), sh, 4) || !read_strict_int(a[1], &blk) || !read_optional_view(a[2], &q) ||
       !read_optional_view(a[3], &k) || !read_ptr(a[4], &scores) || !read_int(a[5], &n_protect) || !read_int(a[6], &k_keep) || !read_int(a[7], &flags) ||
       !read_float(a[8], &scale) || !read_ptr(a[9], &bs) || !read_ptr(a[10], &idx) || !read_ptr(a[11], &cnt) ||
       !read_ptr(a[12], &tok) || !read_ptr(a[13], &pblk) || !read_ptr(a[14], &ws) || !read_numel(a[14], &ws_bytes) ||
@@ -200,7 +206,7 @@ PyObject* py_sparse(PyObject*, PyObject* const* a, Py_ssize_t n) {
   float scale;
   size_t ws_bytes;
   if (!read_shape(a[0], sh, 4) || !read_view(a[0], &q) || !read_view(a[1], &k) || !read_view(a[2], &v) ||
-      !read_ptr(a[3], &idx) || !read_ptr(a[4], &cnt) || !read_int(a[5], &blk) || !read_ptr(a[6], &o) ||
+      !read_ptr(a[3], &idx) || !read_ptr(a[4], &cnt) || !read_strict_int(a[5], &blk) || !read_ptr(a[6], &o) ||
       !read_ptr(a[7], &lse) || !read_float(a[8], &scale) || !read_ptr(a[9], &ws) || !read_numel(a[9], &ws_bytes) ||
       !read_stream(a[0], &stream))
     return nullptr;
@@ -223,7 +229,7 @@ PyObject* py_protected(PyObject*, PyObject* const* a, Py_ssize_t n) {
   float scale;
   size_t ws_bytes;
   if (!read_shape(a[0], sh, 4) || !read_view(a[0], &q) || !read_view(a[1], &k) || !read_view(a[2], &v) ||
-      !read_ptr(a[3], &tok) || !read_int(a[4], &n_protect) || !read_int(a[5], &blk) || !read_ptr(a[6], &o) ||
+      !read_ptr(a[3], &tok) || !read_int(a[4], &n_protect) || !read_strict_int(a[5], &blk) || !read_ptr(a[6], &o) ||
       !read_ptr(a[7], &lse) || !read_float(a[8], &scale) || !read_ptr(a[9], &ws) || !read_numel(a[9], &ws_bytes) ||
       !read_stream(a[0], &stream))
     return nullptr;

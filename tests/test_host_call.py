@@ -75,3 +75,42 @@ def test_given_block_scores_in_host_memory_are_refused(recorded):
         av.avsa_build_block_mask(None, None, None, 0, 1, 64, flags=av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES,
                                  block_scores=bs, shape=(1, 2, 256, 64))
     assert recorded == []
+
+
+class _OnGpu:
+    """Stands for a tensor on cuda:1: what the marshalling reads of one, without the device."""
+
+    def __init__(self, shape, dtype=torch.bfloat16, stride=None, ptr=65536, is_cuda=True):
+        self.shape, self.dtype, self.is_cuda, self._ptr = torch.Size(shape), dtype, is_cuda, ptr
+        dense, n = [], 1
+        for s in reversed(self.shape):
+            dense.insert(0, n)
+            n *= s
+        self._dense, self._n, self._stride = tuple(dense), n, tuple(dense) if stride is None else tuple(stride)
+
+    def stride(self):
+        return self._stride
+
+    def data_ptr(self):
+        return self._ptr
+
+    def numel(self):
+        return self._n
+
+    def get_device(self):
+        return 1 if self.is_cuda else -1
+
+    def is_contiguous(self):
+        return self._stride == self._dense
+
+
+def test_a_block_size_that_is_no_integer_is_refused(recorded):
+    t, f32, u8, ws = _OnGpu((1, 2, 256, 64)), _OnGpu((1, 2, 4, 4), torch.float32), _OnGpu((1, 256), torch.uint8), _OnGpu((999,))
+    out = dict(block_scores=f32, col_idx=f32, col_cnt=f32, prot_tok=u8, prot_blk=u8)
+    for blk in (64.0, 64.9, "64"):
+        for call in (lambda: av.avsa_sparse_self_attn(t, t, t, f32, f32, blk, o=t, ws=ws),
+                     lambda: av.avsa_protected_rows_attn(t, t, t, u8, 1, blk, t, ws=ws),
+                     lambda: av.avsa_build_block_mask(t, t, None, 0, 1, blk, out=out, ws=ws)):
+            with pytest.raises(TypeError):
+                call()
+    assert recorded == []
