@@ -80,6 +80,8 @@ def test_given_block_scores_in_host_memory_are_refused(recorded):
 class _OnGpu:
     """Stands for a tensor on cuda:1: what the marshalling reads of one, without the device."""
 
+    device = torch.device("cuda", 1)
+
     def __init__(self, shape, dtype=torch.bfloat16, stride=None, ptr=65536, is_cuda=True):
         self.shape, self.dtype, self.is_cuda, self._ptr = torch.Size(shape), dtype, is_cuda, ptr
         dense, n = [], 1
