@@ -76,6 +76,17 @@ bool read_tuple(PyObject* tuple, int64_t* out, Py_ssize_t n) {      // steals th
   return ok;
 }
 bool read_shape(PyObject* t, int64_t* shape, Py_ssize_t n) { return read_tuple(PyObject_GetAttr(t, s_shape), shape, n); }
+// one extent of a tensor of any rank
+bool read_extent(PyObject* t, Py_ssize_t axis, int64_t* out) {
+  PyObject* shape = PyObject_GetAttr(t, s_shape);
+  if (shape == nullptr) return false;
+  PyObject* v = PySequence_GetItem(shape, axis);
+  Py_DECREF(shape);
+  if (v == nullptr) return false;
+  *out = PyLong_AsLongLong(v);
+  Py_DECREF(v);
+  return !PyErr_Occurred();
+}
 
 // bf16 [B,H,N,d] on a CUDA device with a contiguous head dimension
 bool read_view(PyObject* t, avsa_bf16_4d* out) {
@@ -244,7 +255,7 @@ PyObject* py_protected(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // indicators(y_v, yhat_v, y_a, yhat_a, prot_tok, s_cur, s_anchor, lambda_p, lambda_s, tau, eps, out, ws) -> status
 PyObject* py_indicators(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!arity(n, 13)) return nullptr;
-  int64_t vs[3], as[3];
+  int64_t vs[3], na;
   void *y[4], *tok, *cur, *anchor, *out, *ws, *stream;
   float lp, ls, tau, eps;
   size_t ws_bytes;
@@ -261,14 +272,14 @@ PyObject* py_indicators(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
     if (!read_ptr(a[i], &y[i])) return nullptr;
   }
-  if (!read_shape(a[0], vs, 3) || !read_shape(a[2], as, 3) || !read_ptr(a[4], &tok) || !read_ptr(a[5], &cur) ||
+  if (!read_shape(a[0], vs, 3) || !read_extent(a[2], 1, &na) || !read_ptr(a[4], &tok) || !read_ptr(a[5], &cur) ||
       !read_ptr(a[6], &anchor) || !read_float(a[7], &lp) || !read_float(a[8], &ls) || !read_float(a[9], &tau) ||
       !read_float(a[10], &eps) || !read_ptr(a[11], &out) || !read_ptr(a[12], &ws) || !read_numel(a[12], &ws_bytes) ||
       !read_stream(a[0], &stream))
     return nullptr;
   int st;
   Py_BEGIN_ALLOW_THREADS;
-  st = f_indicators(static_cast<int>(vs[0]), static_cast<int>(vs[1]), static_cast<int>(as[1]), static_cast<int>(vs[2]), y[0],
+  st = f_indicators(static_cast<int>(vs[0]), static_cast<int>(vs[1]), static_cast<int>(na), static_cast<int>(vs[2]), y[0],
                     y[1], y[2], y[3], static_cast<uint8_t*>(tok), static_cast<float*>(cur), static_cast<float*>(anchor), lp, ls,
                     tau, eps, static_cast<float*>(out), ws, ws_bytes, stream);
   Py_END_ALLOW_THREADS;

@@ -116,3 +116,16 @@ def test_a_block_size_that_is_no_integer_is_refused(recorded):
             with pytest.raises(TypeError):
                 call()
     assert recorded == []
+
+
+def test_audio_features_of_any_rank_keep_their_token_axis(recorded):
+    """The audio tokens are axis 1 of y_a, whatever the channels behind it are split into (the video stream gives B and C)."""
+    y_v, out, ws = _OnGpu((2, 40, 384)), _OnGpu((2, 8), torch.float32), _OnGpu((9999,), torch.uint8)
+    for shape in ((2, 24, 384), (2, 24, 3, 128), (2, 24 * 384)):
+        y_a = _OnGpu(shape)
+        av.avsa_cache_indicators(y_v, y_v, y_a, y_a, out=out, ws=ws)
+        assert recorded.pop()[1][:4] == [2, 40, shape[1], 384]
+    for bad_v in ((80, 384), (2, 40, 3, 128)):
+        with pytest.raises(ValueError):
+            av.avsa_cache_indicators(_OnGpu(bad_v), y_v, y_v, y_v, out=out, ws=ws)
+    assert recorded == []
