@@ -694,6 +694,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
     if (tid == 0) {
       for (int i = 0; i < L::kNumBars; i++) mbar_inval(bar0 + i * 8);
     }
+    __syncwarp();      // thread 0 was alone; attn_launch_regs begins with an instruction that the whole warp executes together
     attn_launch_regs();
     persist_exact_phase<BLK, D, MODE>(&tmq, &tmk, &tmv, &tmo, p);
   }

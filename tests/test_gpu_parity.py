@@ -271,13 +271,13 @@ def test_sparse_attention_single_and_odd_counts():
     _run_sparse_case(w, 3, idx, cnt)
 
 
-@pytest.mark.parametrize("step,expect_redo,heads", [(1.0, False, 4), (16.0, True, 4), (16.0, True, 12)])
+@pytest.mark.parametrize("step,expect_redo,heads", [(1.0, False, 4), (16.0, True, 4), (16.0, True, 12), (16.0, True, 20)])
 def test_sparse_attention_row_maxima_growing_along_the_key_axis(step, expect_redo, heads):
     """Logits that grow from key block to key block.  The fast kernel keeps the first tile's row maximum
     as its reference: a moderate growth stays inside its headroom, a steep one makes it hand the work item
-    to the exact-rescaling kernel (listed behind the status record in the workspace).  Both must match
-    the oracle; in the steep case items must actually have been handed over (with 12 heads more of them than
-    the exact kernel has CTAs, so that its CTAs take several items each)."""
+    to exact rescaling (listed behind the status record in the workspace).  Both must match the oracle; in the
+    steep case items must actually have been handed over.  With 12 heads (6936 tile pairs, below 64 per SM) every
+    CTA of the tile kernel recomputes several of its own, with 20 (11560) every CTA of the grid behind it does."""
     import dataclasses
     w = dataclasses.replace(wl.WORKLOADS["medium128"], H=heads)
     q, k, v = wl.make_self_qkv(w, 6)
@@ -950,11 +950,11 @@ def test_protected_rows_odd_lengths(B, H, N, d, n_protect):
     assert (got_o[~on] == 7.0).all() and (got_l[~on] == 7.0).all()
 
 
-@pytest.mark.parametrize("heads", [20, 40])
-def test_rows_that_outgrow_their_reference_in_short_and_long_calls(heads):
+@pytest.mark.parametrize("heads,d,repeat", [(20, 128, 1), (40, 128, 5), (8, 64, 1), (20, 64, 5)])
+def test_rows_that_outgrow_their_reference_in_short_and_long_calls(heads, d, repeat):
     """Steeply growing logits: a short call recomputes such items inside the tile kernel, a long one in a grid of its
-    own (more than 64 tile pairs per SM, 32 without lists); list and range modes."""
-    d, n, na = 128, 2070, 300
+    own (more than 64 tile pairs per SM, 32 without lists); list and range modes, both tile shapes of either."""
+    n, na = 2070, 300
     g = torch.Generator().manual_seed(heads)
     q, k, v = (torch.randn((1, heads, n, d), generator=g) for _ in range(3))
     u = 1.0 / np.sqrt(d)
@@ -976,13 +976,48 @@ def test_rows_that_outgrow_their_reference_in_short_and_long_calls(heads):
     _close(_np64(o)[:, hs], want_o, "outgrown O")
     _close_lse(_np64(lse)[:, hs], want_l, "outgrown lse")
     qa = q[:, :, :na].contiguous()
-    kc, vc = (torch.cat([t] * 5, dim=2) if heads > 20 else t for t in (k, v))
+    kc, vc = (torch.cat([t] * repeat, dim=2) for t in (k, v))
     oc, lc, _, wc = av.avsa_cross_attn_scores(qa.cuda(), kc.cuda(), vc.cuda(), want_scores=False)
     _status_ok(wc)
     assert av.avsa_redo_count(wc) > 0
     want_o, want_l, _ = orc.cross_attention(_np64(qa)[:, hs], _np64(kc)[:, hs], _np64(vc)[:, hs])
     _close(_np64(oc)[:, hs], want_o, "outgrown cross O")
     _close_lse(_np64(lc)[:, hs], want_l, "outgrown cross lse")
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("H,N,n_protect,short", [
+    (8, 2600, 700, True),       # query tiles in parts of 7 key tiles, recomputed inside the tile kernel
+    (40, 2070, 300, True),      # whole rows stored through the row map, inside the tile kernel
+    (128, 768, 700, True),      # the same with the query tiles off the queue
+    (64, 1500, 1500, False),    # whole rows, in the grid behind it
+    (54, 2688, 2500, False),    # the queue with its end cut: whole rows and parts, in the grid behind it
+])
+def test_protected_rows_that_outgrow_their_reference(H, N, n_protect, short, d):
+    """Dense rows whose logits grow by some 16 per 128 keys, in every form that their exact recomputation takes: the flagged
+    rows are the oracle's, the others stay as they were."""
+    assert (2 * H * -(-n_protect // 128) * -(-N // 128) <= 64 * 148) == short
+    g = torch.Generator(device="cuda").manual_seed(N + d)
+    q, k, v = (torch.randn((1, H, N, d), generator=g, device="cuda") for _ in range(3))
+    u = 1.0 / np.sqrt(d)
+    q = (q + 8.0 * u).to(torch.bfloat16)
+    ramp = torch.arange(N, dtype=torch.float32, device="cuda").div(128, rounding_mode="floor") * 2.0 * np.sqrt(d)
+    k = (k + (ramp * u).view(1, 1, -1, 1)).to(torch.bfloat16)
+    v = v.to(torch.bfloat16)
+    flags = torch.zeros((1, N), dtype=torch.uint8, device="cuda")
+    flags[0, torch.randperm(N, generator=g, device="cuda")[:n_protect]] = 1
+    o = torch.full((1, H, N, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((1, H, N), 7.0, dtype=torch.float32, device="cuda")
+    ws = av.avsa_protected_rows_attn(q, k, v, flags, n_protect, d, o, lse=lse)
+    _status_ok(ws)
+    assert av.avsa_redo_count(ws) >= H * -(-n_protect // 128)      # every query tile, in one part at least
+    hs, on = [0, H - 1], flags[0].bool().cpu().numpy()
+    want_o, want_l = orc.dense_attention(_np64(q[:, hs]), _np64(k[:, hs]), _np64(v[:, hs]))
+    got_o, got_l = _np64(o[:, hs]), _np64(lse[:, hs])
+    _close(got_o[:, :, on], want_o[:, :, on], "outgrown protected O")
+    _close_lse(got_l[:, :, on], want_l[:, :, on], "outgrown protected lse")
+    off = ~flags[0].bool()
+    assert bool((o[:, :, off] == 7.0).all()) and bool((lse[:, :, off] == 7.0).all())
 
 
 @pytest.mark.parametrize("NB", [1, 32, 33, 256, 257, 512, 513, 1024, 1025])
