@@ -37,11 +37,11 @@ struct ColsumSmem {
   static constexpr int kKTile = 128 * D * 2;
   static constexpr int kK = 0;
   static constexpr int kQ = kColStages * kKTile;      // NCH * W * D * 2 bytes follow
-  static int bars_offset(int NCH, int W) { return kQ + NCH * W * D * 2; }
+  static constexpr int bars_offset(int NCH, int W) { return kQ + NCH * W * D * 2; }
   static constexpr int kNumBars = 1 + 2 * kColStages + 4;
   static constexpr int kBarBytes = 128;               // keeps the lse table behind it 16-byte aligned
   static_assert(kNumBars * 8 <= kBarBytes, "barrier area too small");
-  static int total(int NCH, int W) { return bars_offset(NCH, W) + kBarBytes + 512 * 4 + 16; }
+  static constexpr int total(int NCH, int W) { return bars_offset(NCH, W) + kBarBytes + 512 * 4 + 16; }
 };
 
 enum ColWhere { kColQFull = 21, kColKEmpty, kColKFull, kColSEmpty, kColSFull };
@@ -292,11 +292,11 @@ template <int D>
 struct ColsumRevSmem {
   static constexpr int kTile = 128 * D * 2;
   static constexpr int kQ = 0;                              // ring of query chunks
-  __host__ __device__ static int k_offset() { return kRevStages * kTile; }      // NKT resident key tiles follow
-  __host__ __device__ static int lse_offset(int NKT) { return k_offset() + NKT * kTile; }
-  __host__ __device__ static int bars_offset(int NKT) { return lse_offset(NKT) + kRevLseSlots * 512; }
+  __host__ __device__ static constexpr int k_offset() { return kRevStages * kTile; }      // NKT resident key tiles follow
+  __host__ __device__ static constexpr int lse_offset(int NKT) { return k_offset() + NKT * kTile; }
+  __host__ __device__ static constexpr int bars_offset(int NKT) { return lse_offset(NKT) + kRevLseSlots * 512; }
   static constexpr int kNumBars = 1 + 2 * kRevStages + 4;
-  static int total(int NKT) { return bars_offset(NKT) + 128 + 16; }
+  static constexpr int total(int NKT) { return bars_offset(NKT) + 128 + 16; }
 };
 
 enum ColRevWhere { kRevKFull = 51, kRevQEmpty, kRevQFull, kRevSEmpty, kRevSFull };
@@ -695,7 +695,10 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
     const int smem = L::total(c.NKT);
-    if (cudaFuncSetAttribute(colsum_rev_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    // always the same limit (four key tiles), whatever this call needs: the limit belongs to the kernel, and a host thread
+    // with fewer keys must not lower it between another thread's setting and launch
+    constexpr int kMaxSmem = L::total(4);
+    if (cudaFuncSetAttribute(colsum_rev_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
       return AVSA_ERR_CUDA;
     ColsumRevParams rp;
     rp.lse2 = lse2;
@@ -722,7 +725,8 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, c.W)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
     const int smem = L::total(c.NCH, c.W);
-    if (cudaFuncSetAttribute(colsum_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    constexpr int kMaxSmem = L::total(2, 256);      // 512 queries; always the same limit, as above
+    if (cudaFuncSetAttribute(colsum_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
       return AVSA_ERR_CUDA;
     ColsumParams cp;
     cp.part_lse2 = part_lse;

@@ -1051,3 +1051,43 @@ def test_mask_select_over_row_lengths(NB):
         _status_ok(out["ws"])
         assert np.array_equal(out["col_cnt"].cpu().numpy(), cnt)
         assert np.array_equal(out["col_idx"].cpu().numpy(), idx)
+
+
+@pytest.mark.parametrize("reverse", [False, True])
+def test_host_threads_with_short_and_long_axes_do_not_disturb_each_other(reverse):
+    """Two host threads, each with its stream, buffers and shape: the score pass needs 100 to 227 KB of shared memory, by the
+    length of the axis that stays on chip, and no call may fail because of what the other thread's last one asked for."""
+    import threading
+    shapes = ((16, 600), (512, 600))      # (short axis, long axis)
+    inputs, want = [], []
+    for n_short, n_long in shapes:
+        g = torch.Generator(device="cuda").manual_seed(n_short)
+        nq, nk = (n_long, n_short) if reverse else (n_short, n_long)
+        q, k = (torch.randn((1, 1, n, 128), generator=g, device="cuda").bfloat16() for n in (nq, nk))
+        buf = dict(scores=torch.empty((1, nk), device="cuda"), lse=torch.empty((1, 1, nq), device="cuda"),
+                   ws=torch.empty(av.avsa_cross_attn_scores_workspace_bytes(1, 1, nq, nk, 128), dtype=torch.uint8, device="cuda"))
+        inputs.append((q, k, buf))
+        want.append(av.avsa_cross_attn_scores(q, k, k, want_o=False, **buf)[2].clone())
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(i):
+        q, k, buf = inputs[i]
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            for _ in range(2000):
+                try:
+                    av.avsa_cross_attn_scores(q, k, k, want_o=False, **buf)
+                except av.AvsaError as e:
+                    failed.append((i, str(e)))
+                    break
+        stream.synchronize()
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    for (q, k, buf), w in zip(inputs, want):
+        assert torch.equal(buf["scores"], w)
