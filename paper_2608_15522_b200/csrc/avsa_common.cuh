@@ -52,7 +52,11 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, 
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  // The call returns this failure itself.  Left behind as the runtime's last error, it would fail the thread's next call too
+  // (every call ends by reading that error), or the next check of another library in the process.
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 // Resets the status record at the start of every call (first node of the call's launch sequence).
