@@ -100,6 +100,9 @@ bool device_is_sm100();
 // Grid size of the persistent kernels: one CTA per SM of the current device, at most one per work item.
 int persistent_grid(long long items);
 
+// (batch, head) pairs are counted in 32 bits: a product that wrapped to 0 would divide by 0 in the plans of the work
+inline bool pairs_ok(int B, int H) { return static_cast<long long>(B) * H <= 0x7fffffffll; }
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 }  // namespace avsa

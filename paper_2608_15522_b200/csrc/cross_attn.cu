@@ -764,7 +764,7 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
 using namespace avsa;
 
 extern "C" size_t avsa_cross_attn_scores_workspace_bytes(int B, int H, int Nq, int Nk, int d) {
-  if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128)) return 0;
+  if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128) || !pairs_ok(B, H)) return 0;
   return make_cross_plan(B, H, Nq, Nk, d).total;
 }
 
@@ -774,7 +774,7 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
                                       void* stream) {
   if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0) return AVSA_ERR_INVALID_ARG;
   if (d != 64 && d != 128) return AVSA_ERR_UNSUPPORTED;
-  if (H > 65535 || B > 65535) return AVSA_ERR_UNSUPPORTED;
+  if (H > 65535 || B > 65535 || !pairs_ok(B, H)) return AVSA_ERR_UNSUPPORTED;
   // the score pass keeps either the queries or the keys of a head on chip
   if (scores != nullptr && Nq > 512 && Nk > 512) return AVSA_ERR_UNSUPPORTED;
   if (!tensor_ok(q, B, H) || !tensor_ok(k, B, H) || !tensor_ok(v, B, H)) return AVSA_ERR_INVALID_ARG;

@@ -195,7 +195,7 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
 using namespace avsa;
 
 extern "C" size_t avsa_protected_rows_attn_workspace_bytes(int B, int H, int N, int d, int blk, int n_protect) {
-  if (B <= 0 || H <= 0 || N <= 0 || n_protect < 0 || n_protect > N) return 0;
+  if (B <= 0 || H <= 0 || N <= 0 || n_protect < 0 || n_protect > N || !pairs_ok(B, H)) return 0;
   if (!((blk == 128 && d == 128) || (blk == 64 && d == 64))) return 0;
   return make_prot_plan(B, H, N, d, n_protect).total;
 }
@@ -205,7 +205,7 @@ extern "C" int avsa_protected_rows_attn(int B, int H, int N, int d, int blk, avs
                                         float* lse, float softmax_scale, void* ws, size_t ws_bytes, void* stream) {
   if (B <= 0 || H <= 0 || N <= 0 || n_protect < 0 || n_protect > N) return AVSA_ERR_INVALID_ARG;
   if (!((blk == 128 && d == 128) || (blk == 64 && d == 64))) return AVSA_ERR_UNSUPPORTED;
-  if (H > 65535 || B > 65535) return AVSA_ERR_UNSUPPORTED;
+  if (H > 65535 || B > 65535 || !pairs_ok(B, H)) return AVSA_ERR_UNSUPPORTED;
   if (!tensor_ok(q, B, H) || !tensor_ok(k, B, H) || !tensor_ok(v, B, H)) return AVSA_ERR_INVALID_ARG;
   if (prot_tok == nullptr || o_bf16 == nullptr || !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;

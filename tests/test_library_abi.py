@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 from paper_2608_15522_b200 import binding as av
 from paper_2608_15522_b200 import build
@@ -42,3 +44,20 @@ def test_host_only_entry_points():
     assert av.avsa_build_block_mask_workspace_bytes(1, 24, 32760, 128, 128) > 2 * 24 * 256 * 128 * 4
     assert av.avsa_sparse_self_attn_workspace_bytes(1, 24, 32760, 128, 128) >= 16
     assert av.avsa_cross_attn_scores_workspace_bytes(1, 1, 1, 1, 96) == 0
+
+
+def test_more_pairs_than_32_bits_count_are_refused():
+    """2^32 (batch, head) pairs wrap to 0, which the plans of the work divide by: the queries say 0 (not supported) and the calls
+    AVSA_ERR_UNSUPPORTED, before any pointer is followed.  In a process of its own: a division by 0 ends it."""
+    code = """if True:
+        from paper_2608_15522_b200 import binding as av
+        for b, h in ((65536, 65536), (40000, 60000)):
+            assert av.avsa_cross_attn_scores_workspace_bytes(b, h, 4, 4, 64) == 0
+            assert av.avsa_protected_rows_attn_workspace_bytes(b, h, 4, 64, 64, 1) == 0
+        lib, t = av.load_library(), av._Bf16Tensor4(4096, 8, 8, 64)
+        args = (65535, 65535, 4)
+        assert lib.avsa_cross_attn_scores(*args, 4, 64, t, t, t, 4096, 4096, 4096, 0.0, 1.0, 0.0, 4096, 1 << 40, 0) == av.AVSA_ERR_UNSUPPORTED
+        assert lib.avsa_protected_rows_attn(*args, 64, 64, t, t, t, 4096, 1, 4096, 4096, 0.0, 4096, 1 << 40, 0) == av.AVSA_ERR_UNSUPPORTED
+    """
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    assert r.returncode == 0, r.stdout
