@@ -129,3 +129,98 @@ def test_audio_features_of_any_rank_keep_their_token_axis(recorded):
         with pytest.raises(ValueError):
             av.avsa_cache_indicators(_OnGpu(bad_v), y_v, y_v, y_v, out=out, ws=ws)
     assert recorded == []
+
+
+# ------------------------------------------------------------------------- every check by itself, on otherwise good arguments
+_VIEWS = {"cross": ("q", "k", "v"), "mask": ("q", "k"), "sparse": ("q", "k", "v"), "protected": ("q", "k", "v"),
+          "indicators": ("y_v", "yhat_v", "y_a", "yhat_a")}
+
+
+def _good(name):
+    """Arguments of one call that nothing is wrong with: stand-ins on cuda:1, every buffer handed in."""
+    def view(i, n=96):
+        return _OnGpu((2, 3, n, 64), ptr=4096 * i, stride=(3 * n * 64 + 8, n * 64, 64, 1))
+
+    def f32(i):
+        return _OnGpu((2, 3, 2, 2), torch.float32, ptr=4096 * i)
+
+    def feat(i, n):
+        return _OnGpu((2, n, 384), ptr=4096 * i)
+
+    u8, ws = _OnGpu((2, 96), torch.uint8, ptr=4096 * 20), _OnGpu((5000,), torch.uint8, ptr=4096 * 30)
+    if name == "cross":
+        return dict(q=view(1, 32), k=view(2), v=view(3), o=view(4), lse=f32(5), scores=f32(6), score_beta=0.25, score_gamma=0.5,
+                    softmax_scale=0.125, ws=ws)
+    if name == "mask":
+        return dict(q=view(1), k=view(2), scores=f32(3), n_protect=7, k_keep=2, blk=64, flags=0x8001, softmax_scale=0.25,
+                    out=dict(block_scores=f32(4), col_idx=f32(5), col_cnt=f32(6), prot_tok=u8, prot_blk=f32(7)), ws=ws)
+    if name == "sparse":
+        return dict(q=view(1), k=view(2), v=view(3), col_idx=f32(4), col_cnt=f32(5), blk=64, softmax_scale=0.5, o=view(6), lse=f32(7),
+                    ws=ws)
+    if name == "protected":
+        return dict(q=view(1), k=view(2), v=view(3), prot_tok=u8, n_protect=9, blk=64, o=view(6), lse=f32(7), softmax_scale=0.5, ws=ws)
+    return dict(y_v=feat(1, 40), yhat_v=feat(2, 40), y_a=feat(3, 24), yhat_a=feat(4, 24), prot_tok=u8, s_cur=f32(5), s_anchor=f32(6),
+                lambda_p=0.5, lambda_s=0.25, tau=0.125, eps=0.0625, out=f32(7), ws=ws)
+
+
+_ENTRY = {"cross": av.avsa_cross_attn_scores, "mask": av.avsa_build_block_mask, "sparse": av.avsa_sparse_self_attn,
+          "protected": av.avsa_protected_rows_attn, "indicators": av.avsa_cache_indicators}
+
+
+def _at(i, n=96):
+    return (4096 * i, 3 * n * 64 + 8, n * 64, 64)
+
+
+_P = [4096 * i for i in range(8)]
+_FLAGS, _WS = 4096 * 20, [4096 * 30, 5000, 4097]      # workspace, its size, the stream of cuda:1
+
+
+@pytest.mark.parametrize("name,want", [
+    ("cross", [2, 3, 32, 96, 64, _at(1, 32), _at(2), _at(3), _P[4], _P[5], _P[6], 0.25, 0.5, 0.125]),
+    ("mask", [2, 3, 96, 64, 64, _at(1), _at(2), _P[3], 7, 2, 0x8001, 0.25, _P[4], _P[5], _P[6], _FLAGS, _P[7]]),
+    ("sparse", [2, 3, 96, 64, 64, _at(1), _at(2), _at(3), _P[4], _P[5], _P[6], _P[7], 0.5]),
+    ("protected", [2, 3, 96, 64, 64, _at(1), _at(2), _at(3), _FLAGS, 9, _P[6], _P[7], 0.5]),
+    ("indicators", [2, 40, 24, 384, _P[1], _P[2], _P[3], _P[4], _FLAGS, _P[5], _P[6], 0.5, 0.25, 0.125, 0.0625, _P[7]]),
+])
+def test_good_arguments_reach_the_library_as_they_are(recorded, name, want):
+    """Sizes, pointers, strides, counts, the workspace's size and the stream of the tensors' device, in the library's order."""
+    _ENTRY[name](**_good(name))
+    assert recorded == [(name, want + _WS)]
+
+
+def _wrong(t, what):
+    if what == "none":
+        return None
+    new = _OnGpu(t.shape, t.dtype, t.stride(), t.data_ptr())
+    if what == "fp32":
+        new.dtype = torch.float32
+    elif what == "host":
+        new.is_cuda = False
+    elif what == "rank":
+        new.shape, new._stride = new.shape[1:], new._stride[1:]
+    else:      # the innermost axis not contiguous
+        new._stride = new._stride[:-1] + (2,)
+    return new
+
+
+@pytest.mark.parametrize("what,error,match", [
+    ("fp32", ValueError, "bf16"), ("host", ValueError, "CUDA"), ("stride", ValueError, "contiguous"),
+    ("rank", ValueError, "bf16 tensor|dimensions|unpack"), ("none", AttributeError, "NoneType")])
+@pytest.mark.parametrize("name,arg", [(n, a) for n in _VIEWS for a in _VIEWS[n]])
+def test_one_wrong_tensor_is_refused(recorded, name, arg, what, error, match):
+    """Exactly one property of one tensor is wrong, so that only the check meant for it can refuse the call."""
+    args = _good(name)
+    if name == "indicators" and what == "rank" and arg != "y_v":
+        pytest.skip("any rank is taken there")
+    if name == "mask" and what == "none":
+        args[arg] = None      # a null view: the library says whether the flags allow it
+        if arg == "q":
+            args["shape"] = (2, 3, 96, 64)
+            args["block_scores"] = args["out"]["block_scores"]
+        _ENTRY[name](**args)
+        assert recorded.pop()[1][5 + (arg == "k")] == (None, 0, 0, 0)
+        return
+    args[arg] = _wrong(args[arg], what)
+    with pytest.raises(error, match=match):
+        _ENTRY[name](**args)
+    assert recorded == []
