@@ -520,7 +520,7 @@ def test_cross_attention_long_query_axis_two_chunks():
     (1, 96, 300, 520, 128, True),      # the same with the queries in two chunks
 ])
 def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
-    """Every way the (query tile, key tile) work is cut over the CTAs: whole rows, split rows, chunks that do not divide
+    """The ways a stream of (query tile, key tile) pairs is cut over the CTAs: whole rows, split rows, chunks that do not divide
     the query tiles; with O, and with only the LSE asked for (same LSEs)."""
     g = torch.Generator().manual_seed(Nq * 7 + Nk)
     q, k, v = (torch.randn((B, H, n, d), generator=g).to(torch.bfloat16) for n in (Nq, Nk, Nk))
@@ -1103,3 +1103,29 @@ def test_a_refused_launch_fails_its_own_call_only():
     m = av.avsa_build_block_mask(q[:, :2], q[:, :2], None, 0, 1, 64)
     _status_ok(m["ws"])
     assert (m["col_cnt"] == 1).all() and (m["col_idx"] == 0).all()
+
+
+@pytest.mark.parametrize("growth", [0.0, 4.0])
+def test_cross_attention_queue_with_its_end_cut(growth):
+    """240 heads x 4 query tiles x 29 key tiles: long enough for the queue, whose last units are cut in two.  Whole query
+    tiles go out as tiles, the cut ones through the merge, and the score pass takes the LSEs of both.  With logits that grow by
+    4 per 128 keys whole items and parts (15 tiles) outgrow their reference and are recomputed."""
+    B, H, nq, nk, d = 10, 24, 512, 3712, 64
+    g = torch.Generator(device="cuda").manual_seed(17)
+    u = 1.0 / np.sqrt(d)
+    q, k, v = (torch.randn((B, H, n, d), generator=g, device="cuda") for n in (nq, nk, nk))
+    if growth:
+        q = q + 8.0 * u
+        ramp = torch.arange(nk, dtype=torch.float32, device="cuda").div(128, rounding_mode="floor") * growth * np.sqrt(d) / 8.0
+        k = k + (ramp * u).view(1, 1, -1, 1)
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    o, lse, s, ws = av.avsa_cross_attn_scores(q, k, v, score_gamma=1.0 / (H * nq))
+    _status_ok(ws)
+    assert (av.avsa_redo_count(ws) >= B * H * 4) if growth else (av.avsa_redo_count(ws) == 0)
+    for b in (0, B - 1):      # whole rows; cut rows
+        want_o, want_lse, A = orc.cross_attention(_np64(q[b : b + 1]), _np64(k[b : b + 1]), _np64(v[b : b + 1]))
+        _close(_np64(o[b : b + 1]), want_o, "queue O")
+        _close_lse(_np64(lse[b : b + 1]), want_lse, "queue lse")
+        _close_scores(_np64(s[b : b + 1]), orc.column_scores(A, gamma=1.0 / (H * nq)), "queue scores")
+    _, lse2, _, _ = av.avsa_cross_attn_scores(q, k, v, want_scores=False, want_o=False)
+    assert torch.equal(lse, lse2)
