@@ -15,8 +15,8 @@
 // MODE_LIST   key tiles come from an explicit ascending list; the output tile is converted to bf16
 //             and TMA-stored; optional natural-log LSE.
 // MODE_RANGE  key tiles are a contiguous range.  Part of the key axis: the output is a partial result (fp32 rows
-//             normalised by their own sum) for merge_splits_rows.  The whole key axis: output written like MODE_LIST
-//             (unless the caller wants partials throughout).  The log2-domain LSE of the range is written either way.
+//             normalised by their own sum) for merge_splits_rows.  The whole key axis: output written like MODE_LIST,
+//             through a row map, or not at all (AttnParams::store).  The log2-domain LSE of the range is written either way.
 #pragma once
 #include "avsa_common.cuh"
 #include "sm100_ptx.cuh"
@@ -90,8 +90,8 @@ struct RangeSplit {
   __host__ __device__ bool whole_rows() const {      // no query tile is split
     return L > 0 ? L % NKB == 0 : (nA == 1 || unitsA == 0) && (nB == 1 || unitsA == units);
   }
-  // Item: stream: unit * ctas + CTA (below 2^31: one query tile of 128 rows is 16 KB at least, so 2^31 / 148 of them do
-  // not fit the card); queue: the slot.
+  // Item: stream: unit * ctas + CTA (far below 2^31: calls of more than a few thousand units go to the queue, whose cost
+  // per tile is lower); queue: the slot.
   struct Item {
     int u, j, kb0, cnt, slot;      // cnt <= 0: nothing there
   };

@@ -92,8 +92,9 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&r)[8]) 
 }
 
 // MODE_LIST: work item = query tile with an explicit list of key tiles, output bf16 rows + optional LSE
-// (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE: the CTA's items are its segments of
-// the stream described at RangeSplit, fixed by its index; output bf16 rows where the key axis is not split, else
+// (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE: the work is cut as RangeSplit
+// describes; the CTA's items are its segments of the stream, fixed by its index, or come off the queue like the lists
+// (which of the two: make_range_split); output bf16 rows where the key axis is not split, else
 // normalised fp32 partials for merge_splits_rows, and the log2 LSE of the range.
 template <int BLK, int D, int MODE, bool FOLD>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -136,10 +137,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   constexpr int REDO = 8 * kPRing;
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + L::kMisc);   // [0] tmem base, [1] stop
 
-  volatile int* mine = reinterpret_cast<volatile int*>(smem + L::kRedo);
+  volatile int* own_redo = reinterpret_cast<volatile int*>(smem + L::kRedo);      // FOLD: count, then from [4] on the items
 
   if (tid == 0) {
-    if (FOLD) mine[0] = 0;
+    if (FOLD) own_redo[0] = 0;
     for (int s = 0; s < kPQB; s++) {
       mbar_init(BAR(Q_FULL + s), 1);
       mbar_init(BAR(Q_EMPTY + s), 1);
@@ -303,7 +304,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         }
         // The CTA's first item is its own index, the others come off the queue behind those of the whole grid: with
         // one item or less per CTA, a CTA that is a little early must not take a second one from a late CTA.
-        if (FOLD && __any_sync(FULLM, mine[0] >= L::kRedoCap - kPRing)) break;
+        if (FOLD && __any_sync(FULLM, own_redo[0] >= L::kRedoCap - kPRing)) break;
         if (!first) {
           if (lane == 0) id = gridDim.x + atomicAdd(&p.status->next_item, 1);
           id = __shfl_sync(FULLM, id, 0);
@@ -609,8 +610,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         if (redo) {
           redo_list[atomicAdd(&p.status->redo_count, 1)] = it.item;
           if (FOLD) {
-            mine[4 + mine[0]] = it.item;
-            mine[0] = mine[0] + 1;
+            own_redo[4 + own_redo[0]] = it.item;
+            own_redo[0] = own_redo[0] + 1;
           }
         }
       }
@@ -690,7 +691,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   tc_fence_before();
   __syncthreads();
   if (warp == 2) tmem_dealloc(tmem, 512);
-  if (FOLD && mine[0] > 0 && misc[1] == 0u) {          // uniform over the CTA; hardly ever taken
+  if (FOLD && own_redo[0] > 0 && misc[1] == 0u) {          // uniform over the CTA; hardly ever taken
     if (tid == 0) {
       for (int i = 0; i < L::kNumBars; i++) mbar_inval(bar0 + i * 8);
     }

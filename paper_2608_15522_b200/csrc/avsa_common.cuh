@@ -18,8 +18,8 @@ struct StatusRecord {
   int where;      // which wait / check
   int item;       // work item (block index)
   int aux;        // tile index or offending value
-  int redo_count; // sparse attention: work items the fast kernel left to the exact kernel in this call
-  int next_item;  // sparse attention: head of the work queue of the persistent kernel
+  int redo_count; // attention calls: work items whose rows outgrew their reference and were recomputed exactly
+  int next_item;  // attention calls: head of the work queue of the persistent kernel
 };
 constexpr size_t kStatusBytes = 256;   // the record, padded so that what follows stays 256-byte aligned
 
@@ -33,10 +33,20 @@ __device__ __forceinline__ void report_status(StatusRecord* st, int code, int wh
 
 // ------------------------------------------------------------------------------------ programmatic dependent launch
 // Every kernel of the library's calls is launched as a programmatic dependent of the kernel before it on the stream:
-// it is set up while that one drains, waits (pdl_wait) before it touches memory that an earlier kernel may read or
-// write, and then lets its own successor be set up (pdl_launch).  A grid retires only after its own wait, so whatever
-// is ordered behind it is ordered behind everything before it as well.  Between ordinary launches the GPU idles
-// 1.5-4 us each; the smallest layer-step (eleven launches) took 33 us with them.
+// it is set up while that one drains, waits (pdl_wait) for that kernel's end, and lets its own successor be set up
+// (pdl_launch).  Between ordinary launches the GPU idles 1.5-4 us each; the smallest layer-step (eleven launches) took
+// 33 us with them.  What keeps a chain of such launches in order:
+//   - every grid has CTAs that wait, so it retires only after its predecessor has, and whatever waits for it is behind
+//     everything before it as well;
+//   - a kernel may touch memory before its own wait only if the kernel in front of it lets it go no earlier than after a
+//     wait of its own (then everything before that kernel is done) and writes nothing that the early part uses.
+// Most kernels wait first and let their successor go right after.  The others:
+//   - pool_kernel lets its successor go at once, reads q and k and writes the pooled means without waiting; only its last
+//     CTAs wait, before they retire.  token_select_kernel in front of it goes by the rule;
+//   - score_select_kernel lets its successor go before it waits itself: the successor must wait before it touches
+//     anything (every first kernel of a call and expand_blocks_kernel do);
+//   - indicators_finalize_kernel reads the saliencies before its wait; l1_partials_kernel in front of it goes by the rule;
+//   - colsum_kernel and colsum_rev_kernel let their successor go at their end only (the reason stands there).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
