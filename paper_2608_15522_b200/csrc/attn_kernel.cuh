@@ -61,6 +61,9 @@ struct AttnSmem {
 // `chunk` CTAs, and group g takes tiles [g L, (g+1) L).  Every CTA gets the same number of tiles up to one, in at most
 // L/NKB + 2 contiguous segments.  For calls of few tiles per CTA, where equal pieces do not divide over the CTAs (128
 // query tiles on 148 SMs: 20 idle; 340 us as one item each, 323 as a stream).
+//   The shares of a stream are fixed: a CTA that starts late, because another stream's kernel holds its SM, brings its whole share
+// with it, and the call takes up to twice as long (512 queries x 49152 keys, 32 heads, us: 328 alone, 550 with 4 to 32 SMs
+// held; cut into 128 equal items off a queue 377 in both, and 635 from 24 SMs on).
 //   Queue (L == 0): the first unitsA units are cut into nA pieces of tpsA tiles, the rest into smaller ones (nB, tpsB),
 // and the CTAs take them off a queue.  The SMs are not equally fast (a GPC's SMs share their way to L2; equal shares end
 // up to 10 % apart), so for long calls the queue with small pieces at its end is the better balance: 1782 us as a stream,
@@ -582,7 +585,10 @@ __device__ __forceinline__ void attn_fwd_body(const CUtensorMap* tmq, const CUte
 // (128 keys against 128 queries, 0.7 us): an item's own start and end take about four (measured on one-tile items), a
 // merge grid about four; the slowest SM needs 8 % more for an equal share; and beyond ~70 tile streams side by side the
 // DRAM (6.5 TB/s against 64 KB per tile and stream) sets the pace instead of the tensor pipe.
-inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_of_l2) {
+//   `max_run`: key tiles that one accumulator may sum.  The fp32 accumulation of the tensor cores truncates, which draws long
+// sums towards zero: dense rows of 49152 keys in one run were 2.4e-4 of their value low, in runs of 64 tiles 1.3e-4, and
+// their LSEs' error was 5.6e-7 instead of 5.3e-7.
+inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_of_l2, int max_run) {
   RangeSplit best = {};
   double best_cost = 0.0;
   // (more than 32 query tiles side by side share no more, and small chunks divide the CTAs better)
@@ -603,6 +609,7 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
     const long long rows = (even + NKB - 1) / NKB * NKB;         // the same, no query tile split
     for (int v = 0; v < (rows != even ? 2 : 1); v++) {
       const long long L = v == 0 ? rows : even;
+      if ((L < NKB ? L : NKB) > max_run) continue;
       r.L = static_cast<int>(L);
       r.groups = static_cast<int>((tiles + L - 1) / L);
       r.ctas = r.groups * chunk;
@@ -616,10 +623,12 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
     }
   }
   // the queue: pieces of 48 tiles or more (a part of a row costs three tiles more than a whole one: its fp32 rows are
-  // written and read again), the last round of them cut into smaller ones
+  // written and read again), smaller ones only where max_run rules out the rest, and the last round of them cut into
+  // smaller ones
   const int cpb = (NQT + 31) / 32;
   const double share = static_cast<double>(BH) * NQT * NKB / ctas;       // tiles per CTA
-  for (int n = 1; n == 1 || NKB / n >= 48; n++) {
+  const int n0 = (NKB + max_run - 1) / max_run;
+  for (int n = n0; n == n0 || NKB / n >= (best.ctas == 0 ? 8 : 48); n++) {
     RangeSplit r = {};
     r.chunk = (NQT + cpb - 1) / cpb;
     r.cpb = cpb;
@@ -635,12 +644,19 @@ inline RangeSplit make_range_split(int BH, int NQT, int NKB, int ctas, bool out_
     r.nB = (NKB + r.tpsB - 1) / r.tpsB;
     const bool cut_tail = r.tpsB < r.tpsA;
     const double tail = cut_tail ? static_cast<double>(r.tpsA) * ctas * cpb / (static_cast<double>(NQT) * NKB) : 0.0;
-    if (share < 3.0 * r.tpsA || tail + 1.0 > r.units) continue;
+    if (share < 3.0 * r.tpsA || tail + 1.0 > r.units) {
+      // (no plan yet, and the pieces of the next round would be tiny: equal pieces)
+      if (best.ctas != 0 || NKB / (n + 1) >= 8) continue;
+      r.tpsB = r.tpsA;
+      r.nB = r.nA;
+      r.unitsA = r.units;
+      return r;
+    }
     r.unitsA = cut_tail ? r.units - static_cast<int>(tail + 1.0) : r.units;
     const double main_share = cut_tail ? share - r.tpsA : share;
     const double cost = share + (r.nA > 1 ? 7.0 : 4.0) * main_share / r.tpsA + (cut_tail ? 7.0 * r.tpsA / r.tpsB : 0.0) +
                         0.7 * r.tpsB + (r.whole_rows() ? 0.0 : 4.0);
-    if (cost < best_cost) {
+    if (best.ctas == 0 || cost < best_cost) {
       best = r;
       best_cost = cost;
     }

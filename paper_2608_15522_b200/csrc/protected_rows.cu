@@ -103,6 +103,10 @@ struct ProtPlan {
 // make_cross_plan).
 constexpr int kProtTile = 128;
 
+// Key tiles that one accumulator sums (see make_range_split): 64, and with 64 channels 32, as long as the sums were with the 64-key
+// tiles of before.
+constexpr int prot_max_run(int d) { return d / 2; }
+
 static ProtPlan make_prot_plan(int B, int H, int N, int d, int n_protect) {
   constexpr int blk = kProtTile;
   ProtPlan c;
@@ -111,7 +115,7 @@ static ProtPlan make_prot_plan(int B, int H, int N, int d, int n_protect) {
   c.n_pad = c.NQT * blk;
   c.NKB = (N + blk - 1) / blk;
   const long long kv_bytes = 4ll * B * H * N * d;
-  c.rs = make_range_split(B * H, c.NQT, c.NKB, persistent_grid(1 << 30), kv_bytes > kL2KeepBytes);
+  c.rs = make_range_split(B * H, c.NQT, c.NKB, persistent_grid(1 << 30), kv_bytes > kL2KeepBytes, prot_max_run(d));
   size_t off = kStatusBytes;
   const size_t slots = static_cast<size_t>(c.rs.slots());
   c.off_rows = off; off += align_up(static_cast<size_t>(B) * c.n_pad * sizeof(int32_t), 256);

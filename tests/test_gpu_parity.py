@@ -1129,3 +1129,26 @@ def test_cross_attention_queue_with_its_end_cut(growth):
         _close_scores(_np64(s[b : b + 1]), orc.column_scores(A, gamma=1.0 / (H * nq)), "queue scores")
     _, lse2, _, _ = av.avsa_cross_attn_scores(q, k, v, want_scores=False, want_o=False)
     assert torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_long_dense_rows_do_not_drift_towards_zero(d):
+    """The tensor cores' fp32 accumulation truncates, so what one accumulator sums is bounded (64 key tiles, 32 with 64
+    channels).  With values of mean 1 the error along the result shows it: 1.1e-4 to 1.3e-4 of the value in such runs, 2.4e-4
+    when the 384 tiles of this sequence are one run; bf16 rounding averages out over the 32768 (16384) elements compared
+    (1.8e-3 / sqrt(16384) = 1.4e-5)."""
+    H, N, n_protect = 8, 49152, 8192
+    g = torch.Generator(device="cuda").manual_seed(d)
+    q, k, v = (torch.randn((1, H, N, d), generator=g, device="cuda") for _ in range(3))
+    q, k, v = q.to(torch.bfloat16), k.to(torch.bfloat16), (v + 1.0).to(torch.bfloat16)
+    rows = torch.randperm(N, generator=g, device="cuda")[:n_protect]
+    flags = torch.zeros((1, N), dtype=torch.uint8, device="cuda")
+    flags[0, rows] = 1
+    o = torch.zeros_like(q)
+    _status_ok(av.avsa_protected_rows_attn(q, k, v, flags, n_protect, d, o))
+    hs, rows = [0, 1], rows[:128]      # (the last heads are the cut end of the queue)
+    want, _, _ = orc.cross_attention(_np64(q[:, hs][:, :, rows]), _np64(k[:, hs]), _np64(v[:, hs]))
+    got = _np64(o[:, hs][:, :, rows])
+    _close(got, want, "long dense rows")
+    drift = ((got - want) * want).sum() / (want * want).sum()
+    assert abs(drift) <= 1.8e-4, f"drift {drift:.2e}"
