@@ -26,14 +26,15 @@
  *     kernels' work queue.  Calls on the same workspace must not overlap on the GPU.
  *   - The attention calls (cross-attention pass 1, sparse self-attention, protected rows) run a kernel that
  *     normalises each row by the maximum of its first key tile instead of a running maximum (softmax is
- *     invariant to that shift), and behind it an exact-rescaling kernel for the work items whose rows
- *     outgrew that reference (a row whose sum of exp(logit - reference) ends above 2^64 or not finite;
- *     values of v are assumed to stay below 2^60 in magnitude).  Results do not depend on which kernel
- *     produced them beyond rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).
+ *     invariant to that shift), and recompute with exact rescaling the work items whose rows outgrew that
+ *     reference (a row whose sum of exp(logit - reference) ends above 2^64 or not finite; values of v are
+ *     assumed to stay below 2^60 in magnitude): in the same kernel in short calls, in one behind it in
+ *     long ones.  Results do not depend on which way produced them beyond rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).
  *   - Errors detectable on the host return at once with nothing enqueued.  Return values are
  *     avsa_status codes.
- *   - Supported shapes: (blk, d) in {(128,128), (64,64)}; any N >= 1 (the last block may be partial:
- *     pooled means divide by the valid count, invalid keys are masked, rows >= N are not written).
+ *   - Supported shapes: (blk, d) in {(128,128), (64,64)}; B and H up to 65535, B*H below 2^31 (mask: up to
+ *     65535); any N >= 1 (the last block may be partial: pooled means divide by the valid count, invalid
+ *     keys are masked, rows >= N are not written).
  */
 #ifndef AVSA_H_
 #define AVSA_H_
