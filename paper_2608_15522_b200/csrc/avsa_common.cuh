@@ -63,8 +63,8 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-  // The call returns this failure itself.  Left behind as the runtime's last error, it would fail the thread's next call too
-  // (every call ends by reading that error), or the next check of another library in the process.
+  // The call returns this failure itself.  Left behind as the runtime's last error, which every call reads at its end, it
+  // would fail a good call of the same thread: the next one that does not set a kernel attribute (that clears it).
   if (e != cudaSuccess) cudaGetLastError();
   return e;
 }

@@ -1095,14 +1095,16 @@ def test_host_threads_with_short_and_long_axes_do_not_disturb_each_other(reverse
 
 def test_a_refused_launch_fails_its_own_call_only():
     """65536 (batch, head) pairs are one more than the mask's pooling grid can have, which the launch itself reports.  The
-    call fails; the next call on the thread, and PyTorch's next launch, know nothing of it."""
+    call fails; the thread's next call knows nothing of it (the indicators: their call sets no kernel attribute, which would
+    clear the runtime's last error by itself)."""
     q = torch.zeros((1, 65536, 1, 64), dtype=torch.bfloat16, device="cuda")
     with pytest.raises(av.AvsaError) as e:
         av.avsa_build_block_mask(q, q, None, 0, 1, 64)
     assert e.value.status == av.AVSA_ERR_CUDA
-    m = av.avsa_build_block_mask(q[:, :2], q[:, :2], None, 0, 1, 64)
-    _status_ok(m["ws"])
-    assert (m["col_cnt"] == 1).all() and (m["col_idx"] == 0).all()
+    y = torch.ones((1, 8, 64), dtype=torch.bfloat16, device="cuda")
+    out, ws = av.avsa_cache_indicators(y, y, y, y)
+    _status_ok(ws)
+    assert (out[0, :5] == 0.0).all() and out[0, 5] == 1.0
 
 
 @pytest.mark.parametrize("growth", [0.0, 4.0])
