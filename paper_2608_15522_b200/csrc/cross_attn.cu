@@ -3,7 +3,9 @@
 //   pass 1  flash attention, key axis split across CTAs -> partial (O, LSE) -> merge -> O, row LSE
 //   pass 2  for every key tile: S^T = K Q^T on the tensor cores, p = exp2(S^T c - lse_j), summed over
 //           the queries -> per-head column sums -> fixed-order head sum with the beta/gamma blend
+// With at most 256 keys both are one pass over the queries: cross_resident.cuh.
 #include "attn_persist_kernel.cuh"
+#include "cross_resident.cuh"
 
 namespace avsa {
 
@@ -571,11 +573,30 @@ struct CrossPlan {
   int NKT, NCH, W, n_range, tpc, ctas2;      // pass 2 (key tiles of 128), cuts per pair, tiles per CTA, CTAs
   bool reverse;                              // pass 2 with the keys resident (Nq > 512, Nk <= 512)
   int NQC, rev_ranges, rev_cpr, rev_slots;   // query chunks of 128, CTAs per (b,h), chunks per CTA, partial slots
-  size_t off_part_o, off_part_lse, off_lse, off_lse2, off_partial, off_redo, total;
+  bool resident;                             // both passes in one kernel, K and V of a head on chip
+  int res_tiles, res_L, res_ctas;            // query tiles of all pairs, per CTA, CTAs
+  size_t off_part_o, off_part_lse, off_lse, off_lse2, off_partial, off_redo, off_cta, total;
 };
 
 static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
-  CrossPlan c;
+  CrossPlan c = {};
+  // Few keys: everything in one kernel, whatever the number of queries (faster from 2 heads x 32 queries to 64 x 19200, with scores
+  // and without: cross_resident.cuh).  More than 256 keys of 128 channels do not fit an SM's shared memory beside the tiles, nor
+  // their logits its tensor memory.  (Tiles are counted in 32 bits there; calls beyond that go the other way.)
+  const long long tiles = static_cast<long long>(B) * H * ((Nq + 127) / 128);
+  if (Nk <= kResMaxKeys && tiles < (1ll << 30)) {
+    c.resident = true;
+    c.NQT = (Nq + 127) / 128;
+    c.res_tiles = static_cast<int>(tiles);
+    const int grid = persistent_grid(tiles);
+    c.res_L = (c.res_tiles + grid - 1) / grid;
+    c.res_ctas = (c.res_tiles + c.res_L - 1) / c.res_L;
+    size_t off = kStatusBytes;
+    c.off_cta = off; off += align_up(static_cast<size_t>(c.res_ctas) * sizeof(CtaStatus), 256);
+    c.off_partial = off; off += align_up((static_cast<size_t>(c.res_ctas) + B * H) * Nk * sizeof(float), 256);
+    c.total = off;
+    return c;
+  }
   // Tiles of 128 rows for both head sizes.  With 64 channels and 64-row tiles, half of the MMA's 128 rows held nothing,
   // and every hand-over moved half as many keys (24 heads,
   // 256 queries x 32760 keys with scores: 369 us; with these tiles 162; reverse direction 342 -> 212).
@@ -625,6 +646,63 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   c.off_redo = off; off += align_up(slots1 * sizeof(int), 256);
   c.total = off;
   return c;
+}
+
+template <int D, int KG, bool SCORES>
+static int launch_resident(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
+                           const ResidentParams& rp, int ctas, cudaStream_t st) {
+  constexpr int kSmem = ResidentSmem<D, KG>::kTotal;
+  if (cudaFuncSetAttribute(cross_resident_kernel<D, KG, SCORES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+    return AVSA_ERR_CUDA;
+  return launch_pdl(cross_resident_kernel<D, KG, SCORES>, ctas, kResThreads, kSmem, st, tq, tk, tv, to, rp) == cudaSuccess
+             ? AVSA_OK : AVSA_ERR_CUDA;
+}
+
+template <int D>
+static int run_cross_resident(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const avsa_bf16_4d& k, const avsa_bf16_4d& v,
+                              void* o, float* lse, float* scores, float beta, float gamma, float scale, uint8_t* ws,
+                              const CrossPlan& c, cudaStream_t st) {
+  StatusRecord* status = reinterpret_cast<StatusRecord*>(ws);
+  CUtensorMap tq, tk, tv, to;
+  if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
+  if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
+  if (!encode_bf16_tile_map(&tv, v.ptr, B, H, Nk, D, v.stride_b, v.stride_h, v.stride_n, 128)) return AVSA_ERR_CUDA;
+  to = tq;      // not used without an output
+  if (o != nullptr && !encode_bf16_tile_map(&to, o, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 32)) return AVSA_ERR_CUDA;
+  ResidentParams rp = {};
+  rp.lse = lse;
+  rp.partial = reinterpret_cast<float*>(ws + c.off_partial);
+  rp.status = status;
+  rp.cta_status = reinterpret_cast<CtaStatus*>(ws + c.off_cta);
+  rp.H = H;
+  rp.Nq = Nq;
+  rp.NQT = c.NQT;
+  rp.Nk = Nk;
+  rp.tiles = c.res_tiles;
+  rp.L = c.res_L;
+  const int chunks = (Nk + 31) / 32;
+  // The first group has the first 128 keys, not half of them: the exponentials take the same time either way (the groups share
+  // the MUFU), and the more keys the reference maximum covers, the more often the largest probability is exactly 1 (157 keys:
+  // O 2.04e-3 from 64 bits, 2.10e-3 with equal halves).
+  rp.nch0 = chunks < 4 ? chunks : 4;
+  rp.nch1 = chunks - rp.nch0;
+  rp.store_o = o != nullptr ? 1 : 0;
+  rp.scale_log2 = scale * 1.4426950408889634f;
+  int rc;
+  if (scores != nullptr) {
+    rc = Nk > 128 ? launch_resident<D, 2, true>(tq, tk, tv, to, rp, c.res_ctas, st)
+                  : launch_resident<D, 1, true>(tq, tk, tv, to, rp, c.res_ctas, st);
+    if (rc != AVSA_OK) return rc;
+    if (launch_pdl(resident_finalize_kernel, static_cast<unsigned>(B * ((Nk + 31) / 32)), 256, 0, st, rp.partial, c.res_L, c.NQT, B,
+                   H, Nk, beta, gamma, scores, rp.cta_status, c.res_ctas, status) != cudaSuccess)
+      return AVSA_ERR_CUDA;
+  } else {
+    if (launch_pdl(clear_status_kernel, 1, 1, 0, st, status) != cudaSuccess) return AVSA_ERR_CUDA;
+    rc = Nk > 128 ? launch_resident<D, 2, false>(tq, tk, tv, to, rp, c.res_ctas, st)
+                  : launch_resident<D, 1, false>(tq, tk, tv, to, rp, c.res_ctas, st);
+    if (rc != AVSA_OK) return rc;
+  }
+  return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
 template <int BLK, int D>
@@ -786,6 +864,12 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
   uint8_t* base = static_cast<uint8_t*>(ws);
+  if (c.resident && d == 128)
+    return run_cross_resident<128>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c,
+                                   as_stream(stream));
+  if (c.resident)
+    return run_cross_resident<64>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c,
+                                  as_stream(stream));
   if (d == 128)
     return run_cross<128, 128>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c,
                                as_stream(stream));

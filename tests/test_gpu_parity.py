@@ -536,6 +536,58 @@ def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
     assert torch.equal(lse, lse2)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,Nq,Nk", [
+    (1, 1, 1, 32), (1, 2, 127, 33), (2, 3, 1000, 64), (1, 40, 600, 65), (1, 40, 515, 100), (1, 24, 2427, 128),
+    (1, 3, 129, 129), (1, 40, 600, 160), (2, 20, 515, 161), (1, 24, 2427, 200), (1, 2, 128, 255), (1, 40, 600, 256),
+])
+def test_cross_attention_few_keys(B, H, Nq, Nk, d):
+    """K and V of a head on chip, both passes in one kernel: one and two key groups, chunks of 32 keys and their remainders, one
+    and several query tiles and heads per CTA; the same bits without scores and on a second run."""
+    g = torch.Generator().manual_seed(Nq * 7 + Nk)
+    q, k, v = (torch.randn((B, H, n, d), generator=g).to(torch.bfloat16) for n in (Nq, Nk, Nk))
+    hs = sorted({0, H // 2, H - 1})
+    gamma = 1.0 / (H * Nq)
+    qc, kc, vc = (t.transpose(1, 2).contiguous().transpose(1, 2).cuda() for t in (q, k, v))
+    o, lse, s, ws = av.avsa_cross_attn_scores(qc, kc, vc, score_gamma=gamma)
+    _status_ok(ws)
+    assert av.avsa_redo_count(ws) == 0
+    want_s = np.zeros((B, Nk))
+    for h in range(H):
+        want_o, want_lse, A = orc.cross_attention(_np64(q[:, h : h + 1]), _np64(k[:, h : h + 1]), _np64(v[:, h : h + 1]))
+        want_s = orc.column_scores(A, s_prev=want_s, beta=1.0, gamma=gamma)
+        if h in hs:
+            _close(_np64(o[:, h : h + 1]), want_o, "few keys O")
+            _close_lse(_np64(lse[:, h : h + 1]), want_lse, "few keys lse")
+    _close_scores(_np64(s), want_s, "few keys scores")
+    o2, lse2, _, ws2 = av.avsa_cross_attn_scores(qc, kc, vc, want_scores=False)
+    _status_ok(ws2)
+    assert torch.equal(o, o2) and torch.equal(lse, lse2)
+    s3 = av.avsa_cross_attn_scores(qc, kc, vc, want_o=False, score_gamma=gamma)[2]
+    assert torch.equal(s, s3)
+
+
+@pytest.mark.parametrize("step", [30.0, 80.0])
+def test_cross_attention_few_keys_that_outgrow_their_reference(step):
+    """The keys from 128 on have logits larger by 30 nats (43 in base 2: still relative to the first ones' maximum) or 80 (115: the
+    rows take another reference, and their tiles are counted)."""
+    B, H, Nq, Nk, d = 1, 3, 300, 200, 128
+    g = torch.Generator().manual_seed(9)
+    q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, Nk, Nk))
+    u = 1.0 / np.sqrt(d)
+    q = (q + 8.0 * u).to(torch.bfloat16)
+    q[:, :, ::2] = (q[:, :, ::2].float() - 8.0 * u).to(torch.bfloat16)      # every other row keeps its reference
+    k[:, :, 128:] += step * u * np.sqrt(d) / 8.0
+    k, v = k.to(torch.bfloat16), v.to(torch.bfloat16)
+    o, lse, s, ws = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), score_gamma=1.0 / (H * Nq))
+    _status_ok(ws)
+    assert av.avsa_redo_count(ws) == (9 if step > 64 else 0)      # three tiles a head
+    want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+    _close(_np64(o), want_o, "outgrown O")
+    _close_lse(_np64(lse), want_lse, "outgrown lse")
+    _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "outgrown scores")
+
+
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_reverse_direction(name):
     """Video queries attending to audio keys (the other half of the bidirectional pair): outputs, LSE, and the
