@@ -63,6 +63,20 @@ class _Bf16Tensor4(ctypes.Structure):
 
 _lib = None
 _host_module = None
+_alloc_module = None
+
+
+def _extension(name: str):
+    """An extension module that build.py put beside this file."""
+    path = next((p for p in (os.path.join(_HERE, name + e) for e in importlib.machinery.EXTENSION_SUFFIXES)
+                 if os.path.exists(p)), None)
+    if path is None:
+        raise RuntimeError(f"{name} is missing in {_HERE}: run `python -m paper_2608_15522_b200.build` "
+                           "(there is no fallback path)")
+    spec = importlib.util.spec_from_file_location(name, path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
 
 
 def _host():
@@ -70,14 +84,7 @@ def _host():
     global _host_module
     if _host_module is None:
         lib = load_library()
-        path = next((p for p in (os.path.join(_HERE, "_avsa_host" + e) for e in importlib.machinery.EXTENSION_SUFFIXES)
-                     if os.path.exists(p)), None)
-        if path is None:
-            raise RuntimeError(f"_avsa_host is missing in {_HERE}: run `python -m paper_2608_15522_b200.build` "
-                               "(there is no fallback path)")
-        spec = importlib.util.spec_from_file_location("_avsa_host", path)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
+        module = _extension("_avsa_host")
         address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
         module.bind(address(lib.avsa_cross_attn_scores), address(lib.avsa_build_block_mask),
                     address(lib.avsa_sparse_self_attn), address(lib.avsa_protected_rows_attn),
@@ -164,8 +171,32 @@ def _stream(device) -> ctypes.c_void_p:
     return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
 
 
-def _workspace(nbytes: int, device) -> torch.Tensor:
-    return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
+_KINDS = (torch.float32, torch.int32, torch.uint8)      # of the allocating extension
+
+
+def _empty(like, kind: int, *sizes) -> torch.Tensor:
+    """An uninitialised tensor of _KINDS[kind] on the device of ``like`` (csrc/host_alloc.cc; torch.empty for whatever is not
+    a plain tensor)."""
+    if type(like) is not torch.Tensor:
+        return torch.empty(sizes, dtype=_KINDS[kind], device=like.device)
+    global _alloc_module
+    if _alloc_module is None:
+        _alloc_module = _extension("_avsa_alloc")
+    return _alloc_module.empty(like, kind, *sizes)
+
+
+def _empty_as(like) -> torch.Tensor:
+    """An uninitialised bf16 tensor with the shape and strides of ``like``."""
+    if type(like) is not torch.Tensor:
+        return torch.empty_strided(like.shape, like.stride(), dtype=torch.bfloat16, device=like.device)
+    global _alloc_module
+    if _alloc_module is None:
+        _alloc_module = _extension("_avsa_alloc")
+    return _alloc_module.empty_as(like)
+
+
+def _workspace(nbytes: int, like) -> torch.Tensor:
+    return _empty(like, 2, max(int(nbytes), 256))
 
 
 def _check(status: int, where: str) -> None:
@@ -200,15 +231,15 @@ def avsa_cross_attn_scores(q, k, v, scores=None, score_beta=0.0, score_gamma=1.0
                            want_o=True, want_scores=True, o=None, lse=None, ws=None):
     """Eq. 1-2.  q [B,H,Nq,d], k/v [B,H,Nk,d] bf16 CUDA.  Returns (o, lse, scores, ws)."""
     if want_o and o is None:
-        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
+        o = _empty_as(q)
     if lse is None:
-        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
+        lse = _empty(q, 0, *q.shape[:3])
     if want_scores and scores is None:
-        scores = torch.empty((q.shape[0], k.shape[2]), dtype=torch.float32, device=q.device)
+        scores = _empty(q, 0, q.shape[0], k.shape[2])
         score_beta = 0.0
     if ws is None:
         B, H, Nq, d = q.shape
-        ws = _workspace(avsa_cross_attn_scores_workspace_bytes(B, H, Nq, k.shape[2], d), q.device)
+        ws = _workspace(avsa_cross_attn_scores_workspace_bytes(B, H, Nq, k.shape[2], d), q)
     st = (_host_module or _host()).cross(q, k, v, o if want_o else None, lse, scores if want_scores else None, score_beta,
                                          score_gamma, softmax_scale, ws)
     if st != AVSA_OK:
@@ -229,10 +260,12 @@ def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTE
     """
     if q is not None:
         B, H, N, d = shape = q.shape
-        dev = q.device
+        like = q
     else:
         B, H, N, d = shape
-        dev = block_scores.device
+        like = block_scores
+        if like is None:
+            raise AttributeError("without q and k the block scores are an argument")
     out = out or {}
     if block_scores is None:
         block_scores = out.get("block_scores")
@@ -242,17 +275,17 @@ def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTE
     prot_blk = out.get("prot_blk")
     NB = (N + blk - 1) // blk
     if block_scores is None:
-        block_scores = torch.empty((B, H, NB, NB), dtype=torch.float32, device=dev)
+        block_scores = _empty(like, 0, B, H, NB, NB)
     if col_idx is None:
-        col_idx = torch.empty((B, H, NB, NB), dtype=torch.int32, device=dev)
+        col_idx = _empty(like, 1, B, H, NB, NB)
     if col_cnt is None:
-        col_cnt = torch.empty((B, H, NB), dtype=torch.int32, device=dev)
+        col_cnt = _empty(like, 1, B, H, NB)
     if prot_tok is None:
-        prot_tok = torch.empty((B, N), dtype=torch.uint8, device=dev)
+        prot_tok = _empty(like, 2, B, N)
     if prot_blk is None:
-        prot_blk = torch.empty((B, NB), dtype=torch.uint8, device=dev)
+        prot_blk = _empty(like, 2, B, NB)
     if ws is None:
-        ws = _workspace(avsa_build_block_mask_workspace_bytes(B, H, N, d, blk), dev)
+        ws = _workspace(avsa_build_block_mask_workspace_bytes(B, H, N, d, blk), like)
     st = (_host_module or _host()).mask(tuple(shape), blk, q, k, scores, n_protect, k_keep, flags, softmax_scale, block_scores,
                                         col_idx, col_cnt, prot_tok, prot_blk, ws)
     if st != AVSA_OK:
@@ -289,12 +322,12 @@ def avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk) -> int:
 def avsa_sparse_self_attn(q, k, v, col_idx, col_cnt, blk, softmax_scale=0.0, want_lse=False, o=None, lse=None, ws=None):
     """Eq. 10.  Returns (o, lse or None, ws)."""
     if o is None:
-        o = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
+        o = _empty_as(q)
     if want_lse and lse is None:
-        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
+        lse = _empty(q, 0, *q.shape[:3])
     if ws is None:
         B, H, N, d = q.shape
-        ws = _workspace(avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk), q.device)
+        ws = _workspace(avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk), q)
     st = (_host_module or _host()).sparse(q, k, v, col_idx, col_cnt, blk, o, lse, softmax_scale, ws)
     if st != AVSA_OK:
         raise AvsaError(st, "avsa_sparse_self_attn")
@@ -326,7 +359,7 @@ def avsa_protected_rows_attn(q, k, v, prot_tok, n_protect, blk, o, lse=None, sof
     attention rows.  Returns ws."""
     if ws is None:
         B, H, N, d = q.shape
-        ws = _workspace(avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, int(n_protect)), q.device)
+        ws = _workspace(avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, int(n_protect)), q)
     st = (_host_module or _host()).protected_rows(q, k, v, prot_tok, n_protect, blk, o, lse, softmax_scale, ws)
     if st != AVSA_OK:
         raise AvsaError(st, "avsa_protected_rows_attn")
@@ -342,10 +375,10 @@ def avsa_cache_indicators(y_v, yhat_v, y_a, yhat_a, prot_tok=None, s_cur=None, s
     """Eq. 12-15.  y_v/yhat_v bf16 [B,Nv,C], y_a/yhat_a bf16 [B,Na,C] (contiguous).  Returns (out [B,8], ws) with
     out[:, :6] = dv, da, dp, ds, dsync, reuse."""
     if out is None:
-        out = torch.empty((y_v.shape[0], 8), dtype=torch.float32, device=y_v.device)
+        out = _empty(y_v, 0, y_v.shape[0], 8)
     if ws is None:
         B, Nv, C = y_v.shape
-        ws = _workspace(avsa_cache_indicators_workspace_bytes(B, Nv, y_a.shape[1], C), y_v.device)
+        ws = _workspace(avsa_cache_indicators_workspace_bytes(B, Nv, y_a.shape[1], C), y_v)
     st = (_host_module or _host()).indicators(y_v, yhat_v, y_a, yhat_a, prot_tok, s_cur, s_anchor, lambda_p, lambda_s, tau, eps,
                                               out, ws)
     if st != AVSA_OK:

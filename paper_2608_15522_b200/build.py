@@ -1,4 +1,4 @@
-"""Builds libavsa.so and the host extension that calls it in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libavsa.so and the two host extensions of its binding in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
 from __future__ import annotations
 
 import os
@@ -11,6 +11,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libavsa.so")
 HOST = os.path.join(HERE, "_avsa_host" + sysconfig.get_config_var("EXT_SUFFIX"))      # marshalling for this interpreter
+ALLOC = os.path.join(HERE, "_avsa_alloc" + sysconfig.get_config_var("EXT_SUFFIX"))    # tensors for the wrappers
 SOURCES = ["api.cu", "mask.cu", "sparse_attn.cu", "cross_attn.cu", "protected_rows.cu", "cache_indicators.cu"]
 HEADERS = sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")) + [os.path.join("..", "..", "include", "avsa.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -25,29 +26,37 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(HOST):
+    outputs = (LIB, HOST, ALLOC)
+    if not all(os.path.exists(o) for o in outputs):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST))
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["host_call.cc"]]
+    t = min(os.path.getmtime(o) for o in outputs)
+    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["host_call.cc", "host_alloc.cc"]]
     return any(os.path.getmtime(p) > t for p in deps)
 
 
-def _build_host() -> None:
-    src = os.path.join(CSRC, "host_call.cc")
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wall", "-Wno-cast-function-type",
-           "-I" + sysconfig.get_paths()["include"], src, "-o", HOST]
-    r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"g++ failed on host_call.cc:\n{r.stdout}")
+def _start_host_builds():
+    """g++ on the two host extensions: (source, process) each."""
+    import torch
+    base = torch.__path__[0]
+    include = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include")]
+    common = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I" + sysconfig.get_paths()["include"]]
+    host = common + ["-Wall", "-Wno-cast-function-type", os.path.join(CSRC, "host_call.cc"), "-o", HOST]
+    alloc = common + [f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+    alloc += [flag for path in include for flag in ("-isystem", path)]
+    alloc += [os.path.join(CSRC, "host_alloc.cc"), "-o", ALLOC, "-L" + os.path.join(base, "lib"),
+              "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10"]
+    return [(name, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))
+            for name, cmd in (("host_call.cc", host), ("host_alloc.cc", alloc))]
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compiles every .cu of the library, links libavsa.so and builds the host extension; returns the library's path."""
+    """Compiles every .cu of the library, links libavsa.so and builds the host extensions; returns the library's path."""
     if not force and not _stale():
         return LIB
     nvcc = _nvcc()
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
+    host_procs = _start_host_builds()
     procs = []
     for s in SOURCES:
         obj = os.path.join(objdir, s.replace(".cu", ".o"))
@@ -65,7 +74,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}")
-    _build_host()
+    for name, pr in host_procs:
+        out, _ = pr.communicate()
+        if pr.returncode != 0:
+            raise RuntimeError(f"g++ failed on {name}:\n{out}")
     return LIB
 
 
