@@ -47,6 +47,10 @@ enum FastWhere { kFastSFree = 61, kFastPFree, kFastMref };
 // (3,3,1), (3,2,2), (2,3,2), (4,2,1) and (2,4,1) of the seven 32 KB tile slots are within noise of each other; the
 // seventh slot is the staging buffer of the output tile.
 constexpr int kPKS = 3, kPVS = 2, kPQB = 1, kPRing = 4;
+// Range-mode calls that never stage an output tile (store other than kStoreTile, or a stream in which no CTA has a whole row) use that
+// buffer as a third V stage: their keys come from DRAM, and two tiles' time does not cover that latency (24 heads, 157 queries x 17856
+// keys: 57 -> 53 us; 256 x 32760, with scores, the call 171.5 -> 166.3; 512 x 49152 and the dense rows, from L2, as before).
+constexpr int kPVSMax = 3;
 
 template <int BLK, int D>
 struct PersistSmem {
@@ -55,9 +59,9 @@ struct PersistSmem {
   static constexpr int kQ = 0;
   static constexpr int kK = kPQB * kQBytes;
   static constexpr int kV = kK + kPKS * kTileBytes;
-  static constexpr int kStage = kV + kPVS * kTileBytes;         // output tile, 128-byte swizzled, for the TMA store
+  static constexpr int kStage = kV + kPVS * kTileBytes;         // output tile, 128-byte swizzled, for the TMA store; or V stage 2
   static constexpr int kBars = kStage + kQBytes;
-  static constexpr int kNumBars = 2 * kPQB + 2 * kPKS + 2 * kPVS + 18 + 2 * kPRing;
+  static constexpr int kNumBars = 2 * kPQB + 2 * kPKS + 2 * kPVSMax + 18 + 2 * kPRing;
   static constexpr int kStats = kBars + kNumBars * 8;          // float mref[128], lsum[2][128]
   static constexpr int kItems = kStats + 3 * 128 * 4;          // AttnItem[kPRing], two redo flags
   static constexpr int kMisc = kItems + 32 * kPRing + 16;      // tmem base, stop flag
@@ -117,7 +121,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   const uint32_t bar0 = smem_u32(smem + L::kBars);
   auto BAR = [&](int i) { return bar0 + static_cast<uint32_t>(i) * 8u; };
   constexpr int Q_FULL = 0, Q_EMPTY = kPQB, K_FULL = 2 * kPQB, K_EMPTY = K_FULL + kPKS, V_FULL = K_EMPTY + kPKS,
-                V_EMPTY = V_FULL + kPVS, S_FULL = V_EMPTY + kPVS /* + group */, S_FREE = S_FULL + 2,
+                V_EMPTY = V_FULL + kPVSMax, S_FULL = V_EMPTY + kPVSMax /* + group */, S_FREE = S_FULL + 2,
                 P_FULL = S_FREE + 2 /* + 2*group + half */, P_FREE = P_FULL + 4, O_FULL = P_FREE + 2,
                 O_FREE = O_FULL + 1, MREF = O_FREE + 1, ITEM_FULL = MREF + 1 /* + slot */, ITEM_EMPTY = ITEM_FULL + kPRing,
                 QK_DRAIN = ITEM_EMPTY + kPRing, PV_DRAIN = QK_DRAIN + 1, LSUM_A = PV_DRAIN + 1, LSUM_B = LSUM_A + 1,
@@ -149,7 +153,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       mbar_init(BAR(K_FULL + s), 1);
       mbar_init(BAR(K_EMPTY + s), 1);
     }
-    for (int s = 0; s < kPVS; s++) {
+    for (int s = 0; s < kPVSMax; s++) {
       mbar_init(BAR(V_FULL + s), 1);
       mbar_init(BAR(V_EMPTY + s), 1);
     }
@@ -191,6 +195,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   const uint32_t tmem = misc[0];
   pdl_wait();
   pdl_launch();
+
+  const int n_vs = !kListIn && (p.store != kStoreTile || (p.rs.L > 0 && p.rs.L < p.rs.NKB)) ? kPVSMax : kPVS;      // V stages
 
   // A wait that gives up when the CTA has been stopped (a time limit was reached somewhere).
   auto wait_or_stop = [&](int bar, uint32_t parity, int where, int tag) -> bool {
@@ -344,6 +350,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       return true;
     };
     int vc = 0;              // V tiles loaded so far, over all items
+    int sv = 0, fv = 0;      // stage of the next one, and how often the ring has been round
     bool ok = publish(0);
     AttnItem cur = pub, next;                     // item n, whose V tiles are loaded next, and item n + 1
     next.item = -1;
@@ -360,10 +367,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         const int nn = min(32, a_cnt - t0);
         for (int j = 0; j < nn; j++) {
           const int kb = __shfl_sync(FULLM, mine, j);
-          const int s = vc % kPVS;
+          const int s = sv;
           int good = 1;
           if (lane == 0) {
-            if (vc >= kPVS) good = wait_or_stop(V_EMPTY + s, ((vc / kPVS) - 1) & 1, kWhereVEmpty, t0 + j) ? 1 : 0;
+            if (fv > 0) good = wait_or_stop(V_EMPTY + s, (fv - 1) & 1, kWhereVEmpty, t0 + j) ? 1 : 0;
             if (good) {
               mbar_expect_tx(BAR(V_FULL + s), L::kTileBytes);
               for (int pn = 0; pn < NPANEL; pn++)
@@ -377,6 +384,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
             break;
           }
           vc++;
+          if (++sv == n_vs) {
+            sv = 0;
+            fv++;
+          }
         }
       }
       if (!ok) break;
@@ -388,7 +399,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       }
     }
     if (lane == 0 && misc[1] != 0u)
-      for (int c = max(0, vc - kPVS); c < vc; c++) mbar_wait(BAR(V_FULL + c % kPVS), (c / kPVS) & 1);
+      for (int c = max(0, vc - n_vs); c < vc; c++) mbar_wait(BAR(V_FULL + c % n_vs), (c / n_vs) & 1);
   } else if (warp == 1) {
     // ------------------------------------------------------------------ Q K^T issuer
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
@@ -458,7 +469,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         umma_ts(tmem_u + TM_O, tm_buf + ks * 8, desc64(v_lo + ks * (2048 >> 4)), idesc_pv, kk > 0 ? 1u : acc_first);
       }
     };
-    int vc = 0;                 // V tiles consumed so far
+    int sv = 0, fv = 0;         // stage of the next V tile, and how often the ring has been round
     int used[2] = {0, 0};       // P tiles read so far from each group's buffer
     bool ok = true;
     for (int n = 0; ok; n++) {
@@ -466,8 +477,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
       if (!get_item(n, it)) break;
       const int cnt = it.cnt;
       for (int t = 0; t < cnt && ok; t++) {
-        const int j = t & 1, sv = vc % kPVS;
-        ok = wait_all(V_FULL + sv, (vc / kPVS) & 1, kWhereVFull, t);
+        const int j = t & 1;
+        ok = wait_all(V_FULL + sv, fv & 1, kWhereVFull, t);
         if (!ok) break;
         ok = wait_all(P_FULL + 2 * j, used[j] & 1, kWherePFull, t);
         if (!ok) break;
@@ -491,7 +502,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         }
         __syncwarp();
         used[j]++;
-        vc++;
+        if (++sv == n_vs) {
+          sv = 0;
+          fv++;
+        }
       }
       if (ok) item_done(n);
     }
