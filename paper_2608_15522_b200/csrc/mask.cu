@@ -25,21 +25,16 @@ __device__ __forceinline__ uint32_t rank_key(float x) {
 constexpr unsigned kPoolTailCtas = 296;   // CTAs at the end of the pooling grid that wait for the token select
 
 template <int D>
-__global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh,
-                                                   int64_t q_sn, const __nv_bfloat16* __restrict__ k, int64_t k_sb,
-                                                   int64_t k_sh, int64_t k_sn, float* __restrict__ qbar,
-                                                   float* __restrict__ kbar, int H, int N, int blk) {
+__device__ __forceinline__ void pool_block(int nb, int NB, int bh, int which, const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh,
+                                           int64_t q_sn, const __nv_bfloat16* __restrict__ k, int64_t k_sb, int64_t k_sh,
+                                           int64_t k_sn, float* __restrict__ qbar, float* __restrict__ kbar, int H, int N, int blk) {
   constexpr int TPR = D / 8;          // threads per row
   constexpr int RPP = 256 / TPR;      // rows per pass
   __shared__ float part[RPP][D + 4];
-  // lets the block-score grid be staged while this one drains (it waits for this grid before it reads)
-  pdl_launch();
-
-  const int nb = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
   const int b = bh / H, h = bh % H;
   const __nv_bfloat16* src = which == 0 ? q + b * q_sb + h * q_sh : k + b * k_sb + h * k_sh;
   const int64_t sn = which == 0 ? q_sn : k_sn;
-  float* dst = (which == 0 ? qbar : kbar) + (static_cast<int64_t>(bh) * gridDim.x + nb) * D;
+  float* dst = (which == 0 ? qbar : kbar) + (static_cast<int64_t>(bh) * NB + nb) * D;
   const int c = threadIdx.x % TPR, g = threadIdx.x / TPR;
   const int row0 = nb * blk;
   const int valid = min(blk, N - row0);
@@ -74,6 +69,16 @@ __global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restri
     for (int j = 0; j < RPP; j++) s += part[j][threadIdx.x];
     dst[threadIdx.x] = s / static_cast<float>(valid);
   }
+}
+
+template <int D>
+__global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh,
+                                                   int64_t q_sn, const __nv_bfloat16* __restrict__ k, int64_t k_sb,
+                                                   int64_t k_sh, int64_t k_sn, float* __restrict__ qbar,
+                                                   float* __restrict__ kbar, int H, int N, int blk) {
+  // lets the block-score grid be staged while this one drains (it waits for this grid before it reads)
+  pdl_launch();
+  pool_block<D>(blockIdx.x, gridDim.x, blockIdx.y, blockIdx.z, q, q_sb, q_sh, q_sn, k, k_sb, k_sh, k_sn, qbar, kbar, H, N, blk);
   // This grid starts while the token select (its predecessor on the stream) is still running.  The last
   // CTAs wait for it before they retire, so that "pooling finished" implies "token select finished" for the
   // kernels behind (which wait for their predecessor only); by then the select is long done, and no
@@ -170,37 +175,32 @@ __device__ __forceinline__ void warp_pick_digit(const int* bins, int want, int l
 // ------------------------------------------------------------------------------------------------
 constexpr int kSelectSmemKeys = 56 * 1024;   // 224 KB of keys at most
 
-template <bool STAGED>
-__global__ void __launch_bounds__(1024) token_select_kernel(const float* __restrict__ scores, int N, int n_protect,
-                                                            int blk, int NB, int min_tokens,
-                                                            uint8_t* __restrict__ prot_tok,
-                                                            uint8_t* __restrict__ prot_blk, StatusRecord* status) {
-  extern __shared__ uint32_t skeys[];
+template <bool STAGED, int THREADS>
+__device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const float* __restrict__ scores, int N, int n_protect, int blk,
+                                              int NB, int min_tokens, uint8_t* __restrict__ prot_tok,
+                                              uint8_t* __restrict__ prot_blk, StatusRecord* status) {
+  constexpr int WARPS = THREADS / 32;
   __shared__ int bins[256];
   __shared__ int s_digit, s_above, s_in_bin;
-  __shared__ int warp_cnt[32];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int warp_cnt[WARPS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* s = scores + static_cast<int64_t>(b) * N;
   uint8_t* ptok = prot_tok + static_cast<int64_t>(b) * N;
   uint8_t* pblk = prot_blk + static_cast<int64_t>(b) * NB;
-  // nothing launched next on the stream depends on this kernel until the list emission, so let the
-  // pooling kernel start right away (but not before this grid's own predecessors are done: pooling does not wait)
-  pdl_wait();
-  pdl_launch();
   if (b == 0 && tid == 0) {
     status->code = 0;
     status->where = 0;
     status->item = 0;
     status->aux = 0;
   }
-  for (int i = tid; i < NB; i += 1024) pblk[i] = 0;
+  for (int i = tid; i < NB; i += THREADS) pblk[i] = 0;
   if (n_protect <= 0) {
-    for (int i = tid; i < N; i += 1024) ptok[i] = 0;
+    for (int i = tid; i < N; i += THREADS) ptok[i] = 0;
     return;
   }
   if (STAGED) {
 #pragma unroll 8
-    for (int i = tid; i < N; i += 1024) skeys[i] = rank_key(__ldg(s + i));
+    for (int i = tid; i < N; i += THREADS) skeys[i] = rank_key(__ldg(s + i));
   }
   auto key_at = [&](int i) -> uint32_t { return STAGED ? skeys[i] : rank_key(__ldg(s + i)); };
   uint32_t prefix = 0, mask = 0;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
     const int shift = 24 - 8 * pass;
     if (tid < 256) bins[tid] = 0;
     __syncthreads();     // also orders the staging stores before the first reads
-    for (int i0 = 0; i0 < N; i0 += 1024) {
+    for (int i0 = 0; i0 < N; i0 += THREADS) {
       const int i = i0 + tid;
       const bool valid = i < N;
       const uint32_t key = valid ? key_at(i) : 0u;
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
   const uint32_t T = prefix;     // the n_protect-th largest key; `want` ties at T are taken, lowest index first
   // contiguous segment per warp, a whole number of blocks (blk is a multiple of 32), so that every block's
   // count of protected tokens is known to one warp
-  const int seg = ((N + 31) / 32 + blk - 1) / blk * blk;
+  const int seg = ((N + WARPS - 1) / WARPS + blk - 1) / blk * blk;
   const int lo = min(N, warp * seg), hi = min(N, lo + seg);
   int eq_mine = 0;
   for (int i0 = lo; i0 < hi; i0 += 32) {
@@ -264,6 +264,42 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
       if (in_block >= min_tokens && lane == 0) pblk[i0 / blk] = 1;
       in_block = 0;
     }
+  }
+}
+
+template <bool STAGED>
+__global__ void __launch_bounds__(1024) token_select_kernel(const float* __restrict__ scores, int N, int n_protect,
+                                                            int blk, int NB, int min_tokens,
+                                                            uint8_t* __restrict__ prot_tok,
+                                                            uint8_t* __restrict__ prot_blk, StatusRecord* status) {
+  extern __shared__ uint32_t skeys[];
+  // nothing launched next on the stream depends on this kernel until the list emission, so let the
+  // pooling kernel start right away (but not before this grid's own predecessors are done: pooling does not wait)
+  pdl_wait();
+  pdl_launch();
+  select_tokens<STAGED, 1024>(blockIdx.x, skeys, scores, N, n_protect, blk, NB, min_tokens, prot_tok, prot_blk, status);
+}
+
+// Select and pooling of a short sequence in one launch: the first B CTAs select, the others pool a block each.  A launch costs the host
+// 2.1 us, and with few tokens 256 threads select them in the time of 1024 (157 tokens: the mask and attention calls 19.9 -> 18.6
+// us; with 2070 the select takes 8.2 instead of 5.5).
+constexpr int kSelectPoolTokens = 512;
+template <int D>
+__global__ void __launch_bounds__(256) select_pool_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh,
+                                                          int64_t q_sn, const __nv_bfloat16* __restrict__ k, int64_t k_sb,
+                                                          int64_t k_sh, int64_t k_sn, float* __restrict__ qbar,
+                                                          float* __restrict__ kbar, int B, int H, int N, int blk, int NB,
+                                                          const float* __restrict__ scores, int n_protect, int min_tokens,
+                                                          uint8_t* __restrict__ prot_tok, uint8_t* __restrict__ prot_blk,
+                                                          StatusRecord* status) {
+  extern __shared__ uint32_t skeys[];
+  pdl_wait();
+  pdl_launch();
+  if (static_cast<int>(blockIdx.x) < B) {
+    select_tokens<true, 256>(blockIdx.x, skeys, scores, N, n_protect, blk, NB, min_tokens, prot_tok, prot_blk, status);
+  } else {
+    const int i = blockIdx.x - B, pair = i / NB;
+    pool_block<D>(i % NB, NB, pair >> 1, pair & 1, q, q_sb, q_sh, q_sn, k, k_sb, k_sh, k_sn, qbar, kbar, H, N, blk);
   }
 }
 
@@ -642,6 +678,7 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   uint8_t* pblk = prot_blk != nullptr ? prot_blk : base + w.pblk;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
 
+  const bool one_launch = !by_block_sum && !given && N <= kSelectPoolTokens && static_cast<int64_t>(B) * H <= 65535;
   if (by_block_sum) {
     // block sums, then the token select run over the NB sums: its "token" flags are the block flags (its own
     // block lift goes to a scratch array); the token flags are filled in at the end of the call
@@ -654,6 +691,8 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
     if (launch_pdl(token_select_kernel<true>, B, 1024, key_bytes, st, bsum, NB, n_protect, 32, (NB + 31) / 32, 1, pblk,
                    base + w.junk, static_cast<StatusRecord*>(ws)) != cudaSuccess)
       return AVSA_ERR_CUDA;
+  } else if (one_launch) {
+    // (with the pooling, below)
   } else if (N <= kSelectSmemKeys) {
     const size_t key_bytes = static_cast<size_t>(N) * sizeof(uint32_t);
     if (!allow_select_smem()) return AVSA_ERR_CUDA;
@@ -671,15 +710,20 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   if (!given) {
     const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(q.ptr);
     const __nv_bfloat16* kp = static_cast<const __nv_bfloat16*>(k.ptr);
-    // the pooling kernel does not read anything the token select writes: allow it to start early
-    const dim3 pool_grid(NB, B * H, 2);
     cudaError_t e;
-    if (d == 128)
-      e = launch_pdl(pool_kernel<128>, pool_grid, 256, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b,
-                     k.stride_h, k.stride_n, qbar, kbar, H, N, blk);
-    else
-      e = launch_pdl(pool_kernel<64>, pool_grid, 256, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b,
-                     k.stride_h, k.stride_n, qbar, kbar, H, N, blk);
+    if (one_launch) {
+      const unsigned grid = static_cast<unsigned>(B) * (1 + 2 * H * NB);
+      const size_t key_bytes = static_cast<size_t>(N) * sizeof(uint32_t);
+      auto kernel = d == 128 ? select_pool_kernel<128> : select_pool_kernel<64>;
+      e = launch_pdl(kernel, grid, 256, key_bytes, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b, k.stride_h,
+                     k.stride_n, qbar, kbar, B, H, N, blk, NB, scores, n_protect, min_tokens, ptok, pblk, static_cast<StatusRecord*>(ws));
+    } else {
+      // the pooling kernel does not read anything the token select writes: allow it to start early
+      const dim3 pool_grid(NB, B * H, 2);
+      auto kernel = d == 128 ? pool_kernel<128> : pool_kernel<64>;
+      e = launch_pdl(kernel, pool_grid, 256, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b, k.stride_h, k.stride_n,
+                     qbar, kbar, H, N, blk);
+    }
     if (e != cudaSuccess) return AVSA_ERR_CUDA;
     // block scores and lists of 16 query blocks per CTA, staged behind the pooling grid
     if (d == 128)

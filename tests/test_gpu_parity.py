@@ -1072,6 +1072,25 @@ def test_protected_rows_that_outgrow_their_reference(H, N, n_protect, short, d):
     assert bool((o[:, :, off] == 7.0).all()) and bool((lse[:, :, off] == 7.0).all())
 
 
+@pytest.mark.parametrize("n", [1, 63, 256, 257, 511, 512, 513])
+def test_mask_with_the_select_in_the_pooling_grid(n):
+    """Up to 512 tokens one launch selects and pools: token flags and block flags are the oracle's, ties at the threshold included, and
+    the lists those of the block scores that the call itself returns."""
+    B, H, d, n_protect = 3, 2, 64, max(1, n // 9)
+    NB = (n + d - 1) // d
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k = (torch.randn((B, H, n, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    s = torch.round(torch.randn((B, n), generator=g, device="cuda") * 4) / 4
+    k_keep = max(1, NB // 2)
+    m = av.avsa_build_block_mask(q, k, s, n_protect, k_keep, d)
+    _status_ok(m["ws"])
+    idx, cnt, tok, blk = orc.build_block_mask(m["block_scores"].cpu().numpy(), s.cpu().numpy(), n_protect, k_keep, d, n)
+    assert np.array_equal(m["prot_tok"].cpu().numpy(), tok) and np.array_equal(m["prot_blk"].cpu().numpy(), blk)
+    assert np.array_equal(m["col_cnt"].cpu().numpy(), cnt) and np.array_equal(m["col_idx"].cpu().numpy(), idx)
+    want = orc.block_scores(_np64(q), _np64(k), d)
+    assert np.abs(m["block_scores"].cpu().numpy() - want).max() <= 1e-4 * np.abs(want).max()
+
+
 @pytest.mark.parametrize("NB", [1, 32, 33, 256, 257, 512, 513, 1024, 1025])
 def test_mask_select_over_row_lengths(NB):
     """The select's key slots per lane at their limits: distinct scores, heavy ties, one bit of difference, a sign change,
