@@ -96,7 +96,7 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&r)[8]) 
 }
 
 // MODE_LIST: work item = query tile with an explicit list of key tiles, output bf16 rows + optional LSE
-// (block-sparse self-attention; `order` maps queue position to item).  MODE_RANGE: the work is cut as RangeSplit
+// (block-sparse self-attention; `order`, where there is one, maps queue position to item).  MODE_RANGE: the work is cut as RangeSplit
 // describes; the CTA's items are its segments of the stream, fixed by its index, or come off the queue like the lists
 // (which of the two: make_range_split); output bf16 rows where the key axis is not split, else
 // normalised fp32 partials for merge_splits_rows, and the log2 LSE of the range.
@@ -317,28 +317,39 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
         }
         first = false;
         if (id >= n_items) break;
-        if (kListIn) id = order[id];                  // queue position -> query tile (long lists first)
-        pub = decode_item<BLK, MODE>(p, id);
+        if (kListIn && order != nullptr) id = order[id];      // queue position -> query tile (long lists first)
         if (!kListIn) {
+          pub = decode_item<BLK, MODE>(p, id);
           if (pub.cnt <= 0) continue;
           break;
         }
-        const int c = pub.cnt;
+        // The length and the first 32 entries come in one trip to L2, and the last entry out of the check (one after the other,
+        // as decode_item reads them, these trips stood in front of a CTA's first tile).
+        const int32_t* lst = p.col_idx + static_cast<int64_t>(id) * p.NKB;
+        int e = lane < p.NKB ? lst[lane] : 0;
+        const int c = p.col_cnt[id];
         bool bad = (c < 1 || c > p.NKB);
+        int carry = -1;
         if (!bad) {
           // nothing is loaded through a bad list: entries in range and strictly ascending
-          const int32_t* lst = p.col_idx + static_cast<int64_t>(id) * p.NKB;
-          int carry = -1;
           for (int t0 = 0; t0 < c; t0 += 32) {
             const bool have = t0 + lane < c;
-            const int e = have ? lst[t0 + lane] : 0;
+            if (t0 > 0) e = have ? lst[t0 + lane] : 0;
             int prev = __shfl_up_sync(FULLM, e, 1);
             if (lane == 0) prev = carry;
             if (have && (e < 0 || e >= p.NKB || e <= prev)) bad = true;
-            carry = __shfl_sync(FULLM, e, 31);
+            carry = __shfl_sync(FULLM, e, (min(32, c - t0)) - 1);
           }
           bad = __any_sync(FULLM, bad);
         }
+        pub.item = id;
+        pub.cnt = c;
+        pub.qt = id % p.NQT;
+        pub.h = (id / p.NQT) % p.H;
+        pub.b = (id / p.NQT) / p.H;
+        pub.kb0 = 0;
+        pub.slot = 0;
+        pub.valid = carry == p.NKB - 1 ? p.Nk - carry * BLK : BLK;
         if (!bad) break;
         if (lane == 0) report_status(p.status, AVSA_ERR_BAD_MASK, kWhereList, id, c);   // refused, not deferred
       }

@@ -470,6 +470,40 @@ def test_sparse_attention_skips_only_the_malformed_item_of_a_long_queue():
     _close(got, want, "queue with malformed items")
 
 
+@pytest.mark.parametrize("heads", [2, 6])
+@pytest.mark.parametrize("bad", [None, 35])
+def test_sparse_attention_list_lengths(heads, bad):
+    """Lists around the 32 entries that are read at once, and an entry behind them that is out of order; with an item per CTA at
+    most (2 heads x 66 query blocks, the output staged over Q) and off the queue."""
+    B, N, d = 1, 64 * 65 + 9, 64
+    NB = 66
+    g = torch.Generator().manual_seed(heads)
+    q, k, v = (torch.randn((B, heads, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    rng = np.random.default_rng(3)
+    idx = np.full((B, heads, NB, NB), -1, np.int32)
+    cnt = np.zeros((B, heads, NB), np.int32)
+    for h in range(heads):
+        for i in range(NB):
+            c = [1, 2, 3, 31, 32, 33, 63, 64, 65, 66][(h + i) % 10]
+            idx[0, h, i, :c] = np.sort(rng.choice(NB, size=c, replace=False))
+            cnt[0, h, i] = c
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), idx, cnt, d)
+    if bad is not None:
+        assert cnt[0, 1, 5] == 63
+        idx[0, 1, 5, bad] = idx[0, 1, 5, bad - 1]
+        want[0, 1, 5 * d : 6 * d] = 7.0
+    o = torch.full((B, heads, N, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    _, lse, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(),
+                                          d, want_lse=True, o=o)
+    code, detail = av.avsa_read_status(ws)
+    if bad is None:
+        assert code == av.AVSA_OK
+        _close_lse(_np64(lse), want_l, "list lengths lse")
+    else:
+        assert code == av.AVSA_ERR_BAD_MASK and detail[1] == NB + 5
+    _close(_np64(o), want, "list lengths O")
+
+
 # ------------------------------------------------------------------------------------------- cross attention
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_outputs_and_scores(name):
