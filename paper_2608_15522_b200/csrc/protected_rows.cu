@@ -178,7 +178,6 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   m.part_lse2 = part_lse;
   m.Nq = c.n_pad;
   m.H = H;
-  set_merge_rows(m, B * H);
   m.o = static_cast<__nv_bfloat16*>(o);
   m.o_sb = q.stride_b;
   m.o_sh = q.stride_h;
@@ -187,9 +186,8 @@ static int run_protected(int B, int H, int N, int n_protect, const avsa_bf16_4d&
   m.row_map = rows;
   m.row_map_stride = c.n_pad;
   m.n_out = N;
-  constexpr int MRPB = 128 / (D / 4);
-  if (!c.rs.whole_rows() &&
-      launch_pdl(merge_splits_kernel<BLK, D>, (m.total_rows + MRPB - 1) / MRPB, 128, 0, st, m) != cudaSuccess)
+  const int merge_blocks = set_merge_rows(m, B * H, D);
+  if (!c.rs.whole_rows() && launch_pdl(merge_splits_kernel<BLK, D>, merge_blocks, 256, 0, st, m) != cudaSuccess)
     return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }

@@ -552,6 +552,10 @@ def test_cross_attention_long_query_axis_two_chunks():
     (1, 2, 130, 6400, 64, True),
     (1, 100, 40, 1000, 64, True),      # score pass: 800 key tiles cut evenly through the heads
     (1, 96, 300, 520, 128, True),      # the same with the queries in two chunks
+    (1, 1, 100, 6400, 64, True),       # a row in more parts than lanes take at once (50 of 16 and, below, of 32)
+    (1, 1, 130, 6400, 128, True),
+    (1, 40, 400, 900, 64, True),
+    (1, 20, 500, 1700, 128, True),
 ])
 def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
     """The ways a stream of (query tile, key tile) pairs is cut over the CTAs: whole rows, split rows, chunks that do not divide
