@@ -14,69 +14,86 @@ namespace avsa {
 // a range of its 128-key tiles: either one of n_range equal cuts of a pair, or (n_range == 0) one of even cuts of all
 // pairs' tiles in a row, which may lead from one pair into the next: the CTA then loads queries and LSEs again with
 // its pipeline empty (about three tiles).  S^T[key, query] accumulates in tensor memory
-// (two buffers of up to 256 columns); two groups of 128 threads (one thread per key row) turn
-// alternate buffers into row sums of exp2(S^T c - lse2[query]).
-//   warp 0 TMA producer, warp 1 MMA issuer, warp 2 tensor-memory allocation,
-//   warps 4-7 / 8-11 the two reduction groups.
+// by chunks of queries; G groups of 128 threads (one thread per key row), each with its own buffer of 512 / G columns, turn them
+// into row sums of exp2(S^T c - lse2[query]).
+//   warp 0 TMA producer, warp 1 MMA issuer, warp 2 tensor-memory allocation, warps 4 and up the reduction groups.
+//   Bound by the exponentials (H Nq Nk of them, 16 a clock and SM on the MUFU).  Up to 256 queries are one chunk, and two groups
+// take the tiles by turns.  More are four chunks of up to 128, and four groups work on two tiles side by side, two chunks of a
+// tile each: sixteen warps keep the MUFU busy while some wait for a tile or for tensor memory (32 heads x 512 x 49152, the call:
+// 610 us with two groups, 584 with four; with 160 queries, where a tile's work is a third of that, 89 and 93).  A quarter of the
+// exponentials as polynomials on the FMA pipe cost what they saved and more (584 -> 607).
+//   As many key tiles are on their way as the queries leave room for (72 queries x 17856 keys: 74.9 us with three, 73.2 with
+// six; 400 queries of 64 channels x 19200 keys 218 and 212).
 // ------------------------------------------------------------------------------------------------
-constexpr int kColThreads = 384;
-constexpr int kColStages = 3;
+constexpr int kColStages = 6;              // at most
+constexpr int kRevThreads = 384;           // of colsum_rev_kernel
+__host__ __device__ constexpr int col_groups(int Nq) { return Nq > 256 ? 4 : 2; }
+__host__ __device__ constexpr int col_chunks(int G) { return G == 4 ? 4 : 1; }
 
 struct ColsumParams {
   const float* part_lse2;  // log2-domain LSEs of pass 1's key ranges, [slots][blk], merged here
   RangeSplit rs;           // how pass 1 was cut
   int blk;
-  float* partial;          // [NCH][B,H,Nk]
+  float* partial;          // [1 or, with four groups, 2][B,H,Nk]
   StatusRecord* status;
   int H, Nq, Nk, NKT;      // NKT = key tiles of 128
-  int NCH, W;              // query chunks and their width (multiple of 16, <= 256)
+  int W;                   // width of the query chunks (multiple of 16)
   int BH, n_range, tiles_per_cta;
   float scale_log2;
 };
 
-template <int D>
+template <int D, int G>
 struct ColsumSmem {
   static constexpr int kKTile = 128 * D * 2;
-  static constexpr int kK = 0;
-  static constexpr int kQ = kColStages * kKTile;      // NCH * W * D * 2 bytes follow
-  static constexpr int bars_offset(int NCH, int W) { return kQ + NCH * W * D * 2; }
-  static constexpr int kNumBars = 1 + 2 * kColStages + 4;
-  static constexpr int kBarBytes = 128;               // keeps the lse table behind it 16-byte aligned
+  static constexpr int kQ = 0;                        // the queries, then the key tiles
+  __host__ __device__ static constexpr int k_offset(int W) { return col_chunks(G) * W * D * 2; }
+  static constexpr int kNumBars = 1 + 2 * kColStages + 2 * G;
+  static constexpr int kBarBytes = 192;               // keeps the lse table behind it 16-byte aligned
   static_assert(kNumBars * 8 <= kBarBytes, "barrier area too small");
-  static constexpr int total(int NCH, int W) { return bars_offset(NCH, W) + kBarBytes + 512 * 4 + 16; }
+  static constexpr int kTail = kBarBytes + 512 * 4 + 16;      // barriers, LSE table, tensor-memory base and stop flag
+  static constexpr int kMax = 232448;
+  __host__ __device__ static constexpr int stages(int W) {
+    const int room = (kMax - kTail - k_offset(W)) / kKTile;
+    return room < kColStages ? room : kColStages;
+  }
+  __host__ __device__ static constexpr int bars_offset(int W) { return k_offset(W) + stages(W) * kKTile; }
+  static constexpr int total(int W) { return bars_offset(W) + kTail; }
 };
 
 enum ColWhere { kColQFull = 21, kColKEmpty, kColKFull, kColSEmpty, kColSFull };
 
-template <int D>
-__global__ void __launch_bounds__(kColThreads, 1)
+template <int D, int G>
+__global__ void __launch_bounds__(128 + 128 * G, 1)
 colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk, const ColsumParams p) {
-  using L = ColsumSmem<D>;
+  using L = ColsumSmem<D, G>;
+  constexpr int kThreads = 128 + 128 * G, kCols = 512 / G;
+  constexpr int NCH = col_chunks(G), WIDTH = G / 2, SIDE = G / 2;      // chunks; of a tile, and tiles, side by side
   constexpr int NPANEL = D / 64;
   constexpr int KPANEL_BYTES = 128 * 128;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int item = blockIdx.x;
-  const int W = p.W, NCH = p.NCH;
+  const int W = p.W;
   const int q_chunk_bytes = W * D * 2, q_panel_bytes = W * 128;
   if ((smem_u32(smem) & 1023u) != 0u) {
     if (tid == 0) report_status(p.status, AVSA_ERR_CUDA, kWhereSmemAlign, item, 0);
     return;
   }
-  const int bars_off = L::kQ + NCH * q_chunk_bytes;
+  const int n_st = L::stages(W), k_off = L::k_offset(W);
+  const int bars_off = L::bars_offset(W);
   const uint32_t bar0 = smem_u32(smem + bars_off);
   auto BAR = [&](int i) { return bar0 + static_cast<uint32_t>(i) * 8u; };
-  constexpr int Q_FULL = 0, K_FULL = 1, K_EMPTY = 1 + kColStages, S_FULL = 1 + 2 * kColStages, S_EMPTY = S_FULL + 2;
+  constexpr int Q_FULL = 0, K_FULL = 1, K_EMPTY = 1 + kColStages, S_FULL = 1 + 2 * kColStages, S_EMPTY = S_FULL + G;
   float* lse2 = reinterpret_cast<float*>(smem + bars_off + L::kBarBytes);
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + bars_off + L::kBarBytes + 512 * 4);
 
   if (tid == 0) {
     mbar_init(BAR(Q_FULL), 1);
-    for (int s = 0; s < kColStages; s++) {
+    for (int s = 0; s < n_st; s++) {
       mbar_init(BAR(K_FULL + s), 1);
       mbar_init(BAR(K_EMPTY + s), 1);
     }
-    for (int g = 0; g < 2; g++) {
+    for (int g = 0; g < G; g++) {
       mbar_init(BAR(S_FULL + g), 1);
       mbar_init(BAR(S_EMPTY + g), 128);
     }
@@ -96,6 +113,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   pdl_wait();
 
   auto wait_or_abort = [&](int bar, uint32_t parity, int where, int aux) -> bool {
+    if (mbar_try_wait(BAR(bar), parity)) return true;
     if (misc[1] != 0u) return false;
     if (mbar_wait(BAR(bar), parity)) return true;
     report_status(p.status, AVSA_ERR_TIMEOUT, where, item, aux);
@@ -111,6 +129,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   }
   pos_end = min(pos_end, pos + p.tiles_per_cta);
   int kc = 0;                               // key tiles of the segments before
+  int uses[G] = {};                         // chunks that went to each group's buffer (one group's own: uses[0])
   for (int seg = 0; pos < pos_end; seg++) {
     const int bh = pos / p.NKT, kt0 = pos % p.NKT, h = bh % p.H, b = bh / p.H;
     const int ntile = min(p.NKT - kt0, pos_end - pos);
@@ -118,7 +137,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
     // (straight from the partial LSEs of pass 1's key ranges: the same maximum-and-sum as in merge_splits_rows, so that
     // nothing has to be merged between the passes)
     // (warp 0 has no part in this: the first tiles and the queries are on their way meanwhile)
-    for (int j = tid - 32; j < NCH * W; j += kColThreads - 32) {
+    for (int j = tid - 32; j < NCH * W; j += kThreads - 32) {
       if (warp == 0) break;
       float v = -INFINITY;
       if (j < p.Nq) {
@@ -135,8 +154,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
       }
       lse2[j] = v;
     }
-    if (warp != 0) asm volatile("bar.sync 1, 352;" ::: "memory");      // the table is there (kColThreads - 32 threads)
-    const int n_units = ntile * NCH;
+    if (warp != 0) asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");      // the table is there
     if (warp == 0) {
       if (lane == 0) {
         mbar_expect_tx(BAR(Q_FULL), NCH * q_chunk_bytes);
@@ -146,12 +164,12 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
                         ch * W, h, b);
         bool ok = true;
         for (int t = 0; t < ntile && ok; t++) {
-          const int s = (kc + t) % kColStages, f = (kc + t) / kColStages;
+          const int s = (kc + t) % n_st, f = (kc + t) / n_st;
           if (f > 0) ok = wait_or_abort(K_EMPTY + s, (f - 1) & 1, kColKEmpty, t);
           if (!ok) break;
           mbar_expect_tx(BAR(K_FULL + s), L::kKTile);
           for (int pn = 0; pn < NPANEL; pn++)
-            tma_load_4d(smem_u32(smem + L::kK) + s * L::kKTile + pn * KPANEL_BYTES, &tmk, BAR(K_FULL + s), pn * 64,
+            tma_load_4d(smem_u32(smem + k_off) + s * L::kKTile + pn * KPANEL_BYTES, &tmk, BAR(K_FULL + s), pn * 64,
                         (kt0 + t) * 128, h, b);
         }
       }
@@ -162,96 +180,96 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
       const uint32_t idesc = make_idesc_bf16(128, W, 0, 0);
       constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
       auto desc64 = [](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
-      const uint32_t k_lo0 = ((smem_u32(smem + L::kK) & 0x3FFFFu) >> 4) | (1u << 16);
+      const uint32_t k_lo0 = ((smem_u32(smem + k_off) & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t q_lo0 = ((smem_u32(smem + L::kQ) & 0x3FFFFu) >> 4) | (1u << 16);
       auto wait_all = [&](int bar, uint32_t parity, int where, int aux) -> bool {
         return __all_sync(0xffffffffu, wait_or_abort(bar, parity, where, aux));
       };
       bool ok = wait_all(Q_FULL, seg & 1, kColQFull, 0);
-      for (int t = 0; t < ntile && ok; t++) {
-        const int s = (kc + t) % kColStages, f = (kc + t) / kColStages;
-        ok = wait_all(K_FULL + s, f & 1, kColKFull, t);
-        if (!ok) break;
-        const uint32_t k_lo = k_lo0 + s * (L::kKTile >> 4);
-        for (int ch = 0; ch < NCH && ok; ch++) {
-          const int u = (kc + t) * NCH + ch, g = u & 1, i = u >> 1;
-          if (i > 0) ok = wait_all(S_EMPTY + g, (i - 1) & 1, kColSEmpty, u);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t q_lo = q_lo0 + ch * (q_chunk_bytes >> 4);
-          if (leader) {
+      for (int t0 = 0; t0 < ntile && ok; t0 += SIDE) {
+        const int n = min(SIDE, ntile - t0);
+        for (int ch0 = 0; ch0 < NCH && ok; ch0 += WIDTH) {
+          for (int t = t0; t < t0 + n && ok; t++) {
+            const int s = (kc + t) % n_st, f = (kc + t) / n_st;
+            if (ch0 == 0) ok = wait_all(K_FULL + s, f & 1, kColKFull, t);
+            const uint32_t k_lo = k_lo0 + s * (L::kKTile >> 4);
+            for (int c = 0; c < WIDTH && ok; c++) {
+              const int g = (t & 1) * WIDTH + c;
+              int used = 0;
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ks++) {
-              const uint32_t koff = ((ks >> 2) * KPANEL_BYTES + (ks & 3) * 32) >> 4;
-              const uint32_t qoff = ((ks >> 2) * q_panel_bytes + (ks & 3) * 32) >> 4;
-              umma_ss(tmem + g * 256, desc64(k_lo + koff), desc64(q_lo + qoff), idesc, ks > 0 ? 1u : 0u);
+              for (int i = 0; i < G; i++)
+                if (i == g) used = uses[i]++;
+              if (used > 0) ok = wait_all(S_EMPTY + g, (used - 1) & 1, kColSEmpty, t);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t q_lo = q_lo0 + (ch0 + c) * (q_chunk_bytes >> 4);
+              if (leader) {
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ks++) {
+                  const uint32_t koff = ((ks >> 2) * KPANEL_BYTES + (ks & 3) * 32) >> 4;
+                  const uint32_t qoff = ((ks >> 2) * q_panel_bytes + (ks & 3) * 32) >> 4;
+                  umma_ss(tmem + g * kCols, desc64(k_lo + koff), desc64(q_lo + qoff), idesc, ks > 0 ? 1u : 0u);
+                }
+                umma_commit(BAR(S_FULL + g));
+                if (ch0 + c == NCH - 1) umma_commit(BAR(K_EMPTY + s));
+              }
+              __syncwarp();
             }
-            umma_commit(BAR(S_FULL + g));
-            if (ch == NCH - 1) umma_commit(BAR(K_EMPTY + s));
           }
-          __syncwarp();
         }
       }
     } else if (warp >= 4) {
       const int g = (warp - 4) >> 2;
       const int row = ((warp & 3) << 5) + lane;
       const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
+      const int first_ch = g % WIDTH;
+      const uint32_t base = tmem + g * kCols + lane_off;
+      const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
       bool ok = true;
-      const int u0 = kc * NCH;      // units of the segments before: unit u goes to buffer and group u mod 2
-      for (int u = u0 + ((g ^ u0) & 1); u < u0 + n_units && ok; u += 2) {
-        const int i = u >> 1, t = u / NCH - kc, ch = u % NCH;
-        ok = wait_or_abort(S_FULL + g, i & 1, kColSFull, u);
-        if (!ok) break;
-        tc_fence_after();
-        const float* l2 = lse2 + ch * W;
-        const uint32_t base = tmem + g * 256 + lane_off;
-        const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
+      // the group's tiles, and of each its chunks one after the other
+      for (int t = g / WIDTH; t < ntile && ok; t += 2) {
         uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-        // sum over 32 (or 16) queries of exp2(s*c - lse2), two values per packed FMA / add
-        auto reduce32 = [&](const uint32_t (&sv)[32], const float* nl) {
+        for (int ch = first_ch; ch < NCH && ok; ch += WIDTH) {
+          ok = wait_or_abort(S_FULL + g, uses[0] & 1, kColSFull, t);
+          if (!ok) break;
+          uses[0]++;
+          tc_fence_after();
+          const float* nl0 = lse2 + ch * W;
+          // sum over 16 queries of exp2(s*c - lse2), two values per packed FMA / add
+          auto reduce16 = [&](const uint32_t (&sv)[16], const float* nl) {
 #pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const ulonglong2 nv = *reinterpret_cast<const ulonglong2*>(nl + j);      // four negated LSEs
-            float x0, x1, x2, x3;
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nv.x), x0, x1);
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3])), c2, nv.y), x2, x3);
-            acc[(j >> 2) & 3] = add_f32x2(acc[(j >> 2) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-            acc[((j >> 2) + 2) & 3] = add_f32x2(acc[((j >> 2) + 2) & 3], pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
+            for (int j = 0; j < 16; j += 4) {
+              const ulonglong2 nv = *reinterpret_cast<const ulonglong2*>(nl + j);      // four negated LSEs
+              float x0, x1, x2, x3, y0, y1;
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nv.x), x0, x1);
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3])), c2, nv.y), x2, x3);
+              y0 = fast_exp2(x0);
+              y1 = fast_exp2(x1);
+              acc[(j >> 1) & 3] = add_f32x2(acc[(j >> 1) & 3], pack_f32x2(y0, y1));
+              acc[((j >> 1) + 1) & 3] = add_f32x2(acc[((j >> 1) + 1) & 3], pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
+            }
+          };
+          const int n16 = W / 16;
+          uint32_t sa[16], sb[16];
+          tmem_ld16(base, sa);
+          for (int c = 0; c < n16; c += 2) {
+            tmem_wait_ld_regs(sa);
+            if (c + 1 < n16) tmem_ld16(base + (c + 1) * 16, sb);      // in flight under the exponentials of piece c
+            reduce16(sa, nl0 + c * 16);
+            if (c + 1 < n16) {
+              tmem_wait_ld_regs(sb);
+              if (c + 2 < n16) tmem_ld16(base + (c + 2) * 16, sa);
+              reduce16(sb, nl0 + (c + 1) * 16);
+            }
           }
-        };
-        const int n32 = W / 32;           // whole 32-column pieces; W is a multiple of 16, so 16 columns may remain
-        uint32_t sa[32], sb[32];
-        if (n32 > 0) tmem_ld32(base, sa);
-        for (int c = 0; c < n32; c += 2) {
-          tmem_wait_ld();
-          if (c + 1 < n32) tmem_ld32(base + (c + 1) * 32, sb);      // in flight under the exponentials of piece c
-          reduce32(sa, l2 + c * 32);
-          if (c + 1 < n32) {
-            tmem_wait_ld();
-            if (c + 2 < n32) tmem_ld32(base + (c + 2) * 32, sa);
-            reduce32(sb, l2 + (c + 1) * 32);
-          }
-        }
-        if (n32 * 32 < W) {
-          uint32_t st[16];
-          tmem_ld16(base + n32 * 32, st);
-          tmem_wait_ld();
-          const float* nl = l2 + n32 * 32;
-#pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            float x0, x1;
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(st[j]), __uint_as_float(st[j + 1])), c2,
-                                   *reinterpret_cast<const uint64_t*>(nl + j)), x0, x1);
-            acc[(j >> 1) & 3] = add_f32x2(acc[(j >> 1) & 3], pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-          }
+          tc_fence_before();
+          mbar_arrive(BAR(S_EMPTY + g));
         }
         float sum0, sum1;
         unpack_f32x2(add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3])), sum0, sum1);
-        tc_fence_before();
-        mbar_arrive(BAR(S_EMPTY + g));
         const int key = (kt0 + t) * 128 + row;
-        if (key < p.Nk)
-          p.partial[(static_cast<int64_t>(ch) * p.BH + bh) * p.Nk + key] = sum0 + sum1;
+        if (ok && key < p.Nk)
+          p.partial[(static_cast<int64_t>(first_ch) * p.BH + bh) * p.Nk + key] = sum0 + sum1;
       }
     }
     pos += ntile;
@@ -305,7 +323,7 @@ struct ColsumRevSmem {
 enum ColRevWhere { kRevKFull = 51, kRevQEmpty, kRevQFull, kRevSEmpty, kRevSFull };
 
 template <int D>
-__global__ void __launch_bounds__(kColThreads, 1)
+__global__ void __launch_bounds__(kRevThreads, 1)
 colsum_rev_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                   const ColsumRevParams p) {
   using L = ColsumRevSmem<D>;
@@ -576,7 +594,8 @@ __global__ void __launch_bounds__(256) head_sum_wide_kernel(const float* __restr
 struct CrossPlan {
   int blk, NQT, NKB;                         // pass 1 (key tiles of blk)
   RangeSplit rs;
-  int NKT, NCH, W, n_range, tpc, ctas2;      // pass 2 (key tiles of 128), cuts per pair, tiles per CTA, CTAs
+  int NKT, NCH, W, n_range, tpc, ctas2;      // pass 2 (key tiles of 128), query chunks, cuts per pair, tiles per CTA, CTAs
+  int slots2;                                // sums per key
   bool reverse;                              // pass 2 with the keys resident (Nq > 512, Nk <= 512)
   int NQC, rev_ranges, rev_cpr, rev_slots;   // query chunks of 128, CTAs per (b,h), chunks per CTA, partial slots
   bool resident;                             // both passes in one kernel, K and V of a head on chip
@@ -613,8 +632,9 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   const long long kv_bytes = 4ll * B * H * Nk * d;
   c.rs = make_range_split(B * H, c.NQT, c.NKB, target, kv_bytes > kL2KeepBytes, c.NKB);
   c.NKT = (Nk + 127) / 128;
-  c.NCH = Nq > 256 ? 2 : 1;
+  c.NCH = col_chunks(col_groups(Nq));
   c.W = (((Nq + c.NCH - 1) / c.NCH) + 15) / 16 * 16;
+  c.slots2 = col_groups(Nq) / 2;
   // equal cuts of every pair, or even cuts through all of them where that is shorter by more than the reload it costs
   // (32 heads x 384 tiles, 512 queries on 148 SMs: 96 tiles on 128 of them 645 us for the call, 84 on all 612; 32 x 157 with
   // 100 queries: 110 us as 40 tiles on 128, 112 as 34 on all)
@@ -647,7 +667,7 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   c.off_part_lse = off; off += align_up(slots1 * c.blk * sizeof(float), 256);
   c.off_lse = off; off += align_up(static_cast<size_t>(B) * H * Nq * sizeof(float), 256);
   c.off_lse2 = off; off += c.reverse ? align_up(static_cast<size_t>(B) * H * c.NQC * 128 * sizeof(float), 256) : 0;
-  const size_t slots = c.reverse ? static_cast<size_t>(c.rev_slots) : static_cast<size_t>(c.NCH);
+  const size_t slots = c.reverse ? static_cast<size_t>(c.rev_slots) : static_cast<size_t>(c.slots2);
   c.off_partial = off; off += align_up(slots * B * H * Nk * sizeof(float), 256);
   c.off_redo = off; off += align_up(slots1 * sizeof(int), 256);
   c.total = off;
@@ -709,6 +729,14 @@ static int run_cross_resident(int B, int H, int Nq, int Nk, const avsa_bf16_4d& 
     if (rc != AVSA_OK) return rc;
   }
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
+}
+
+template <int D, int G>
+static int launch_colsum(const CUtensorMap& tq, const CUtensorMap& tk, const ColsumParams& cp, int ctas, cudaStream_t st) {
+  using L = ColsumSmem<D, G>;
+  // always the same limit, as in the reverse direction
+  if (cudaFuncSetAttribute(colsum_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kMax) != cudaSuccess) return AVSA_ERR_CUDA;
+  return launch_pdl(colsum_kernel<D, G>, ctas, 128 + 128 * G, L::total(cp.W), st, tq, tk, cp) == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
 template <int BLK, int D>
@@ -780,7 +808,7 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     const int smem = L::total(c.NKT);
     // always the same limit (four key tiles), whatever this call needs: the limit belongs to the kernel, and a host thread
     // with fewer keys must not lower it between another thread's setting and launch
-    constexpr int kMaxSmem = L::total(4);
+    constexpr int kMaxSmem = 232448;      // always the same limit, as above
     if (cudaFuncSetAttribute(colsum_rev_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
       return AVSA_ERR_CUDA;
     ColsumRevParams rp;
@@ -794,7 +822,7 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     rp.n_range = c.rev_ranges;
     rp.chunks_per_range = c.rev_cpr;
     rp.scale_log2 = scale * 1.4426950408889634f;
-    if (launch_pdl(colsum_rev_kernel<D>, dim3(c.rev_ranges, H, B), kColThreads, smem, st, tq, tk, rp) != cudaSuccess)
+    if (launch_pdl(colsum_rev_kernel<D>, dim3(c.rev_ranges, H, B), kRevThreads, smem, st, tq, tk, rp) != cudaSuccess)
       return AVSA_ERR_CUDA;
     const int64_t n = static_cast<int64_t>(B) * Nk;
     if (launch_pdl(head_sum_wide_kernel, static_cast<unsigned>((n + 7) / 8), 256, 0, st, partial, c.rev_slots, B, H, Nk, beta,
@@ -803,14 +831,9 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
   }
   // ---- pass 2, queries resident (at most 512 queries)
   if (scores != nullptr && !c.reverse) {
-    using L = ColsumSmem<D>;
     CUtensorMap tq, tk;
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, c.W)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
-    const int smem = L::total(c.NCH, c.W);
-    constexpr int kMaxSmem = L::total(2, 256);      // 512 queries; always the same limit, as above
-    if (cudaFuncSetAttribute(colsum_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
-      return AVSA_ERR_CUDA;
     ColsumParams cp;
     cp.part_lse2 = part_lse;
     cp.rs = c.rs;
@@ -821,21 +844,21 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     cp.Nq = Nq;
     cp.Nk = Nk;
     cp.NKT = c.NKT;
-    cp.NCH = c.NCH;
     cp.W = c.W;
     cp.BH = B * H;
     cp.n_range = c.n_range;
     cp.tiles_per_cta = c.tpc;
     cp.scale_log2 = scale * 1.4426950408889634f;
-    if (launch_pdl(colsum_kernel<D>, c.ctas2, kColThreads, smem, st, tq, tk, cp) != cudaSuccess) return AVSA_ERR_CUDA;
+    const int rc = col_groups(Nq) == 4 ? launch_colsum<D, 4>(tq, tk, cp, c.ctas2, st) : launch_colsum<D, 2>(tq, tk, cp, c.ctas2, st);
+    if (rc != AVSA_OK) return rc;
     const int64_t n = static_cast<int64_t>(B) * Nk;
     const int hs_blocks = static_cast<int>((n + kHeadSumKeys - 1) / kHeadSumKeys);
     if (merge_late) {
-      if (launch_pdl(cross_finalize_kernel<BLK, D>, hs_blocks + merge_blocks, 256, 0, st, hs_blocks, partial, c.NCH, B,
+      if (launch_pdl(cross_finalize_kernel<BLK, D>, hs_blocks + merge_blocks, 256, 0, st, hs_blocks, partial, c.slots2, B,
                      H, Nk, beta, gamma, scores, m) != cudaSuccess)
         return AVSA_ERR_CUDA;
     } else {
-      if (launch_pdl(head_sum_kernel, hs_blocks, 256, 0, st, partial, c.NCH, B, H, Nk, beta, gamma, scores) != cudaSuccess)
+      if (launch_pdl(head_sum_kernel, hs_blocks, 256, 0, st, partial, c.slots2, B, H, Nk, beta, gamma, scores) != cudaSuccess)
         return AVSA_ERR_CUDA;
     }
   }

@@ -551,10 +551,15 @@ def test_cross_attention_long_query_axis_two_chunks():
     (1, 22, 2427, 200, 128, True),     # reverse: 19 query tiles in chunks of 4, whole rows, score pass over the keys
     (1, 2, 130, 6400, 64, True),
     (1, 100, 40, 1000, 64, True),      # score pass: 800 key tiles cut evenly through the heads
-    (1, 96, 300, 520, 128, True),      # the same with the queries in two chunks
+    (1, 96, 300, 520, 128, True),      # the same with the queries in four chunks
+    (1, 3, 128, 700, 64, True),        # one chunk, tiles by turns over four groups
+    (1, 3, 129, 650, 128, True),       # two chunks of 80
+    (1, 2, 256, 515, 128, True),
+    (1, 2, 257, 900, 64, True),        # four chunks of 80
+    (2, 2, 512, 640, 128, True),
     (1, 1, 100, 6400, 64, True),       # a row in more parts than lanes take at once (50 of 16 and, below, of 32)
     (1, 1, 130, 6400, 128, True),
-    (1, 40, 400, 900, 64, True),
+    (1, 40, 400, 900, 64, True),       # more than 8192 split rows
     (1, 20, 500, 1700, 128, True),
 ])
 def test_cross_attention_work_split(B, H, Nq, Nk, d, scores):
