@@ -1117,8 +1117,8 @@ def test_protected_rows_that_outgrow_their_reference(H, N, n_protect, short, d):
 
 @pytest.mark.parametrize("n", [1, 63, 256, 257, 511, 512, 513])
 def test_mask_with_the_select_in_the_pooling_grid(n):
-    """Up to 512 tokens one launch selects and pools: token flags and block flags are the oracle's, ties at the threshold included, and
-    the lists those of the block scores that the call itself returns."""
+    """Up to 512 tokens one launch selects and pools: token flags and block flags are the oracle's, ties at the threshold included,
+    block scores are its up to fp32 sums, and the lists hold the largest of the scores that the call returns."""
     B, H, d, n_protect = 3, 2, 64, max(1, n // 9)
     NB = (n + d - 1) // d
     g = torch.Generator(device="cuda").manual_seed(n)
@@ -1127,11 +1127,17 @@ def test_mask_with_the_select_in_the_pooling_grid(n):
     k_keep = max(1, NB // 2)
     m = av.avsa_build_block_mask(q, k, s, n_protect, k_keep, d)
     _status_ok(m["ws"])
-    idx, cnt, tok, blk = orc.build_block_mask(m["block_scores"].cpu().numpy(), s.cpu().numpy(), n_protect, k_keep, d, n)
-    assert np.array_equal(m["prot_tok"].cpu().numpy(), tok) and np.array_equal(m["prot_blk"].cpu().numpy(), blk)
-    assert np.array_equal(m["col_cnt"].cpu().numpy(), cnt) and np.array_equal(m["col_idx"].cpu().numpy(), idx)
     want = orc.block_scores(_np64(q), _np64(k), d)
-    assert np.abs(m["block_scores"].cpu().numpy() - want).max() <= 1e-4 * np.abs(want).max()
+    _, _, tok, blk = orc.build_block_mask(want, s.cpu().numpy(), n_protect, k_keep, d, n)
+    assert np.array_equal(m["prot_tok"].cpu().numpy(), tok) and np.array_equal(m["prot_blk"].cpu().numpy(), blk)
+    bs, idx, cnt = (m[x].cpu().numpy() for x in ("block_scores", "col_idx", "col_cnt"))
+    assert np.abs(bs - want).max() <= 1e-4 * np.abs(want).max()
+    assert np.array_equal(cnt, np.broadcast_to(np.where(blk != 0, NB, k_keep)[:, None, :], cnt.shape))
+    for row, scores_row, c in zip(idx.reshape(-1, NB), bs.reshape(-1, NB), cnt.reshape(-1)):
+        kept = row[:c]
+        assert (np.diff(kept) > 0).all() and (row[c:] == -1).all()
+        rest = np.setdiff1d(np.arange(NB), kept)
+        assert rest.size == 0 or scores_row[kept].min() >= scores_row[rest].max()
 
 
 @pytest.mark.parametrize("NB", [1, 32, 33, 256, 257, 512, 513, 1024, 1025])
