@@ -10,7 +10,7 @@
 //   What bounds it: a tile's phases follow one another in the softmax warps (24 heads x 32760 queries x 256 keys, cycles a
 // tile: logits and maximum 700, exponentials 2330, which is the MUFU's rate, row sums 200-500, column sums 850, O 1000, waits
 // for S 350-800), because tensor memory holds one tile (KG = 2).  Against the calls that it replaces (attention over two-tile
-// items 160 us, LSE conversion 5, S^T and its exponentials again 70, head sum 4): 254 -> 162 us; 100 keys 223 -> 80;
+// items 160 us, LSE conversion 5, S^T and its exponentials again 70, head sum 4): 255 -> 159 us; 100 keys 223 -> 80;
 // 24 keys of 64 channels, 32 heads x 49152 queries 382 -> 93; 8 heads x 2070 x 72 keys 19.4 -> 10.3; 2 heads x 32 queries x 256
 // keys 13.8 -> 8.3.  Without scores (256 keys) 157 -> 124.
 //
@@ -328,9 +328,10 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         tc_fence_after();
         // ---- the row's maximum, over batches of 64 logits (two chunks); the last batch stays in registers
         uint32_t s[64];
+        // (one load of 64 columns, of which the second half may be no keys' and is left alone; as two of 32 the call with 256 keys took
+        // 144.6 us instead of 141.5)
         auto load_batch = [&](int c0) {
-          tmem_ld32(tm_s + c0 * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-          if (c0 + 1 < nch) tmem_ld32(tm_s + c0 * 32 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+          tmem_ld64(tm_s + c0 * 32, s);
           tmem_wait_ld_regs(s);
         };
         float m8[8];
@@ -485,8 +486,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           __syncwarp();
 #pragma unroll
           for (int c = 0; c < COLS / 64; c++) {
-            tmem_ld32(tm_o + (kSplitO ? w * 64 : c * 64), *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-            tmem_ld32(tm_o + (kSplitO ? w * 64 : c * 64) + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+            tmem_ld64(tm_o + (kSplitO ? w * 64 : c * 64), s);
             tmem_wait_ld_regs(s);
             if (c == COLS / 64 - 1) {
               tc_fence_before();
