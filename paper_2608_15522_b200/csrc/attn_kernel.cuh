@@ -724,18 +724,18 @@ struct MergeParams {
   int row_map_stride, n_out;
 };
 
-// A CTA of 256 threads merges eight rows of a query tile (sixteen with 64 channels): in every part they are 4 KB in a row, and eight parts'
-// loads are in flight.  Where the rows are is worked out once for all of them, and a row's LSEs are loaded by its 32 (16)
-// lanes side by side, so that two trips to L2 and one more for every eight parts are all there is.  (A row a warp, one LSE after
-// the other and parts by fours: 896 rows x 24 heads of 3 to 6 parts 22.5 us, 21.3 now; 576 rows of 17 parts, with their head sums, 9.5, 5.7 now.
-// Four times the rows a CTA, four float4 a thread and part: 20.5 and, with head sums, 32 heads x 512 rows 18.8 instead of 19.2.)
+// A CTA of 256 threads merges eight rows of a query tile (sixteen with 64 channels): in every part they are 4 KB in a row, and
+// eight parts' loads are in flight.  Where the rows are is worked out once for all of them, and a row's LSEs are loaded by its 32
+// (16) lanes side by side, together with the first parts: one trip to L2 and one more for every eight further parts are all there
+// is.  (A row a warp, one LSE after the other and parts by fours: 896 rows x 24 heads of 3 to 6 parts 22.5 us, 18.2 now; 576 rows
+// of 17 parts, with their head sums, 9.5, 5.3 now.  The parts asked for only when their weights were known: 21.3 and 5.7.)
 // `block`: index of the group of rows.
 __host__ __device__ constexpr int merge_rows(int D) { return 1024 / D; }
 constexpr int kMergeParts = 128;
 template <int BLK, int D>
 __device__ __forceinline__ void merge_splits_rows(int block, const MergeParams& m) {
   constexpr int ROWS = merge_rows(D), LANES = 256 / ROWS, V = D / 4, U = 8;       // lanes of a row, float4 of a row, parts in flight
-  static_assert(BLK % ROWS == 0 && ROWS * V == 256, "a group of rows lies in one query tile, a part of it is a float4 a thread");
+  static_assert(BLK % ROWS == 0 && LANES == V, "a group of rows lies in one query tile, a part of it is a float4 a thread");
   __shared__ float weight[kMergeParts][ROWS];
   __shared__ float total[ROWS];
   const int tid = threadIdx.x;
@@ -747,8 +747,23 @@ __device__ __forceinline__ void merge_splits_rows(int block, const MergeParams& 
   if (n == 1) return;
   const int64_t row0 = (static_cast<int64_t>(first) * m.rs.chunk + qt % m.rs.chunk) * BLK + q0 % BLK;
   const int64_t step = static_cast<int64_t>(m.rs.chunk) * BLK;
-  // the largest LSE of a row, then what every part weighs beside it
+  // this thread's row (LANES threads have one, which is as many as it has float4) and where it goes
   const int wr = tid / LANES, wl = tid % LANES;
+  int out_row = q0 + wr < m.Nq ? q0 + wr : -1;
+  if (m.row_map != nullptr && out_row >= 0) {
+    out_row = m.row_map[static_cast<int64_t>(b) * m.row_map_stride + out_row];
+    if (out_row >= m.n_out) out_row = -1;
+  }
+  // the first parts are asked for together with the LSEs
+  const float4* src = reinterpret_cast<const float4*>(m.part_o + row0 * D) + tid;
+  float4 v[U];
+  auto load_parts = [&](int s0) {
+#pragma unroll
+    for (int k = 0; k < U; k++)
+      v[k] = m.o != nullptr && s0 + k < n ? __ldg(src + (s0 + k) * step * V) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  load_parts(0);
+  // the largest LSE of a row, then what every part weighs beside it
   const float* pl = m.part_lse2 + row0 + wr;
   const float mine = wl < n ? __ldg(pl + wl * step) : -INFINITY;
   float M = mine;
@@ -763,38 +778,26 @@ __device__ __forceinline__ void merge_splits_rows(int block, const MergeParams& 
   }
 #pragma unroll
   for (int off = LANES / 2; off > 0; off >>= 1) W += __shfl_xor_sync(0xffffffffu, W, off);
-  auto out_row = [&](int r) -> int {
-    const int qrow = q0 + r;
-    if (qrow >= m.Nq) return -1;
-    if (m.row_map == nullptr) return qrow;
-    const int o = m.row_map[static_cast<int64_t>(b) * m.row_map_stride + qrow];
-    return o < m.n_out ? o : -1;
-  };
   if (wl == 0) {
     total[wr] = W;
-    const int o = out_row(wr);
-    if (m.lse != nullptr && o >= 0) m.lse[static_cast<int64_t>(bh) * m.n_out + o] = (M + log2f(W)) * 0.6931471805599453f;
+    if (m.lse != nullptr && out_row >= 0)
+      m.lse[static_cast<int64_t>(bh) * m.n_out + out_row] = (M + log2f(W)) * 0.6931471805599453f;
   }
   if (m.o == nullptr) return;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int r = tid / V, c4 = tid % V;
-  const float4* src = reinterpret_cast<const float4*>(m.part_o + row0 * D) + tid;
   for (int c0 = 0; c0 < n; c0 += kMergeParts) {
     const int nc = min(kMergeParts, n - c0);
     if (c0 > 0) {      // (hardly ever: more parts than the table holds)
       __syncthreads();
       for (int s = wl; s < nc; s += LANES) weight[s][wr] = exp2f(__ldg(pl + (c0 + s) * step) - M);
     }
+    __syncthreads();      // the weights are there
     for (int s0 = 0; s0 < nc; s0 += U) {
-      float4 v[U];
-#pragma unroll
-      for (int k = 0; k < U; k++)
-        v[k] = s0 + k < nc ? __ldg(src + (c0 + s0 + k) * step * V) : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (s0 == 0) __syncthreads();      // the weights are there (the first loads are on their way)
+      if (c0 + s0 > 0) load_parts(c0 + s0);
 #pragma unroll
       for (int k = 0; k < U; k++) {
         if (s0 + k >= nc) break;
-        const float w = weight[s0 + k][r];
+        const float w = weight[s0 + k][wr];
         acc.x = fmaf(w, v[k].x, acc.x);
         acc.y = fmaf(w, v[k].y, acc.y);
         acc.z = fmaf(w, v[k].z, acc.z);
@@ -802,13 +805,12 @@ __device__ __forceinline__ void merge_splits_rows(int block, const MergeParams& 
       }
     }
   }
-  const int o = out_row(r);
-  if (o < 0) return;
-  const float inv = 1.0f / total[r];
+  if (out_row < 0) return;
+  const float inv = 1.0f / total[wr];
   uint2 pk;
   pk.x = pack_bf16x2(acc.x * inv, acc.y * inv);
   pk.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-  *reinterpret_cast<uint2*>(m.o + b * m.o_sb + h * m.o_sh + o * m.o_sn + c4 * 4) = pk;
+  *reinterpret_cast<uint2*>(m.o + b * m.o_sb + h * m.o_sh + out_row * m.o_sn + wl * 4) = pk;
 }
 
 // returns the number of groups of rows

@@ -505,8 +505,8 @@ __global__ void __launch_bounds__(256) lse_to_log2_kernel(const float* __restric
 // scores[b,i] = beta * scores[b,i] + gamma * sum_h sum_ch partial[ch][b,h,i] for 64 keys; all 256 threads of the CTA call it.
 // A fixed order: each of four threads a key adds a quarter of the terms, heads ascending, then the quarters are added.  Sixteen
 // loads a thread are in flight.  (A thread a key and eight loads left a quarter as many threads waiting for eight round trips:
-// 32 heads x 2 chunks x 49152 keys with its merge 19.8 us, now 19.2;
-// 8 heads x 2070 keys with the merge of 576 rows 9.5, now 5.7.)
+// 32 heads x 2 chunks x 49152 keys with its merge 19.8 us, now 17.8;
+// 8 heads x 2070 keys with the merge of 576 rows 9.5, now 5.3.)
 constexpr int kHeadSumKeys = 64;
 __device__ __forceinline__ void head_sum_keys(int block, int tid, const float* __restrict__ partial, int NCH, int B,
                                               int H, int Nk, float beta, float gamma, float* __restrict__ scores) {
