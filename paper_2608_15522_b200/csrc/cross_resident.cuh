@@ -19,7 +19,8 @@
 //   warp 2      tensor-memory allocation
 //   warps 4-7, 8-11  two softmax groups, one thread per row
 // KG = 2 (129 to 256 keys): both groups work on the same tile, the first on keys 0-127, the second on the rest.  The first
-// one's maximum is the reference of both; the row sums are exchanged in pairs of warps.
+// one's maximum is the reference of both (where a row outgrows it, the second group takes another one and rescales the first's
+// P); the row sums are exchanged in pairs of warps.
 //   tensor memory: S, then p (fp32, 256 columns) | P (bf16, 128) | O (128)
 // KG = 1 (at most 128 keys): the groups take alternate tiles.
 //   tensor memory: S/p of group 0 | of group 1 (128 each) | P of group 0 | of group 1 (64 each) | O (128)
@@ -256,6 +257,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           const int nch = i == 0 ? p.nch0 : p.nch1, key0 = i * p.nch0 * 32;
           if (part == 1 && nch <= 2) continue;
           ok = wait_all(P_FULL + 2 * g + part, uses & 1, kResPFull, T);
+          // (the second group may rescale the first's P until it hands over the first part of its own)
+          if (ok && KG == 2 && part == 0 && i == 0) ok = wait_all(P_FULL + 2, uses & 1, kResPFull, T);
           if (!ok) break;
           tc_fence_after();
           // steps of 16 keys: of more than two chunks those behind the second come first
@@ -361,8 +364,10 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         float first = 1.f;    // (second group) what the first group's are multiplied by
         if (KG == 2) {
           // The first group's maximum is the reference of the whole row (it goes ahead with it), unless the second group's lies
-          // beyond it by more than 2^64.  Then the second group takes its own, less 60: its probabilities reach 2^60, beside
-          // which the first group's, at most 1 in the accumulator of O where they should be 2^-4 or less, are nothing.
+          // beyond it by more than 2^57.  Then the second takes the least reference 2^k times the first's (which makes a power of
+          // two of the factor) beside which none of its probabilities exceeds 2^57.  So a row's sum is about 2^64 at most (128 keys
+          // of 2^57): values of v up to 2^60 leave the accumulator of O finite.
+          // (Both groups waiting for both maxima, and taking the same reference: 142 -> 149 us, without scores 122 -> 133.)
           if (w == 0) {
             exch[row] = m;
             mbar_arrive(BAR(MAX + quad));
@@ -370,10 +375,10 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             ok = wait_all(MAX + quad, T & 1, kResMax, T);
             if (!ok) break;
             const float ma = exch[row];
-            if (m - ma > 64.f) {
-              m -= 60.f;
+            if (m - ma > 57.f) {
+              if (m - ma > 64.f && atomicMax(const_cast<int*>(&misc[6]), T + 1) < T + 1) atomicAdd(const_cast<int*>(&misc[7]), 1);
+              m = ma + ceilf(m - ma - 57.f);
               first = exp2f(ma - m);
-              if (atomicMax(const_cast<int*>(&misc[6]), T + 1) < T + 1) atomicAdd(const_cast<int*>(&misc[7]), 1);
             } else {
               m = ma;
             }
@@ -402,6 +407,22 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             tmem_st16(tm_p + (c0 + c) * 16, pk);
             if (SCORES) tmem_st32(tm_s + (c0 + c) * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
           }
+          if (upper && bar == P_FULL + 2 && __any_sync(FULLM, first != 1.f)) {
+            // Rows with another reference: the first group's P in proportion, before any of it is multiplied with V (the issuer
+            // waits for this hand-over first), so that every key weighs what it should, however large its v is.
+            for (int part = 0; part < 2 && ok; part++) ok = wait_all(P_FULL + part, T & 1, kResPFull, T);
+            if (!ok) return;
+            tc_fence_after();
+            for (int c = 0; c < 4; c++) {
+              uint32_t pk[16];
+              tmem_ld16(tmem + lane_off + TM_P + c * 16, pk);
+              tmem_wait_ld_regs(pk);
+#pragma unroll
+              for (int j = 0; j < 16; j++)
+                pk[j] = pack_bf16x2(__uint_as_float(pk[j] << 16) * first, __uint_as_float(pk[j] & 0xffff0000u) * first);
+              tmem_st16(tmem + lane_off + TM_P + c * 16, pk);
+            }
+          }
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(BAR(bar));
@@ -412,12 +433,14 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         };
         if (nch > 2) {      // the batch at hand first
           exp_batch(2, P_FULL + 2 * w);
+          if (!ok) break;
           load_batch(0);
           if (!SCORES) s_free();
           exp_batch(0, P_FULL + 2 * w + 1);
         } else {
           if (!SCORES) s_free();
           exp_batch(0, P_FULL + 2 * w);
+          if (!ok) break;
         }
         float lsum;
         {

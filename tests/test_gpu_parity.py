@@ -631,6 +631,32 @@ def test_cross_attention_few_keys_that_outgrow_their_reference(step):
     _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "outgrown scores")
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("nk", [200, 256])
+@pytest.mark.parametrize("gap,v_first,v_rest", [(50, 59, 59), (63, 59, 59), (66, 59, 59), (61, 59, 0), (66, 59, 0), (200, 0, 59)])
+def test_cross_attention_few_keys_with_large_values(gap, v_first, v_rest, nk, d):
+    """The keys from 128 on have logits larger by ``gap`` in base 2 (within 2), and the values of either half are of magnitude 2^v:
+    no accumulator overflows, and the first half keeps its weight where large values make it count (128 2^(59 - 61) beside
+    72).  The tiles with a gap beyond 64 are counted."""
+    B, H, Nq = 1, 2, 150
+    g = torch.Generator().manual_seed(11)
+    q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, nk, nk))
+    q, k = 0.5 * q, 0.5 * k
+    q[..., 0], k[..., 0] = 8.0, 0.0
+    k[:, :, 128:, 0] = gap / 8.0 * np.log(2.0) * np.sqrt(d)
+    v = 1.0 + 0.25 * v
+    v[:, :, :128] *= 2.0**v_first
+    v[:, :, 128:] *= 2.0**v_rest
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+    o, lse, s, ws = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), score_gamma=1.0 / (H * Nq))
+    _status_ok(ws)
+    assert av.avsa_redo_count(ws) == (2 * H if gap > 64 else 0)
+    _close(_np64(o) / 2.0**v_rest, want_o / 2.0**v_rest, "large values O")
+    _close_lse(_np64(lse), want_lse, "large values lse")
+    _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "large values scores")
+
+
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_reverse_direction(name):
     """Video queries attending to audio keys (the other half of the bidirectional pair): outputs, LSE, and the
