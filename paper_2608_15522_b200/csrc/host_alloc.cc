@@ -1,11 +1,23 @@
 // Uninitialised tensors for the wrappers of binding.py: torch.empty without the parsing of its Python arguments, which costs
 // twice what the allocation does (2.2 us a tensor; the audio branch's own mask and attention, called without buffers, make
-// eight of them in a pass of 40 us).  The same operators through the same dispatcher, caching allocator and current stream.
+// eight of them in a pass of 40 us).  The same operators through the same dispatcher, caching allocator and current stream, and
+// as there without the interpreter lock: an allocation may wait for the GPU.
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
+#include <ATen/DimVector.h>
 
 namespace {
+
+// What `allocate` returns, called without the interpreter lock (which is taken again if it throws, too).
+template <typename F>
+at::Tensor without_lock(F&& allocate) {
+  struct Lock {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Lock() { PyEval_RestoreThread(state); }
+  } lock;
+  return allocate();
+}
 
 // empty(like, kind, *sizes): kind 0 fp32, 1 int32, 2 uint8, 3 bf16, on the device of `like`
 PyObject* py_empty(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -20,8 +32,8 @@ PyObject* py_empty(PyObject*, PyObject* const* a, Py_ssize_t n) {
     sizes[i - 2] = PyLong_AsLongLong(a[i]);
     if (sizes[i - 2] == -1 && PyErr_Occurred()) return nullptr;
   }
-  const at::Tensor& like = THPVariable_Unpack(a[0]);
-  return THPVariable_Wrap(at::empty(at::IntArrayRef(sizes, n - 2), at::TensorOptions().dtype(kinds[kind]).device(like.device())));
+  const auto options = at::TensorOptions().dtype(kinds[kind]).device(THPVariable_Unpack(a[0]).device());
+  return THPVariable_Wrap(without_lock([&] { return at::empty(at::IntArrayRef(sizes, n - 2), options); }));
   END_HANDLE_TH_ERRORS
 }
 
@@ -30,8 +42,9 @@ PyObject* py_empty_as(PyObject*, PyObject* like) {
   HANDLE_TH_ERRORS
   TORCH_CHECK_TYPE(THPVariable_Check(like), "expected a tensor");
   const at::Tensor& t = THPVariable_Unpack(like);
-  return THPVariable_Wrap(
-      at::empty_strided(t.sizes(), t.strides(), at::TensorOptions().dtype(at::kBFloat16).device(t.device())));
+  const at::DimVector sizes(t.sizes()), strides(t.strides());      // (another thread may change the tensor meanwhile)
+  const auto options = at::TensorOptions().dtype(at::kBFloat16).device(t.device());
+  return THPVariable_Wrap(without_lock([&] { return at::empty_strided(sizes, strides, options); }));
   END_HANDLE_TH_ERRORS
 }
 
