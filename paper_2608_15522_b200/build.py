@@ -12,6 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libavsa.so")
 HOST = os.path.join(HERE, "_avsa_host" + sysconfig.get_config_var("EXT_SUFFIX"))      # marshalling for this interpreter
 ALLOC = os.path.join(HERE, "_avsa_alloc" + sysconfig.get_config_var("EXT_SUFFIX"))    # tensors for the wrappers
+ALLOC_FOR = os.path.join(HERE, "build", "alloc_built_for.txt")      # the PyTorch that ALLOC was compiled against
 SOURCES = ["api.cu", "mask.cu", "sparse_attn.cu", "cross_attn.cu", "protected_rows.cu", "cache_indicators.cu"]
 HEADERS = sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")) + [os.path.join("..", "..", "include", "avsa.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -25,10 +26,19 @@ def _nvcc() -> str:
     return exe
 
 
+def _torch_abi() -> str:
+    """What the allocating extension is bound to besides its source."""
+    import torch
+    return f"torch {torch.__version__} cxx11 abi {int(torch.compiled_with_cxx11_abi())}"
+
+
 def _stale() -> bool:
     outputs = (LIB, HOST, ALLOC)
-    if not all(os.path.exists(o) for o in outputs):
+    if not all(os.path.exists(o) for o in outputs + (ALLOC_FOR,)):
         return True
+    with open(ALLOC_FOR) as f:
+        if f.read() != _torch_abi():
+            return True
     t = min(os.path.getmtime(o) for o in outputs)
     deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["host_call.cc", "host_alloc.cc"]]
     return any(os.path.getmtime(p) > t for p in deps)
@@ -78,6 +88,8 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         out, _ = pr.communicate()
         if pr.returncode != 0:
             raise RuntimeError(f"g++ failed on {name}:\n{out}")
+    with open(ALLOC_FOR, "w") as f:
+        f.write(_torch_abi())
     return LIB
 
 
