@@ -66,28 +66,24 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     nvcc = _nvcc()
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
-    host_procs = _start_host_builds()
-    procs = []
+    procs = []      # (source, object or None, process), all at once
+    for name, pr in _start_host_builds():
+        procs.append((name, None, pr))
     for s in SOURCES:
         obj = os.path.join(objdir, s.replace(".cu", ".o"))
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", os.path.join(CSRC, s), "-o", obj]
         procs.append((s, obj, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    objs = []
-    for s, obj, pr in procs:
-        out, _ = pr.communicate()
-        if verbose and out:
+    outputs = [pr.communicate()[0] for _, _, pr in procs]      # (all of them end before the first failure is reported)
+    for (name, obj, pr), out in zip(procs, outputs):
+        if verbose and out and obj is not None:
             print(out)
         if pr.returncode != 0:
-            raise RuntimeError(f"nvcc failed on {s}:\n{out}")
-        objs.append(obj)
+            raise RuntimeError(f"{'g++' if obj is None else 'nvcc'} failed on {name}:\n{out}")
+    objs = [obj for _, obj, _ in procs if obj is not None]
     cmd = [nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"]
     r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}")
-    for name, pr in host_procs:
-        out, _ = pr.communicate()
-        if pr.returncode != 0:
-            raise RuntimeError(f"g++ failed on {name}:\n{out}")
     with open(ALLOC_FOR, "w") as f:
         f.write(_torch_abi())
     return LIB
