@@ -9,24 +9,32 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-static EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
+typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
+
+struct DriverFns {
+  EncodeTiledFn encode = nullptr;
+  CtxGetCurrentFn current = nullptr;
+};
+
+static const DriverFns& driver_fns() {
+  static DriverFns fns;
   static std::once_flag once;
   std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess) {
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
+    auto get = [](const char* name) -> void* {
+      void* p = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      return cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess ? p : nullptr;
+    };
+    fns.encode = reinterpret_cast<EncodeTiledFn>(get("cuTensorMapEncodeTiled"));
+    fns.current = reinterpret_cast<CtxGetCurrentFn>(get("cuCtxGetCurrent"));
   });
-  return fn;
+  return fns;
 }
 
 bool encode_bf16_tile_map(CUtensorMap* map, const void* ptr, int B, int H, int N, int d, int64_t stride_b,
                           int64_t stride_h, int64_t stride_n, int box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return false;
+  const DriverFns& fns = driver_fns();
+  if (fns.encode == nullptr || fns.current == nullptr) return false;
   // A dimension of extent 1 never has its stride used for addressing, but the encoder still wants a
   // multiple of 16 bytes; give it a harmless one.
   const int64_t sn = stride_n;
@@ -39,12 +47,15 @@ bool encode_bf16_tile_map(CUtensorMap* map, const void* ptr, int B, int H, int N
   cuuint32_t box[4] = {64u, static_cast<cuuint32_t>(box_rows), 1u, 1u};
   cuuint32_t elem[4] = {1u, 1u, 1u, 1u};
   auto encode = [&] {
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, elem,
+    return fns.encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, elem,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
   if (encode()) return true;
-  // A host thread whose first CUDA call this is has no context yet: the runtime makes one current with the device.
+  // A host thread whose first CUDA call this is has no context yet: the runtime makes one current with the device.  (A thread that
+  // has one keeps it: then the map itself was refused.)
+  CUcontext ctx = nullptr;
+  if (fns.current(&ctx) == CUDA_SUCCESS && ctx != nullptr) return false;
   int dev = 0;
   return cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && encode();
 }

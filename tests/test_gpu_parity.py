@@ -1253,6 +1253,35 @@ def test_a_refused_launch_fails_its_own_call_only():
     assert (out[0, :5] == 0.0).all() and out[0, 5] == 1.0
 
 
+def test_a_refused_tensor_map_leaves_the_thread_its_context():
+    """A head stride that no tensor map can hold is refused on the host with nothing enqueued; a thread that works in a context of its
+    own still does so afterwards."""
+    import ctypes
+    import threading
+    driver = ctypes.CDLL("libcuda.so.1")
+    lib = av.load_library()
+    t = torch.zeros((2, 64, 64), dtype=torch.bfloat16, device="cuda")
+    lse, ws = torch.empty((2, 64), device="cuda"), torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    device = t.device.index
+    seen = {}
+
+    def work():
+        own, current, dev = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_int()
+        assert driver.cuDeviceGet(ctypes.byref(dev), device) == 0
+        assert driver.cuCtxCreate_v2(ctypes.byref(own), 0, dev) == 0      # (and makes it current)
+        far = av._Bf16Tensor4(t.data_ptr(), 0, 1 << 40, 64)
+        seen["status"] = lib.avsa_cross_attn_scores(1, 2, 64, 64, 64, far, far, far, None, lse.data_ptr(), None, 0.0, 1.0, 0.0,
+                                                    ws.data_ptr(), ws.numel(), None)
+        assert driver.cuCtxGetCurrent(ctypes.byref(current)) == 0
+        seen["kept"] = current.value == own.value
+        assert driver.cuCtxDestroy_v2(own) == 0
+
+    thread = threading.Thread(target=work)
+    thread.start()
+    thread.join()
+    assert seen == {"status": av.AVSA_ERR_CUDA, "kept": True}
+
+
 @pytest.mark.parametrize("growth", [0.0, 4.0])
 def test_cross_attention_queue_with_its_end_cut(growth):
     """240 heads x 4 query tiles x 29 key tiles: long enough for the queue, whose last units are cut in two.  Whole query
