@@ -532,15 +532,15 @@ def test_cross_attention_outputs_and_scores(name):
     assert torch.equal(s, s3)
 
 
-def test_cross_attention_long_query_axis_two_chunks():
-    """More than 256 queries: the column-sum pass splits the query axis in two."""
+def test_cross_attention_long_query_axis_in_chunks():
+    """More than 256 queries: the column-sum pass splits the query axis in four."""
     w = wl.Workload("x", 1, 2, 128, 2, 9, 17, 300, 128, 50, 10, 1.0, ((0, 1, 1, 3, 2, 4),))
     (qa, kc, vc), want_o, want_lse, want_s = _oracle_scores(w, 7)
     o, lse, s, ws = av.avsa_cross_attn_scores(qa.cuda(), kc.cuda(), vc.cuda(), score_gamma=1.0 / (w.H * w.n_audio))
     _status_ok(ws)
     _close(_np64(o), want_o, "cross O")
     _close_lse(_np64(lse), want_lse, "cross lse")
-    _close_scores(_np64(s), want_s, "scores, two query chunks")
+    _close_scores(_np64(s), want_s, "scores, four query chunks")
 
 
 @pytest.mark.parametrize("B,H,Nq,Nk,d,scores", [
@@ -548,17 +548,26 @@ def test_cross_attention_long_query_axis_two_chunks():
     (1, 1, 600, 3000, 128, False),     # 5 query tiles in chunks of 4, 24 key tiles cut into twelve ranges
     (1, 2, 300, 2900, 128, True),      # 3 query tiles, split rows, the LSEs of the score pass from the parts
     (2, 3, 140, 333, 64, True),        # few tiles: whole rows, written by the tile kernel itself
-    (1, 22, 2427, 200, 128, True),     # reverse: 19 query tiles in chunks of 4, whole rows, score pass over the keys
+    (1, 22, 2427, 200, 128, True),     # few keys: both passes in one kernel, 418 query tiles over the CTAs
+    (1, 22, 2427, 300, 128, True),     # reverse: 19 query tiles, score pass with three key tiles resident
+    (1, 22, 2427, 300, 64, True),
+    (2, 2, 600, 257, 64, True),        # reverse with one key in the last tile
+    (2, 2, 600, 257, 128, True),
+    (1, 4, 700, 385, 128, True),
+    (1, 2, 513, 512, 64, True),        # the fewest queries and the most keys of the reverse direction
+    (1, 3, 1000, 512, 128, True),
     (1, 2, 130, 6400, 64, True),
     (1, 100, 40, 1000, 64, True),      # score pass: 800 key tiles cut evenly through the heads
     (1, 96, 300, 520, 128, True),      # the same with the queries in four chunks
-    (1, 3, 128, 700, 64, True),        # one chunk, tiles by turns over four groups
-    (1, 3, 129, 650, 128, True),       # two chunks of 80
+    (1, 3, 128, 700, 64, True),        # one chunk, tiles by turns over two groups
+    (1, 3, 129, 650, 128, True),       # one chunk of 144
     (1, 2, 256, 515, 128, True),
     (1, 2, 257, 900, 64, True),        # four chunks of 80
     (2, 2, 512, 640, 128, True),
     (1, 1, 100, 6400, 64, True),       # a row in more parts than lanes take at once (50 of 16 and, below, of 32)
     (1, 1, 130, 6400, 128, True),
+    (1, 1, 100, 17000, 64, True),      # more parts (133 and, with as many as there are SMs, 148) than the merge's table of weights holds
+    (1, 1, 100, 18900, 128, True),
     (1, 40, 400, 900, 64, True),       # more than 8192 split rows
     (1, 20, 500, 1700, 128, True),
 ])
@@ -688,7 +697,7 @@ def test_cross_attention_row_maxima_growing_along_the_key_axis(reverse):
     w = dataclasses.replace(wl.WORKLOADS["medium128"], H=12)      # forward: 24 query tiles -> key splits of 3 tiles
     qa, kc, vc = wl.make_cross_qkv(w, 3)
     if reverse:
-        qa, kc, vc = kc, torch.cat([qa, qa, qa], dim=2), torch.cat([qa, qa, qa], dim=2).flip(2)   # 2070 queries, 216 keys
+        qa, kc, vc = kc, torch.cat([qa] * 5, dim=2), torch.cat([qa] * 5, dim=2).flip(2)   # 2070 queries, 360 keys
     u = 1.0 / np.sqrt(w.d)
     qa = (qa.float() + 8.0 * u).to(torch.bfloat16)
     nk = kc.shape[2]
@@ -1201,10 +1210,12 @@ def test_mask_select_over_row_lengths(NB):
 
 @pytest.mark.parametrize("reverse", [False, True])
 def test_host_threads_with_short_and_long_axes_do_not_disturb_each_other(reverse):
-    """Two host threads, each with its stream, buffers and shape: the score pass needs 100 to 227 KB of shared memory, by the
-    length of the axis that stays on chip, and no call may fail because of what the other thread's last one asked for."""
+    """Two host threads, each with its stream, buffers and shape: both run the same score pass (272 and 512 queries the one with
+    four reduction groups, 272 and 512 keys the reverse one), which needs more or less shared memory by the length of the axis
+    that stays on chip (210 and 226 KB; 195 and 227 KB), and no call may fail because of what the other thread's last one asked
+    for."""
     import threading
-    shapes = ((16, 600), (512, 600))      # (short axis, long axis)
+    shapes = ((272, 600), (512, 600))      # (short axis, long axis)
     inputs, want = [], []
     for n_short, n_long in shapes:
         g = torch.Generator(device="cuda").manual_seed(n_short)
