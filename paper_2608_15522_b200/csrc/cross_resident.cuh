@@ -105,7 +105,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
       mbar_init(BAR(Q_EMPTY + s), 1);
       mbar_init(BAR(S_FULL + s), 1);
       mbar_init(BAR(S_FREE + s), 128);
-      mbar_init(BAR(P_FULL + 2 * s), 128);
+      mbar_init(BAR(P_FULL + 2 * s), KG == 2 && s == 0 ? 132 : 128);      // (the second group's warps release the first's P)
       mbar_init(BAR(P_FULL + 2 * s + 1), 128);
       mbar_init(BAR(FLUSH + s), 256);
     }
@@ -257,8 +257,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           const int nch = i == 0 ? p.nch0 : p.nch1, key0 = i * p.nch0 * 32;
           if (part == 1 && nch <= 2) continue;
           ok = wait_all(P_FULL + 2 * g + part, uses & 1, kResPFull, T);
-          // (the second group may rescale the first's P until it hands over the first part of its own)
-          if (ok && KG == 2 && part == 0 && i == 0) ok = wait_all(P_FULL + 2, uses & 1, kResPFull, T);
           if (!ok) break;
           tc_fence_after();
           // steps of 16 keys: of more than two chunks those behind the second come first
@@ -367,7 +365,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           // beyond it by more than 2^57.  Then the second takes the least reference 2^k times the first's (which makes a power of
           // two of the factor) beside which none of its probabilities exceeds 2^57.  So a row's sum is about 2^64 at most (128 keys
           // of 2^57): values of v up to 2^60 leave the accumulator of O finite.
-          // (Both groups waiting for both maxima, and taking the same reference: 142 -> 149 us, without scores 122 -> 133.)
+          // (us with / without scores, 256 keys: 142 / 121 this way, as without any of it; both groups waiting for both maxima and
+          // taking the same reference 149 / 133; the issuer waiting for the second group's first P 143 / 128.)
           if (w == 0) {
             exch[row] = m;
             mbar_arrive(BAR(MAX + quad));
@@ -383,6 +382,29 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
               m = ma;
             }
             exch[row] = m;      // (the first group has its own maximum in a register and reads this after the sums' barrier)
+            if (__any_sync(FULLM, first != 1.f)) {
+              // Rows with another reference: the first group's P in proportion, so that every key weighs what it should, however
+              // large its v is.  (The logits at hand are read again afterwards: nothing is held in registers across this.)
+              ok = wait_all(P_FULL + 1, T & 1, kResPFull, T);      // all of it is there
+              if (!ok) break;
+              tc_fence_after();
+#pragma unroll 1
+              for (int c = 0; c < 4; c++) {
+                uint32_t pk[16];
+                tmem_ld16(tmem + lane_off + TM_P + c * 16, pk);
+                tmem_wait_ld_regs(pk);
+#pragma unroll
+                for (int j = 0; j < 16; j++)
+                  pk[j] = pack_bf16x2(__uint_as_float(pk[j] << 16) * first, __uint_as_float(pk[j] & 0xffff0000u) * first);
+                tmem_st16(tmem + lane_off + TM_P + c * 16, pk);
+              }
+              tmem_wait_st();
+              tc_fence_before();
+              __syncwarp();
+              load_batch(nch > 2 ? 2 : 0);
+              max_batch(nch > 2 ? 2 : 0);
+            }
+            if (lane == 0) mbar_arrive(BAR(P_FULL));      // before this none of the first group's P is multiplied with V
           }
         }
         // ---- exponentials: P (bf16) for the second product, p (fp32) over the logits for the column sums
@@ -407,22 +429,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             tmem_st16(tm_p + (c0 + c) * 16, pk);
             if (SCORES) tmem_st32(tm_s + (c0 + c) * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
           }
-          if (upper && bar == P_FULL + 2 && __any_sync(FULLM, first != 1.f)) {
-            // Rows with another reference: the first group's P in proportion, before any of it is multiplied with V (the issuer
-            // waits for this hand-over first), so that every key weighs what it should, however large its v is.
-            for (int part = 0; part < 2 && ok; part++) ok = wait_all(P_FULL + part, T & 1, kResPFull, T);
-            if (!ok) return;
-            tc_fence_after();
-            for (int c = 0; c < 4; c++) {
-              uint32_t pk[16];
-              tmem_ld16(tmem + lane_off + TM_P + c * 16, pk);
-              tmem_wait_ld_regs(pk);
-#pragma unroll
-              for (int j = 0; j < 16; j++)
-                pk[j] = pack_bf16x2(__uint_as_float(pk[j] << 16) * first, __uint_as_float(pk[j] & 0xffff0000u) * first);
-              tmem_st16(tmem + lane_off + TM_P + c * 16, pk);
-            }
-          }
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(BAR(bar));
@@ -433,14 +439,12 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         };
         if (nch > 2) {      // the batch at hand first
           exp_batch(2, P_FULL + 2 * w);
-          if (!ok) break;
           load_batch(0);
           if (!SCORES) s_free();
           exp_batch(0, P_FULL + 2 * w + 1);
         } else {
           if (!SCORES) s_free();
           exp_batch(0, P_FULL + 2 * w);
-          if (!ok) break;
         }
         float lsum;
         {
