@@ -18,8 +18,8 @@ struct StatusRecord {
   int where;      // which wait / check
   int item;       // work item (block index)
   int aux;        // tile index or offending value
-  int redo_count; // attention calls: work items whose rows outgrew their reference and were recomputed exactly (with at most 256
-                  // keys of the cross-attention: given another reference)
+  int redo_count; // attention calls: work items whose rows outgrew their reference and were recomputed exactly (cross-attention
+                  // against at most 256 keys: query tiles in which the keys from 128 on outgrew the first ones' maximum by 2^64)
   int next_item;  // attention calls: head of the work queue of the persistent kernel
 };
 constexpr size_t kStatusBytes = 256;   // the record, padded so that what follows stays 256-byte aligned

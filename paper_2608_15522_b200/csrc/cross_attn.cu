@@ -134,8 +134,8 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
     const int bh = pos / p.NKT, kt0 = pos % p.NKT, h = bh % p.H, b = bh / p.H;
     const int ntile = min(p.NKT - kt0, pos_end - pos);
     // negated log2-domain LSEs (one packed FMA then gives s*c - lse2); queries beyond Nq get -inf: exp2 = 0
-    // (straight from the partial LSEs of pass 1's key ranges: the same maximum-and-sum as in merge_splits_rows, so that
-    // nothing has to be merged between the passes)
+    // (straight from the partial LSEs of pass 1's key ranges: the maximum and sum of merge_splits_rows, added in the order of
+    // the parts, so that nothing has to be merged between the passes)
     // (warp 0 has no part in this: the first tiles and the queries are on their way meanwhile)
     for (int j = tid - 32; j < NCH * W; j += kThreads - 32) {
       if (warp == 0) break;
@@ -282,9 +282,9 @@ colsum_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ C
   }
   tc_fence_before();
   __syncthreads();
-  // Only now: CTAs of the next grid that are staged earlier share the SMs with this one's last ones.  Measured both ways, this /
-  // right after the wait, us: 32.9 / 33.3 (a layer-step of 256 tokens), 64.0 / 65.6 (2070 tokens, batch of two), 698 / 707
-  // (512 queries x 49152 keys, which fills all SMs), 254 / 259 (reverse direction).
+  // Only now: CTAs of the next grid that are staged earlier share the SMs with this one's last ones.  Measured both ways with two
+  // groups, this / right after the wait, us: 64.0 / 65.6 (a layer-step of 2070 tokens, 72 queries, batch of two), 698 / 707 (512
+  // queries x 49152 keys, which fills all SMs).
   pdl_launch();
   if (warp == 2) tmem_dealloc(tmem, 512);
 }
@@ -608,6 +608,10 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
   // Few keys: everything in one kernel, whatever the number of queries (faster from 2 heads x 32 queries to 64 x 19200, with scores
   // and without: cross_resident.cuh).  More than 256 keys of 128 channels do not fit an SM's shared memory beside the tiles, nor
   // their logits its tensor memory.  (Tiles are counted in 32 bits there; calls beyond that go the other way.)
+  // The CTAs' shares are fixed: one that starts late, because another stream's kernel holds its SM, brings its whole share with it.
+  // us with 0 / 1 / 2 / 4 / 8 / 16 / 32 SMs held, 24 heads x 32760 queries x 256 keys: 165 / 166 / 199 / 288 / 287 / 290 / 293 (two-tile
+  // items off a queue and the score pass behind them, with 0 / 4 / 8 / 16 / 32: 253 / 271 / 331 / 340 / 358); x 17856 x 160: 91 / 94 / 95 / 147 /
+  // 148 / 148 / 149 (162 / 174 / 207 / 207 / 223).
   const long long tiles = static_cast<long long>(B) * H * ((Nq + 127) / 128);
   if (Nk <= kResMaxKeys && tiles < (1ll << 30)) {
     c.resident = true;
@@ -623,8 +627,7 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
     return c;
   }
   // Tiles of 128 rows for both head sizes.  With 64 channels and 64-row tiles, half of the MMA's 128 rows held nothing,
-  // and every hand-over moved half as many keys (24 heads,
-  // 256 queries x 32760 keys with scores: 369 us; with these tiles 162; reverse direction 342 -> 212).
+  // and every hand-over moved half as many keys (24 heads, 256 queries x 32760 keys with scores: 369 us; with these tiles 162).
   c.blk = 128;
   c.NQT = (Nq + c.blk - 1) / c.blk;
   c.NKB = (Nk + c.blk - 1) / c.blk;
@@ -806,9 +809,9 @@ static int run_cross(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const 
     if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
     if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
     const int smem = L::total(c.NKT);
-    // always the same limit (four key tiles), whatever this call needs: the limit belongs to the kernel, and a host thread
-    // with fewer keys must not lower it between another thread's setting and launch
-    constexpr int kMaxSmem = 232448;      // always the same limit, as above
+    // always the same limit, whatever this call needs: the limit belongs to the kernel, and a host thread with fewer keys must
+    // not lower it between another thread's setting and launch
+    constexpr int kMaxSmem = 232448;
     if (cudaFuncSetAttribute(colsum_rev_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
       return AVSA_ERR_CUDA;
     ColsumRevParams rp;

@@ -10,9 +10,9 @@
 //   What bounds it: a tile's phases follow one another in the softmax warps (24 heads x 32760 queries x 256 keys, cycles a
 // tile: logits and maximum 700, exponentials 2330, which is the MUFU's rate, row sums 200-500, column sums 850, O 1000, waits
 // for S 350-800), because tensor memory holds one tile (KG = 2).  Against the calls that it replaces (attention over two-tile
-// items 160 us, LSE conversion 5, S^T and its exponentials again 70, head sum 4): 255 -> 159 us; 100 keys 223 -> 80;
+// items 160 us, LSE conversion 5, S^T and its exponentials again 70, head sum 4): 255 -> 161 us; 100 keys 223 -> 80;
 // 24 keys of 64 channels, 32 heads x 49152 queries 382 -> 93; 8 heads x 2070 x 72 keys 19.4 -> 10.3; 2 heads x 32 queries x 256
-// keys 13.8 -> 8.3.  Without scores (256 keys) 157 -> 124.
+// keys 13.8 -> 8.3.  Without scores (256 keys) 157 -> 121.
 //
 //   warp 0      TMA producer: K and V of a head once, query tiles through a two-slot ring
 //   warp 1      MMA issuer: S = Q K^T (by key group), O = P V (P in tensor memory)
