@@ -621,8 +621,8 @@ def test_cross_attention_few_keys(B, H, Nq, Nk, d):
 
 @pytest.mark.parametrize("step", [30.0, 80.0])
 def test_cross_attention_few_keys_that_outgrow_their_reference(step):
-    """The keys from 128 on have logits larger by 30 nats (43 in base 2: still relative to the first ones' maximum) or 80 (115: the
-    rows take another reference, and their tiles are counted)."""
+    """The keys from 128 on have logits larger by 30 nats (43 in base 2, up to 62 in some rows: not counted, and most rows stay
+    relative to the first ones' maximum) or 80 (115: the rows take another reference, and their tiles are counted)."""
     B, H, Nq, Nk, d = 1, 3, 300, 200, 128
     g = torch.Generator().manual_seed(9)
     q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, Nk, Nk))
