@@ -726,6 +726,15 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
   }
 }
 
+template <int BLK, int D, int MODE>
+inline bool launch_redo(int grid, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                        const CUtensorMap& to, const AttnParams& prm, int* redo) {
+  constexpr int kExactSmem = AttnSmem<BLK, D>::kTotal;
+  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kExactSmem) != cudaSuccess)
+    return false;
+  return launch_pdl(attn_redo_kernel<BLK, D, MODE>, grid, kAttnThreads, kExactSmem, st, tq, tk, tv, to, prm, redo) == cudaSuccess;
+}
+
 // The persistent kernel and, unless it recomputes its items itself, the redo grid behind it.
 template <int BLK, int D, int MODE>
 inline bool launch_attention(int grid, bool fold, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
@@ -735,11 +744,7 @@ inline bool launch_attention(int grid, bool fold, cudaStream_t st, const CUtenso
   auto kernel = fold ? attn_persist_kernel<BLK, D, MODE, true> : attn_persist_kernel<BLK, D, MODE, false>;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal) != cudaSuccess) return false;
   if (launch_pdl(kernel, grid, kAttnThreads, L::kTotal, st, tq, tk, tv, to, prm, redo, order, n_items) != cudaSuccess) return false;
-  if (fold) return true;
-  constexpr int kExactSmem = AttnSmem<BLK, D>::kTotal;
-  if (cudaFuncSetAttribute(attn_redo_kernel<BLK, D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kExactSmem) != cudaSuccess)
-    return false;
-  return launch_pdl(attn_redo_kernel<BLK, D, MODE>, grid, kAttnThreads, kExactSmem, st, tq, tk, tv, to, prm, redo) == cudaSuccess;
+  return fold || launch_redo<BLK, D, MODE>(grid, st, tq, tk, tv, to, prm, redo);
 }
 
 }  // namespace avsa

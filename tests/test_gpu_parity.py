@@ -504,6 +504,68 @@ def test_sparse_attention_list_lengths(heads, bad):
     _close(_np64(o), want, "list lengths O")
 
 
+@pytest.mark.parametrize("case", ["random", "nothing_shared", "first_blocks_swapped", "dense_beside_short", "outgrown", "nan_value",
+                                  "both_malformed", "window"])
+def test_sparse_attention_pairs_of_64_blocks(case):
+    """Query blocks of 64 rows are taken two at a time with the union of their lists: an odd number of blocks (the last pair has one
+    block, of 9 rows), lists that share nothing or begin elsewhere, a block that one of a pair does not list and whose values are no
+    numbers, rows that outgrow their reference in one block of a pair, a pair without a list, and more than the 1024 key blocks that
+    are joined at a time."""
+    B, H, NB, d = (1, 1, 1061, 64) if case == "window" else (1, 5, 35, 64)
+    N = (NB - 1) * d + 9
+    g = torch.Generator().manual_seed(3)
+    q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    rng = np.random.default_rng(11)
+    idx = np.full((B, H, NB, NB), -1, np.int32)
+    cnt = np.zeros((B, H, NB), np.int32)
+    for h in range(H):
+        for i in range(NB):
+            cols = rng.choice(NB, size=1 + int(rng.integers(6)) if case == "window" else 1 + int(rng.integers(NB)), replace=False)
+            if case == "window":
+                cols = np.union1d(cols, [[0, 1023, 1024], [1024], [1060], [1023]][i % 4])
+            elif case == "nothing_shared":
+                cols = np.arange(i % 2, NB, 2 + i % 3 * 2)
+            elif case == "first_blocks_swapped":
+                cols = np.arange(7 + i % 5 if i % 4 in (0, 3) else i % 5, NB)
+            elif case == "dense_beside_short":
+                cols = np.arange(NB) if (i // 2) % 2 == i % 2 else np.array([(5 * i) % NB])
+            elif case == "nan_value":
+                cols = np.union1d(cols[cols != 7], [0] if i != 8 else [7])
+            cols = np.sort(cols)
+            idx[0, h, i, : len(cols)], cnt[0, h, i] = cols, len(cols)
+    if case == "outgrown":      # keys that grow from block to block, for the rows of every other block of a pair
+        q[:, :, (torch.arange(N) // d) % 2 == 1] *= 0.01
+        k = (k.float() * (1 + 3 * (torch.arange(N) // d))[None, None, :, None]).to(torch.bfloat16)
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), idx, cnt, d)
+    if case == "nan_value":
+        v[:, :, 7 * d : 8 * d] = float("nan")
+        want[:, :, 8 * d : 9 * d] = 7.0
+    if case == "both_malformed":
+        cnt[0, 2, 10], cnt[0, 2, 11] = 0, NB + 1
+        want[0, 2, 10 * d : 12 * d] = want_l[0, 2, 10 * d : 12 * d] = 7.0
+    o = torch.full((B, H, N, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((B, H, N), 7.0, device="cuda")
+    _, _, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), d,
+                                        want_lse=True, o=o, lse=lse)
+    code, detail = av.avsa_read_status(ws)
+    if case == "both_malformed":
+        assert code == av.AVSA_ERR_BAD_MASK and detail[1] in (2 * NB + 10, 2 * NB + 11)
+    else:
+        assert code == av.AVSA_OK
+    got = _np64(o)
+    n_redo, items = av.avsa_sparse_self_attn_redo_items(ws)
+    if case == "nan_value":
+        assert np.all(np.isnan(got[:, :, 8 * d : 9 * d]))      # these rows list the block
+        got[:, :, 8 * d : 9 * d] = 7.0
+    elif case == "outgrown":
+        assert n_redo > 0 and len(set(items.tolist())) == n_redo and np.all(cnt.reshape(-1)[items] > 1)
+        assert np.all(items % NB % 2 == 0)
+    else:
+        assert n_redo == 0
+    _close(got, want, f"pairs {case} O")
+    _close_lse(_np64(lse), want_l, f"pairs {case} lse")
+
+
 # ------------------------------------------------------------------------------------------- cross attention
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_outputs_and_scores(name):
