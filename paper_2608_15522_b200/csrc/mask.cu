@@ -108,80 +108,58 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// Adds one warp's digits to a shared-memory histogram.  When every participating lane holds the same
-// digit (the usual case for the leading byte of like-signed scores) one lane adds the whole count;
-// otherwise each lane adds its own (the hardware serialises only lanes that really collide).
-__device__ __forceinline__ void warp_hist_add(int* bins, bool in, uint32_t dgt, int lane) {
-  const unsigned inmask = __ballot_sync(0xffffffffu, in);
-  if (inmask == 0u) return;
-  const int leader = __ffs(inmask) - 1;
-  const uint32_t d0 = __shfl_sync(0xffffffffu, dgt, leader);
-  const bool uniform = __all_sync(0xffffffffu, !in || dgt == d0);
-  if (uniform) {
-    if (lane == leader) atomicAdd(&bins[d0], __popc(inmask));
-  } else if (in) {
-    atomicAdd(&bins[dgt], 1);
-  }
-}
-
 // ------------------------------------------------------------------------------------------------
-// Radix-select helper: given 256 digit counts (descending scan), find the digit that holds the
-// want-th largest element.  One warp; lane l owns digits 255-8l .. 248-8l.
-// ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void warp_pick_digit(const int* bins, int want, int lane, int& digit, int& above,
-                                                int& in_bin) {
-  int local[8];
-  int sum = 0;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    local[i] = bins[255 - (lane * 8 + i)];
-    sum += local[i];
-  }
-  int incl = sum;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    int t = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += t;
-  }
-  const int excl = incl - sum;
-  const bool mine = (excl < want) && (want <= incl);
-  int dg = 0, ab = 0, ib = 0;
-  if (mine) {
-    int run = excl;
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-      if (run < want && want <= run + local[i]) {
-        dg = 255 - (lane * 8 + i);
-        ab = run;
-        ib = local[i];
-      }
-      run += local[i];
-    }
-  }
-  const unsigned who = __ballot_sync(0xffffffffu, mine);
-  const int src = __ffs(who) - 1;
-  digit = __shfl_sync(0xffffffffu, dg, src);
-  above = __shfl_sync(0xffffffffu, ab, src);
-  in_bin = __shfl_sync(0xffffffffu, ib, src);
-}
-
-// ------------------------------------------------------------------------------------------------
-// (iii) protected token set: one CTA of 1024 threads per batch item.  The canonical keys are staged
-// in shared memory once (global memory is re-read instead when they do not fit); a radix select
-// (4 x 8 bits, warp-aggregated histogram) finds the n_protect-th largest key; then every warp walks
-// its own contiguous segment in index order, taking every larger key and the lowest-index ties,
-// writes the token flags and raises the flag of every block that holds one.  Block 0 also resets
-// the status record of the call.
+// (iii) protected token set: one CTA per batch item.  The canonical keys are staged in shared memory once (global memory is re-read
+// instead when they do not fit).  The n_protect-th largest is found by histograms of 512 equal bins, the first over the range that the
+// keys really span, the next over the bin that holds it, until every key of the bin is taken or it is one value wide; scores are
+// spread over such bins, so that two passes are the rule and few lanes meet in a counter.  Then every warp walks its own
+// contiguous segment in index order, taking every larger key and the lowest-index ties, and writes the flags of the tokens, four a
+// lane, and of the blocks that hold enough of them.  Block 0 also resets the status record of the call.
+//   Bound by one CTA's passes, above all by the counters of the first histogram.  us for the mask call where pooling does not cover the
+// select, against digits of eight bits with one key a lane and vote: 2 heads x 18600 tokens 35.0 -> 27.7, x 49152 71 -> 52; 4 heads x 2070
+// 12.5 -> 11.4.
 // ------------------------------------------------------------------------------------------------
 constexpr int kSelectSmemKeys = 56 * 1024;   // 224 KB of keys at most
+constexpr int kSelectBins = 512;
+
+// Given the counts of the bins, the one that holds the want-th largest key, how many keys lie above it and in it.  One warp.
+__device__ __forceinline__ void warp_pick_bin(const int* bins, int want, int lane, int& bin, int& above, int& in_bin) {
+  constexpr int GROUPS = kSelectBins / 32;      // of 32 bins, from the largest keys down
+  int mine[GROUPS], run = 0, g_found = 0, g_above = 0;
+#pragma unroll
+  for (int g = 0; g < GROUPS; g++) mine[g] = bins[kSelectBins - 1 - (g * 32 + lane)];
+#pragma unroll
+  for (int g = 0; g < GROUPS; g++) {
+    const int sum = __reduce_add_sync(0xffffffffu, mine[g]);
+    if (run < want && want <= run + sum) {
+      g_found = g;
+      g_above = run;
+    }
+    run += sum;
+  }
+  const int n = bins[kSelectBins - 1 - (g_found * 32 + lane)];
+  int incl = n;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += t;
+  }
+  const int excl = g_above + incl - n;
+  const int src = __ffs(__ballot_sync(0xffffffffu, excl < want && want <= excl + n)) - 1;
+  bin = kSelectBins - 1 - (g_found * 32 + src);
+  above = __shfl_sync(0xffffffffu, excl, src);
+  in_bin = __shfl_sync(0xffffffffu, n, src);
+}
 
 template <bool STAGED, int THREADS>
 __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const float* __restrict__ scores, int N, int n_protect, int blk,
                                               int NB, int min_tokens, uint8_t* __restrict__ prot_tok,
                                               uint8_t* __restrict__ prot_blk, StatusRecord* status) {
   constexpr int WARPS = THREADS / 32;
-  __shared__ int bins[256];
-  __shared__ int s_digit, s_above, s_in_bin;
+  constexpr unsigned FULLM = 0xffffffffu;
+  __shared__ int bins[kSelectBins];
+  __shared__ uint32_t warp_min[WARPS], warp_max[WARPS];
+  __shared__ int s_bin, s_above, s_in_bin;
   __shared__ int warp_cnt[WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* s = scores + static_cast<int64_t>(b) * N;
@@ -193,77 +171,138 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
     status->item = 0;
     status->aux = 0;
   }
-  for (int i = tid; i < NB; i += THREADS) pblk[i] = 0;
   if (n_protect <= 0) {
+    for (int i = tid; i < NB; i += THREADS) pblk[i] = 0;
     for (int i = tid; i < N; i += THREADS) ptok[i] = 0;
     return;
   }
-  if (STAGED) {
-#pragma unroll 8
-    for (int i = tid; i < N; i += THREADS) skeys[i] = rank_key(__ldg(s + i));
+  // four keys from index i (a multiple of four) on; how many of them there are
+  auto load4 = [&](int i, uint32_t (&k)[4]) -> int {
+    const int n = min(4, N - i);
+    if (STAGED) {
+      const uint4 v = *reinterpret_cast<const uint4*>(skeys + i);      // (the last four may end in unused memory)
+      k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; j++) k[j] = j < n ? rank_key(__ldg(s + i + j)) : 0u;
+    }
+    return n;
+  };
+  // ---- the keys, and the range that they span
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  constexpr int U = THREADS == 1024 ? 16 : 2;      // loads in flight
+  for (int i0 = tid; i0 < N; i0 += THREADS * U) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) v[u] = i0 + u * THREADS < N ? __ldg(s + i0 + u * THREADS) : 0.f;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      if (i0 + u * THREADS >= N) break;
+      const uint32_t key = rank_key(v[u]);
+      if (STAGED) skeys[i0 + u * THREADS] = key;
+      kmin = min(kmin, key);
+      kmax = max(kmax, key);
+    }
   }
-  auto key_at = [&](int i) -> uint32_t { return STAGED ? skeys[i] : rank_key(__ldg(s + i)); };
-  uint32_t prefix = 0, mask = 0;
+  kmin = __reduce_min_sync(FULLM, kmin);
+  kmax = __reduce_max_sync(FULLM, kmax);
+  if (lane == 0) {
+    warp_min[warp] = kmin;
+    warp_max[warp] = kmax;
+  }
+  for (int i = tid; i < kSelectBins; i += THREADS) bins[i] = 0;
+  __syncthreads();
+  kmin = __reduce_min_sync(FULLM, warp_min[lane % WARPS]);
+  kmax = __reduce_max_sync(FULLM, warp_max[lane % WARPS]);
+  // ---- the n_protect-th largest key is one of [base, base + span]; `want` of those are taken
+  uint32_t base = kmin, span = kmax - kmin;
   int want = n_protect;
-  for (int pass = 0; pass < 4; pass++) {
-    const int shift = 24 - 8 * pass;
-    if (tid < 256) bins[tid] = 0;
-    __syncthreads();     // also orders the staging stores before the first reads
-    for (int i0 = 0; i0 < N; i0 += THREADS) {
-      const int i = i0 + tid;
-      const bool valid = i < N;
-      const uint32_t key = valid ? key_at(i) : 0u;
-      const bool in = valid && ((key & mask) == prefix);
-      warp_hist_add(bins, in, (key >> shift) & 255u, lane);
+  bool whole = want == N;        // all of them
+  while (!whole && span > 0) {
+    const int shift = max(0, 32 - __clz(span) - 9);
+    for (int i = 4 * tid; i < N; i += 4 * THREADS) {
+      uint32_t k[4];
+      const int n = load4(i, k);
+#pragma unroll
+      for (int j = 0; j < 4; j++)
+        if (j < n && k[j] - base <= span) atomicAdd(&bins[(k[j] - base) >> shift], 1);
     }
     __syncthreads();
     if (warp == 0) {
-      int dg, ab, ib;
-      warp_pick_digit(bins, want, lane, dg, ab, ib);
+      int bin, above, in_bin;
+      warp_pick_bin(bins, want, lane, bin, above, in_bin);
       if (lane == 0) {
-        s_digit = dg;
-        s_above = ab;
-        s_in_bin = ib;
+        s_bin = bin;
+        s_above = above;
+        s_in_bin = in_bin;
       }
     }
     __syncthreads();
     want -= s_above;
-    prefix |= static_cast<uint32_t>(s_digit) << shift;
-    mask |= 255u << shift;
-    const bool whole_bin = (s_in_bin == want);   // every key of the bin is taken: no need to refine further
+    whole = s_in_bin == want;
+    base += static_cast<uint32_t>(s_bin) << shift;
+    span = (1u << shift) - 1u;
+    if (whole || span == 0) break;
+    for (int i = tid; i < kSelectBins; i += THREADS) bins[i] = 0;
     __syncthreads();
-    if (whole_bin) break;
   }
-  const uint32_t T = prefix;     // the n_protect-th largest key; `want` ties at T are taken, lowest index first
-  // contiguous segment per warp, a whole number of blocks (blk is a multiple of 32), so that every block's
-  // count of protected tokens is known to one warp
+  // every key from `base` on is taken, or those above it and the first `want` of its own value
+  // contiguous segment per warp, a whole number of blocks (blk is 32, 64 or 128), so that a block's tokens are one step's of one warp
   const int seg = ((N + WARPS - 1) / WARPS + blk - 1) / blk * blk;
   const int lo = min(N, warp * seg), hi = min(N, lo + seg);
-  int eq_mine = 0;
-  for (int i0 = lo; i0 < hi; i0 += 32) {
-    const int i = i0 + lane;
-    eq_mine += __popc(__ballot_sync(0xffffffffu, i < hi && key_at(i) == T));
-  }
-  if (lane == 0) warp_cnt[warp] = eq_mine;
-  __syncthreads();
   int eq_seen = 0;
-  for (int w2 = 0; w2 < warp; w2++) eq_seen += warp_cnt[w2];
-  int in_block = 0;     // protected tokens of the block being walked
-  for (int i0 = lo; i0 < hi; i0 += 32) {
-    const int i = i0 + lane;
-    const bool valid = i < hi;
-    const uint32_t key = valid ? key_at(i) : 0u;
-    const bool gt = valid && key > T;
-    const bool eq = valid && key == T;
-    const unsigned eqm = __ballot_sync(0xffffffffu, eq);
-    const bool keep = gt || (eq && (eq_seen + __popc(eqm & ((1u << lane) - 1u))) < want);
-    eq_seen += __popc(eqm);
-    if (valid) ptok[i] = keep ? 1 : 0;
-    in_block += __popc(__ballot_sync(0xffffffffu, keep));
-    if ((i0 + 32) % blk == 0 || i0 + 32 >= hi) {          // last 32 tokens of the block (or of the sequence)
-      if (in_block >= min_tokens && lane == 0) pblk[i0 / blk] = 1;
-      in_block = 0;
+  if (!whole) {
+    int mine = 0;
+    for (int i = lo + 4 * lane; i < hi; i += 128) {
+      uint32_t k[4];
+      const int n = load4(i, k);
+#pragma unroll
+      for (int j = 0; j < 4; j++) mine += j < n && k[j] == base ? 1 : 0;
     }
+    mine = __reduce_add_sync(FULLM, mine);
+    if (lane == 0) warp_cnt[warp] = mine;
+    __syncthreads();
+    eq_seen = __reduce_add_sync(FULLM, lane < warp ? warp_cnt[lane % WARPS] : 0);
+  }
+  const bool words = (reinterpret_cast<uintptr_t>(ptok) & 3u) == 0u;
+  const int group = blk / 4;      // lanes that hold a block
+  const unsigned group_mask = (group == 32 ? FULLM : (1u << group) - 1u) << (lane / group * group);
+  for (int i0 = lo; i0 < hi; i0 += 128) {
+    const int i = i0 + 4 * lane;
+    uint32_t k[4] = {0u, 0u, 0u, 0u};
+    const int n = i < hi ? load4(i, k) : 0;
+    bool keep[4];
+    if (whole) {
+#pragma unroll
+      for (int j = 0; j < 4; j++) keep[j] = j < n && k[j] >= base;
+    } else {
+      unsigned before = 0, total = 0;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const unsigned m = __ballot_sync(FULLM, j < n && k[j] == base);
+        before += __popc(m & ((1u << lane) - 1u));
+        total += __popc(m);
+      }
+      int rank = eq_seen + static_cast<int>(before);
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const bool eq = j < n && k[j] == base;
+        keep[j] = j < n && (k[j] > base || (eq && rank < want));
+        rank += eq ? 1 : 0;
+      }
+      eq_seen += static_cast<int>(total);
+    }
+    if (words && n == 4) {
+      *reinterpret_cast<uint32_t*>(ptok + i) = (keep[0] ? 1u : 0u) | (keep[1] ? 0x100u : 0u) | (keep[2] ? 0x10000u : 0u) | (keep[3] ? 0x1000000u : 0u);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; j++)
+        if (j < n) ptok[i + j] = keep[j] ? 1 : 0;
+    }
+    int in_block = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) in_block += __popc(__ballot_sync(FULLM, keep[j]) & group_mask);
+    if (lane % group == 0 && i < hi) pblk[i / blk] = in_block >= min_tokens ? 1 : 0;
   }
 }
 
@@ -272,7 +311,7 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
                                                             int blk, int NB, int min_tokens,
                                                             uint8_t* __restrict__ prot_tok,
                                                             uint8_t* __restrict__ prot_blk, StatusRecord* status) {
-  extern __shared__ uint32_t skeys[];
+  extern __shared__ __align__(16) uint32_t skeys[];
   // nothing launched next on the stream depends on this kernel until the list emission, so let the
   // pooling kernel start right away (but not before this grid's own predecessors are done: pooling does not wait)
   pdl_wait();
@@ -292,7 +331,7 @@ __global__ void __launch_bounds__(256) select_pool_kernel(const __nv_bfloat16* _
                                                           const float* __restrict__ scores, int n_protect, int min_tokens,
                                                           uint8_t* __restrict__ prot_tok, uint8_t* __restrict__ prot_blk,
                                                           StatusRecord* status) {
-  extern __shared__ uint32_t skeys[];
+  extern __shared__ __align__(16) uint32_t skeys[];
   pdl_wait();
   pdl_launch();
   if (static_cast<int>(blockIdx.x) < B) {
@@ -590,7 +629,7 @@ __global__ void __launch_bounds__(256) expand_blocks_kernel(const uint8_t* __res
 // rows each): sixteen warps with one row each shorten a CTA's own latency chain, but the 512-thread CTAs, staged
 // while the pooling grid drains, took thread slots from its last CTAs and the call came out slower (0.118 against
 // 0.103 ms on the Ovi-class shape).
-template <int D, int KPL, int WARPS>
+template <int D, int KPL, int WARPS, int NT>
 static cudaError_t launch_score_select_as(cudaStream_t st, int B, int NB, const float* qbar, const float* kbar,
                                           float* bs, const uint8_t* pblk, int H, float scale, int k_keep, int pr, int pc,
                                           int32_t* col_idx, int32_t* col_cnt) {
@@ -686,7 +725,7 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
     if (n_protect > 0 &&
         launch_pdl(block_sum_kernel, dim3((NB + 7) / 8, B), 256, 0, st, scores, N, blk, NB, bsum) != cudaSuccess)
       return AVSA_ERR_CUDA;
-    const size_t key_bytes = static_cast<size_t>(NB) * sizeof(uint32_t);
+    const size_t key_bytes = align_up(static_cast<size_t>(NB) * sizeof(uint32_t), 16);
     if (!allow_select_smem()) return AVSA_ERR_CUDA;
     if (launch_pdl(token_select_kernel<true>, B, 1024, key_bytes, st, bsum, NB, n_protect, 32, (NB + 31) / 32, 1, pblk,
                    base + w.junk, static_cast<StatusRecord*>(ws)) != cudaSuccess)
@@ -694,7 +733,7 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   } else if (one_launch) {
     // (with the pooling, below)
   } else if (N <= kSelectSmemKeys) {
-    const size_t key_bytes = static_cast<size_t>(N) * sizeof(uint32_t);
+    const size_t key_bytes = align_up(static_cast<size_t>(N) * sizeof(uint32_t), 16);
     if (!allow_select_smem()) return AVSA_ERR_CUDA;
     if (launch_pdl(token_select_kernel<true>, B, 1024, key_bytes, st, scores, N, n_protect, blk, NB, min_tokens, ptok, pblk,
                    static_cast<StatusRecord*>(ws)) != cudaSuccess)
@@ -713,7 +752,7 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
     cudaError_t e;
     if (one_launch) {
       const unsigned grid = static_cast<unsigned>(B) * (1 + 2 * H * NB);
-      const size_t key_bytes = static_cast<size_t>(N) * sizeof(uint32_t);
+      const size_t key_bytes = align_up(static_cast<size_t>(N) * sizeof(uint32_t), 16);
       auto kernel = d == 128 ? select_pool_kernel<128> : select_pool_kernel<64>;
       e = launch_pdl(kernel, grid, 256, key_bytes, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b, k.stride_h,
                      k.stride_n, qbar, kbar, B, H, N, blk, NB, scores, n_protect, min_tokens, ptok, pblk, static_cast<StatusRecord*>(ws));

@@ -156,6 +156,38 @@ def test_mask_long_sequence_beyond_the_shared_memory_key_cache():
     assert np.array_equal(out["col_idx"].cpu().numpy(), idx)
 
 
+@pytest.mark.parametrize("n", [1, 3, 129, 511, 513, 4099, 57344, 57347])
+@pytest.mark.parametrize("kind", ["log_normal", "outliers", "constant", "two_values", "one_above", "signs"])
+def test_mask_token_select_over_ranges_of_scores(n, kind):
+    """The select's bins follow the range that the scores span: narrow and wide ranges, ranges stretched by infinities, one value, ties
+    at the edge, both signs; lengths around four tokens a lane, a CTA's step and the keys kept in shared memory; a second batch item
+    whose flags may begin at any byte."""
+    B, H, d, blk = 2, 1, 128, 128
+    NB = (n + blk - 1) // blk
+    rng = np.random.default_rng(n)
+    s = np.exp(0.3 * rng.standard_normal((B, n))).astype(np.float32)
+    if kind == "outliers":
+        s[0, 0], s[1, n // 2], s[1, n - 1] = np.inf, -np.inf, 1e-30
+    elif kind == "constant":
+        s[:] = 0.25
+    elif kind == "two_values":
+        s = np.where(s > 1.2, np.float32(3.0), np.float32(2.0))
+    elif kind == "one_above":
+        s = np.full((B, n), 1.0, np.float32)
+        s[:, n // 3] = np.nextafter(np.float32(1.0), np.float32(2.0))
+    elif kind == "signs":
+        s = rng.standard_normal((B, n)).astype(np.float32)
+    bs = np.zeros((B, H, NB, NB), np.float32)
+    for n_protect in sorted({1, (n + 19) // 20, n // 2 + 1, max(1, n - 1), n}):
+        _, _, ptok, pblk = orc.build_block_mask(bs, s, n_protect, 1, blk, n)
+        out = av.avsa_build_block_mask(None, None, torch.from_numpy(s).cuda(), n_protect, 1, blk,
+                                       flags=av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES,
+                                       block_scores=torch.from_numpy(bs).cuda(), shape=(B, H, n, d))
+        _status_ok(out["ws"])
+        assert np.array_equal(out["prot_tok"].cpu().numpy(), ptok), n_protect
+        assert np.array_equal(out["prot_blk"].cpu().numpy(), pblk), n_protect
+
+
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_block_scores_and_selection_from_pooled_qk(name):
     w = wl.WORKLOADS[name]
