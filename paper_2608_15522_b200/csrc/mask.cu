@@ -454,14 +454,17 @@ constexpr int kStripRows = 16;
 template <int D>
 __host__ __device__ constexpr int strip_pitch(int NB) { return (NB + 31) / 32 * 32 + 4; }
 
-template <int D, int KPL, int WARPS>
+// NT: 8-column MMA tiles a warp and pass, one to four, so that short rows occupy all warps too.  gridDim.z CTAs share a strip: each
+// computes its scores and takes its share of the rows through the select (two where that still leaves every CTA an SM).  us for the
+// mask call before -> with both: 4 heads x 17 blocks 11.4 -> 10.1, 24 x 17 11.9 -> 11.4, 2 x 146 27.7 -> 23.7, 2 x 384 52.1 -> 44.9.
+template <int D, int KPL, int WARPS, int NT>
 __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
                                                                   float* __restrict__ bs, const uint8_t* __restrict__ prot_blk,
                                                                   int H, int NB, float scale, int k_keep, int protect_rows,
                                                                   int protect_cols, int32_t* __restrict__ col_idx,
                                                                   int32_t* __restrict__ col_cnt) {
   constexpr int PITCH = D + 4;
-  constexpr int NT = 32 / WARPS;              // 8-column MMA tiles per warp and pass: 4 with 8 warps, 2 with 16
+  constexpr int TPH = NT < 2 ? NT : 2, HPG = NT / TPH;      // tiles of a half-step, half-steps of a 16-channel group
   constexpr int CHUNK = NT * 8;               // columns per warp and pass
   extern __shared__ __align__(16) float strip_smem[];
   uint32_t* sq_hi = reinterpret_cast<uint32_t*>(strip_smem);            // [16][PITCH] pooled queries of the strip,
@@ -469,7 +472,7 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   const int SP = strip_pitch<D>(NB);
   float* strip = strip_smem + 2 * kStripRows * PITCH;       // [16][SP] block scores of the strip
   float4* ring = reinterpret_cast<float4*>(strip + kStripRows * SP);    // [WARPS][4 slots][2 tiles][32 lanes]
-  static_assert(NT == 4, "the key ring holds two tile pairs per 16-channel group");
+  static_assert(NT == 1 || NT == 2 || NT == 4, "the key ring holds at most two tiles a half-step");
   // Staged behind the pooling grid (programmatic dependent launch) and waits for it here; the pooling grid in
   // turn retires only after the token select, so the block flags are final too.
   pdl_launch();
@@ -483,12 +486,12 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   // held): the pieces of three half-steps ahead are in flight under the MMAs of the current one, and the first
   // three of a warp's first chunk already under the load of the strip's queries.  A plain load per step left every
   // step waiting for its own L2 round trip (1500 cycles each, eight in a row).
-  constexpr int HS = (D / 16) * 2;            // half-steps: (16-channel group jg, tile pair hp)
+  constexpr int HS = (D / 16) * HPG;          // half-steps: (16-channel group jg, tile pair hp)
   const uint32_t ring_base = smem_u32_of(ring) + (warp * 4 * 2 * 32 + lane) * 16;
   auto issue = [&](int j0, int hs) {
-    const int jg = hs >> 1, hp = hs & 1;
+    const int jg = hs / HPG, hp = hs % HPG;
 #pragma unroll
-    for (int n2 = 0; n2 < 2; n2++) {
+    for (int n2 = 0; n2 < TPH; n2++) {
       const int col = j0 + (hp * 2 + n2) * 8 + g;
       const bool valid = col < NB;                          // beyond the last key block: zero fill
       const float* src = kb + static_cast<int64_t>(valid ? col : 0) * D + 4 * t + 16 * jg;
@@ -534,7 +537,7 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
     uint32_t ah[2][4], al[2][4];
 #pragma unroll
     for (int hs = 0; hs < HS; hs++) {
-      const int jg = hs >> 1, hp = hs & 1;
+      const int jg = hs / HPG, hp = hs % HPG;
       if (hs + 3 < HS) issue(j0, hs + 3);
       asm volatile("cp.async.commit_group;" ::: "memory");      // (an empty group near the end keeps the count uniform)
       asm volatile("cp.async.wait_group 3;" ::: "memory");       // the pieces of half-step hs have landed
@@ -550,8 +553,8 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
         al[1][0] = qal.z; al[1][1] = qcl.z; al[1][2] = qal.w; al[1][3] = qcl.w;
       }
 #pragma unroll
-      for (int n2 = 0; n2 < 2; n2++) {
-        const int ni = hp * 2 + n2;
+      for (int n2 = 0; n2 < TPH; n2++) {
+        const int ni = hp * TPH + n2;
         const float4 kvp = ring[(warp * 4 * 2 + (hs & 3) * 2 + n2) * 32 + lane];
         uint32_t bhh[2][2], bl[2][2];
         split_tf32(kvp.x, bhh[0][0], bl[0][0]);
@@ -577,11 +580,10 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   __syncthreads();
   const int b = bh / H;
   const uint8_t* pb = prot_blk + static_cast<int64_t>(b) * NB;
+  const int rows = kStripRows / static_cast<int>(gridDim.z), r_end = min(static_cast<int>(blockIdx.z + 1) * rows, NB - i0);
 #pragma unroll 1
-  for (int rr = 0; rr < kStripRows / WARPS; rr++) {
-    const int r = warp * (kStripRows / WARPS) + rr;
+  for (int r = blockIdx.z * rows + warp; r < r_end; r += WARPS) {
     const int qi = i0 + r;
-    if (qi >= NB) break;
     const int64_t row = static_cast<int64_t>(bh) * NB + qi;
     const float* src = strip + r * SP;
     float* dst = bs + row * NB;
@@ -637,23 +639,29 @@ static cudaError_t launch_score_select_as(cudaStream_t st, int B, int NB, const 
                              sizeof(float) + WARPS * 4 * 2 * 32 * 16;
   // always the same limit (the largest NB the call accepts), so concurrent callers never race on its value
   constexpr int kMaxSmem = (2 * kStripRows * (D + 4) + kStripRows * strip_pitch<D>(kMaxBlocksPerRow)) * 4 + WARPS * 4 * 2 * 32 * 16;
-  cudaError_t e = cudaFuncSetAttribute(score_select_kernel<D, KPL, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(score_select_kernel<D, KPL, WARPS, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMaxSmem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(score_select_kernel<D, KPL, WARPS>, dim3((NB + kStripRows - 1) / kStripRows, B * H, 1), WARPS * 32, smem, st,
+  const int strips = (NB + kStripRows - 1) / kStripRows;
+  const unsigned share = 2ll * strips * B * H <= persistent_grid(1 << 30) ? 2 : 1;
+  return launch_pdl(score_select_kernel<D, KPL, WARPS, NT>, dim3(strips, B * H, share), WARPS * 32, smem, st,
                     qbar, kbar, bs, pblk, H, NB, scale, k_keep, pr, pc, col_idx, col_cnt);
 }
 template <int D>
 static cudaError_t launch_score_select(cudaStream_t st, int B, int NB, const float* qbar, const float* kbar, float* bs,
                                        const uint8_t* pblk, int H, float scale, int k_keep, int pr, int pc,
                                        int32_t* col_idx, int32_t* col_cnt) {
+  if (NB <= 64)
+    return launch_score_select_as<D, 2, 8, 1>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+  if (NB <= 128)
+    return launch_score_select_as<D, 4, 8, 2>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   if (NB <= 256)
-    return launch_score_select_as<D, 8, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+    return launch_score_select_as<D, 8, 8, 4>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   if (NB <= 512)
-    return launch_score_select_as<D, 16, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+    return launch_score_select_as<D, 16, 8, 4>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
   if (NB <= 1024)      // (64 keys a lane are 230 registers, one CTA per SM)
-    return launch_score_select_as<D, 32, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
-  return launch_score_select_as<D, 64, 8>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+    return launch_score_select_as<D, 32, 8, 4>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
+  return launch_score_select_as<D, 64, 8, 4>(st, B, NB, qbar, kbar, bs, pblk, H, scale, k_keep, pr, pc, col_idx, col_cnt);
 }
 
 // The staged token select may use up to kSelectSmemKeys keys of dynamic shared memory.  The limit is always set
