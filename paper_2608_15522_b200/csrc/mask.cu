@@ -580,10 +580,12 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
   __syncthreads();
   const int b = bh / H;
   const uint8_t* pb = prot_blk + static_cast<int64_t>(b) * NB;
-  const int rows = kStripRows / static_cast<int>(gridDim.z), r_end = min(static_cast<int>(blockIdx.z + 1) * rows, NB - i0);
+  const int rows = kStripRows / static_cast<int>(gridDim.z), per = rows / WARPS;      // of the CTA, of a warp
 #pragma unroll 1
-  for (int r = blockIdx.z * rows + warp; r < r_end; r += WARPS) {
+  for (int rr = 0; rr < per; rr++) {
+    const int r = blockIdx.z * rows + warp * per + rr;
     const int qi = i0 + r;
+    if (qi >= NB) break;
     const int64_t row = static_cast<int64_t>(bh) * NB + qi;
     const float* src = strip + r * SP;
     float* dst = bs + row * NB;
