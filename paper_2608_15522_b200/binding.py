@@ -93,6 +93,20 @@ def _host():
     return _host_module
 
 
+def _alloc():
+    """The extension module that allocates tensors and takes plain tensors through a whole call, bound to the loaded library."""
+    global _alloc_module
+    if _alloc_module is None:
+        lib = load_library()
+        module = _extension("_avsa_alloc")
+        entries = ("avsa_cross_attn_scores", "avsa_build_block_mask", "avsa_sparse_self_attn", "avsa_protected_rows_attn")
+        address = lambda name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value
+        module.bind(*(address(e) for e in entries), *(address(e + "_workspace_bytes") for e in entries),
+                    getattr(torch._C, "_cuda_getCurrentRawStream", None))
+        _alloc_module = module
+    return _alloc_module
+
+
 def load_library() -> ctypes.CDLL:
     """Loads libavsa.so (built in-tree by ``build.py``) and declares the prototypes."""
     global _lib
@@ -179,20 +193,14 @@ def _empty(like, kind: int, *sizes) -> torch.Tensor:
     a plain tensor)."""
     if type(like) is not torch.Tensor:
         return torch.empty(sizes, dtype=_KINDS[kind], device=like.device)
-    global _alloc_module
-    if _alloc_module is None:
-        _alloc_module = _extension("_avsa_alloc")
-    return _alloc_module.empty(like, kind, *sizes)
+    return (_alloc_module or _alloc()).empty(like, kind, *sizes)
 
 
 def _empty_as(like) -> torch.Tensor:
     """An uninitialised bf16 tensor with the shape and strides of ``like``."""
     if type(like) is not torch.Tensor:
         return torch.empty_strided(like.shape, like.stride(), dtype=torch.bfloat16, device=like.device)
-    global _alloc_module
-    if _alloc_module is None:
-        _alloc_module = _extension("_avsa_alloc")
-    return _alloc_module.empty_as(like)
+    return (_alloc_module or _alloc()).empty_as(like)
 
 
 def _workspace(nbytes: int, like) -> torch.Tensor:
@@ -230,6 +238,11 @@ def avsa_cross_attn_scores_workspace_bytes(B, H, Nq, Nk, d) -> int:
 def avsa_cross_attn_scores(q, k, v, scores=None, score_beta=0.0, score_gamma=1.0, softmax_scale=0.0,
                            want_o=True, want_scores=True, o=None, lse=None, ws=None):
     """Eq. 1-2.  q [B,H,Nq,d], k/v [B,H,Nk,d] bf16 CUDA.  Returns (o, lse, scores, ws)."""
+    done = (_alloc_module or _alloc()).cross(q, k, v, scores, score_beta, score_gamma, softmax_scale, want_o, want_scores, o, lse, ws)
+    if done is not None:
+        if done[0] != AVSA_OK:
+            raise AvsaError(done[0], "avsa_cross_attn_scores")
+        return done[1:]
     if want_o and o is None:
         o = _empty_as(q)
     if lse is None:
@@ -251,6 +264,9 @@ def avsa_build_block_mask_workspace_bytes(B, H, N, d, blk) -> int:
     return int(load_library().avsa_build_block_mask_workspace_bytes(B, H, N, d, blk))
 
 
+_MASK_RESULT = ("block_scores", "col_idx", "col_cnt", "prot_tok", "prot_blk", "ws")
+
+
 def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTECT_ROWS, softmax_scale=0.0,
                           block_scores=None, shape=None, out=None, ws=None):
     """Eq. 8-9 plus the block-score top-k.  Returns dict(block_scores, col_idx, col_cnt, prot_tok, prot_blk, ws).
@@ -258,6 +274,19 @@ def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTE
     With AVSA_USE_GIVEN_BLOCK_SCORES pass ``block_scores`` [B,H,NB,NB] fp32 and ``shape`` = (B,H,N,d);
     q and k may then be None.
     """
+    out = out or {}
+    if block_scores is None:
+        block_scores = out.get("block_scores")
+    col_idx = out.get("col_idx")
+    col_cnt = out.get("col_cnt")
+    prot_tok = out.get("prot_tok")
+    prot_blk = out.get("prot_blk")
+    done = (_alloc_module or _alloc()).mask(q, k, scores, n_protect, k_keep, blk, flags, softmax_scale, block_scores, col_idx, col_cnt,
+                                            prot_tok, prot_blk, ws)
+    if done is not None:
+        if done[0] != AVSA_OK:
+            raise AvsaError(done[0], "avsa_build_block_mask")
+        return dict(zip(_MASK_RESULT, done[1:]))
     if q is not None:
         B, H, N, d = shape = q.shape
         like = q
@@ -266,13 +295,6 @@ def avsa_build_block_mask(q, k, scores, n_protect, k_keep, blk, flags=AVSA_PROTE
         like = block_scores
         if like is None:
             raise AttributeError("without q and k the block scores are an argument")
-    out = out or {}
-    if block_scores is None:
-        block_scores = out.get("block_scores")
-    col_idx = out.get("col_idx")
-    col_cnt = out.get("col_cnt")
-    prot_tok = out.get("prot_tok")
-    prot_blk = out.get("prot_blk")
     NB = (N + blk - 1) // blk
     if block_scores is None:
         block_scores = _empty(like, 0, B, H, NB, NB)
@@ -321,6 +343,11 @@ def avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk) -> int:
 
 def avsa_sparse_self_attn(q, k, v, col_idx, col_cnt, blk, softmax_scale=0.0, want_lse=False, o=None, lse=None, ws=None):
     """Eq. 10.  Returns (o, lse or None, ws)."""
+    done = (_alloc_module or _alloc()).sparse(q, k, v, col_idx, col_cnt, blk, softmax_scale, want_lse, o, lse, ws)
+    if done is not None:
+        if done[0] != AVSA_OK:
+            raise AvsaError(done[0], "avsa_sparse_self_attn")
+        return done[1:]
     if o is None:
         o = _empty_as(q)
     if want_lse and lse is None:
@@ -359,6 +386,11 @@ def avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, n_protect) -> int:
 def avsa_protected_rows_attn(q, k, v, prot_tok, n_protect, blk, o, lse=None, softmax_scale=0.0, ws=None):
     """Eq. 9 / Eq. 11 on tokens: overwrites the rows of the protected tokens in ``o`` (and ``lse``) with dense
     attention rows.  Returns ws."""
+    done = (_alloc_module or _alloc()).protected_rows(q, k, v, prot_tok, n_protect, blk, o, lse, softmax_scale, ws)
+    if done is not None:
+        if done[0] != AVSA_OK:
+            raise AvsaError(done[0], "avsa_protected_rows_attn")
+        return done[1]
     if ws is None:
         B, H, N, d = q.shape
         ws = _workspace(avsa_protected_rows_attn_workspace_bytes(B, H, N, d, blk, int(n_protect)), q)

@@ -1459,3 +1459,57 @@ def test_long_dense_rows_do_not_drift_towards_zero(d):
     _close(got, want, "long dense rows")
     drift = ((got - want) * want).sum() / (want * want).sum()
     assert abs(drift) <= 1.8e-4, f"drift {drift:.2e}"
+
+
+# ------------------------------------------------------------------------------------------- whole calls in native code
+@pytest.mark.parametrize("given", [False, True])
+def test_whole_calls_give_what_the_general_way_gives(monkeypatch, given):
+    """Plain tensors go through one native call a wrapper; the same calls the general way (as for any other class of tensor) give
+    the same bits, objects that the caller brings come back as they are, and refusals are the same."""
+    w = wl.WORKLOADS["tiny"]
+    q, k, v = (t.cuda() for t in wl.make_self_qkv(w, 3))
+    qa, kc, vc = (t.cuda() for t in wl.make_cross_qkv(w, 3))
+    s = torch.rand((w.B, w.n_video), device="cuda")
+    NB, N, n_protect = w.n_blocks, w.n_video, 20
+
+    def layer():
+        kw = [{}, {}, {}, {}]
+        if given:
+            kw = [dict(out=dict(block_scores=torch.empty((w.B, w.H, NB, NB), device="cuda"), prot_blk=torch.empty((w.B, NB), dtype=torch.uint8, device="cuda"))),
+                  dict(o=torch.empty_like(q), lse=torch.empty((w.B, w.H, N), device="cuda")),
+                  dict(scores=torch.full((w.B, N), 0.25, device="cuda"), score_beta=0.5, o=torch.empty_like(qa)),
+                  dict(ws=torch.empty(av.avsa_protected_rows_attn_workspace_bytes(w.B, w.H, N, w.d, w.blk, n_protect), dtype=torch.uint8, device="cuda"))]
+        m = av.avsa_build_block_mask(q, k, s, n_protect, 2, w.blk, flags=av.AVSA_PROTECT_TOKENS, **kw[0])
+        o, lse, ws = av.avsa_sparse_self_attn(q, k, v, m["col_idx"], m["col_cnt"], w.blk, want_lse=True, **kw[1])
+        wp = av.avsa_protected_rows_attn(q, k, v, m["prot_tok"], n_protect, w.blk, o, lse=lse, **kw[3])
+        oc, lc, sc, wc = av.avsa_cross_attn_scores(qa, kc, vc, **kw[2])
+        plain = av.avsa_cross_attn_scores(qa, kc, vc, want_o=False, want_scores=False)
+        assert plain[0] is None and plain[2] is None
+        if given:
+            assert m["block_scores"] is kw[0]["out"]["block_scores"] and m["prot_blk"] is kw[0]["out"]["prot_blk"]
+            assert o is kw[1]["o"] and lse is kw[1]["lse"] and oc is kw[2]["o"] and sc is kw[2]["scores"] and wp is kw[3]["ws"]
+        for x in (m["ws"], ws, wp, wc, plain[3]):
+            _status_ok(x)
+        torch.cuda.synchronize()
+        return [m[key].clone() for key in ("block_scores", "col_idx", "col_cnt", "prot_tok", "prot_blk")] + [o, lse, oc, lc, sc, plain[1]]
+
+    def refusals():
+        got = []
+        for call in (lambda: av.avsa_sparse_self_attn(q, k, v, None, None, w.blk), lambda: av.avsa_sparse_self_attn(q.float(), k, v, q, q, w.blk),
+                     lambda: av.avsa_build_block_mask(q[0], k, s, 1, 1, w.blk), lambda: av.avsa_build_block_mask(q, k, s, 1, 1, 64.5),
+                     lambda: av.avsa_build_block_mask(q, k, s, N + 1, 1, w.blk), lambda: av.avsa_cross_attn_scores(qa, kc.cpu(), vc),
+                     lambda: av.avsa_cross_attn_scores(qa, kc, vc, ws=torch.empty(256, dtype=torch.uint8, device="cuda"))):
+            with pytest.raises(Exception) as e:
+                call()
+            got.append((e.type, str(e.value)))
+        return got
+
+    native, native_refusals = layer(), refusals()
+
+    class General:
+        empty, empty_as = av._alloc().empty, av._alloc().empty_as
+        cross = mask = sparse = protected_rows = staticmethod(lambda *a: None)
+    monkeypatch.setattr(av, "_alloc_module", General)
+    for a, b in zip(native, layer()):
+        assert a.dtype == b.dtype and a.shape == b.shape and a.stride() == b.stride() and torch.equal(a, b)
+    assert native_refusals == refusals()
