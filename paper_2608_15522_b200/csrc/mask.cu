@@ -114,7 +114,8 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 // keys really span, the next over the bin that holds it, until every key of the bin is taken or it is one value wide; scores are
 // spread over such bins, so that two passes are the rule and few lanes meet in a counter.  Then every warp walks its own
 // contiguous segment in index order, taking every larger key and the lowest-index ties, and writes the flags of the tokens, four a
-// lane, and of the blocks that hold enough of them.  Block 0 also resets the status record of the call.
+// lane, and of the blocks that hold enough of them.  The kernel's first block also resets the call's
+// status record.
 //   Bound by one CTA's passes, above all by the counters of the first histogram.  us for the mask call where pooling does not cover the
 // select, against digits of eight bits with one key a lane and vote: 2 heads x 18600 tokens 35.0 -> 27.7, x 49152 71 -> 52; 4 heads x 2070
 // 12.5 -> 11.4.
@@ -151,10 +152,11 @@ __device__ __forceinline__ void warp_pick_bin(const int* bins, int want, int lan
   in_bin = __shfl_sync(0xffffffffu, n, src);
 }
 
-template <bool STAGED, int THREADS>
-__device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const float* __restrict__ scores, int N, int n_protect, int blk,
-                                              int NB, int min_tokens, uint8_t* __restrict__ prot_tok,
-                                              uint8_t* __restrict__ prot_blk, StatusRecord* status) {
+// One batch item's scores `s` to its flags `ptok` and `pblk`, by the first THREADS threads of the CTA: all of it, or (BARRIER) beside
+// others, with a barrier of their own.
+template <bool STAGED, int THREADS, int BARRIER = 0>
+__device__ __forceinline__ void select_tokens(uint32_t* skeys, const float* __restrict__ s, int N, int n_protect, int blk, int NB,
+                                              int min_tokens, uint8_t* ptok, uint8_t* pblk) {
   constexpr int WARPS = THREADS / 32;
   constexpr unsigned FULLM = 0xffffffffu;
   __shared__ int bins[kSelectBins];
@@ -162,15 +164,10 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
   __shared__ int s_bin, s_above, s_in_bin;
   __shared__ int warp_cnt[WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* s = scores + static_cast<int64_t>(b) * N;
-  uint8_t* ptok = prot_tok + static_cast<int64_t>(b) * N;
-  uint8_t* pblk = prot_blk + static_cast<int64_t>(b) * NB;
-  if (b == 0 && tid == 0) {
-    status->code = 0;
-    status->where = 0;
-    status->item = 0;
-    status->aux = 0;
-  }
+  auto sync = [] {
+    if (BARRIER == 0) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"n"(BARRIER), "n"(THREADS) : "memory");
+  };
   if (n_protect <= 0) {
     for (int i = tid; i < NB; i += THREADS) pblk[i] = 0;
     for (int i = tid; i < N; i += THREADS) ptok[i] = 0;
@@ -211,7 +208,7 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
     warp_max[warp] = kmax;
   }
   for (int i = tid; i < kSelectBins; i += THREADS) bins[i] = 0;
-  __syncthreads();
+  sync();
   kmin = __reduce_min_sync(FULLM, warp_min[lane % WARPS]);
   kmax = __reduce_max_sync(FULLM, warp_max[lane % WARPS]);
   // ---- the n_protect-th largest key is one of [base, base + span]; `want` of those are taken
@@ -227,7 +224,7 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
       for (int j = 0; j < 4; j++)
         if (j < n && k[j] - base <= span) atomicAdd(&bins[(k[j] - base) >> shift], 1);
     }
-    __syncthreads();
+    sync();
     if (warp == 0) {
       int bin, above, in_bin;
       warp_pick_bin(bins, want, lane, bin, above, in_bin);
@@ -237,14 +234,14 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
         s_in_bin = in_bin;
       }
     }
-    __syncthreads();
+    sync();
     want -= s_above;
     whole = s_in_bin == want;
     base += static_cast<uint32_t>(s_bin) << shift;
     span = (1u << shift) - 1u;
     if (whole || span == 0) break;
     for (int i = tid; i < kSelectBins; i += THREADS) bins[i] = 0;
-    __syncthreads();
+    sync();
   }
   // every key from `base` on is taken, or those above it and the first `want` of its own value
   // contiguous segment per warp, a whole number of blocks (blk is 32, 64 or 128), so that a block's tokens are one step's of one warp
@@ -261,7 +258,7 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
     }
     mine = __reduce_add_sync(FULLM, mine);
     if (lane == 0) warp_cnt[warp] = mine;
-    __syncthreads();
+    sync();
     eq_seen = __reduce_add_sync(FULLM, lane < warp ? warp_cnt[lane % WARPS] : 0);
   }
   const bool words = (reinterpret_cast<uintptr_t>(ptok) & 3u) == 0u;
@@ -306,6 +303,13 @@ __device__ __forceinline__ void select_tokens(int b, uint32_t* skeys, const floa
   }
 }
 
+__device__ __forceinline__ void reset_mask_status(StatusRecord* status) {
+  status->code = 0;
+  status->where = 0;
+  status->item = 0;
+  status->aux = 0;
+}
+
 template <bool STAGED>
 __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restrict__ scores, int N, int n_protect,
                                                             int blk, int NB, int min_tokens,
@@ -316,7 +320,10 @@ __global__ void __launch_bounds__(1024) token_select_kernel(const float* __restr
   // pooling kernel start right away (but not before this grid's own predecessors are done: pooling does not wait)
   pdl_wait();
   pdl_launch();
-  select_tokens<STAGED, 1024>(blockIdx.x, skeys, scores, N, n_protect, blk, NB, min_tokens, prot_tok, prot_blk, status);
+  const int b = blockIdx.x;
+  if (b == 0 && threadIdx.x == 0) reset_mask_status(status);
+  select_tokens<STAGED, 1024>(skeys, scores + static_cast<int64_t>(b) * N, N, n_protect, blk, NB, min_tokens,
+                              prot_tok + static_cast<int64_t>(b) * N, prot_blk + static_cast<int64_t>(b) * NB);
 }
 
 // Select and pooling of a short sequence in one launch: the first B CTAs select, the others pool a block each.  A launch costs the host
@@ -335,7 +342,10 @@ __global__ void __launch_bounds__(256) select_pool_kernel(const __nv_bfloat16* _
   pdl_wait();
   pdl_launch();
   if (static_cast<int>(blockIdx.x) < B) {
-    select_tokens<true, 256>(blockIdx.x, skeys, scores, N, n_protect, blk, NB, min_tokens, prot_tok, prot_blk, status);
+    const int b = blockIdx.x;
+    if (b == 0 && threadIdx.x == 0) reset_mask_status(status);
+    select_tokens<true, 256>(skeys, scores + static_cast<int64_t>(b) * N, N, n_protect, blk, NB, min_tokens,
+                             prot_tok + static_cast<int64_t>(b) * N, prot_blk + static_cast<int64_t>(b) * NB);
   } else {
     const int i = blockIdx.x - B, pair = i / NB;
     pool_block<D>(i % NB, NB, pair >> 1, pair & 1, q, q_sb, q_sh, q_sn, k, k_sb, k_sh, k_sn, qbar, kbar, H, N, blk);
@@ -596,6 +606,105 @@ __global__ void __launch_bounds__(WARPS * 32) score_select_kernel(const float* _
 }
 
 // ------------------------------------------------------------------------------------------------
+// The whole mask of a short sequence in one launch, a CTA per (batch, head) pair: eight warps select the protected tokens (every CTA
+// for itself; the first head's writes the flags), sixteen pool the head's queries and keys meanwhile, then all take block scores (plain
+// fp32, a warp a score) and lists.  Two launches, with the pooled means and the flags through L2 between them, cost more than what
+// every head repeats, as long as a head is short and has an SM: us for the mask call 7.0 -> 4.2 (2 heads x 256 tokens of 64 channels) and
+// 4.5 (24 x 157 of 128), with the attention behind it 14.7 -> 13.1 and 15.8 -> 14.3; with 405 tokens of 128 channels 18.2 -> 18.8, 500 of 64
+// 26.0 -> 27.3, two batches of 32 heads x 320 of 128 23.5 -> 24.5.
+// ------------------------------------------------------------------------------------------------
+__host__ __device__ constexpr int short_tokens(int d) { return d == 128 ? 256 : 320; }
+constexpr int kShortThreads = 768;
+template <int D>
+__global__ void __launch_bounds__(kShortThreads) mask_short_kernel(
+    const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh, int64_t q_sn, const __nv_bfloat16* __restrict__ k, int64_t k_sb,
+    int64_t k_sh, int64_t k_sn, int H, int N, int NB, const float* __restrict__ scores, int n_protect, int min_tokens, float scale,
+    int k_keep, int protect_rows, int protect_cols, float* __restrict__ bs, int32_t* __restrict__ col_idx, int32_t* __restrict__ col_cnt,
+    uint8_t* prot_tok, uint8_t* prot_blk, StatusRecord* status) {
+  constexpr int BLK = D, TOKENS = short_tokens(D), MAX_NB = TOKENS / BLK, TPR = D / 8, RPW = 32 / TPR;      // threads of a row, rows of a warp's load
+  constexpr int POOL_WARPS = 16, SELECT_WARPS = 8;
+  __shared__ __align__(16) uint32_t skeys[TOKENS];
+  __shared__ uint8_t own_tok[TOKENS], own_blk[MAX_NB];
+  __shared__ float part[POOL_WARPS][D], mean[2 * MAX_NB][D];
+  __shared__ float strip[MAX_NB][MAX_NB];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bh = blockIdx.x, h = bh % H, b = bh / H;
+  uint8_t* ptok = h == 0 ? prot_tok + static_cast<int64_t>(b) * N : own_tok;
+  uint8_t* pblk = h == 0 ? prot_blk + static_cast<int64_t>(b) * NB : own_blk;
+  pdl_wait();
+  pdl_launch();
+  if (bh == 0 && tid == 0) reset_mask_status(status);
+  // a (tensor, block) pair's rows are shared by WPP warps
+  const int pairs = 2 * NB, WPP = POOL_WARPS / pairs;
+  if (warp < SELECT_WARPS) {
+    select_tokens<true, 32 * SELECT_WARPS, 1>(skeys, scores + static_cast<int64_t>(b) * N, N, n_protect, BLK, NB, min_tokens, ptok, pblk);
+  } else {
+    const int pw = warp - SELECT_WARPS, pair = pw / WPP, nb = pair >> 1;
+    if (pair < pairs) {
+      const __nv_bfloat16* src = (pair & 1) == 0 ? q + b * q_sb + h * q_sh : k + b * k_sb + h * k_sh;
+      const int64_t sn = (pair & 1) == 0 ? q_sn : k_sn;
+      const int row0 = nb * BLK, rows = min(BLK, N - row0);
+      float acc[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) acc[i] = 0.f;
+      constexpr int U = 8;      // loads in flight
+      for (int r0 = (pw % WPP) * RPW + lane / TPR; r0 < rows; r0 += WPP * RPW * U) {
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const int r = r0 + u * WPP * RPW;
+          v[u] = make_uint4(0u, 0u, 0u, 0u);
+          if (r < rows) v[u] = __ldg(reinterpret_cast<const uint4*>(src + (row0 + r) * sn + (lane % TPR) * 8));
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+          for (int i = 0; i < 4; i++) {
+            acc[2 * i] += __uint_as_float(w[i] << 16);
+            acc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+#pragma unroll
+        for (int off = TPR; off < 32; off <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+      }
+      if (lane < TPR) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) part[pw][lane * 8 + i] = acc[i];
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < pairs * D; e += kShortThreads) {
+    const int pair = e / D, c = e % D;
+    float sum = 0.f;
+    for (int i = 0; i < WPP; i++) sum += part[pair * WPP + i][c];
+    mean[pair][c] = sum / static_cast<float>(min(BLK, N - (pair >> 1) * BLK));
+  }
+  __syncthreads();
+  for (int e = warp; e < NB * NB; e += kShortThreads / 32) {
+    const int i = e / NB, j = e % NB;
+    float sum = 0.f;
+#pragma unroll
+    for (int c = 0; c < D / 32; c++) sum = fmaf(mean[2 * i][c * 32 + lane], mean[2 * j + 1][c * 32 + lane], sum);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if (lane == 0) {
+      strip[i][j] = sum * scale;
+      bs[static_cast<int64_t>(bh) * NB * NB + e] = sum * scale;
+    }
+  }
+  __syncthreads();
+  if (warp < NB) {
+    const int64_t row = static_cast<int64_t>(bh) * NB + warp;
+    select_row<1>(strip[warp], pblk, protect_rows && pblk[warp] != 0, NB, k_keep, protect_cols, lane, col_idx + row * NB, col_cnt + row);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
 // Optional block-sum protection (AVSA_PROTECT_BLOCK_SUM): the response of a block is the sum of its tokens'
 // scores, accumulated in fp64 (for 128 fp32 terms of like magnitude that sum is exact, so its value does not
 // depend on the order of the adds) and rounded to fp32; the top-n blocks are then chosen by the same select
@@ -728,6 +837,16 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
 
   const bool one_launch = !by_block_sum && !given && N <= kSelectPoolTokens && static_cast<int64_t>(B) * H <= 65535;
+  if (one_launch && N <= short_tokens(d) && static_cast<int64_t>(B) * H <= persistent_grid(1 << 30)) {
+    const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(q.ptr);
+    const __nv_bfloat16* kp = static_cast<const __nv_bfloat16*>(k.ptr);
+    auto kernel = d == 128 ? mask_short_kernel<128> : mask_short_kernel<64>;
+    if (launch_pdl(kernel, B * H, kShortThreads, 0, st, qp, q.stride_b, q.stride_h, q.stride_n, kp, k.stride_b, k.stride_h, k.stride_n, H, N,
+                   NB, scores, n_protect, min_tokens, scale, k_keep, (flags & AVSA_PROTECT_ROWS) ? 1 : 0, (flags & AVSA_PROTECT_COLS) ? 1 : 0,
+                   block_scores, col_idx, col_cnt, ptok, pblk, static_cast<StatusRecord*>(ws)) != cudaSuccess)
+      return AVSA_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
+  }
   if (by_block_sum) {
     // block sums, then the token select run over the NB sums: its "token" flags are the block flags (its own
     // block lift goes to a scratch array); the token flags are filled in at the end of the call

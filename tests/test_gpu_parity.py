@@ -1294,6 +1294,28 @@ def test_mask_with_the_select_in_the_pooling_grid(n):
         assert rest.size == 0 or scores_row[kept].min() >= scores_row[rest].max()
 
 
+@pytest.mark.parametrize("d,n,heads", [(128, 1, 2), (128, 127, 3), (128, 129, 74), (128, 256, 5), (128, 257, 5), (128, 200, 75), (64, 65, 4),
+                                       (64, 257, 3), (64, 320, 6), (64, 321, 6)])
+@pytest.mark.parametrize("flags", [av.AVSA_PROTECT_ROWS, av.AVSA_PROTECT_ROWS | av.AVSA_PROTECT_COLS, av.AVSA_PROTECT_TOKENS])
+def test_mask_of_a_short_sequence_in_one_launch(d, n, heads, flags):
+    """A CTA per (batch, head) pair pools, selects, scores and lists: block counts that share the pooling warps unevenly, the last
+    length of each head size and the next, as many heads as SMs and more, none protected, and [B,N,H,d] storage."""
+    B, NB = 2, (n + d - 1) // d
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k = (torch.randn((B, n, heads, d), generator=g, device="cuda").bfloat16().transpose(1, 2) for _ in range(2))
+    s = torch.round(torch.randn((B, n), generator=g, device="cuda") * 4) / 4
+    k_keep = max(1, NB // 2)
+    for n_protect in (0, max(1, n // 9)):
+        m = av.avsa_build_block_mask(q, k, s if n_protect else None, n_protect, k_keep, d, flags=flags)
+        _status_ok(m["ws"])
+        want, got = orc.block_scores(_np64(q), _np64(k), d), m["block_scores"].cpu().numpy()
+        assert np.abs(got - want).max() <= 1e-5 * np.abs(want).max()      # (fp32 sums of 128 means and products)
+        idx, cnt, tok, blk = orc.build_block_mask(got, s.cpu().numpy(), n_protect, k_keep, d, n,
+                                                  protect_rows=bool(flags & av.AVSA_PROTECT_ROWS), protect_cols=bool(flags & av.AVSA_PROTECT_COLS))
+        for key, x in (("col_idx", idx), ("col_cnt", cnt), ("prot_tok", tok), ("prot_blk", blk)):
+            assert np.array_equal(m[key].cpu().numpy(), x), key
+
+
 @pytest.mark.parametrize("NB", [1, 32, 33, 256, 257, 512, 513, 1024, 1025])
 def test_mask_select_over_row_lengths(NB):
     """The select's key slots per lane at their limits: distinct scores, heavy ties, one bit of difference, a sign change,
