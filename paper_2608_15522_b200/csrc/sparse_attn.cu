@@ -204,11 +204,11 @@ __global__ void __launch_bounds__(32) bounded_wait_selftest_kernel(StatusRecord*
 // Lists of 64-blocks are run in pairs (attn_pair_kernel) unless every query block has a CTA of its own or the sequence is short: joining
 // the lists takes a launch more, and pairs of short lists that share little save nothing.  us as items of 64 rows / in pairs, lists of
 // 10 % drawn at random, of 25 % with a third of the rows dense, of all blocks: 148 items of 148 blocks 15 / 23, 76 / 72, 77 / 73; 180 of
-// 90 18 / 19, 51 / 50, 92 / 51; 592 of 148 39 / 33, 166 / 129, 281 / 132; 576 of 24 17 / 17, 38 / 35, 56 / 36; 288 of 24 12 / 14, 26 / 25, 33 / 26.
-constexpr int kPairMinBlocks = 32;
+// 90 18 / 19, 51 / 50, 92 / 51; 592 of 148 39 / 33, 166 / 129, 281 / 132; 888 of 37 24 / 27, 69 / 58, 116 / 81; 396 of 33, the mask's own lists of
+// 10 %, 16 / 19; 288 of 24 12 / 14, 26 / 25, 33 / 26.
 static bool runs_pairs(int B, int H, int d, int NB) {
   const long long items = static_cast<long long>(B) * H * NB;
-  return d == 64 && NB >= kPairMinBlocks && persistent_grid(items) < items;
+  return d == 64 && (NB >= 64 ? persistent_grid(items) < items : NB >= 32 && items >= 4ll * persistent_grid(items));
 }
 
 static int launch_pair_attn(int B, int H, int N, const avsa_bf16_4d& q, const avsa_bf16_4d& k, const avsa_bf16_4d& v, void* o,
