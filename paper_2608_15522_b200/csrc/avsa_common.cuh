@@ -52,23 +52,32 @@ __device__ __forceinline__ void report_status(StatusRecord* st, int code, int wh
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// (in clusters of `cluster` CTAs)
 template <class... Params, class... Args>
-inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchAttribute attr[1];
+inline cudaError_t launch_pdl_clusters(void (*kernel)(Params...), unsigned cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                       Args&&... args) {
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim = {cluster, 1, 1};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
   // The call returns this failure itself.  Left behind as the runtime's last error, which every call reads at its end, it
   // would fail a good call of the same thread: the next one that does not set a kernel attribute (that clears it).
   if (e != cudaSuccess) cudaGetLastError();
   return e;
+}
+
+template <class... Params, class... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_pdl_clusters(kernel, 1, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // Resets the status record at the start of every call (first node of the call's launch sequence).

@@ -3,7 +3,10 @@
 //   pass 1  flash attention, key axis split across CTAs -> partial (O, LSE) -> merge -> O, row LSE
 //   pass 2  for every key tile: S^T = K Q^T on the tensor cores, p = exp2(S^T c - lse_j), summed over
 //           the queries -> per-head column sums -> fixed-order head sum with the beta/gamma blend
-// With at most 256 keys both are one pass over the queries: cross_resident.cuh.
+// With at most 256 keys both are one pass over the queries, and in short calls with at most 4096, sliced over a cluster of CTAs:
+// cross_resident.cuh.
+#include <atomic>
+
 #include "attn_persist_kernel.cuh"
 #include "cross_resident.cuh"
 
@@ -558,6 +561,72 @@ __global__ void __launch_bounds__(256) cross_finalize_kernel(int hs_blocks, cons
   }
 }
 
+// End of a sliced call (cross_resident.cuh) in one grid: the first `hs_blocks` CTAs sum the score partials over heads, the next ones add
+// the slices' O (eight rows a CTA, sixteen with 64 channels, all slices' loads in flight), the last one collects the CTAs' records.
+struct SlicedFinalize {
+  const float* part_o;      // [pair][slice][rows][D]
+  int slices, rows, Nq, H, groups;
+  __nv_bfloat16* o;
+  int64_t o_sb, o_sh, o_sn;
+  const CtaStatus* cta_status;
+  int n_ctas;
+  StatusRecord* status;
+};
+template <int D>
+__global__ void __launch_bounds__(256) sliced_finalize_kernel(int hs_blocks, const float* __restrict__ partial, int B, int sums, int Nk,
+                                                              float beta, float gamma, float* __restrict__ scores,
+                                                              const __grid_constant__ SlicedFinalize m) {
+  pdl_wait();
+  pdl_launch();
+  const int tid = threadIdx.x;
+  if (static_cast<int>(blockIdx.x) < hs_blocks) {
+    head_sum_keys(blockIdx.x, tid, partial, 1, B, sums, Nk, beta, gamma, scores);      // (a sum per head and query tile)
+  } else if (blockIdx.x + 1 < gridDim.x) {
+    constexpr int LANES = D / 4, ROWS = 256 / LANES;
+    const int block = static_cast<int>(blockIdx.x) - hs_blocks, bh = block / m.groups;
+    const int row = (block % m.groups) * ROWS + tid / LANES, col = (tid % LANES) * 4;
+    if (row >= m.Nq) return;
+    const float4* src = reinterpret_cast<const float4*>(m.part_o + (static_cast<int64_t>(bh) * m.slices * m.rows + row) * D + col);
+    float4 v[kResMaxSlices], acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kResMaxSlices; c++)
+      v[c] = c < m.slices ? __ldg(src + static_cast<int64_t>(c) * m.rows * LANES) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kResMaxSlices; c++) {
+      acc.x += v[c].x;
+      acc.y += v[c].y;
+      acc.z += v[c].z;
+      acc.w += v[c].w;
+    }
+    uint2 pk;
+    pk.x = pack_bf16x2(acc.x, acc.y);
+    pk.y = pack_bf16x2(acc.z, acc.w);
+    *reinterpret_cast<uint2*>(m.o + bh / m.H * m.o_sb + bh % m.H * m.o_sh + row * m.o_sn + col) = pk;
+  } else {
+    __shared__ int first, redo;
+    if (tid == 0) {
+      first = 0x7fffffff;
+      redo = 0;
+    }
+    __syncthreads();
+    for (int g = tid; g < m.n_ctas; g += 256) {
+      if (m.cta_status[g].code != 0) atomicMin(&first, g);
+      if (m.cta_status[g].redo != 0) atomicAdd(&redo, m.cta_status[g].redo);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      CtaStatus s = {};
+      if (first != 0x7fffffff) s = m.cta_status[first];
+      m.status->code = s.code;
+      m.status->where = s.where;
+      m.status->item = s.item;
+      m.status->aux = s.aux;
+      m.status->redo_count = redo;
+      m.status->next_item = 0;
+    }
+  }
+}
+
 // The same sum for few keys and many partial slots (the reverse direction: at most 512 keys, two slots per CTA of the
 // score pass): one warp per key.  Lane l adds the terms j = l, l + 32, ... in ascending order, then the 32 lane sums
 // are combined by a fixed butterfly, so the result is reproducible bit for bit (the order differs from the kernel
@@ -600,10 +669,57 @@ struct CrossPlan {
   int NQC, rev_ranges, rev_cpr, rev_slots;   // query chunks of 128, CTAs per (b,h), chunks per CTA, partial slots
   bool resident;                             // both passes in one kernel, K and V of a head on chip
   int res_tiles, res_L, res_ctas;            // query tiles of all pairs, per CTA, CTAs
+  int slices;                                // more than 0: the same with the keys of a pair over this many CTAs
   size_t off_part_o, off_part_lse, off_lse, off_lse2, off_partial, off_redo, off_cta, total;
 };
 
-static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
+// How many clusters of `slices` CTAs the current device runs side by side (asked once per device: it depends on the sizes of its GPCs);
+// none where it cannot say.
+template <int D, bool SCORES>
+static cudaError_t allow_sliced() {
+  auto kernel = cross_resident_kernel<D, 2, SCORES, true>;
+  // (more than 8 CTAs are not portable to every device)
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ResidentSmem<D, 2, true>::kTotal);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+template <int D, bool SCORES>
+static int sliced_clusters(int slices) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][kResMaxSlices + 1];      // one more than the number; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  if (dev >= 0 && dev < kDevices) {
+    const int k = known[dev][slices].load(std::memory_order_relaxed);
+    if (k > 0) return k - 1;
+  }
+  int n = 0;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {static_cast<unsigned>(slices), 1, 1};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = static_cast<unsigned>(slices);
+  cfg.blockDim = kResThreads;
+  cfg.dynamicSmemBytes = ResidentSmem<D, 2, true>::kTotal;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (dev < 0 || allow_sliced<D, SCORES>() != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, cross_resident_kernel<D, 2, SCORES, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (dev < kDevices) known[dev][slices].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+// Query tiles that a sliced call takes at most: as many clusters as run side by side.  us with scores, the two passes / sliced, 100
+// queries, 128 channels: 16 tiles of 2 slices 17.2 / 11.6, 74 19.6 / 13.7, 85 21.4 / 22.8; 24 of 5 20.9 / 12.8, 28 21.4 / 21.8; 14 of 8 20.3 /
+// 12.2, 18 20.9 / 22.1, 35 25.2 / 32.8; 7 of 16 21.1 / 14.4, 8 21.3 / 25.1.  Without scores the one pass of before is as short where
+// two slices fill the SMs with tiles of 128 channels (32 tiles 10.8 / 10.8, 74 11.0 / 12.6; 64 channels 10.2 / 9.3; 32 tiles of 4 15.3 / 11.8).
+static long long max_sliced_tiles(int slices, int d, bool scores) {
+  const int n = d == 128 ? (scores ? sliced_clusters<128, true>(slices) : sliced_clusters<128, false>(slices))
+                         : (scores ? sliced_clusters<64, true>(slices) : sliced_clusters<64, false>(slices));
+  return slices == 2 && d == 128 && !scores && n > 32 ? 32 : n;
+}
+static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool scores) {
   CrossPlan c = {};
   // Few keys: everything in one kernel, whatever the number of queries (faster from 2 heads x 32 queries to 64 x 19200, with scores
   // and without: cross_resident.cuh).  More than 256 keys of 128 channels do not fit an SM's shared memory beside the tiles, nor
@@ -623,6 +739,18 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d) {
     size_t off = kStatusBytes;
     c.off_cta = off; off += align_up(static_cast<size_t>(c.res_ctas) * sizeof(CtaStatus), 256);
     c.off_partial = off; off += align_up((static_cast<size_t>(c.res_ctas) + B * H) * Nk * sizeof(float), 256);
+    c.total = off;
+    return c;
+  }
+  const int slices = (Nk + kResMaxKeys - 1) / kResMaxKeys;
+  if (slices <= kResMaxSlices && Nq <= kResSlicedQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
+    c.slices = slices;
+    c.NQT = (Nq + 127) / 128;
+    c.res_ctas = static_cast<int>(tiles) * slices;
+    size_t off = kStatusBytes;
+    c.off_cta = off; off += align_up(static_cast<size_t>(c.res_ctas) * sizeof(CtaStatus), 256);
+    c.off_partial = off; off += align_up(static_cast<size_t>(tiles) * Nk * sizeof(float), 256);
+    c.off_part_o = off; off += align_up(static_cast<size_t>(c.res_ctas) * 128 * d * sizeof(float), 256);
     c.total = off;
     return c;
   }
@@ -681,9 +809,9 @@ template <int D, int KG, bool SCORES>
 static int launch_resident(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                            const ResidentParams& rp, int ctas, cudaStream_t st) {
   constexpr int kSmem = ResidentSmem<D, KG>::kTotal;
-  if (cudaFuncSetAttribute(cross_resident_kernel<D, KG, SCORES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+  if (cudaFuncSetAttribute(cross_resident_kernel<D, KG, SCORES, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
     return AVSA_ERR_CUDA;
-  return launch_pdl(cross_resident_kernel<D, KG, SCORES>, ctas, kResThreads, kSmem, st, tq, tk, tv, to, rp) == cudaSuccess
+  return launch_pdl(cross_resident_kernel<D, KG, SCORES, false>, ctas, kResThreads, kSmem, st, tq, tk, tv, to, rp) == cudaSuccess
              ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -731,6 +859,60 @@ static int run_cross_resident(int B, int H, int Nq, int Nk, const avsa_bf16_4d& 
                   : launch_resident<D, 1, false>(tq, tk, tv, to, rp, c.res_ctas, st);
     if (rc != AVSA_OK) return rc;
   }
+  return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
+}
+
+template <int D, bool SCORES>
+static int launch_sliced(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const ResidentParams& rp, int ctas,
+                         cudaStream_t st) {
+  constexpr int kSmem = ResidentSmem<D, 2, true>::kTotal;
+  auto kernel = cross_resident_kernel<D, 2, SCORES, true>;
+  if (allow_sliced<D, SCORES>() != cudaSuccess) return AVSA_ERR_CUDA;
+  return launch_pdl_clusters(kernel, static_cast<unsigned>(rp.slices), ctas, kResThreads, kSmem, st, tq, tk, tv, tq, rp) == cudaSuccess
+             ? AVSA_OK : AVSA_ERR_CUDA;
+}
+
+template <int D>
+static int run_cross_sliced(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q, const avsa_bf16_4d& k, const avsa_bf16_4d& v,
+                            void* o, float* lse, float* scores, float beta, float gamma, float scale, uint8_t* ws, const CrossPlan& c,
+                            cudaStream_t st) {
+  CUtensorMap tq, tk, tv;
+  if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
+  if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
+  if (!encode_bf16_tile_map(&tv, v.ptr, B, H, Nk, D, v.stride_b, v.stride_h, v.stride_n, 128)) return AVSA_ERR_CUDA;
+  ResidentParams rp = {};
+  rp.lse = lse;
+  rp.partial = reinterpret_cast<float*>(ws + c.off_partial);
+  rp.part_o = o != nullptr ? reinterpret_cast<float*>(ws + c.off_part_o) : nullptr;
+  rp.cta_status = reinterpret_cast<CtaStatus*>(ws + c.off_cta);
+  rp.H = H;
+  rp.Nq = Nq;
+  rp.NQT = c.NQT;
+  rp.Nk = Nk;
+  rp.slices = c.slices;
+  rp.scale_log2 = scale * 1.4426950408889634f;
+  const int rc = scores != nullptr ? launch_sliced<D, true>(tq, tk, tv, rp, c.res_ctas, st) : launch_sliced<D, false>(tq, tk, tv, rp, c.res_ctas, st);
+  if (rc != AVSA_OK) return rc;
+  SlicedFinalize m = {};
+  m.part_o = rp.part_o;
+  m.slices = c.slices;
+  m.rows = c.NQT * 128;
+  m.Nq = Nq;
+  m.H = H;
+  m.groups = (Nq + merge_rows(D) - 1) / merge_rows(D);
+  m.o = static_cast<__nv_bfloat16*>(o);
+  m.o_sb = q.stride_b;
+  m.o_sh = q.stride_h;
+  m.o_sn = q.stride_n;
+  m.cta_status = rp.cta_status;
+  m.n_ctas = c.res_ctas;
+  m.status = reinterpret_cast<StatusRecord*>(ws);
+  const int64_t n = static_cast<int64_t>(B) * Nk;
+  const int hs_blocks = scores != nullptr ? static_cast<int>((n + kHeadSumKeys - 1) / kHeadSumKeys) : 0;
+  const int merge_blocks = o != nullptr ? B * H * m.groups : 0;
+  if (launch_pdl(sliced_finalize_kernel<D>, hs_blocks + merge_blocks + 1, 256, 0, st, hs_blocks, rp.partial, B, H * c.NQT, Nk, beta, gamma, scores,
+                 m) != cudaSuccess)
+    return AVSA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -874,7 +1056,8 @@ using namespace avsa;
 
 extern "C" size_t avsa_cross_attn_scores_workspace_bytes(int B, int H, int Nq, int Nk, int d) {
   if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128) || !pairs_ok(B, H)) return 0;
-  return make_cross_plan(B, H, Nq, Nk, d).total;
+  const size_t with = make_cross_plan(B, H, Nq, Nk, d, true).total, without = make_cross_plan(B, H, Nq, Nk, d, false).total;
+  return with > without ? with : without;
 }
 
 extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_bf16_4d q, avsa_bf16_4d k,
@@ -889,7 +1072,7 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (!tensor_ok(q, B, H) || !tensor_ok(k, B, H) || !tensor_ok(v, B, H)) return AVSA_ERR_INVALID_ARG;
   if (o_bf16 != nullptr && !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
-  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d);
+  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, scores != nullptr);
   if (ws == nullptr || ws_bytes < c.total) return AVSA_ERR_WORKSPACE;
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
@@ -900,6 +1083,9 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (c.resident)
     return run_cross_resident<64>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c,
                                   as_stream(stream));
+  if (c.slices > 0)
+    return d == 128 ? run_cross_sliced<128>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c, as_stream(stream))
+                    : run_cross_sliced<64>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c, as_stream(stream));
   if (d == 128)
     return run_cross<128, 128>(B, H, Nq, Nk, q, k, v, o_bf16, lse, scores, score_beta, score_gamma, scale, base, c,
                                as_stream(stream));

@@ -568,7 +568,7 @@ def test_sparse_attention_pairs_of_64_blocks(case):
     block, of 9 rows), lists that share nothing or begin elsewhere, a block that one of a pair does not list and whose values are no
     numbers, rows that outgrow their reference in one block of a pair, a pair without a list, and more than the 1024 key blocks that
     are joined at a time."""
-    B, H, NB, d = (1, 1, 1061, 64) if case == "window" else (1, 5, 35, 64)
+    B, H, NB, d = (1, 1, 1061, 64) if case == "window" else (1, 17, 35, 64)
     N = (NB - 1) * d + 9
     g = torch.Generator().manual_seed(3)
     q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
@@ -805,6 +805,42 @@ def test_cross_attention_reverse_direction(name):
     _close_scores(got_s, want_s, f"{name} reverse scores")
     _, _, s2, _ = av.avsa_cross_attn_scores(q_video.cuda(), k_audio.cuda(), v_audio.cuda(), score_gamma=gamma)
     assert torch.equal(s, s2)                                              # fixed summation order
+
+
+@pytest.mark.parametrize("B,H,Nq,Nk,d", [
+    (1, 2, 72, 257, 128), (1, 3, 1, 288, 64), (1, 2, 127, 289, 128), (1, 72, 20, 512, 64), (1, 73, 20, 512, 64),      # two slices
+    (1, 33, 60, 400, 128), (2, 3, 129, 513, 128), (1, 8, 512, 769, 64), (1, 24, 33, 1280, 128), (2, 5, 200, 1537, 64),
+    (1, 14, 128, 2048, 128), (1, 20, 128, 2048, 128), (1, 3, 300, 2047, 64), (2, 4, 72, 2070, 128), (1, 2, 100, 4096, 64),
+    (1, 3, 40, 4003, 128), (1, 2, 100, 4097, 128)])
+@pytest.mark.parametrize("growth", [0.0, 30.0, 90.0])
+def test_cross_attention_sliced_keys(B, H, Nq, Nk, d, growth):
+    """Short calls against 257 to 4096 keys: a cluster of CTAs takes a query tile, each some of the keys.  Slices of four chunks of 32 keys
+    and of eight, the last key alone in its chunk, several query tiles, as many clusters as run side by side and one more, the first
+    length beyond; logits that grow along the keys (base 2, per 128 keys), so that the reference changes inside a slice and from slice
+    to slice; [B,N,H,d] storage; with and without scores."""
+    g = torch.Generator().manual_seed(Nk + Nq)
+    q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, Nk, Nk))
+    if growth:
+        u = 1.0 / np.sqrt(d)
+        q = q * 0.1 + 8.0 * u
+        ramp = torch.arange(Nk, dtype=torch.float32).div(128, rounding_mode="floor") * growth * np.log(2) * np.sqrt(d) / 8.0
+        k = k + (ramp * u).view(1, 1, -1, 1)
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+    qs, ks, vs = (t.cuda().transpose(1, 2).contiguous().transpose(1, 2) for t in (q, k, v))
+    prev = torch.rand((B, Nk), generator=g).cuda()
+    o, lse, s, ws = av.avsa_cross_attn_scores(qs, ks, vs, scores=prev.clone(), score_beta=0.5, score_gamma=0.5 / (H * Nq))
+    _status_ok(ws)
+    assert o.stride() == qs.stride()
+    _close(_np64(o), want_o, "sliced O")
+    _close_lse(_np64(lse), want_lse, "sliced lse")
+    _close_scores(_np64(s), 0.5 * _np64(prev) + orc.column_scores(A, gamma=0.5 / (H * Nq)), "sliced scores")
+    again = av.avsa_cross_attn_scores(qs, ks, vs, scores=prev.clone(), score_beta=0.5, score_gamma=0.5 / (H * Nq))
+    assert torch.equal(again[0], o) and torch.equal(again[1], lse) and torch.equal(again[2], s)
+    o2, lse2, _, ws2 = av.avsa_cross_attn_scores(qs, ks, vs, want_scores=False)
+    _status_ok(ws2)
+    _close(_np64(o2), want_o, "sliced O without scores")
+    _close_lse(_np64(lse2), want_lse, "sliced lse without scores")
 
 
 @pytest.mark.parametrize("reverse", [False, True])
