@@ -30,8 +30,9 @@
  *     that reference (a row whose sum of exp(logit - reference) ends above 2^64 or not finite): in the same kernel
  *     in short calls, in one behind it in long ones (of query blocks of 64 rows also those with an output that is
  *     not finite).  Results do not depend on which way produced them beyond
- *     rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).  Cross-attention against at
- *     most 256 keys, and short calls against at most 4096 (of 129 to 256 each per CTA), recompute nothing: a row whose keys from 128 on outgrow the maximum of the first 128 by more
+ *     rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).  Cross-attention in short calls
+ *     against at most 4096 keys recomputes nothing (every part of a row takes its own maximum), nor does it
+ *     against at most 256 keys: there a row whose keys from 128 on outgrow the maximum of the first 128 by more
  *     than 2^57 (as factors of exp) takes a larger reference on the way, and the int32 counts the tiles of 128
  *     queries in which one did so by more than 2^64.  Values of v are assumed to stay below 2^60 in magnitude.
  *   - Errors detectable on the host return at once with nothing enqueued.  Return values are

@@ -3,12 +3,12 @@
 //   pass 1  flash attention, key axis split across CTAs -> partial (O, LSE) -> merge -> O, row LSE
 //   pass 2  for every key tile: S^T = K Q^T on the tensor cores, p = exp2(S^T c - lse_j), summed over
 //           the queries -> per-head column sums -> fixed-order head sum with the beta/gamma blend
-// With at most 256 keys both are one pass over the queries, and in short calls with at most 4096, sliced over a cluster of CTAs:
-// cross_resident.cuh.
+// With at most 256 keys both are one pass over the queries (cross_resident.cuh), and in short calls with at most 4096 too, the keys
+// sliced over a cluster of CTAs (cross_sliced.cuh).
 #include <atomic>
 
 #include "attn_persist_kernel.cuh"
-#include "cross_resident.cuh"
+#include "cross_sliced.cuh"
 
 namespace avsa {
 
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256) cross_finalize_kernel(int hs_blocks, cons
   }
 }
 
-// End of a sliced call (cross_resident.cuh) in one grid: the first `hs_blocks` CTAs sum the score partials over heads, the next ones add
+// End of a sliced call (cross_sliced.cuh) in one grid: the first `hs_blocks` CTAs sum the score partials over heads, the next ones add
 // the slices' O (eight rows a CTA, sixteen with 64 channels, all slices' loads in flight), the last one collects the CTAs' records.
 struct SlicedFinalize {
   const float* part_o;      // [pair][slice][rows][D]
@@ -587,12 +587,12 @@ __global__ void __launch_bounds__(256) sliced_finalize_kernel(int hs_blocks, con
     const int row = (block % m.groups) * ROWS + tid / LANES, col = (tid % LANES) * 4;
     if (row >= m.Nq) return;
     const float4* src = reinterpret_cast<const float4*>(m.part_o + (static_cast<int64_t>(bh) * m.slices * m.rows + row) * D + col);
-    float4 v[kResMaxSlices], acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 v[kSlicedMaxSlices], acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < kResMaxSlices; c++)
+    for (int c = 0; c < kSlicedMaxSlices; c++)
       v[c] = c < m.slices ? __ldg(src + static_cast<int64_t>(c) * m.rows * LANES) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < kResMaxSlices; c++) {
+    for (int c = 0; c < kSlicedMaxSlices; c++) {
       acc.x += v[c].x;
       acc.y += v[c].y;
       acc.z += v[c].z;
@@ -677,15 +677,15 @@ struct CrossPlan {
 // none where it cannot say.
 template <int D, bool SCORES>
 static cudaError_t allow_sliced() {
-  auto kernel = cross_resident_kernel<D, 2, SCORES, true>;
+  auto kernel = cross_sliced_kernel<D, SCORES>;
   // (more than 8 CTAs are not portable to every device)
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ResidentSmem<D, 2, true>::kTotal);
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SlicedSmem<D>::kTotal);
   return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 template <int D, bool SCORES>
 static int sliced_clusters(int slices) {
   constexpr int kDevices = 64;
-  static std::atomic<int> known[kDevices][kResMaxSlices + 1];      // one more than the number; 0: not asked yet
+  static std::atomic<int> known[kDevices][kSlicedMaxSlices + 1];      // one more than the number; 0: not asked yet
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
   if (dev >= 0 && dev < kDevices) {
@@ -698,12 +698,12 @@ static int sliced_clusters(int slices) {
   attr[0].val.clusterDim = {static_cast<unsigned>(slices), 1, 1};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = static_cast<unsigned>(slices);
-  cfg.blockDim = kResThreads;
-  cfg.dynamicSmemBytes = ResidentSmem<D, 2, true>::kTotal;
+  cfg.blockDim = kSlicedThreads;
+  cfg.dynamicSmemBytes = SlicedSmem<D>::kTotal;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (dev < 0 || allow_sliced<D, SCORES>() != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, cross_resident_kernel<D, 2, SCORES, true>, &cfg) != cudaSuccess) {
+      cudaOccupancyMaxActiveClusters(&n, cross_sliced_kernel<D, SCORES>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -742,8 +742,8 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool score
     c.total = off;
     return c;
   }
-  const int slices = (Nk + kResMaxKeys - 1) / kResMaxKeys;
-  if (slices <= kResMaxSlices && Nq <= kResSlicedQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
+  const int slices = (Nk + kSlicedKeys - 1) / kSlicedKeys;
+  if (slices <= kSlicedMaxSlices && Nq <= kSlicedMaxQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
     c.slices = slices;
     c.NQT = (Nq + 127) / 128;
     c.res_ctas = static_cast<int>(tiles) * slices;
@@ -809,9 +809,9 @@ template <int D, int KG, bool SCORES>
 static int launch_resident(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                            const ResidentParams& rp, int ctas, cudaStream_t st) {
   constexpr int kSmem = ResidentSmem<D, KG>::kTotal;
-  if (cudaFuncSetAttribute(cross_resident_kernel<D, KG, SCORES, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+  if (cudaFuncSetAttribute(cross_resident_kernel<D, KG, SCORES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
     return AVSA_ERR_CUDA;
-  return launch_pdl(cross_resident_kernel<D, KG, SCORES, false>, ctas, kResThreads, kSmem, st, tq, tk, tv, to, rp) == cudaSuccess
+  return launch_pdl(cross_resident_kernel<D, KG, SCORES>, ctas, kResThreads, kSmem, st, tq, tk, tv, to, rp) == cudaSuccess
              ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -863,12 +863,12 @@ static int run_cross_resident(int B, int H, int Nq, int Nk, const avsa_bf16_4d& 
 }
 
 template <int D, bool SCORES>
-static int launch_sliced(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const ResidentParams& rp, int ctas,
+static int launch_sliced(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const SlicedParams& rp, int ctas,
                          cudaStream_t st) {
-  constexpr int kSmem = ResidentSmem<D, 2, true>::kTotal;
-  auto kernel = cross_resident_kernel<D, 2, SCORES, true>;
+  constexpr int kSmem = SlicedSmem<D>::kTotal;
+  auto kernel = cross_sliced_kernel<D, SCORES>;
   if (allow_sliced<D, SCORES>() != cudaSuccess) return AVSA_ERR_CUDA;
-  return launch_pdl_clusters(kernel, static_cast<unsigned>(rp.slices), ctas, kResThreads, kSmem, st, tq, tk, tv, tq, rp) == cudaSuccess
+  return launch_pdl_clusters(kernel, static_cast<unsigned>(rp.slices), ctas, kSlicedThreads, kSmem, st, tq, tk, tv, rp) == cudaSuccess
              ? AVSA_OK : AVSA_ERR_CUDA;
 }
 
@@ -880,7 +880,7 @@ static int run_cross_sliced(int B, int H, int Nq, int Nk, const avsa_bf16_4d& q,
   if (!encode_bf16_tile_map(&tq, q.ptr, B, H, Nq, D, q.stride_b, q.stride_h, q.stride_n, 128)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tk, k.ptr, B, H, Nk, D, k.stride_b, k.stride_h, k.stride_n, 128)) return AVSA_ERR_CUDA;
   if (!encode_bf16_tile_map(&tv, v.ptr, B, H, Nk, D, v.stride_b, v.stride_h, v.stride_n, 128)) return AVSA_ERR_CUDA;
-  ResidentParams rp = {};
+  SlicedParams rp = {};
   rp.lse = lse;
   rp.partial = reinterpret_cast<float*>(ws + c.off_partial);
   rp.part_o = o != nullptr ? reinterpret_cast<float*>(ws + c.off_part_o) : nullptr;

@@ -43,24 +43,18 @@ struct CtaStatus {
 
 struct ResidentParams {
   float* lse;               // [B,H,Nq] natural log, or null
-  float* partial;           // [CTA + pair][Nk] column sums (SLICED: [query tile][Nk])
+  float* partial;           // [CTA + pair][Nk] column sums
   StatusRecord* status;     // without scores: cleared in front of the kernel
   CtaStatus* cta_status;    // with scores: [gridDim.x]
   int H, Nq, NQT, Nk;
   int tiles, L;             // query tiles of all pairs, and per CTA
-  int slices;               // SLICED: CTAs of a query tile
-  float* part_o;            // SLICED: [pair][slice][NQT * 128][D] fp32, or null
   int nch0, nch1;           // chunks of 32 keys of the first group (both, with KG == 1), of the second
   int store_o;
   float scale_log2;
 };
 
-constexpr int kResMaxSlices = 16;          // the largest cluster there is (beyond 8 the kernel has to allow it)
-constexpr int kResSlicedQueries = 512;      // the most queries of a sliced call
-
-template <int D, int KG, bool SLICED = false>
+template <int D, int KG>
 struct ResidentSmem {
-  static constexpr int kQS = SLICED ? 1 : 2;                   // query tiles on chip
   static constexpr int kRows = KG * 128;                       // key rows held
   static constexpr int kPanel = kRows * 128;                   // 64 channels of them
   static constexpr int kKV = kRows * D * 2;
@@ -71,30 +65,23 @@ struct ResidentSmem {
   static constexpr int kK = 0;
   static constexpr int kV = kK + kKV;
   static constexpr int kQ = kV + kKV;
-  static constexpr int kStage = kQ + kQS * kQBytes;
+  static constexpr int kStage = kQ + 2 * kQBytes;
   static constexpr int kBars = kStage + 8 * kStageWarp;
-  static constexpr int kNumBars = 4 + 3 + 4 + 4 + 3 + 8 + 2 + 1 + (SLICED ? 4 : 0);
+  static constexpr int kNumBars = 4 + 3 + 4 + 4 + 3 + 8 + 2 + 1;
   static constexpr int kExch = kBars + (kNumBars * 8 + 15) / 16 * 16;      // float max[128], sum[2 sets][2][128]
-  static constexpr int kSlice = kExch + 5 * 128 * 4;           // SLICED: float2 (maximum, sum) [kResMaxSlices][128]
-  static constexpr int kMisc = kSlice + (SLICED ? kResMaxSlices * 128 * 8 : 0);      // tmem base, stop flag, first error (4), recomputed items (2)
+  static constexpr int kMisc = kExch + 5 * 128 * 4;            // tmem base, stop flag, first error (4), recomputed items (2)
   static constexpr int kTotal = kMisc + 32;
   static_assert(kTotal <= 232448, "shared memory of a CTA exceeded");
 };
 
 enum ResidentWhere { kResQEmpty = 81, kResKVEmpty, kResQFull, kResKFull, kResVFull, kResSFree, kResSFull, kResPFull, kResOFree,
-                     kResOFull, kResMax, kResSum, kResFlush, kResAlign, kResSlice };
+                     kResOFull, kResMax, kResSum, kResFlush, kResAlign };
 
-// SLICED (257 to 4096 keys, short calls): a cluster of CTAs takes a query tile of a pair, each CTA 129 to 256 of its keys (KG = 2).  They
-// tell each other their rows' maxima and sums (through distributed shared memory, a barrier for each quarter of the rows); from then on
-// every probability's weight is known where it is, as with few keys.  O leaves as fp32 in proportion, and sliced_finalize_kernel adds
-// the slices.  Two launches instead of four, and every exponential once: 8 heads x 72 queries x 2048 keys 19.6 -> 12.1 us, 2 x 72 x 300 15.7
-// -> 10.1, 24 x 109 x 1100 24.0 -> 13.3.
-template <int D, int KG, bool SCORES, bool SLICED>
+template <int D, int KG, bool SCORES>
 __global__ void __launch_bounds__(kResThreads, 1)
 cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                       const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmo, const ResidentParams p) {
-  using L = ResidentSmem<D, KG, SLICED>;
-  static_assert(!SLICED || KG == 2, "a slice is 129 to 256 keys");
+  using L = ResidentSmem<D, KG>;
   constexpr int NPANEL = D / 64;
   constexpr int QPANEL = 128 * 128;
   constexpr unsigned FULLM = 0xffffffffu;
@@ -104,8 +91,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
   auto BAR = [&](int i) { return bar0 + static_cast<uint32_t>(i) * 8u; };
   constexpr int Q_FULL = 0, Q_EMPTY = 2, K_FULL = 4, V_FULL = 5, KV_EMPTY = 6, S_FULL = 7 /* + group */, S_FREE = 9,
                 P_FULL = 11 /* + 2*group + part */, O_FULL = 15 /* + tile's group, KG == 1 */, O_FREE = 17, MAX = 18 /* + row quarter */,
-                SUM = 22, FLUSH = 26, DRAIN = 28, SLICE = 29 /* + row quarter */;
-  static_assert(DRAIN + 1 + (SLICED ? 4 : 0) <= L::kNumBars, "barrier table too small");
+                SUM = 22, FLUSH = 26, DRAIN = 28;
+  static_assert(DRAIN + 1 <= L::kNumBars, "barrier table too small");
   constexpr uint32_t TM_P = 256, TM_O = 384;
   // who reads O out: every thread half of its row's channels, or one group the whole rows
   constexpr bool kSplitO = KG == 2 && D == 128;
@@ -133,8 +120,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
       mbar_init(BAR(SUM + q), 64);
     }
     mbar_init(BAR(DRAIN), 1);
-    if (SLICED)
-      for (int q = 0; q < 4; q++) mbar_init(BAR(SLICE + q), p.slices);
     for (int i = 1; i < 8; i++) misc[i] = 0;
     fence_mbar_init();
     prefetch_tmap(&tmq);
@@ -149,7 +134,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (SLICED) cluster_sync_all();      // everyone's barriers are there
   const uint32_t tmem = static_cast<uint32_t>(misc[0]);
   pdl_wait();
 
@@ -179,21 +163,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
   };
 
   // The CTA's share of the stream of query tiles; a segment is the part of it that lies in one (batch, head) pair.
-  int pos0 = static_cast<int>(blockIdx.x) * p.L;
-  int pos_end = min(p.tiles, pos0 + p.L);
-  // its keys: from `kbase` on, in chunks of 32 for the two groups (both have all of them with KG == 1)
-  int kbase = 0, nkeys = p.Nk, nch0 = p.nch0, nch1 = p.nch1;
-  const int slice = SLICED ? static_cast<int>(blockIdx.x) % p.slices : 0;
-  if (SLICED) {
-    pos0 = static_cast<int>(blockIdx.x) / p.slices;
-    pos_end = pos0 + 1;
-    const int chunks = (p.Nk + 31) / 32, least = chunks / p.slices, more = chunks % p.slices;
-    const int n = least + (slice < more ? 1 : 0);
-    kbase = (slice * least + min(slice, more)) * 32;
-    nkeys = min(p.Nk - kbase, n * 32);
-    nch0 = 4;
-    nch1 = max(1, n - 4);      // (of a slice of four, of which there are few, the second group has keys that are left out)
-  }
+  const int pos0 = static_cast<int>(blockIdx.x) * p.L;
+  const int pos_end = min(p.tiles, pos0 + p.L);
 
   if ((smem_u32(smem) & 1023u) != 0u) {
     if (tid == 0) fail(AVSA_ERR_CUDA, kResAlign, 0);
@@ -210,14 +181,14 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           mbar_expect_tx(BAR(bar), L::kKV);
           for (int kt = 0; kt < KG; kt++)
             for (int pn = 0; pn < NPANEL; pn++)
-              tma_load_4d(smem_u32(smem + off) + pn * L::kPanel + kt * 128 * 128, tm, BAR(bar), pn * 64, kbase + kt * 128, h, b);
+              tma_load_4d(smem_u32(smem + off) + pn * L::kPanel + kt * 128 * 128, tm, BAR(bar), pn * 64, kt * 128, h, b);
         };
         if (k_loads > 0) ok = wait_or_stop(KV_EMPTY, (k_loads - 1) & 1, kResKVEmpty, k_loads);      // the pair before is done
         if (!ok) break;
         load_kv(K_FULL, L::kK, &tmk);
         k_loads++;
         for (int at = at0; at < at1; at++) {
-          const int s = T % L::kQS, f = T / L::kQS;
+          const int s = T & 1, f = T >> 1;
           if (f > 0) ok = wait_or_stop(Q_EMPTY + s, (f - 1) & 1, kResQEmpty, T);
           if (!ok) break;
           mbar_expect_tx(BAR(Q_FULL + s), L::kQBytes);
@@ -232,7 +203,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         pos += at1 - at0;
       }
       if (misc[1] != 0) {      // stopped: loads in flight must land before this CTA's shared memory is given away
-        for (int c = max(0, T - L::kQS); c < T; c++) mbar_wait(BAR(Q_FULL + c % L::kQS), (c / L::kQS) & 1);
+        for (int c = max(0, T - 2); c < T; c++) mbar_wait(BAR(Q_FULL + (c & 1)), (c >> 1) & 1);
         if (k_loads > 0) mbar_wait(BAR(K_FULL), (k_loads - 1) & 1);
         if (v_loads > 0) mbar_wait(BAR(V_FULL), (v_loads - 1) & 1);
       }
@@ -253,25 +224,24 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
     bool ok = true;
     // S of tile T; with KG == 2 the two halves of the keys by themselves (each group frees its own half)
     auto issue_qk = [&](int T, bool first, int seg) {
-      const int qs = T % L::kQS;
-      ok = wait_all(Q_FULL + qs, (T / L::kQS) & 1, kResQFull, T);
+      ok = wait_all(Q_FULL + (T & 1), (T >> 1) & 1, kResQFull, T);
       if (ok && first) ok = wait_all(K_FULL, seg & 1, kResKFull, T);
       for (int i = 0; i < KG && ok; i++) {
         const int g = KG == 2 ? i : T & 1, uses = KG == 2 ? T : T >> 1;
         if (uses > 0) ok = wait_all(S_FREE + g, (uses - 1) & 1, kResSFree, T);
         if (!ok) break;
         tc_fence_after();
-        const int key0 = i * nch0 * 32;
-        const uint32_t idesc = make_idesc_bf16(128, (i == 0 ? nch0 : nch1) * 32, 0, 0);
+        const int key0 = i * p.nch0 * 32;
+        const uint32_t idesc = make_idesc_bf16(128, (i == 0 ? p.nch0 : p.nch1) * 32, 0, 0);
         const uint32_t tm_s = tmem_u + (KG == 2 ? key0 : g * 128);
-        const uint32_t k_lo = k_lo0 + key0 * (128 >> 4), q_lo = q_lo0 + qs * (L::kQBytes >> 4);
+        const uint32_t k_lo = k_lo0 + key0 * (128 >> 4), q_lo = q_lo0 + (T & 1) * (L::kQBytes >> 4);
         if (leader) {
 #pragma unroll
           for (int ks = 0; ks < D / 16; ks++)
             umma_ss(tm_s, desc64(q_lo + (((ks >> 2) * QPANEL + (ks & 3) * 32) >> 4)),
                     desc64(k_lo + (((ks >> 2) * L::kPanel + (ks & 3) * 32) >> 4)), idesc, ks > 0 ? 1u : 0u);
           umma_commit(BAR(S_FULL + g));
-          if (i == KG - 1) umma_commit(BAR(Q_EMPTY + qs));
+          if (i == KG - 1) umma_commit(BAR(Q_EMPTY + (T & 1)));
         }
         __syncwarp();
       }
@@ -284,7 +254,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
       for (int part = 0; part < 2 && ok; part++) {
         for (int i = 0; i < KG && ok; i++) {
           const int g = KG == 2 ? i : T & 1, uses = KG == 2 ? T : T >> 1;
-          const int nch = i == 0 ? nch0 : nch1, key0 = i * nch0 * 32;
+          const int nch = i == 0 ? p.nch0 : p.nch1, key0 = i * p.nch0 * 32;
           if (part == 1 && nch <= 2) continue;
           ok = wait_all(P_FULL + 2 * g + part, uses & 1, kResPFull, T);
           if (!ok) break;
@@ -333,8 +303,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
     const int w = (warp - 4) >> 2, quad = warp & 3, row = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     const bool upper = KG == 2 && w == 1;            // the second half of the keys (with KG == 1 both groups have them all)
-    const int nch = upper ? nch1 : nch0, key0 = upper ? nch0 * 32 : 0;
-    const int kv = min(nkeys - key0, nch * 32);       // keys that exist
+    const int nch = upper ? p.nch1 : p.nch0, key0 = upper ? p.nch0 * 32 : 0;
+    const int kv = min(p.Nk - key0, nch * 32);       // keys that exist
     const uint32_t tm_s = tmem + lane_off + (KG == 2 ? key0 : w * 128);
     const uint32_t tm_p = tmem + lane_off + TM_P + (KG == 2 ? key0 / 2 : w * 64);
     const uint32_t tm_o = tmem + lane_off + TM_O;
@@ -342,16 +312,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
     const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
     uint64_t acc[SCORES ? 16 : 1];                   // column sums (8 i + 2 (lane mod 4) and the next) over a quarter of the rows
     bool ok = true;
-    // SLICED: all slices' maxima and sums are there
-    auto wait_slices = [&]() -> bool {
-      bool there = mbar_try_wait_cluster(BAR(SLICE + quad), 0);
-      const long long t0 = clock64();
-      while (!there && misc[1] == 0) {
-        there = mbar_try_wait_cluster(BAR(SLICE + quad), 0);
-        if (!there && clock64() - t0 > AVSA_WAIT_LIMIT_CYCLES) fail(AVSA_ERR_TIMEOUT, kResSlice, 0);
-      }
-      return __all_sync(FULLM, there);
-    };
     int T = 0, seg = 0;
     for (int pos = pos0; pos < pos_end && ok; seg++) {
       const int bh = pos / p.NQT, h = bh % p.H, b = bh / p.H;
@@ -512,25 +472,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             lsum = fmaf(other, first, lsum);
           }
         }
-        float inv = 1.0f / lsum;
-        if (SLICED) {
-          // ---- what the rows' maxima and sums are over all slices, in the slices' order
-          const float2* of_slice = reinterpret_cast<const float2*>(smem + L::kSlice) + row;
-          if (w == 0) {
-            const uint32_t mine = smem_u32(of_slice + slice * 128);
-            for (int c = 0; c < p.slices; c++) cluster_store_f32x2(cluster_addr(mine, c), m, lsum);
-            __syncwarp();
-            if (lane < p.slices) cluster_arrive(cluster_addr(BAR(SLICE + quad), lane));
-          }
-          ok = wait_slices();
-          if (!ok) break;
-          float M = -INFINITY, all = 0.f;
-          for (int c = 0; c < p.slices; c++) M = fmaxf(M, of_slice[c * 128].x);
-          for (int c = 0; c < p.slices; c++) all = fmaf(of_slice[c * 128].y, exp2f(of_slice[c * 128].x - M), all);
-          inv = exp2f(m - M) / all;
-          m = M;
-          lsum = all;
-        }
+        const float inv = 1.0f / lsum;
         if (SCORES) {
           // ---- column sums: a quarter of the rows a lane (rows beyond the last query add nothing)
           const float wt = qrow < p.Nq ? own * inv : 0.f;
@@ -557,7 +499,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             }
           }
         }
-        if (p.lse != nullptr && (KG == 1 || w == 0) && slice == 0 && qrow < p.Nq)
+        if (p.lse != nullptr && (KG == 1 || w == 0) && qrow < p.Nq)
           p.lse[static_cast<int64_t>(bh) * p.Nq + qrow] = (m + log2f(lsum)) * 0.6931471805599453f;
         // ---- O
         // (KG == 1: a barrier of the group's own, whose phases it sees one by one; of a common one it would wait for every other
@@ -567,10 +509,8 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
         tc_fence_after();
         if (KG == 1 || kSplitO || (T & 1) == w) {
           constexpr int COLS = kSplitO ? 64 : D;
-          if (!SLICED) {
-            if (lane == 0) tma_store_wait_read();      // the warp's last store has read its staging block
-            __syncwarp();
-          }
+          if (lane == 0) tma_store_wait_read();      // the warp's last store has read its staging block
+          __syncwarp();
 #pragma unroll
           for (int c = 0; c < COLS / 64; c++) {
             tmem_ld64(tm_o + (kSplitO ? w * 64 : c * 64), s);
@@ -578,19 +518,6 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
             if (c == COLS / 64 - 1) {
               tc_fence_before();
               mbar_arrive(BAR(O_FREE));
-            }
-            if (SLICED) {
-              if (p.part_o != nullptr && qrow < p.Nq) {
-                float* dst = p.part_o + ((static_cast<int64_t>(bh) * p.slices + slice) * p.NQT * 128 + qrow) * D + (kSplitO ? w * 64 : c * 64);
-#pragma unroll
-                for (int g = 0; g < 8; g++) {
-                  uint32_t r[8];
-#pragma unroll
-                  for (int i = 0; i < 8; i++) r[i] = __float_as_uint(__uint_as_float(s[g * 8 + i]) * inv);
-                  st_global_v8(dst + g * 8, r);
-                }
-              }
-              continue;
             }
 #pragma unroll
             for (int g = 0; g < 8; g++) {
@@ -602,9 +529,9 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
               *reinterpret_cast<uint4*>(stage + c * 4096 + lane * 128 + ((g ^ (lane & 7)) << 4)) = val;
             }
           }
-          if (!SLICED) fence_proxy_async();
+          fence_proxy_async();
           __syncwarp();
-          if (!SLICED && lane == 0 && p.store_o) {
+          if (lane == 0 && p.store_o) {
             for (int pn = 0; pn < COLS / 64; pn++)
               tma_store_4d(&tmo, smem_u32(stage) + pn * 4096, (kSplitO ? w * 64 : 0) + pn * 64, (at0 + t) * 128 + quad * 32, h, b);
             tma_store_commit();
@@ -634,7 +561,7 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
           float s = 0.f;
           for (int i = 0; i < (KG == 2 ? 4 : 8); i++)
             s += reinterpret_cast<const float*>(smem + L::kStage + ((KG == 2 ? w * 4 : 0) + i) * L::kStageWarp)[row];
-          p.partial[(SLICED ? static_cast<int64_t>(pos0) : static_cast<int64_t>(blockIdx.x) + bh) * p.Nk + kbase + key0 + row] = s;
+          p.partial[(static_cast<int64_t>(blockIdx.x) + bh) * p.Nk + key0 + row] = s;
         }
         mbar_arrive(BAR(FLUSH + 1));
         ok = wait_all(FLUSH + 1, seg & 1, kResFlush, seg);
@@ -645,11 +572,10 @@ cross_resident_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_cons
   }
   tc_fence_before();
   __syncthreads();
-  if (SLICED) cluster_sync_all();      // nobody writes into this CTA's shared memory any more
   pdl_launch();      // not earlier: CTAs staged behind this grid would share the SMs with its last ones
   if (warp == 2) tmem_dealloc(tmem, 512);
   if (tid == 0) {
-    if (SCORES || SLICED) {
+    if (SCORES) {
       p.cta_status[blockIdx.x] = CtaStatus{misc[2], misc[3], misc[4], misc[5], misc[7], {0, 0, 0}};
     } else {
       if (misc[2] != 0) report_status(p.status, misc[2], misc[3], misc[4], misc[5]);

@@ -242,6 +242,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld32(taddr, r); }
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[64]) { tmem_ld64(taddr, r); }
 // The wait, and the loaded registers through it: nothing that uses them can be scheduled in front of it.
 __device__ __forceinline__ void tie_regs(uint32_t (&r)[32]) {
   asm volatile(""
