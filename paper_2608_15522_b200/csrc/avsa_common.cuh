@@ -47,7 +47,7 @@ __device__ __forceinline__ void report_status(StatusRecord* st, int code, int wh
 //   - score_select_kernel lets its successor go before it waits itself: the successor must wait before it touches
 //     anything (every first kernel of a call and expand_blocks_kernel do);
 //   - indicators_finalize_kernel reads the saliencies before its wait; l1_partials_kernel in front of it goes by the rule;
-//   - colsum_kernel, colsum_rev_kernel and cross_resident_kernel let their successor go at their end only (the reason stands
+//   - colsum_kernel, colsum_rev_kernel, cross_resident_kernel and cross_sliced_kernel let their successor go at their end only (the reason stands
 //     at the first).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

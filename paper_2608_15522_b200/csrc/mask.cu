@@ -450,9 +450,9 @@ __global__ void __launch_bounds__(128) row_select_kernel(const float* __restrict
 // ------------------------------------------------------------------------------------------------
 // (ii)+(iv) fused: block scores Bs[bh, i, j] = qbar[bh,i,:] . kbar[bh,j,:] * scale for a strip of 16 query
 // blocks against every key block, kept in shared memory, then the lists of those 16 rows straight from
-// there.  One CTA of 8 warps per strip: each warp computes 32-column chunks of the strip with 3xTF32 m16n8k8 MMAs
+// there.  A CTA of 8 warps, or two, per strip: each warp computes chunks of 8 to 32 columns of the strip with 3xTF32 m16n8k8 MMAs
 // (A = the strip's pooled queries from shared memory, B = pooled keys read from L2 as 16-byte pieces), then takes
-// two rows of the strip through the select (see select_row).  Against separate score and list kernels
+// its rows of the strip through the select (see select_row).  Against separate score and list kernels
 // this saves a launch, a drain and a round trip of the scores through L2 on the latency chain behind the
 // pooling kernel.
 //   The channel order inside each group of 16 is permuted identically for both operands (lane t of a
