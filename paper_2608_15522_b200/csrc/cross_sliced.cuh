@@ -222,10 +222,9 @@ cross_sliced_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_consta
 #pragma unroll
       for (int j = 16; j < 128; j += 2) m8[(j >> 1) & 7] = max3f(m8[(j >> 1) & 7], __uint_as_float(s[j]), __uint_as_float(s[j + 1]));
       m = p.scale_log2 * fmaxf(max3f(m8[0], m8[1], m8[2]), fmaxf(max3f(m8[3], m8[4], m8[5]), fmaxf(m8[6], m8[7])));
-      if (kv <= 0) m = -INFINITY;
       // ---- exponentials: P (bf16) for the product with V, p (fp32) over the logits for the column sums
       const uint64_t c2 = pack_f32x2(p.scale_log2, p.scale_log2);
-      const float ref = kv > 0 ? m : 0.f;      // (without keys: probabilities of 0, a maximum that weighs nothing)
+      const float ref = fmaxf(m, -3.402823466e38f);      // (no keys, or none with a logit above -inf: probabilities of 0, and no weight)
       const uint64_t nm2 = pack_f32x2(-ref, -ref);
       uint64_t sum2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll

@@ -843,6 +843,25 @@ def test_cross_attention_sliced_keys(B, H, Nq, Nk, d, growth):
     _close_lse(_np64(lse2), want_lse, "sliced lse without scores")
 
 
+@pytest.mark.parametrize("Nq,Nk,d", [(40, 333, 64), (40, 400, 128), (130, 700, 64), (72, 2048, 128)])
+@pytest.mark.parametrize("first,last", [(0, 128), (128, 256), (224, 333), (0, 332)])
+def test_cross_attention_sliced_keys_that_all_have_logits_of_minus_infinity(Nq, Nk, d, first, last):
+    """Keys that mask themselves (products below the range of fp32) fill a half of a slice, a slice, or all but a few keys: they weigh
+    nothing, and the rest of the row is as without them."""
+    B, H = 1, 3
+    g = torch.Generator().manual_seed(Nk)
+    q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, Nk, Nk))
+    q = q.abs() + 0.1
+    k[:, :, first:last] = -3e38
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+    o, lse, s, ws = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), score_gamma=1.0 / (H * Nq))
+    _status_ok(ws)
+    _close(_np64(o), want_o, "masked keys O")
+    _close_lse(_np64(lse), want_lse, "masked keys lse")
+    _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "masked keys scores")
+
+
 @pytest.mark.parametrize("reverse", [False, True])
 def test_cross_attention_row_maxima_growing_along_the_key_axis(reverse):
     """Pass 1 runs on the fast kernel too (key axis split across work items, or one item per query tile in the
