@@ -24,6 +24,9 @@
  *     when a device-side check fails (a wait that ran out of time, or a malformed column list) -- then at
  *     byte 16 a count of work items or query tiles (see below) and at byte 20 the head of the persistent
  *     kernels' work queue.  Calls on the same workspace must not overlap on the GPU.
+ *   - Alignment of `ws`: 32 bytes are enough for every call, 4 bytes for sparse self-attention, for cross-attention
+ *     against at most 256 keys and for a mask under given block scores.  With less than a call's kernels need
+ *     (16 or 32 bytes, by shape) it returns AVSA_ERR_INVALID_ARG and enqueues nothing.
  *   - The attention calls (cross-attention against more than 256 keys that is not short, sparse self-attention, protected rows) run
  *     a kernel that normalises each row by the maximum of its first key tile instead of a running maximum
  *     (softmax is invariant to that shift), and recompute with exact rescaling the work items whose rows outgrew
@@ -59,7 +62,7 @@ extern "C" {
 
 typedef enum {
   AVSA_OK = 0,
-  AVSA_ERR_INVALID_ARG = 1,  /* null pointer, bad size, bad alignment or stride */
+  AVSA_ERR_INVALID_ARG = 1,  /* null pointer, bad size, bad stride or alignment (of a tensor or of ws) */
   AVSA_ERR_UNSUPPORTED = 2,  /* (blk, d) combination or device not supported */
   AVSA_ERR_WORKSPACE = 3,    /* ws is NULL or smaller than *_workspace_bytes() */
   AVSA_ERR_CUDA = 4,         /* a CUDA runtime / driver call failed */

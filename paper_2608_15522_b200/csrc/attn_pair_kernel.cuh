@@ -162,12 +162,16 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant_
   auto list_of = [&](int item) { return p.entries + static_cast<int64_t>(item) * (2 * p.NP); };
   // loads the tiles of an item through a ring of stages: `full`, `empty` its barriers, `c` the tiles loaded so far over all items
   auto load_tiles = [&](const AttnItem& it, const CUtensorMap* tm, int off, int stages, int full, int empty, int where, int& c) -> bool {
-    const int2* list = reinterpret_cast<const int2*>(list_of(it.item));
+    const int32_t* list = list_of(it.item);
     for (int t0 = 0; t0 < it.cnt; t0 += 32) {
-      const int2 mine = t0 + lane < it.cnt ? list[t0 + lane] : make_int2(0, 0);
+      int mine0 = 0, mine1 = 0;      // (two loads: the workspace need not be aligned to 8 bytes)
+      if (t0 + lane < it.cnt) {
+        mine0 = list[2 * (t0 + lane)];
+        mine1 = list[2 * (t0 + lane) + 1];
+      }
       const int nn = min(32, it.cnt - t0);
       for (int j = 0; j < nn; j++) {
-        const int kb0 = __shfl_sync(FULLM, mine.x, j) & kPairBlock, kb1 = __shfl_sync(FULLM, mine.y, j) & kPairBlock;
+        const int kb0 = __shfl_sync(FULLM, mine0, j) & kPairBlock, kb1 = __shfl_sync(FULLM, mine1, j) & kPairBlock;
         const int s = c % stages, f = c / stages;
         int good = 1;
         if (lane == 0) {

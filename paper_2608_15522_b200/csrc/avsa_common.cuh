@@ -99,6 +99,12 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The widest access of a call to its workspace (whose parts begin at multiples of 256 bytes) needs this alignment of it.
+inline bool ws_aligned(const void* ws, size_t bytes) { return (reinterpret_cast<uintptr_t>(ws) & (bytes - 1)) == 0; }
+constexpr size_t kWsInts = 4;       // the status record, counts, indices, single floats
+constexpr size_t kWsVectors = 16;   // float4, cp.async, tensor maps
+constexpr size_t kWsParts = 32;     // fp32 parts of O (st_global_v8)
+
 // A bf16 [B,H,N,d] view is usable when its base is 16-byte aligned and its strides are multiples of
 // 8 elements (so every row starts on a 16-byte boundary) and positive.
 inline bool tensor_ok(const avsa_bf16_4d& t, int B, int H) {

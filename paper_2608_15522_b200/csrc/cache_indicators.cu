@@ -205,6 +205,7 @@ extern "C" int avsa_cache_indicators(int B, int Nv, int Na, int C, const void* y
   if (B > 65535) return AVSA_ERR_UNSUPPORTED;
   const IndPlan p = make_ind_plan(B, Nv, Na);
   if (ws == nullptr || ws_bytes < p.total) return AVSA_ERR_WORKSPACE;
+  if (!ws_aligned(ws, kWsVectors)) return AVSA_ERR_INVALID_ARG;
   cudaStream_t st = as_stream(stream);
   uint8_t* base = static_cast<uint8_t*>(ws);
   float* pv = reinterpret_cast<float*>(base + p.off_v);

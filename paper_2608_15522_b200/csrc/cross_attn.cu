@@ -5,6 +5,7 @@
 //           the queries -> per-head column sums -> fixed-order head sum with the beta/gamma blend
 // With at most 256 keys both are one pass over the queries (cross_resident.cuh), and in short calls with at most 4096 too, the keys
 // sliced over a cluster of CTAs (cross_sliced.cuh).
+#include <algorithm>
 #include <atomic>
 
 #include "attn_persist_kernel.cuh"
@@ -719,7 +720,7 @@ static long long max_sliced_tiles(int slices, int d, bool scores) {
                          : (scores ? sliced_clusters<64, true>(slices) : sliced_clusters<64, false>(slices));
   return slices == 2 && d == 128 && !scores && n > 32 ? 32 : n;
 }
-static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool scores) {
+static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool scores, bool may_slice) {
   CrossPlan c = {};
   // Few keys: everything in one kernel, whatever the number of queries (faster from 2 heads x 32 queries to 64 x 19200, with scores
   // and without: cross_resident.cuh).  More than 256 keys of 128 channels do not fit an SM's shared memory beside the tiles, nor
@@ -743,7 +744,7 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool score
     return c;
   }
   const int slices = (Nk + kSlicedKeys - 1) / kSlicedKeys;
-  if (slices <= kSlicedMaxSlices && Nq <= kSlicedMaxQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
+  if (may_slice && slices <= kSlicedMaxSlices && Nq <= kSlicedMaxQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
     c.slices = slices;
     c.NQT = (Nq + 127) / 128;
     c.res_ctas = static_cast<int>(tiles) * slices;
@@ -1056,8 +1057,10 @@ using namespace avsa;
 
 extern "C" size_t avsa_cross_attn_scores_workspace_bytes(int B, int H, int Nq, int Nk, int d) {
   if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128) || !pairs_ok(B, H)) return 0;
-  const size_t with = make_cross_plan(B, H, Nq, Nk, d, true).total, without = make_cross_plan(B, H, Nq, Nk, d, false).total;
-  return with > without ? with : without;
+  // what any call of this shape may take: with scores and without, sliced and not
+  const size_t with = make_cross_plan(B, H, Nq, Nk, d, true, true).total, without = make_cross_plan(B, H, Nq, Nk, d, false, true).total;
+  const size_t unsliced = make_cross_plan(B, H, Nq, Nk, d, true, false).total;
+  return std::max({with, without, unsliced});
 }
 
 extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_bf16_4d q, avsa_bf16_4d k,
@@ -1072,8 +1075,11 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (!tensor_ok(q, B, H) || !tensor_ok(k, B, H) || !tensor_ok(v, B, H)) return AVSA_ERR_INVALID_ARG;
   if (o_bf16 != nullptr && !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
-  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, scores != nullptr);
+  // (a workspace that is not aligned for the slices' parts of O takes the two passes, which write none where no row is cut)
+  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, scores != nullptr, ws_aligned(ws, kWsParts));
   if (ws == nullptr || ws_bytes < c.total) return AVSA_ERR_WORKSPACE;
+  const size_t widest = c.resident || c.slices > 0 ? kWsInts : !c.rs.whole_rows() ? kWsParts : scores != nullptr && c.reverse ? kWsVectors : kWsInts;
+  if (!ws_aligned(ws, widest)) return AVSA_ERR_INVALID_ARG;
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
   uint8_t* base = static_cast<uint8_t*>(ws);

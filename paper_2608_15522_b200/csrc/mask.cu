@@ -828,6 +828,10 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   if (min_tokens > blk) return AVSA_ERR_INVALID_ARG;
   const MaskWorkspace w = mask_ws_layout(B, H, N, d, blk);
   if (ws == nullptr || ws_bytes < w.total) return AVSA_ERR_WORKSPACE;
+  // short sequences in one launch keep their pooled means on chip, given scores need none
+  const bool one_launch = !by_block_sum && !given && N <= kSelectPoolTokens && static_cast<int64_t>(B) * H <= 65535;
+  const bool whole = one_launch && N <= short_tokens(d) && static_cast<int64_t>(B) * H <= persistent_grid(1 << 30);
+  if (!ws_aligned(ws, given || whole ? kWsInts : kWsVectors)) return AVSA_ERR_INVALID_ARG;
   cudaStream_t st = as_stream(stream);
   uint8_t* base = static_cast<uint8_t*>(ws);
   float* qbar = reinterpret_cast<float*>(base + w.qbar);
@@ -836,8 +840,7 @@ extern "C" int avsa_build_block_mask(int B, int H, int N, int d, int blk, avsa_b
   uint8_t* pblk = prot_blk != nullptr ? prot_blk : base + w.pblk;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
 
-  const bool one_launch = !by_block_sum && !given && N <= kSelectPoolTokens && static_cast<int64_t>(B) * H <= 65535;
-  if (one_launch && N <= short_tokens(d) && static_cast<int64_t>(B) * H <= persistent_grid(1 << 30)) {
+  if (whole) {
     const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(q.ptr);
     const __nv_bfloat16* kp = static_cast<const __nv_bfloat16*>(k.ptr);
     auto kernel = d == 128 ? mask_short_kernel<128> : mask_short_kernel<64>;

@@ -213,6 +213,8 @@ extern "C" int avsa_protected_rows_attn(int B, int H, int N, int d, int blk, avs
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
   const ProtPlan c = make_prot_plan(B, H, N, d, n_protect);
   if (ws == nullptr || ws_bytes < c.total) return AVSA_ERR_WORKSPACE;
+  // (the gathered queries, and the parts of rows that are cut)
+  if (!ws_aligned(ws, n_protect == 0 ? kWsInts : c.rs.whole_rows() ? kWsVectors : kWsParts)) return AVSA_ERR_INVALID_ARG;
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   const float scale = softmax_scale != 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d));
   if (n_protect == 0) {

@@ -265,6 +265,7 @@ using namespace avsa;
 
 extern "C" int avsa_selftest_bounded_wait(void* ws, size_t ws_bytes, long long limit_cycles, void* stream) {
   if (ws == nullptr || ws_bytes < kStatusBytes) return AVSA_ERR_WORKSPACE;
+  if (!ws_aligned(ws, kWsInts)) return AVSA_ERR_INVALID_ARG;
   if (limit_cycles < 0 || limit_cycles > 2000000000ll) return AVSA_ERR_INVALID_ARG;     // about a second at most
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   bounded_wait_selftest_kernel<<<1, 32, 0, as_stream(stream)>>>(static_cast<StatusRecord*>(ws), limit_cycles);
@@ -289,6 +290,7 @@ extern "C" int avsa_sparse_self_attn(int B, int H, int N, int d, int blk, avsa_b
   if (col_idx == nullptr || col_cnt == nullptr || o_bf16 == nullptr || !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
   if (ws == nullptr || ws_bytes < avsa_sparse_self_attn_workspace_bytes(B, H, N, d, blk)) return AVSA_ERR_WORKSPACE;
+  if (!ws_aligned(ws, kWsInts)) return AVSA_ERR_INVALID_ARG;
   if (!device_is_sm100()) return AVSA_ERR_UNSUPPORTED;
   cudaStream_t st = as_stream(stream);
   AttnParams prm = {};

@@ -1147,6 +1147,54 @@ def test_host_side_argument_errors():
 
 
 # ------------------------------------------------------------------------------------------- caller-owned scratch
+@pytest.mark.parametrize("offset", [4, 16])
+def test_workspaces_cut_out_of_an_arena(offset):
+    """Workspaces at 4 and 16 bytes from an aligned address: the bits of the aligned call, or refused where wider accesses are made.  Short
+    cross-attention against more than 256 keys goes another way there (the sliced one writes parts of O 32 bytes at a time): the
+    same within the bars, or refused where that way cuts rows too."""
+    g = torch.Generator(device="cuda").manual_seed(4)
+    R = lambda *s: torch.randn(s, generator=g, device="cuda").bfloat16()
+
+    def check(call, nbytes, takes, exact=True):
+        """`takes`: the alignment that the call takes (None: either way)."""
+        n = max(nbytes, 256)
+        ws = torch.empty(n + 32, dtype=torch.uint8, device="cuda")[offset:offset + n]
+        assert ws.data_ptr() % 32 == offset
+        try:
+            got = call(ws)
+        except av.AvsaError as e:
+            assert e.status == av.AVSA_ERR_INVALID_ARG and (takes is None or offset % takes != 0)
+            return
+        assert takes is None or offset % takes == 0
+        _status_ok(ws)
+        for x, y in zip(call(None), got):
+            assert torch.equal(x, y) if exact else (x.float() - y.float()).abs().max() <= 2e-2      # (O; LSE and scores differ less)
+
+    for H, N, d in ((3, 700, 128), (5, 64 * 70 + 9, 64), (2, 300, 64)):
+        q, k, v = R(1, H, N, d), R(1, H, N, d), R(1, H, N, d)
+        s = torch.rand((1, N), generator=g, device="cuda")
+        NB, n_protect = (N + d - 1) // d, N // 9
+        names = ("block_scores", "col_idx", "col_cnt", "prot_tok", "prot_blk")
+        mask = lambda ws, **kw: [av.avsa_build_block_mask(q, k, s, n_protect, max(1, NB // 4), d, ws=ws, **kw)[x] for x in names]
+        m, n = mask(None), av.avsa_build_block_mask_workspace_bytes(1, H, N, d, d)
+        check(mask, n, 4 if N == 300 else 16)
+        check(lambda ws: mask(ws, block_scores=m[0], flags=av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES), n, 4)
+        check(lambda ws: av.avsa_sparse_self_attn(q, k, v, m[1], m[2], d, want_lse=True, ws=ws)[:2],
+              av.avsa_sparse_self_attn_workspace_bytes(1, H, N, d, d), 4)
+
+        def rows(ws):
+            o = torch.zeros_like(q)
+            av.avsa_protected_rows_attn(q, k, v, m[3], n_protect, d, o, ws=ws)
+            return (o,)
+        check(rows, av.avsa_protected_rows_attn_workspace_bytes(1, H, N, d, d, n_protect), 16 if offset < 16 else None)
+    for B, H, Nq, Nk, d, takes in ((1, 3, 700, 200, 128, 4), (2, 3, 140, 333, 64, None), (1, 40, 100, 400, 128, None), (1, 2, 60, 9000, 64, 32)):
+        q, k, v = R(B, H, Nq, d), R(B, H, Nk, d), R(B, H, Nk, d)
+        check(lambda ws: av.avsa_cross_attn_scores(q, k, v, ws=ws, score_gamma=1.0 / (H * Nq))[:3],
+              av.avsa_cross_attn_scores_workspace_bytes(B, H, Nq, Nk, d), takes, exact=Nk <= 256)
+    y = [R(1, 64, 64) for _ in range(4)]
+    check(lambda ws: av.avsa_cache_indicators(*y, ws=ws)[:1], av.avsa_cache_indicators_workspace_bytes(1, 64, 64, 64), 16)
+
+
 @pytest.mark.parametrize("name", ["tiny", "medium128"])
 def test_results_do_not_depend_on_what_the_buffers_held_before(name):
     """Workspaces and outputs are caller-owned and arrive with arbitrary contents: every call must produce the

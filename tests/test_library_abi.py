@@ -5,6 +5,9 @@ import re
 import subprocess
 import sys
 
+import pytest
+import torch
+
 from paper_2608_15522_b200 import binding as av
 from paper_2608_15522_b200 import build
 
@@ -61,3 +64,35 @@ def test_more_pairs_than_32_bits_count_are_refused():
     """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     assert r.returncode == 0, r.stdout
+
+
+_T = av._Bf16Tensor4(4096, 64 * 4096, 4096, 64)
+_T128 = av._Bf16Tensor4(4096, 128 * 4096, 4096, 128)
+
+
+def _call(name, ws):
+    """A call that nothing is wrong with but, perhaps, the alignment of its workspace."""
+    lib, p, big = av.load_library(), 8192, 1 << 40
+    cross = lambda nq, nk, t, d, scores: lib.avsa_cross_attn_scores(1, 2, nq, nk, d, t, t, t, p, p, p if scores else None, 0.0, 1.0, 0.0, ws, big, 0)
+    mask = lambda n, flags: lib.avsa_build_block_mask(1, 2, n, 64, 64, _T, _T, p, 3, 1, flags, 0.0, p, p, p, p, p, ws, big, 0)
+    sparse = lambda n, t, d: lib.avsa_sparse_self_attn(1, 24, n, d, d, t, t, t, p, p, p, p, 0.0, ws, big, 0)
+    protected = lambda n_protect: lib.avsa_protected_rows_attn(1, 2, 4096, 128, 128, _T128, _T128, _T128, p, n_protect, p, p, 0.0, ws, big, 0)
+    return {"sparse": lambda: sparse(4096, _T128, 128), "sparse_pairs": lambda: sparse(64 * 64, _T, 64),
+            "mask": lambda: mask(4096, av.AVSA_PROTECT_ROWS), "mask_select_in_pooling": lambda: mask(500, av.AVSA_PROTECT_ROWS),
+            "mask_short": lambda: mask(200, av.AVSA_PROTECT_ROWS), "mask_given": lambda: mask(4096, av.AVSA_PROTECT_ROWS | av.AVSA_USE_GIVEN_BLOCK_SCORES),
+            "cross_few_keys": lambda: cross(4096, 200, _T, 64, True), "cross_parts": lambda: cross(100, 32768, _T, 64, True),
+            "cross_whole_rows": lambda: cross(64 * 1024, 300, _T, 64, False), "cross_whole_rows_reverse": lambda: cross(64 * 1024, 300, _T, 64, True),
+            "protected_none": lambda: protected(0), "protected_parts": lambda: protected(200),
+            "indicators": lambda: lib.avsa_cache_indicators(1, 64, 64, 64, 4096, 4096, 4096, 4096, None, None, None, 0.5, 0.1, 0.2, 1e-6, p, ws, big, 0)}[name]()
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the accepted calls would be launched")
+@pytest.mark.parametrize("name,needs", [
+    ("sparse", 4), ("sparse_pairs", 4), ("mask", 16), ("mask_select_in_pooling", 16), ("mask_short", 4), ("mask_given", 4),
+    ("cross_few_keys", 4), ("cross_parts", 32), ("cross_whole_rows", 4), ("cross_whole_rows_reverse", 16), ("protected_none", 4),
+    ("protected_parts", 32), ("indicators", 16)])
+def test_a_workspace_less_aligned_than_its_accesses_is_refused(name, needs):
+    """By every call, before anything is enqueued; where only words of 4 bytes are touched, 4 bytes are enough."""
+    for offset in (1, 2, 4, 8, 16, 32):
+        refused = _call(name, (1 << 20) + offset) == av.AVSA_ERR_INVALID_ARG
+        assert refused == (offset % needs != 0), offset
