@@ -19,7 +19,8 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  No call reads device
  *     data on the host, so the calls may be recorded into a CUDA graph by stream capture (not on the legacy
  *     default stream) and replayed; pointers, sizes and counts are fixed at capture time.
- *   - `ws` is scratch of at least the matching *_workspace_bytes().  Its first AVSA_STATUS_BYTES (256) bytes
+ *   - `ws` is scratch of at least the matching *_workspace_bytes(), which depends on the shape and on the number of SMs
+ *     of the current device (148 are assumed where there is none) and makes no context.  Its first AVSA_STATUS_BYTES (256) bytes
  *     are reserved for a 24-byte status record of six int32: code (avsa_status), where, item, aux -- filled
  *     when a device-side check fails (a wait that ran out of time, or a malformed column list) -- then at
  *     byte 16 a count of work items or query tiles (see below) and at byte 20 the head of the persistent

@@ -10,10 +10,20 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
+typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
+typedef CUresult (*CtxGetDeviceFn)(CUdevice*);
+typedef CUresult (*PrimaryStateFn)(CUdevice, unsigned int*, int*);
+typedef CUresult (*PrimaryRetainFn)(CUcontext*, CUdevice);
+typedef CUresult (*PrimaryReleaseFn)(CUdevice);
 
 struct DriverFns {
   EncodeTiledFn encode = nullptr;
   CtxGetCurrentFn current = nullptr;
+  CtxGetIdFn id = nullptr;
+  CtxGetDeviceFn device = nullptr;
+  PrimaryStateFn primary_state = nullptr;
+  PrimaryRetainFn primary_retain = nullptr;
+  PrimaryReleaseFn primary_release = nullptr;
 };
 
 static const DriverFns& driver_fns() {
@@ -27,6 +37,11 @@ static const DriverFns& driver_fns() {
     };
     fns.encode = reinterpret_cast<EncodeTiledFn>(get("cuTensorMapEncodeTiled"));
     fns.current = reinterpret_cast<CtxGetCurrentFn>(get("cuCtxGetCurrent"));
+    fns.id = reinterpret_cast<CtxGetIdFn>(get("cuCtxGetId"));
+    fns.device = reinterpret_cast<CtxGetDeviceFn>(get("cuCtxGetDevice"));
+    fns.primary_state = reinterpret_cast<PrimaryStateFn>(get("cuDevicePrimaryCtxGetState"));
+    fns.primary_retain = reinterpret_cast<PrimaryRetainFn>(get("cuDevicePrimaryCtxRetain"));
+    fns.primary_release = reinterpret_cast<PrimaryReleaseFn>(get("cuDevicePrimaryCtxRelease"));
   });
   return fns;
 }
@@ -58,6 +73,27 @@ bool encode_bf16_tile_map(CUtensorMap* map, const void* ptr, int B, int H, int N
   if (fns.current(&ctx) == CUDA_SUCCESS && ctx != nullptr) return false;
   int dev = 0;
   return cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && encode();
+}
+
+uint64_t current_context_id() {
+  unsigned long long id = 0;
+  const DriverFns& fns = driver_fns();
+  return fns.id != nullptr && fns.id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+bool primary_context_is_current() {
+  const DriverFns& f = driver_fns();
+  if (f.current == nullptr || f.device == nullptr || f.primary_state == nullptr || f.primary_retain == nullptr || f.primary_release == nullptr)
+    return false;
+  CUcontext ctx = nullptr, primary = nullptr;
+  CUdevice dev = 0;
+  unsigned int flags = 0;
+  int active = 0;
+  if (f.current(&ctx) != CUDA_SUCCESS || ctx == nullptr || f.device(&dev) != CUDA_SUCCESS) return false;
+  // (asked first: retaining one that is not there would make it)
+  if (f.primary_state(dev, &flags, &active) != CUDA_SUCCESS || active == 0 || f.primary_retain(&primary, dev) != CUDA_SUCCESS) return false;
+  f.primary_release(dev);
+  return primary == ctx;
 }
 
 bool device_is_sm100() {

@@ -124,6 +124,11 @@ bool encode_bf16_tile_map(CUtensorMap* map, const void* ptr, int B, int H, int N
 // True when the current device is compute capability 10.x.
 bool device_is_sm100();
 
+// Id of the current context, unique for the life of the program; 0 where there is none yet.
+uint64_t current_context_id();
+// Whether that is its device's primary context: others may have a part of the SMs only.
+bool primary_context_is_current();
+
 // Grid size of the persistent kernels: one CTA per SM of the current device, at most one per work item.
 int persistent_grid(long long items);
 

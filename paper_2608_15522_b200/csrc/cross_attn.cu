@@ -674,8 +674,6 @@ struct CrossPlan {
   size_t off_part_o, off_part_lse, off_lse, off_lse2, off_partial, off_redo, off_cta, total;
 };
 
-// How many clusters of `slices` CTAs the current device runs side by side (asked once per device: it depends on the sizes of its GPCs);
-// none where it cannot say.
 template <int D, bool SCORES>
 static cudaError_t allow_sliced() {
   auto kernel = cross_sliced_kernel<D, SCORES>;
@@ -683,16 +681,15 @@ static cudaError_t allow_sliced() {
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SlicedSmem<D>::kTotal);
   return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
-template <int D, bool SCORES>
+// How many clusters of `slices` CTAs the device runs side by side (it depends on the sizes of its GPCs).  None where it cannot say, and
+// in any context but the device's primary one, which may have too few SMs of a GPC for a cluster.  Asked once per context.
+template <int D>
 static int sliced_clusters(int slices) {
-  constexpr int kDevices = 64;
-  static std::atomic<int> known[kDevices][kSlicedMaxSlices + 1];      // one more than the number; 0: not asked yet
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-  if (dev >= 0 && dev < kDevices) {
-    const int k = known[dev][slices].load(std::memory_order_relaxed);
-    if (k > 0) return k - 1;
-  }
+  constexpr int kContexts = 64;      // (more of them than that ask again)
+  static std::atomic<uint64_t> known[kContexts][kSlicedMaxSlices + 1];      // context (its id, not 0) << 16 | number
+  uint64_t ctx = current_context_id();
+  const uint64_t k = known[ctx % kContexts][slices].load(std::memory_order_relaxed);
+  if (ctx != 0 && k >> 16 == ctx) return static_cast<int>(k & 0xffff);
   int n = 0;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -703,12 +700,16 @@ static int sliced_clusters(int slices) {
   cfg.dynamicSmemBytes = SlicedSmem<D>::kTotal;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (dev < 0 || allow_sliced<D, SCORES>() != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, cross_sliced_kernel<D, SCORES>, &cfg) != cudaSuccess) {
+  // (the attribute first: it makes the primary context current in a thread that has none)
+  if (allow_sliced<D, true>() != cudaSuccess) {
     cudaGetLastError();
-    return 0;
+  } else if (primary_context_is_current() && cudaOccupancyMaxActiveClusters(&n, cross_sliced_kernel<D, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();      // (no failure of the call, which takes the other way)
+    n = 0;
   }
-  if (dev < kDevices) known[dev][slices].store(n + 1, std::memory_order_relaxed);
+  n = std::min(n, persistent_grid(1 << 30) / slices);      // (what the workspace is sized for; a CTA takes an SM)
+  ctx = current_context_id();
+  if (ctx != 0) known[ctx % kContexts][slices].store(ctx << 16 | static_cast<uint64_t>(n), std::memory_order_relaxed);
   return n;
 }
 // Query tiles that a sliced call takes at most: as many clusters as run side by side.  us with scores, the two passes / sliced, 100
@@ -716,11 +717,13 @@ static int sliced_clusters(int slices) {
 // 12.2, 18 20.9 / 22.1, 35 25.2 / 32.8; 7 of 16 21.1 / 14.4, 8 21.3 / 25.1.  Without scores the one pass of before is as short where
 // two slices fill the SMs with tiles of 128 channels (32 tiles 10.8 / 10.8, 74 11.0 / 12.6; 64 channels 10.2 / 9.3; 32 tiles of 4 15.3 / 11.8).
 static long long max_sliced_tiles(int slices, int d, bool scores) {
-  const int n = d == 128 ? (scores ? sliced_clusters<128, true>(slices) : sliced_clusters<128, false>(slices))
-                         : (scores ? sliced_clusters<64, true>(slices) : sliced_clusters<64, false>(slices));
+  const int n = d == 128 ? sliced_clusters<128>(slices) : sliced_clusters<64>(slices);
   return slices == 2 && d == 128 && !scores && n > 32 ? 32 : n;
 }
-static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool scores, bool may_slice) {
+static int cross_slices(int Nk) { return (Nk + kSlicedKeys - 1) / kSlicedKeys; }
+static bool may_slice(int Nq, int Nk) { return Nk > kResMaxKeys && Nk <= kSlicedMaxSlices * kSlicedKeys && Nq <= kSlicedMaxQueries; }
+// `sliced_tiles`: with how many query tiles at most the call may be sliced
+static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, long long sliced_tiles) {
   CrossPlan c = {};
   // Few keys: everything in one kernel, whatever the number of queries (faster from 2 heads x 32 queries to 64 x 19200, with scores
   // and without: cross_resident.cuh).  More than 256 keys of 128 channels do not fit an SM's shared memory beside the tiles, nor
@@ -743,11 +746,10 @@ static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, bool score
     c.total = off;
     return c;
   }
-  const int slices = (Nk + kSlicedKeys - 1) / kSlicedKeys;
-  if (may_slice && slices <= kSlicedMaxSlices && Nq <= kSlicedMaxQueries && tiles <= max_sliced_tiles(slices, d, scores)) {
-    c.slices = slices;
+  if (tiles <= sliced_tiles) {
+    c.slices = cross_slices(Nk);
     c.NQT = (Nq + 127) / 128;
-    c.res_ctas = static_cast<int>(tiles) * slices;
+    c.res_ctas = static_cast<int>(tiles) * c.slices;
     size_t off = kStatusBytes;
     c.off_cta = off; off += align_up(static_cast<size_t>(c.res_ctas) * sizeof(CtaStatus), 256);
     c.off_partial = off; off += align_up(static_cast<size_t>(tiles) * Nk * sizeof(float), 256);
@@ -1057,10 +1059,9 @@ using namespace avsa;
 
 extern "C" size_t avsa_cross_attn_scores_workspace_bytes(int B, int H, int Nq, int Nk, int d) {
   if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128) || !pairs_ok(B, H)) return 0;
-  // what any call of this shape may take: with scores and without, sliced and not
-  const size_t with = make_cross_plan(B, H, Nq, Nk, d, true, true).total, without = make_cross_plan(B, H, Nq, Nk, d, false, true).total;
-  const size_t unsliced = make_cross_plan(B, H, Nq, Nk, d, true, false).total;
-  return std::max({with, without, unsliced});
+  // What any call of this shape may take, sliced or not, whatever context it is made in: a cluster has an SM a CTA.
+  const size_t sliced = make_cross_plan(B, H, Nq, Nk, d, may_slice(Nq, Nk) ? persistent_grid(1 << 30) / cross_slices(Nk) : 0).total;
+  return std::max(sliced, make_cross_plan(B, H, Nq, Nk, d, 0).total);
 }
 
 extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_bf16_4d q, avsa_bf16_4d k,
@@ -1076,7 +1077,8 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (o_bf16 != nullptr && !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
   // (a workspace that is not aligned for the slices' parts of O takes the two passes, which write none where no row is cut)
-  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, scores != nullptr, ws_aligned(ws, kWsParts));
+  const bool slice = may_slice(Nq, Nk) && ws_aligned(ws, kWsParts);
+  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, slice ? max_sliced_tiles(cross_slices(Nk), d, scores != nullptr) : 0);
   if (ws == nullptr || ws_bytes < c.total) return AVSA_ERR_WORKSPACE;
   const size_t widest = c.resident || c.slices > 0 ? kWsInts : !c.rs.whole_rows() ? kWsParts : scores != nullptr && c.reverse ? kWsVectors : kWsInts;
   if (!ws_aligned(ws, widest)) return AVSA_ERR_INVALID_ARG;

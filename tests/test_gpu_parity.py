@@ -6,6 +6,10 @@ grid itself is coarser than 1e-2 there).  fp32 log-sum-exps: max-abs 1e-3, unsca
 (Eq. 2): every element within 1e-3 of its own value (plus 1e-6 of the largest score), so that a few wrong
 columns cannot hide in a norm.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -16,6 +20,8 @@ from paper_2608_15522_b200 import workloads as wl
 from parity_bars import close_lse as _close_lse, close_o as _close, close_scores as _close_scores, np64 as _np64
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
 
 def _status_ok(ws):
     code, detail = av.avsa_read_status(ws)
@@ -1147,6 +1153,31 @@ def test_host_side_argument_errors():
 
 
 # ------------------------------------------------------------------------------------------- caller-owned scratch
+def test_workspace_sizes_are_the_same_wherever_they_are_asked():
+    """How short cross-attention runs depends on what the device can hold; its workspace does not: the sizes are those of a process
+    that sees no device, every call of the shape is content with them, and asking makes no context on the device."""
+    shapes = [(1, 8, 72, 2048, 128), (1, 24, 109, 1100, 128), (2, 3, 140, 333, 64), (1, 48, 100, 400, 128), (1, 74, 128, 512, 128), (1, 7, 128, 4096, 128),
+              (1, 9, 128, 4096, 128), (1, 2, 72, 300, 128), (1, 24, 256, 32760, 128)]
+    code = f"""if True:
+        import ctypes
+        from paper_2608_15522_b200 import binding as av
+        print([av.avsa_cross_attn_scores_workspace_bytes(*s) for s in {shapes}])
+        cu, flags, active = ctypes.CDLL("libcuda.so.1"), ctypes.c_uint(), ctypes.c_int()
+        assert cu.cuInit(0) != 0 or cu.cuDevicePrimaryCtxGetState(0, ctypes.byref(flags), ctypes.byref(active)) == 0
+        assert active.value == 0, "a context was made"
+    """
+    seen = []
+    for env in ({}, {"CUDA_VISIBLE_DEVICES": ""}):
+        r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env={**os.environ, **env}, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        assert r.returncode == 0, r.stdout
+        seen.append(r.stdout.strip())
+    assert seen[0] == seen[1] == str([av.avsa_cross_attn_scores_workspace_bytes(*s) for s in shapes])
+    for (B, H, Nq, Nk, d), n in zip(shapes, eval(seen[0])):
+        q, k = (torch.zeros((B, H, x, d), dtype=torch.bfloat16, device="cuda") for x in (Nq, Nk))
+        for scores in (True, False):
+            _status_ok(av.avsa_cross_attn_scores(q, k, k, want_scores=scores, ws=torch.empty(n, dtype=torch.uint8, device="cuda"))[3])
+
+
 @pytest.mark.parametrize("offset", [4, 16])
 def test_workspaces_cut_out_of_an_arena(offset):
     """Workspaces at 4 and 16 bytes from an aligned address: the bits of the aligned call, or refused where wider accesses are made.  Short
