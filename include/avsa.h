@@ -113,7 +113,8 @@ typedef struct {
  * softmax_scale == 0 means 1/sqrt(d).  When scores are requested min(Nq, Nk) <= 512 (the score pass keeps the
  * shorter axis of a head on chip: the audio queries, or, in the reverse video->audio direction of the
  * bidirectional pair, the audio keys); without scores any Nq and Nk.  The head sum is taken in a fixed order, so
- * results reproduce bit for bit.  `o` has strides (o_stride_b, o_stride_h, o_stride_n) = q's.
+ * results reproduce bit for bit, and o and lse are the same bits with scores and without.  `o` has strides
+ * (o_stride_b, o_stride_h, o_stride_n) = q's.
  */
 AVSA_API int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_bf16_4d q, avsa_bf16_4d k, avsa_bf16_4d v,
                            void* o_bf16, float* lse, float* scores, float score_beta, float score_gamma,

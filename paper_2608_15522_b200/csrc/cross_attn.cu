@@ -712,16 +712,23 @@ static int sliced_clusters(int slices) {
   if (ctx != 0) known[ctx % kContexts][slices].store(ctx << 16 | static_cast<uint64_t>(n), std::memory_order_relaxed);
   return n;
 }
+static int cross_slices(int Nk) { return (Nk + kSlicedKeys - 1) / kSlicedKeys; }
 // Query tiles that a sliced call takes at most: as many clusters as run side by side.  us with scores, the two passes / sliced, 100
 // queries, 128 channels: 16 tiles of 2 slices 17.2 / 11.6, 74 19.6 / 13.7, 85 21.4 / 22.8; 24 of 5 20.9 / 12.8, 28 21.4 / 21.8; 14 of 8 20.3 /
-// 12.2, 18 20.9 / 22.1, 35 25.2 / 32.8; 7 of 16 21.1 / 14.4, 8 21.3 / 25.1.  Without scores the one pass of before is as short where
-// two slices fill the SMs with tiles of 128 channels (32 tiles 10.8 / 10.8, 74 11.0 / 12.6; 64 channels 10.2 / 9.3; 32 tiles of 4 15.3 / 11.8).
-static long long max_sliced_tiles(int slices, int d, bool scores) {
-  const int n = d == 128 ? sliced_clusters<128>(slices) : sliced_clusters<64>(slices);
-  return slices == 2 && d == 128 && !scores && n > 32 ? 32 : n;
+// 12.2, 18 20.9 / 22.1, 35 25.2 / 32.8; 7 of 16 21.1 / 14.4, 8 21.3 / 25.1.
+static long long max_sliced_tiles(int slices, int d) { return d == 128 ? sliced_clusters<128>(slices) : sliced_clusters<64>(slices); }
+// Whether a call of these sizes may be sliced at all.  Not by whether it wants scores: with and without them O and the LSE are the same
+// bits.  Without scores the other way is one pass, the shorter the fewer the keys, while the slices' parts of O cost by the row: two and
+// three slices of 128 channels, and a second slice of hardly any keys, are kept to rows with which that call loses nothing.  us without scores,
+// one pass / sliced, tiles of 128 rows: 128 channels, 257 keys: 16 tiles 10.4 / 10.5, 32 10.5 / 11.1, 74 10.9 / 13.4 (with scores 20 / 13.9); 300: 20
+// 10.5 / 9.8, 32 10.4 / 10.6, 48 10.5 / 11.4; 400: 36 11.1 / 10.7, 44 11.1 / 11.4, 74 11.4 / 12.8; 640, three slices: 32 11.6 / 11.0, 44 11.6 / 12.1; four
+// always gain (800: 30 13.2 / 11.6).  64 channels, 257 keys: 48 11.1 / 9.7, 60 9.8 / 10.0, 74 10.0 / 10.7; 300: 74 10.0 / 9.9.
+static bool may_slice(int B, int H, int Nq, int Nk, int d) {
+  if (Nk <= kResMaxKeys || Nk > kSlicedMaxSlices * kSlicedKeys || Nq > kSlicedMaxQueries) return false;
+  const long long rows = static_cast<long long>(B) * H * Nq;
+  if (Nk <= kResMaxKeys + 32) return rows <= (d == 128 ? 2048 : 6144);
+  return d != 128 || cross_slices(Nk) > 3 || rows <= (Nk <= 384 ? 4096 : 4608);
 }
-static int cross_slices(int Nk) { return (Nk + kSlicedKeys - 1) / kSlicedKeys; }
-static bool may_slice(int Nq, int Nk) { return Nk > kResMaxKeys && Nk <= kSlicedMaxSlices * kSlicedKeys && Nq <= kSlicedMaxQueries; }
 // `sliced_tiles`: with how many query tiles at most the call may be sliced
 static CrossPlan make_cross_plan(int B, int H, int Nq, int Nk, int d, long long sliced_tiles) {
   CrossPlan c = {};
@@ -1060,7 +1067,7 @@ using namespace avsa;
 extern "C" size_t avsa_cross_attn_scores_workspace_bytes(int B, int H, int Nq, int Nk, int d) {
   if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || (d != 64 && d != 128) || !pairs_ok(B, H)) return 0;
   // What any call of this shape may take, sliced or not, whatever context it is made in: a cluster has an SM a CTA.
-  const size_t sliced = make_cross_plan(B, H, Nq, Nk, d, may_slice(Nq, Nk) ? persistent_grid(1 << 30) / cross_slices(Nk) : 0).total;
+  const size_t sliced = make_cross_plan(B, H, Nq, Nk, d, may_slice(B, H, Nq, Nk, d) ? persistent_grid(1 << 30) / cross_slices(Nk) : 0).total;
   return std::max(sliced, make_cross_plan(B, H, Nq, Nk, d, 0).total);
 }
 
@@ -1077,8 +1084,8 @@ extern "C" int avsa_cross_attn_scores(int B, int H, int Nq, int Nk, int d, avsa_
   if (o_bf16 != nullptr && !aligned16(o_bf16)) return AVSA_ERR_INVALID_ARG;
   if (softmax_scale < 0.f || softmax_scale != softmax_scale) return AVSA_ERR_INVALID_ARG;
   // (a workspace that is not aligned for the slices' parts of O takes the two passes, which write none where no row is cut)
-  const bool slice = may_slice(Nq, Nk) && ws_aligned(ws, kWsParts);
-  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, slice ? max_sliced_tiles(cross_slices(Nk), d, scores != nullptr) : 0);
+  const bool slice = may_slice(B, H, Nq, Nk, d) && ws_aligned(ws, kWsParts);
+  const CrossPlan c = make_cross_plan(B, H, Nq, Nk, d, slice ? max_sliced_tiles(cross_slices(Nk), d) : 0);
   if (ws == nullptr || ws_bytes < c.total) return AVSA_ERR_WORKSPACE;
   const size_t widest = c.resident || c.slices > 0 ? kWsInts : !c.rs.whole_rows() ? kWsParts : scores != nullptr && c.reverse ? kWsVectors : kWsInts;
   if (!ws_aligned(ws, widest)) return AVSA_ERR_INVALID_ARG;

@@ -817,7 +817,7 @@ def test_cross_attention_reverse_direction(name):
     (1, 2, 72, 257, 128), (1, 3, 1, 288, 64), (1, 2, 127, 289, 128), (1, 72, 20, 512, 64), (1, 73, 20, 512, 64),      # two slices
     (1, 33, 60, 400, 128), (2, 3, 129, 513, 128), (1, 8, 512, 769, 64), (1, 24, 33, 1280, 128), (2, 5, 200, 1537, 64),
     (1, 14, 128, 2048, 128), (1, 20, 128, 2048, 128), (1, 3, 300, 2047, 64), (2, 4, 72, 2070, 128), (1, 2, 100, 4096, 64),
-    (1, 3, 40, 4003, 128), (1, 2, 100, 4097, 128)])
+    (1, 3, 40, 4003, 128), (1, 2, 100, 4097, 128), (1, 24, 157, 400, 128), (1, 32, 128, 400, 128), (1, 33, 128, 400, 128)])
 @pytest.mark.parametrize("growth", [0.0, 30.0, 90.0])
 def test_cross_attention_sliced_keys(B, H, Nq, Nk, d, growth):
     """Short calls against 257 to 4096 keys: a cluster of CTAs takes a query tile, each some of the keys.  Slices of four chunks of 32 keys
@@ -847,6 +847,7 @@ def test_cross_attention_sliced_keys(B, H, Nq, Nk, d, growth):
     _status_ok(ws2)
     _close(_np64(o2), want_o, "sliced O without scores")
     _close_lse(_np64(lse2), want_lse, "sliced lse without scores")
+    assert torch.equal(o2, o) and torch.equal(lse2, lse)
 
 
 @pytest.mark.parametrize("Nq,Nk,d", [(40, 333, 64), (40, 400, 128), (130, 700, 64), (72, 2048, 128)])
@@ -866,6 +867,21 @@ def test_cross_attention_sliced_keys_that_all_have_logits_of_minus_infinity(Nq, 
     _close(_np64(o), want_o, "masked keys O")
     _close_lse(_np64(lse), want_lse, "masked keys lse")
     _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "masked keys scores")
+
+
+@pytest.mark.parametrize("B,H,Nq,Nk,d", [
+    (1, 24, 157, 400, 128), (1, 74, 55, 512, 128), (1, 74, 128, 512, 128), (1, 20, 128, 257, 128), (1, 44, 128, 640, 128), (1, 60, 128, 257, 64),
+    (2, 4, 200, 1500, 64), (2, 3, 700, 100, 64), (1, 5, 700, 200, 128), (1, 4, 160, 6000, 128), (1, 6, 900, 300, 64)])
+def test_cross_attention_gives_the_same_rows_with_scores_and_without(B, H, Nq, Nk, d):
+    """The way a shape is computed does not depend on whether the response scores are wanted: sliced keys and the limits of that way, few
+    keys, two passes, the reverse direction."""
+    g = torch.Generator(device="cuda").manual_seed(Nk + Nq)
+    q, k, v = (torch.randn((B, H, n, d), generator=g, device="cuda").bfloat16() for n in (Nq, Nk, Nk))
+    o, lse, _, ws = av.avsa_cross_attn_scores(q, k, v)
+    o2, lse2, _, ws2 = av.avsa_cross_attn_scores(q, k, v, want_scores=False)
+    for x in (ws, ws2):
+        _status_ok(x)
+    assert torch.equal(o, o2) and torch.equal(lse, lse2)
 
 
 @pytest.mark.parametrize("reverse", [False, True])
