@@ -1,7 +1,7 @@
-// Whole calls for the wrappers of binding.py (below), and for their general way uninitialised tensors: torch.empty without the parsing of its Python arguments, which costs
-// twice what the allocation does (2.2 us a tensor; the audio branch's own mask and attention, called without buffers, make
-// eight of them in a pass of 40 us).  The same operators through the same dispatcher, caching allocator and current stream, and
-// as there without the interpreter lock: an allocation may wait for the GPU.
+// Whole calls for the wrappers of binding.py (below), and for their general way uninitialised tensors: torch.empty without the parsing
+// of its Python arguments, which costs twice what the allocation does (2.2 us a tensor; the audio branch's own mask and attention,
+// called without buffers, make eight of them in a pass of 40 us).  The same operators through the same dispatcher, caching allocator
+// and current stream, and as there without the interpreter lock: an allocation may wait for the GPU.
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
@@ -56,10 +56,11 @@ PyObject* py_empty_as(PyObject*, PyObject* like) {
 // ------------------------------------------------------------------------------------------------ whole calls
 // A wrapper's call in one step for what programs pass: plain tensors on a GPU, ints, floats.  Shapes, strides and pointers are read
 // from the tensors themselves instead of through a dozen Python attributes, what the caller did not bring is allocated here, and
-// the interpreter lock is free for allocations, workspace query and launches together.  Whatever is not as expected (another class,
-// type, rank, device, a missing tensor) is left to the general way with its errors: the function then returns None and has
-// done nothing.  (us: the audio branch's mask and attention without buffers 29.6 -> 21.8; the smallest layer-step, three calls with
-// buffers, on the host 21.4 -> 17.0.)
+// the interpreter lock is free for allocations, workspace query and launches together.  Arguments of another class (a subclass of a tensor,
+// an int for a float, no tensor where one has to be), and q, k or v of another type, rank, layout or kind of device, are left to the
+// general way with its errors: the function then returns None and has done nothing.  Of the other tensors nothing but the class
+// is looked at, as in the general way.  (us: the audio branch's mask and attention without buffers 29.6 -> 21.8; the smallest layer-step,
+// three calls with buffers, on the host 21.4 -> 17.0.)
 
 decltype(&avsa_cross_attn_scores) f_cross;
 decltype(&avsa_cross_attn_scores_workspace_bytes) f_cross_ws;
@@ -71,24 +72,44 @@ decltype(&avsa_protected_rows_attn) f_protected;
 decltype(&avsa_protected_rows_attn_workspace_bytes) f_protected_ws;
 PyObject* o_raw_stream;
 
-// A tensor argument: none, or one held for the length of the call (another thread may drop or change the caller's).
+// A tensor argument: none, or one held for the length of the call (another thread may drop the caller's).  Another thread may also
+// resize it or give it other data: where these are and how many is read once, with the interpreter lock, as are the sizes and
+// strides of q, k and v, and nothing is asked of the caller's tensors after that.
 struct Arg {
   at::Tensor t;
+  void* ptr = nullptr;
+  int64_t numel = 0;
   bool there() const { return t.defined(); }
-  void* ptr() const { return t.defined() ? t.data_ptr() : nullptr; }
+  void read() {
+    ptr = t.data_ptr();
+    numel = t.numel();
+  }
 };
 bool take(PyObject* o, Arg& a, bool optional) {
   if (o == Py_None) return optional;
   if (!THPVariable_CheckExact(o)) return false;
   a.t = THPVariable_Unpack(o);
+  a.read();
   return true;
 }
 // bf16 [B,H,N,d] on a GPU with a contiguous head dimension
-bool is_view(const Arg& a) {
-  return a.there() && a.t.is_cuda() && a.t.scalar_type() == at::kBFloat16 && a.t.layout() == at::kStrided && a.t.dim() == 4 && a.t.stride(3) == 1;
+struct View : Arg {
+  int64_t size[4], stride[4];
+  operator avsa_bf16_4d() const { return avsa_bf16_4d{ptr, stride[0], stride[1], stride[2]}; }
+  int dim(int i) const { return static_cast<int>(size[i]); }
+};
+bool take_view(PyObject* o, View& a) {
+  if (!THPVariable_CheckExact(o)) return false;
+  const at::Tensor& t = THPVariable_Unpack(o);
+  if (!t.is_cuda() || t.scalar_type() != at::kBFloat16 || t.layout() != at::kStrided || t.dim() != 4 || t.stride(3) != 1) return false;
+  a.t = t;
+  a.read();
+  for (int i = 0; i < 4; i++) {
+    a.size[i] = t.size(i);
+    a.stride[i] = t.stride(i);
+  }
+  return true;
 }
-avsa_bf16_4d view(const Arg& a) { return avsa_bf16_4d{a.t.data_ptr(), a.t.stride(0), a.t.stride(1), a.t.stride(2)}; }
-bool take_view(PyObject* o, Arg& a) { return take(o, a, false) && is_view(a); }
 bool take_int(PyObject* o, int* out) {
   if (!PyLong_CheckExact(o)) return false;
   int overflow;
@@ -102,25 +123,31 @@ bool take_float(PyObject* o, float* out) {
   *out = static_cast<float>(PyFloat_AS_DOUBLE(o));
   return true;
 }
-// the current stream of the tensor's device
-void* stream_of(const Arg& a) {
-  THPObjectPtr index(PyLong_FromLong(a.t.get_device()));
-  if (!index) throw python_error();
-  THPObjectPtr raw(PyObject_CallOneArg(o_raw_stream, index.get()));
-  if (!raw) throw python_error();
-  void* p = PyLong_AsVoidPtr(raw.get());
-  if (p == nullptr && PyErr_Occurred()) throw python_error();
-  return p;
-}
-void make(Arg& a, const Arg& like, at::ScalarType type, at::IntArrayRef sizes) {
-  if (!a.there()) a.t = at::empty(sizes, at::TensorOptions().dtype(type).device(like.t.device()));
-}
-void make_as(Arg& a, const Arg& like) {
-  if (!a.there()) a.t = at::empty_strided(like.t.sizes(), like.t.strides(), at::TensorOptions().dtype(at::kBFloat16).device(like.t.device()));
-}
-void make_ws(Arg& a, const Arg& like, size_t bytes) {
-  make(a, like, at::kByte, {static_cast<int64_t>(bytes > 256 ? bytes : 256)});
-}
+// Where a call runs and what it allocates there: the device of q and its current stream.
+struct Place {
+  at::Device device;
+  void* stream;
+  explicit Place(const View& q) : device(q.t.device()), stream(nullptr) {
+    THPObjectPtr index(PyLong_FromLong(q.t.get_device()));
+    if (!index) throw python_error();
+    THPObjectPtr raw(PyObject_CallOneArg(o_raw_stream, index.get()));
+    if (!raw) throw python_error();
+    stream = PyLong_AsVoidPtr(raw.get());
+    if (stream == nullptr && PyErr_Occurred()) throw python_error();
+  }
+  at::TensorOptions options(at::ScalarType type) const { return at::TensorOptions().dtype(type).device(device); }
+  void make(Arg& a, at::ScalarType type, at::IntArrayRef sizes) const {      // what the caller did not bring
+    if (a.there()) return;
+    a.t = at::empty(sizes, options(type));
+    a.read();
+  }
+  void make_as(Arg& a, const View& like) const {
+    if (a.there()) return;
+    a.t = at::empty_strided(like.size, like.stride, options(at::kBFloat16));
+    a.read();
+  }
+  void make_ws(Arg& a, size_t bytes) const { make(a, at::kByte, {static_cast<int64_t>(bytes > 256 ? bytes : 256)}); }
+};
 // The caller's own object where there was one.
 PyObject* give(PyObject* given, Arg& a) { return given != Py_None ? Py_NewRef(given) : a.there() ? THPVariable_Wrap(a.t) : Py_NewRef(Py_None); }
 template <int N>
@@ -139,33 +166,33 @@ PyObject* result(int status, PyObject* (&items)[N]) {
   for (int i = 0; i < N; i++) PyTuple_SET_ITEM(r, i + 1, items[i]);
   return r;
 }
-int dim(const Arg& a, int i) { return static_cast<int>(a.t.size(i)); }
 
 // cross(q, k, v, scores, score_beta, score_gamma, softmax_scale, want_o, want_scores, o, lse, ws) -> (status, o, lse, scores, ws)
 PyObject* py_cross(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   TORCH_CHECK_TYPE(n == 12 && f_cross != nullptr, "wrong number of arguments, or bind() has not been called");
-  Arg q, k, v, scores, o, lse, ws;
+  View q, k, v;
+  Arg scores, o, lse, ws;
   float beta, gamma, scale;
   if (!PyBool_Check(a[7]) || !PyBool_Check(a[8]) || !take_view(a[0], q) || !take_view(a[1], k) || !take_view(a[2], v) ||
-      !take(a[3], scores, true) || !take_float(a[4], &beta) || !take_float(a[5], &gamma) || !take_float(a[6], &scale) ||
-      !take(a[9], o, true) || !take(a[10], lse, true) || !take(a[11], ws, true))
+      !take(a[8] == Py_True ? a[3] : Py_None, scores, true) || !take_float(a[4], &beta) || !take_float(a[5], &gamma) || !take_float(a[6], &scale) ||
+      !take(a[7] == Py_True ? a[9] : Py_None, o, true) || !take(a[10], lse, true) || !take(a[11], ws, true))
     Py_RETURN_NONE;
   const bool want_o = a[7] == Py_True, want_scores = a[8] == Py_True;
-  void* stream = stream_of(q);
-  const int B = dim(q, 0), H = dim(q, 1), Nq = dim(q, 2), Nk = dim(k, 2), d = dim(q, 3);
+  const Place place(q);
+  const int B = q.dim(0), H = q.dim(1), Nq = q.dim(2), Nk = k.dim(2), d = q.dim(3);
   int st;
   without_lock([&] {
-    if (want_o) make_as(o, q);
-    make(lse, q, at::kFloat, {B, H, Nq});
+    if (want_o) place.make_as(o, q);
+    place.make(lse, at::kFloat, {B, H, Nq});
     if (want_scores && !scores.there()) {
-      make(scores, q, at::kFloat, {B, Nk});
+      place.make(scores, at::kFloat, {B, Nk});
       beta = 0.f;
     }
-    if (!ws.there()) make_ws(ws, q, f_cross_ws(B, H, Nq, Nk, d));
-    st = f_cross(B, H, Nq, Nk, d, view(q), view(k), view(v), want_o ? o.ptr() : nullptr, static_cast<float*>(lse.ptr()),
-                 want_scores ? static_cast<float*>(scores.ptr()) : nullptr, beta, gamma, scale, ws.ptr(),
-                 static_cast<size_t>(ws.t.numel()), stream);
+    if (!ws.there()) place.make_ws(ws, f_cross_ws(B, H, Nq, Nk, d));
+    st = f_cross(B, H, Nq, Nk, d, q, k, v, want_o ? o.ptr : nullptr, static_cast<float*>(lse.ptr),
+                 want_scores ? static_cast<float*>(scores.ptr) : nullptr, beta, gamma, scale, ws.ptr,
+                 static_cast<size_t>(ws.numel), place.stream);
     return at::Tensor();
   });
   PyObject* items[] = {give(a[9], o), give(a[10], lse), give(a[3], scores), give(a[11], ws)};
@@ -178,27 +205,28 @@ PyObject* py_cross(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   TORCH_CHECK_TYPE(n == 14 && f_mask != nullptr, "wrong number of arguments, or bind() has not been called");
-  Arg q, k, scores, bs, idx, cnt, tok, pblk, ws;
+  View q, k;
+  Arg scores, bs, idx, cnt, tok, pblk, ws;
   int n_protect, k_keep, blk, flags;
   float scale;
   if (!take_view(a[0], q) || !take_view(a[1], k) || !take(a[2], scores, true) || !take_int(a[3], &n_protect) || !take_int(a[4], &k_keep) ||
       !take_int(a[5], &blk) || blk <= 0 || !take_int(a[6], &flags) || !take_float(a[7], &scale) || !take(a[8], bs, true) ||
       !take(a[9], idx, true) || !take(a[10], cnt, true) || !take(a[11], tok, true) || !take(a[12], pblk, true) || !take(a[13], ws, true))
     Py_RETURN_NONE;
-  void* stream = stream_of(q);
-  const int B = dim(q, 0), H = dim(q, 1), N = dim(q, 2), d = dim(q, 3);
+  const Place place(q);
+  const int B = q.dim(0), H = q.dim(1), N = q.dim(2), d = q.dim(3);
   const int64_t NB = (static_cast<int64_t>(N) + blk - 1) / blk;
   int st;
   without_lock([&] {
-    make(bs, q, at::kFloat, {B, H, NB, NB});
-    make(idx, q, at::kInt, {B, H, NB, NB});
-    make(cnt, q, at::kInt, {B, H, NB});
-    make(tok, q, at::kByte, {B, N});
-    make(pblk, q, at::kByte, {B, NB});
-    if (!ws.there()) make_ws(ws, q, f_mask_ws(B, H, N, d, blk));
-    st = f_mask(B, H, N, d, blk, view(q), view(k), static_cast<float*>(scores.ptr()), n_protect, k_keep, static_cast<unsigned>(flags), scale,
-                static_cast<float*>(bs.ptr()), static_cast<int32_t*>(idx.ptr()), static_cast<int32_t*>(cnt.ptr()),
-                static_cast<uint8_t*>(tok.ptr()), static_cast<uint8_t*>(pblk.ptr()), ws.ptr(), static_cast<size_t>(ws.t.numel()), stream);
+    place.make(bs, at::kFloat, {B, H, NB, NB});
+    place.make(idx, at::kInt, {B, H, NB, NB});
+    place.make(cnt, at::kInt, {B, H, NB});
+    place.make(tok, at::kByte, {B, N});
+    place.make(pblk, at::kByte, {B, NB});
+    if (!ws.there()) place.make_ws(ws, f_mask_ws(B, H, N, d, blk));
+    st = f_mask(B, H, N, d, blk, q, k, static_cast<float*>(scores.ptr), n_protect, k_keep, static_cast<unsigned>(flags), scale,
+                static_cast<float*>(bs.ptr), static_cast<int32_t*>(idx.ptr), static_cast<int32_t*>(cnt.ptr),
+                static_cast<uint8_t*>(tok.ptr), static_cast<uint8_t*>(pblk.ptr), ws.ptr, static_cast<size_t>(ws.numel), place.stream);
     return at::Tensor();
   });
   PyObject* items[] = {give(a[8], bs), give(a[9], idx), give(a[10], cnt), give(a[11], tok), give(a[12], pblk), give(a[13], ws)};
@@ -210,22 +238,23 @@ PyObject* py_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_sparse(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   TORCH_CHECK_TYPE(n == 11 && f_sparse != nullptr, "wrong number of arguments, or bind() has not been called");
-  Arg q, k, v, idx, cnt, o, lse, ws;
+  View q, k, v;
+  Arg idx, cnt, o, lse, ws;
   int blk;
   float scale;
   if (!PyBool_Check(a[7]) || !take_view(a[0], q) || !take_view(a[1], k) || !take_view(a[2], v) || !take(a[3], idx, false) ||
       !take(a[4], cnt, false) || !take_int(a[5], &blk) || !take_float(a[6], &scale) || !take(a[8], o, true) || !take(a[9], lse, true) ||
       !take(a[10], ws, true))
     Py_RETURN_NONE;
-  void* stream = stream_of(q);
-  const int B = dim(q, 0), H = dim(q, 1), N = dim(q, 2), d = dim(q, 3);
+  const Place place(q);
+  const int B = q.dim(0), H = q.dim(1), N = q.dim(2), d = q.dim(3);
   int st;
   without_lock([&] {
-    make_as(o, q);
-    if (a[7] == Py_True) make(lse, q, at::kFloat, {B, H, N});
-    if (!ws.there()) make_ws(ws, q, f_sparse_ws(B, H, N, d, blk));
-    st = f_sparse(B, H, N, d, blk, view(q), view(k), view(v), static_cast<int32_t*>(idx.ptr()), static_cast<int32_t*>(cnt.ptr()), o.ptr(),
-                  static_cast<float*>(lse.ptr()), scale, ws.ptr(), static_cast<size_t>(ws.t.numel()), stream);
+    place.make_as(o, q);
+    if (a[7] == Py_True) place.make(lse, at::kFloat, {B, H, N});
+    if (!ws.there()) place.make_ws(ws, f_sparse_ws(B, H, N, d, blk));
+    st = f_sparse(B, H, N, d, blk, q, k, v, static_cast<int32_t*>(idx.ptr), static_cast<int32_t*>(cnt.ptr), o.ptr,
+                  static_cast<float*>(lse.ptr), scale, ws.ptr, static_cast<size_t>(ws.numel), place.stream);
     return at::Tensor();
   });
   PyObject* items[] = {give(a[8], o), give(a[9], lse), give(a[10], ws)};
@@ -237,19 +266,20 @@ PyObject* py_sparse(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_protected(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   TORCH_CHECK_TYPE(n == 10 && f_protected != nullptr, "wrong number of arguments, or bind() has not been called");
-  Arg q, k, v, tok, o, lse, ws;
+  View q, k, v;
+  Arg tok, o, lse, ws;
   int n_protect, blk;
   float scale;
   if (!take_view(a[0], q) || !take_view(a[1], k) || !take_view(a[2], v) || !take(a[3], tok, false) || !take_int(a[4], &n_protect) ||
       !take_int(a[5], &blk) || !take(a[6], o, false) || !take(a[7], lse, true) || !take_float(a[8], &scale) || !take(a[9], ws, true))
     Py_RETURN_NONE;
-  void* stream = stream_of(q);
-  const int B = dim(q, 0), H = dim(q, 1), N = dim(q, 2), d = dim(q, 3);
+  const Place place(q);
+  const int B = q.dim(0), H = q.dim(1), N = q.dim(2), d = q.dim(3);
   int st;
   without_lock([&] {
-    if (!ws.there()) make_ws(ws, q, f_protected_ws(B, H, N, d, blk, n_protect));
-    st = f_protected(B, H, N, d, blk, view(q), view(k), view(v), static_cast<uint8_t*>(tok.ptr()), n_protect, o.ptr(),
-                     static_cast<float*>(lse.ptr()), scale, ws.ptr(), static_cast<size_t>(ws.t.numel()), stream);
+    if (!ws.there()) place.make_ws(ws, f_protected_ws(B, H, N, d, blk, n_protect));
+    st = f_protected(B, H, N, d, blk, q, k, v, static_cast<uint8_t*>(tok.ptr), n_protect, o.ptr,
+                     static_cast<float*>(lse.ptr), scale, ws.ptr, static_cast<size_t>(ws.numel), place.stream);
     return at::Tensor();
   });
   PyObject* items[] = {give(a[9], ws)};
