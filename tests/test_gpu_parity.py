@@ -629,6 +629,153 @@ def test_sparse_attention_pairs_of_64_blocks(case):
     _close_lse(_np64(lse), want_l, f"pairs {case} lse")
 
 
+def _random_lists(rng, B, H, NB, longest):
+    idx, cnt = np.full((B, H, NB, NB), -1, np.int32), np.zeros((B, H, NB), np.int32)
+    for at in np.ndindex(B, H, NB):
+        c = NB if rng.integers(12) == 0 and longest > 8 else 1 + int(rng.integers(longest))
+        idx[at][:c], cnt[at] = np.sort(rng.choice(NB, size=c, replace=False)), c
+    return idx, cnt
+
+
+def _runs_in_pairs(B, H, N):
+    """The workspace has room for the joint lists of two query blocks each."""
+    NB, up = (N + 63) // 64, lambda x: (x + 255) // 256 * 256
+    NP = (NB + 1) // 2
+    return av.avsa_sparse_self_attn_workspace_bytes(B, H, N, 64, 64) == 256 + up(B * H * NB * 8) + up(B * H * NP * (2 * NP + 1) * 4)
+
+
+@pytest.mark.parametrize("layout", ["bhnd", "bnhd", "padded"])
+def test_sparse_attention_pairs_in_batches_layouts_and_used_buffers(layout):
+    """Two batch items with lists of their own and an odd number of blocks, read through strides: the same bits as from contiguous tensors,
+    whatever workspace and outputs held before, launch by launch, and from a CUDA graph."""
+    B, H, NB, d = 2, 2, 67, 64
+    N = (NB - 1) * d + 9
+    assert _runs_in_pairs(B, H, N)
+    g = torch.Generator().manual_seed(8)
+    cpu = [torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3)]
+    idx, cnt = _random_lists(np.random.default_rng(5), B, H, NB, NB // 2)
+    idx_d, cnt_d = torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda()
+    want_o, want_lse, ws = av.avsa_sparse_self_attn(*(t.cuda() for t in cpu), idx_d, cnt_d, d, want_lse=True)
+    _status_ok(ws)
+    if layout == "bhnd":
+        ref_o, ref_lse = orc.masked_attention(*(_np64(t) for t in cpu), idx, cnt, d)
+        _close(_np64(want_o), ref_o, "pairs of two batch items O")
+        _close_lse(_np64(want_lse), ref_lse, "pairs of two batch items lse")
+
+    def store(t):
+        if layout == "bnhd":
+            return t.cuda().transpose(1, 2).contiguous().transpose(1, 2)
+        buf = torch.zeros(t.shape[:-1] + (d + (8 if layout == "padded" else 0),), dtype=t.dtype, device="cuda")
+        buf[..., :d] = t.cuda()
+        return buf[..., :d]
+    q, k, v = (store(t) for t in cpu)
+    n = av.avsa_sparse_self_attn_workspace_bytes(B, H, N, d, d)
+    for fill in (0x00, 0xFF):
+        ws = torch.full((n,), fill, dtype=torch.uint8, device="cuda")
+        o, lse = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device="cuda"), torch.empty((B, H, N), device="cuda")
+        for _ in range(3):
+            o.fill_(float(fill))
+            lse.fill_(float(fill))
+            av.avsa_sparse_self_attn(q, k, v, idx_d, cnt_d, d, o=o, lse=lse, ws=ws)
+            _status_ok(ws)
+            assert torch.equal(o, want_o) and torch.equal(lse, want_lse)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        av.avsa_sparse_self_attn(q, k, v, idx_d, cnt_d, d, o=o, lse=lse, ws=ws)
+    for _ in range(2):
+        o.zero_()
+        lse.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(o, want_o) and torch.equal(lse, want_lse)
+
+
+def test_sparse_attention_pairs_whose_blocks_both_outgrow_their_reference():
+    """Keys that grow from block to block for every row, in two batch items: both blocks of a pair are recomputed, each with its list."""
+    B, H, NB, d = 2, 3, 65, 64
+    N = NB * d
+    assert _runs_in_pairs(B, H, N)
+    g = torch.Generator().manual_seed(6)
+    q, k, v = (torch.randn((B, H, N, d), generator=g) for _ in range(3))
+    k[:, 1:] *= (1 + 3 * (torch.arange(N) // d))[None, None, :, None]      # (the first head's keys do not grow)
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    idx, cnt = _random_lists(np.random.default_rng(9), B, H, NB, 12)
+    o, lse, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), d, want_lse=True)
+    _status_ok(ws)
+    n_redo, items = av.avsa_sparse_self_attn_redo_items(ws)
+    assert n_redo > 0 and len(set(items.tolist())) == n_redo and np.all(cnt.reshape(-1)[items] > 1)
+    b, h, block = items // (H * NB), items // NB % H, items % NB
+    assert np.all(h > 0) and set(b.tolist()) == {0, 1}
+    assert len({(x, y, z // 2) for x, y, z in zip(b, h, block)}) < n_redo      # both of a pair, somewhere
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), idx, cnt, d)
+    _close(_np64(o), want, "pairs recomputed O")
+    _close_lse(_np64(lse), want_l, "pairs recomputed lse")
+
+
+@pytest.mark.parametrize("b,h,block,bad", [(1, 1, 66, "empty"), (1, 0, 5, "order"), (1, 1, 4, "range"), (0, 1, 7, "long")])
+def test_sparse_attention_pairs_with_a_malformed_list_in_either_batch_item(b, h, block, bad):
+    """The item that is reported is the query block's, its rows stay as they were, and its neighbour in the pair has its own list."""
+    B, H, NB, d = 2, 2, 67, 64
+    N = (NB - 1) * d + 9
+    assert _runs_in_pairs(B, H, N)
+    g = torch.Generator().manual_seed(7)
+    q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    idx, cnt = _random_lists(np.random.default_rng(3), B, H, NB, 7)
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), idx, cnt, d)
+    row = idx[b, h, block]
+    if bad == "order":
+        row[:2], cnt[b, h, block] = (9, 9), 2
+    elif bad == "range":
+        row[0], cnt[b, h, block] = NB, 1
+    else:
+        cnt[b, h, block] = 0 if bad == "empty" else NB + 1
+    want[b, h, block * d:(block + 1) * d] = want_l[b, h, block * d:(block + 1) * d] = 7.0
+    o, lse = torch.full((B, H, N, d), 7.0, dtype=torch.bfloat16, device="cuda"), torch.full((B, H, N), 7.0, device="cuda")
+    _, _, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), d, o=o, lse=lse)
+    code, detail = av.avsa_read_status(ws)
+    assert code == av.AVSA_ERR_BAD_MASK and detail[1:] == ((b * H + h) * NB + block, cnt[b, h, block])
+    _close(_np64(o), want, f"pairs, {bad} list O")
+    _close_lse(_np64(lse), want_l, f"pairs, {bad} list lse")
+
+
+@pytest.mark.parametrize("flags", [av.AVSA_PROTECT_ROWS, av.AVSA_PROTECT_ROWS | av.AVSA_PROTECT_COLS])
+def test_sparse_attention_pairs_under_the_masks_own_lists(flags):
+    """Mask and attention of 64-blocks with protected rows, and protected columns too."""
+    B, H, N, d = 2, 4, 70 * 64 + 9, 64
+    assert _runs_in_pairs(B, H, N)
+    g = torch.Generator().manual_seed(2)
+    q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    s = torch.rand((B, N), generator=g)
+    s[:, 1000:1400] += 1.0
+    m = av.avsa_build_block_mask(q.cuda(), k.cuda(), s.cuda(), 300, 7, d, flags=flags)
+    _status_ok(m["ws"])
+    o, lse, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), m["col_idx"], m["col_cnt"], d, want_lse=True)
+    _status_ok(ws)
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), m["col_idx"].cpu().numpy(), m["col_cnt"].cpu().numpy(), d)
+    _close(_np64(o), want, "pairs under a mask O")
+    _close_lse(_np64(lse), want_l, "pairs under a mask lse")
+
+
+def test_sparse_attention_pairs_of_more_than_two_windows_of_blocks():
+    """Lists are joined 1024 key blocks at a time: three windows, entries at their edges, the last pair a single block."""
+    B, H, NB, d = 1, 1, 2101, 64
+    N = (NB - 1) * d + 33
+    assert _runs_in_pairs(B, H, N)
+    g = torch.Generator().manual_seed(1)
+    q, k, v = (torch.randn((B, H, N, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    rng = np.random.default_rng(4)
+    idx, cnt = np.full((B, H, NB, NB), -1, np.int32), np.zeros((B, H, NB), np.int32)
+    for i in range(NB):
+        cols = np.union1d(rng.choice(NB, size=int(rng.integers(1, 4))), [[0, 1023, 1024], [2047, 2048], [1024, 2100], [2048], []][i % 5]).astype(np.int32)
+        idx[0, 0, i, :len(cols)], cnt[0, 0, i] = cols, len(cols)
+    o, lse, ws = av.avsa_sparse_self_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), d, want_lse=True)
+    _status_ok(ws)
+    want, want_l = orc.masked_attention(_np64(q), _np64(k), _np64(v), idx, cnt, d)
+    _close(_np64(o), want, "three windows O")
+    _close_lse(_np64(lse), want_l, "three windows lse")
+
+
 # ------------------------------------------------------------------------------------------- cross attention
 @pytest.mark.parametrize("name", ["tiny", "small128", "medium128"])
 def test_cross_attention_outputs_and_scores(name):
@@ -817,13 +964,13 @@ def test_cross_attention_reverse_direction(name):
     (1, 2, 72, 257, 128), (1, 3, 1, 288, 64), (1, 2, 127, 289, 128), (1, 72, 20, 512, 64), (1, 73, 20, 512, 64),      # two slices
     (1, 33, 60, 400, 128), (2, 3, 129, 513, 128), (1, 8, 512, 769, 64), (1, 24, 33, 1280, 128), (2, 5, 200, 1537, 64),
     (1, 14, 128, 2048, 128), (1, 20, 128, 2048, 128), (1, 3, 300, 2047, 64), (2, 4, 72, 2070, 128), (1, 2, 100, 4096, 64),
-    (1, 3, 40, 4003, 128), (1, 2, 100, 4097, 128), (1, 24, 157, 400, 128), (1, 32, 128, 400, 128), (1, 33, 128, 400, 128)])
+    (1, 3, 40, 4003, 128), (1, 2, 100, 4097, 128), (1, 24, 157, 400, 128), (1, 36, 128, 400, 128), (1, 37, 128, 400, 128)])
 @pytest.mark.parametrize("growth", [0.0, 30.0, 90.0])
 def test_cross_attention_sliced_keys(B, H, Nq, Nk, d, growth):
     """Short calls against 257 to 4096 keys: a cluster of CTAs takes a query tile, each some of the keys.  Slices of four chunks of 32 keys
-    and of eight, the last key alone in its chunk, several query tiles, as many clusters as run side by side and one more, the first
-    length beyond; logits that grow along the keys (base 2, per 128 keys), so that the reference changes inside a slice and from slice
-    to slice; [B,N,H,d] storage; with and without scores."""
+    and of eight, the last key alone in its chunk, several query tiles, the limits of that way and the first length beyond
+    (test_which_short_cross_attention_calls_slice_their_keys says which calls go it); logits that grow along the keys (base 2, per
+    128 keys), so that the reference changes inside a slice and from slice to slice; [B,N,H,d] storage; with and without scores."""
     g = torch.Generator().manual_seed(Nk + Nq)
     q, k, v = (torch.randn((B, H, n, d), generator=g) for n in (Nq, Nk, Nk))
     if growth:
@@ -867,6 +1014,46 @@ def test_cross_attention_sliced_keys_that_all_have_logits_of_minus_infinity(Nq, 
     _close(_np64(o), want_o, "masked keys O")
     _close_lse(_np64(lse), want_lse, "masked keys lse")
     _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * Nq)), "masked keys scores")
+
+
+def _went_sliced(B, H, Nq, Nk, d, **kw):
+    """Runs a call of this shape on random tensors and tells by its workspace whether a cluster took each query tile: then a record per
+    CTA begins behind the status record, all zeros where nothing went wrong."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn((B, H, n, d), generator=g, device="cuda").bfloat16() for n in (Nq, Nk, Nk))
+    ws = torch.full((av.avsa_cross_attn_scores_workspace_bytes(B, H, Nq, Nk, d),), 0xFF, dtype=torch.uint8, device="cuda")
+    av.avsa_cross_attn_scores(q, k, v, ws=ws, **kw)
+    _status_ok(ws)
+    ctas = B * H * ((Nq + 127) // 128) * ((Nk + 255) // 256)
+    return bool((ws[256:256 + 32 * ctas] == 0).all())
+
+
+@pytest.mark.parametrize("B,H,Nq,Nk,d,sliced", [
+    (1, 2, 72, 257, 128, True), (1, 3, 1, 288, 64, True), (1, 16, 128, 257, 128, True), (1, 17, 128, 257, 128, False), (1, 49, 128, 257, 64, False),
+    (1, 32, 128, 300, 128, True), (1, 33, 128, 300, 128, False), (1, 36, 128, 400, 128, True), (1, 37, 128, 400, 128, False), (1, 24, 157, 400, 128, True),
+    (1, 72, 20, 512, 64, True), (1, 36, 128, 640, 128, True), (1, 37, 128, 640, 128, False), (1, 24, 33, 1280, 128, True), (2, 4, 72, 2070, 128, True),
+    (1, 2, 100, 4096, 64, True), (1, 2, 100, 4097, 128, False), (1, 2, 513, 400, 128, False), (1, 80, 20, 512, 64, False), (1, 20, 128, 2048, 128, False)])
+def test_which_short_cross_attention_calls_slice_their_keys(B, H, Nq, Nk, d, sliced):
+    """The limits of the sliced way on both sides, and its parity shapes: the tests that mean it reach it."""
+    assert _went_sliced(B, H, Nq, Nk, d) == sliced
+    assert _went_sliced(B, H, Nq, Nk, d, want_scores=False) == sliced
+
+
+@pytest.mark.parametrize("Nk,d", [(1100, 64), (2048, 128), (4000, 128)])
+def test_cross_attention_with_as_many_clusters_as_run_and_one_more(Nk, d):
+    """The last number of query tiles that the device's clusters hold side by side, and the next: both against the oracle."""
+    slices = (Nk + 255) // 256
+    heads = next(h for h in range(1, 148 // slices + 2) if not _went_sliced(1, h, 128, Nk, d)) - 1
+    assert heads >= 148 // slices // 2
+    for H in (heads, heads + 1):
+        g = torch.Generator().manual_seed(H)
+        q, k, v = (torch.randn((1, H, n, d), generator=g).to(torch.bfloat16) for n in (128, Nk, Nk))
+        o, lse, s, ws = av.avsa_cross_attn_scores(q.cuda(), k.cuda(), v.cuda(), score_gamma=1.0 / (H * 128))
+        _status_ok(ws)
+        want_o, want_lse, A = orc.cross_attention(_np64(q), _np64(k), _np64(v))
+        _close(_np64(o), want_o, "clusters O")
+        _close_lse(_np64(lse), want_lse, "clusters lse")
+        _close_scores(_np64(s), orc.column_scores(A, gamma=1.0 / (H * 128)), "clusters scores")
 
 
 @pytest.mark.parametrize("B,H,Nq,Nk,d", [
