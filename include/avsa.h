@@ -32,9 +32,9 @@
  *     a kernel that normalises each row by the maximum of its first key tile instead of a running maximum
  *     (softmax is invariant to that shift), and recompute with exact rescaling the work items whose rows outgrew
  *     that reference (a row whose sum of exp(logit - reference) ends above 2^64 or not finite): in the same kernel
- *     in short calls, in one behind it in long ones (of query blocks of 64 rows also those with an output that is
- *     not finite).  Results do not depend on which way produced them beyond
- *     rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).  Cross-attention in short calls
+ *     in short calls, in one behind it in long ones (with 64 channels and many blocks, where two query blocks are run
+ *     at a time, also those with an output that is not finite).  Results do not depend on which way produced them
+ *     beyond rounding; the int32 at byte 16 of ws counts the recomputed items (diagnostic).  Cross-attention in short calls
  *     against at most 4096 keys recomputes nothing (every part of a row takes its own maximum), nor does it
  *     against at most 256 keys: there a row whose keys from 128 on outgrow the maximum of the first 128 by more
  *     than 2^57 (as factors of exp) takes a larger reference on the way, and the int32 counts the tiles of 128

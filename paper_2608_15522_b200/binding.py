@@ -363,9 +363,9 @@ def avsa_sparse_self_attn(q, k, v, col_idx, col_cnt, blk, softmax_scale=0.0, wan
 
 def avsa_redo_count(ws: torch.Tensor) -> int:
     """Diagnostic: number of work items that the last attention call on this workspace (sparse self-attention,
-    cross-attention pass 1, protected rows) recomputed with the exact-rescaling kernel.  Cross-attention against at most 256
-    keys has none: there it is the number of query tiles with a row whose keys from 128 on outgrew the first ones' maximum by
-    more than 2^64."""
+    cross-attention pass 1, protected rows) recomputed with the exact-rescaling kernel.  Cross-attention in short calls
+    against at most 4096 keys has none, nor has it against at most 256 keys: there it is the number of query tiles with a
+    row whose keys from 128 on outgrew the first ones' maximum by more than 2^64."""
     torch.cuda.synchronize(ws.device)
     return int(ws[16:20].view(torch.int32).item())
 

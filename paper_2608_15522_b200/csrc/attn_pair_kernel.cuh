@@ -12,7 +12,7 @@
 // piece of a tile to do or nothing.  With the MMA side at half the work of 128 channels the softmax warps set the pace, and four of them
 // on an SM's quarter hide each other's latencies where two do not (4 heads x 296 blocks, us: lists of all blocks 580 with eight
 // softmax warps, 505 with sixteen (XU pipe 63 and 76 % busy); of half the blocks, drawn at random, 354 and 309, and 554 as items of 64
-// rows).  Not in two versions of the loop (with and without a quarter to leave out): then these warps wait for instructions, 458.
+// rows; in a loop of 40 calls on a cool chip 458 and 312, as items of 64 rows 1098 and 560).  Not in two versions of the loop (with and without a quarter to leave out): then these warps wait for instructions, 458.
 //
 // P = 0 does not keep a value of V that is no number out of a row whose list leaves it out: a row that ends non-finite goes to
 // the redo list too, whose kernel takes every query block with its own list.

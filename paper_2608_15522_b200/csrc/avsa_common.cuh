@@ -19,7 +19,8 @@ struct StatusRecord {
   int item;       // work item (block index)
   int aux;        // tile index or offending value
   int redo_count; // attention calls: work items whose rows outgrew their reference and were recomputed exactly (cross-attention
-                  // against at most 256 keys: query tiles in which the keys from 128 on outgrew the first ones' maximum by 2^64)
+                  // against at most 256 keys: query tiles in which the keys from 128 on outgrew the first ones' maximum by 2^64;
+                  // against up to 4096 in short calls: none)
   int next_item;  // attention calls: head of the work queue of the persistent kernel
 };
 constexpr size_t kStatusBytes = 256;   // the record, padded so that what follows stays 256-byte aligned
@@ -47,8 +48,8 @@ __device__ __forceinline__ void report_status(StatusRecord* st, int code, int wh
 //   - score_select_kernel lets its successor go before it waits itself: the successor must wait before it touches
 //     anything (every first kernel of a call and expand_blocks_kernel do);
 //   - indicators_finalize_kernel reads the saliencies before its wait; l1_partials_kernel in front of it goes by the rule;
-//   - colsum_kernel, colsum_rev_kernel, cross_resident_kernel and cross_sliced_kernel let their successor go at their end only (the reason stands
-//     at the first).
+//   - colsum_kernel, colsum_rev_kernel, cross_resident_kernel and cross_sliced_kernel let their successor go at their end only
+//     (the reason stands at the first).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -716,6 +716,10 @@ static int cross_slices(int Nk) { return (Nk + kSlicedKeys - 1) / kSlicedKeys; }
 // Query tiles that a sliced call takes at most: as many clusters as run side by side.  us with scores, the two passes / sliced, 100
 // queries, 128 channels: 16 tiles of 2 slices 17.2 / 11.6, 74 19.6 / 13.7, 85 21.4 / 22.8; 24 of 5 20.9 / 12.8, 28 21.4 / 21.8; 14 of 8 20.3 /
 // 12.2, 18 20.9 / 22.1, 35 25.2 / 32.8; 7 of 16 21.1 / 14.4, 8 21.3 / 25.1.
+//   A cluster starts when as many SMs of one GPC as it has CTAs are free at the same time.  us of a call by itself, with its launches, while
+// another stream's kernel holds 0 / 16 / 32 / 48 / 64 / 96 / 120 SMs (the two passes): 7 tiles of 16 slices 26 / 26 / 48 / 49 and from 64 on not before
+// that kernel ends (35 / 35 / 35 / 47 / 47 / 60 / 73); 14 of 8 23 / 24 / 32 / 34 / 33 / 64, with 120 not before it ends (34 / 34 / 34 / 47 / 47 / 59 / 73);
+// 24 of 5 22 / 22 / 32 / 34 / 33 / 44 / 91 (38 / 38 / 42 / 49 / 50 / 60 / 83).
 static long long max_sliced_tiles(int slices, int d) { return d == 128 ? sliced_clusters<128>(slices) : sliced_clusters<64>(slices); }
 // Whether a call of these sizes may be sliced at all.  Not by whether it wants scores: with and without them O and the LSE are the same
 // bits.  Without scores the other way is one pass, the shorter the fewer the keys, while the slices' parts of O cost by the row: two and

@@ -6,7 +6,8 @@
 // column sums take it from tensor memory as in cross_resident.cuh, and O leaves as fp32 in proportion, for sliced_finalize_kernel to
 // add the slices.  So a call is two launches instead of four (status, attention, score pass, sums and merge), computes every exponential
 // once, and nothing in it is longer than a tile: bound by the latencies of that.  us: 8 heads x 72 queries x 2048 keys 19.6 -> 12.2, 2 x 72 x 300
-// 15.7 -> 10.3, 24 x 109 x 1100 24.0 -> 12.8.  (One part of a whole CTA's keys, with the reference and the sums exchanged between its groups, as in
+// 15.7 -> 10.3, 24 x 109 x 1100 24.0 -> 12.8; with the clamp that lets a half weigh nothing whose logits are all -inf, 0.1-0.3 more with scores and 128
+// channels (16 x 100 x 300 11.43 -> 11.56, 4 x 100 x 4096 14.39 -> 14.61: the exponentials are short of registers).  (One part of a whole CTA's keys, with the reference and the sums exchanged between its groups, as in
 // cross_resident.cuh: 12.5, 10.2, 13.0, without scores 10.5 against 9.5 (24 x 99 x 420), and O 3 % further from 64 bits, whose
 // largest probability of every 128 keys is exact here.)
 //

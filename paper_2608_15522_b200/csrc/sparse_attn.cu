@@ -206,6 +206,11 @@ __global__ void __launch_bounds__(32) bounded_wait_selftest_kernel(StatusRecord*
 // 10 % drawn at random, of 25 % with a third of the rows dense, of all blocks: 148 items of 148 blocks 15 / 23, 76 / 72, 77 / 73; 180 of
 // 90 18 / 19, 51 / 50, 92 / 51; 592 of 148 39 / 33, 166 / 129, 281 / 132; 888 of 37 24 / 27, 69 / 58, 116 / 81; 396 of 33, the mask's own lists of
 // 10 %, 16 / 19; 288 of 24 12 / 14, 26 / 25, 33 / 26.
+//   What decides is how much two lists share and how full the pairs leave their last wave; the rule sees sizes alone.  Thirty sizes from
+// 180 items on, lists of the mask's kind, gain: 5 % of the tokens protected 1.10-2.14 x (10, 25 and 50 % kept), none protected and 25 or 50 % kept
+// 0.94-1.80, 10 % kept 0.88-1.45.  Below 1 there are twelve of the thirty, all between 192 and 888 items (0.88 with 592 items of 37 blocks and 608 of
+// 32, which are 2.05 pairs a CTA); lists of 10 % drawn at random lose up to 18 % at the same sizes.  From 1152 items on (8 a CTA) none lost
+// anything.  To start there would give away the first figures at all the sizes below.
 static bool runs_pairs(int B, int H, int d, int NB) {
   const long long items = static_cast<long long>(B) * H * NB;
   return d == 64 && (NB >= 64 ? persistent_grid(items) < items : NB >= 32 && items >= 4ll * persistent_grid(items));
